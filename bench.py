@@ -979,7 +979,7 @@ def run_small(args):
         "host_us_per_call": {"verify": us_verify_host, "commit": us_commit_host,
                              "note": "wall time of one call on the host (Python binding + C entry point: argument checks, tensor maps, "
                                      "launches), GPU idle beforehand"},
-        "gpu_launches": (3 if chain and args.route == 1 else 4) * K,
+        "gpu_launches": (3 if args.route == 0 or (chain and args.route == 1) else 4) * K,
         "clocks": clocks,
     }
     print(json.dumps(out))

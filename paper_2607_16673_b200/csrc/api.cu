@@ -77,6 +77,18 @@ int verify_common(const speca_dims *dims, const float *S0, const uint16_t *q, co
     if (dims->route == SPECA_ROUTE_EFFECTIVE && !effective_supported(dims)) return SPECA_ERR_UNSUPPORTED;
     const bool eff = dims->route == SPECA_ROUTE_EFFECTIVE || (tensor && !fact && effective_supported(dims));
     if (dims->route == SPECA_ROUTE_FACTORIZED && !fact && !eff) return SPECA_ERR_UNSUPPORTED;
+    // Small trees go to the kernel that streams the state through registers (its loads are 32 bytes wide); it needs no
+    // plan.  A chain longer than max_depth <= 16 is a fault that it reports itself.
+    if (dims->route == SPECA_ROUTE_AUTO && u == nullptr && (reinterpret_cast<uintptr_t>(S0) & 31u) == 0) {
+        int most = dims->max_nodes < total_nodes ? dims->max_nodes : total_nodes;
+        if (chain && most > dims->max_depth) most = dims->max_depth;
+        const int limit = direct_limit(p, dims->d_k, most, fact || eff);
+        if (limit > 0) {
+            rc = cuda_rc(launch_verify_direct(p, dims->d_k, most, limit, st));
+            if (rc != SPECA_OK || most <= limit) return rc;
+            p.skip_nodes = limit;
+        }
+    }
     if (!chain || fact || eff || tf32) {
         // with parent == NULL (chain entry point) the plan kernel assumes parent[i] = i - 1
         rc = cuda_rc(launch_plan(p, st));

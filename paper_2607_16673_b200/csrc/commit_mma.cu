@@ -260,21 +260,6 @@ commit_long_kernel(Params p)
 constexpr int kMinTilesPerWarp = 128;
 std::atomic<int> g_min_tiles_per_warp{kMinTilesPerWarp};
 
-// SM count per device (asked once per device)
-int sm_count_of_current_device()
-{
-    static std::atomic<int> cache[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    const bool cached = dev >= 0 && dev < 64;
-    int sms = cached ? cache[dev].load(std::memory_order_relaxed) : 0;
-    if (sms == 0) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-        if (cached) cache[dev].store(sms, std::memory_order_relaxed);
-    }
-    return sms;
-}
-
 }  // namespace
 
 // Shapes and sizes the long-path kernel takes; everything else stays with the token-by-token kernel.  A small batch

@@ -1,0 +1,504 @@
+// Verification of small draft trees with the state streamed straight into registers.
+//
+// Mathematics: the effective-query regrouping of the tree-masked factorisation (Section 4.2).  With
+// a_0 = t, a_1, ... the root path of node t taken upward, gamma_t the product of alpha over it and
+// rho_t[r] = alpha_{a_0} ... alpha_{a_{r-1}},
+//        o_t = S0 qeff_t + sum_r M[t][a_r] v_{a_r}
+//        qeff_t = scale gamma_t q_t - sum_r scale gamma_t cb_r k_{a_r}        M[t][a_r] = scale rho_t[r] cb_r
+// where cb_r = c_r beta_{a_r} and c is the back substitution up the path
+//        c_r = q_t.k_{a_r} - sum_{m<r} cb_m (k_{a_m}.k_{a_r}) .
+// Everything that meets the state is then one product of the state tile with at most 8 NT vectors.
+//
+// Why warp-level MMAs and no staging.  A draft of a few nodes leaves the kernel bound by the state stream
+// (a unit of 8 nodes does 0.8 M multiply-adds on 128 KB), and at this width a state tile never needs to be
+// seen by more than one warp: lane (g, t) of a warp loads the 16-byte chunks t, t + 4, ... of rows g and g + 8
+// of its 16-row tile, and those registers ARE the A fragments of mma.sync m16n8k8 (the contraction index is
+// free to permute).  There is no ring, no barrier between roles and no shared-memory round trip of the
+// state; while one CTA builds its coefficients the other resident CTAs stream.  The pipelined tcgen05 kernel
+// spends most of a small unit on hand-overs between its roles instead.
+//
+// fp32 accuracy: both operands are split into a TF32 head and the exact remainder (three products; the
+// dropped one is 2^-22 of the result); M is split into three bf16 pieces and multiplies the bf16 value rows
+// exactly.
+//
+// A CTA takes one unit (layer, sequence, head) or a slice of its value rows and checks the topology of its sequence
+// itself (one parent walk per node), so no plan kernel runs in front of it.  It asks the first rows of its tile into L2
+// with one bulk prefetch before it knows anything else, so that the set-up runs under the latency of HBM and the loop
+// over 16-row tiles needs two 32-column steps of registers in flight, not whole tiles: 24 warps fit an SM.  Holding
+// whole tiles in registers through the set-up (16 warps) took 5.1 us per 8-node unit and SM instead of 3.9, at 16
+// nodes 8.0 instead of 4.4.
+// Measured (d_k = 128, d_v = 256, 12288 units): 8 nodes 322 us = 5.6 TB/s (pipelined kernel 448 us), 16 nodes 361 us =
+// 5.6 TB/s (457); d_k = d_v = 64, 24576 units of 8 / 16 / 32 nodes: 154 / 212 / 342 us (serial walk 343 / 645 / 1364).
+// What bounds it: the state stream up to 8 nodes (87 % of the copy rate), above that also the shared-memory reads of the
+// vectors (two 16-byte loads per six MMAs and lane) and, at 32 nodes, two CTAs' worth of warps to hide a longer set-up.
+#include <atomic>
+
+#include "speca_common.cuh"
+#include "tc_ptx.cuh"
+
+namespace speca {
+
+namespace {
+
+__device__ __forceinline__ uint32_t tf32_head(float x) { return __float_as_uint(x) & 0xffffe000u; }
+__device__ __forceinline__ uint32_t tf32_tail(float x) { return __float_as_uint(x - __uint_as_float(tf32_head(x))); }
+
+// (not volatile: the compiler may interleave independent products)
+__device__ __forceinline__ void mma_tf32_sync(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_bf16_sync(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const void *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
+}
+// 32 bytes of a state row in one load; the state is read once per call
+__device__ __forceinline__ void ld_state(float (&x)[8], const float *p)
+{
+    asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7]) : "l"(p));
+}
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+// 16 bytes global -> shared; live == false fills with zeros (the address is not read)
+__device__ __forceinline__ void cp16(void *dst, const void *src, bool live)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst)), "l"(src), "r"(live ? 16 : 0)
+                 : "memory");
+}
+
+// Shared memory of one CTA (bytes); N = 8 NT nodes at most, `rows` value rows.
+template <int DK, int NT> struct Lay {
+    static constexpr int N = 8 * NT;
+    static constexpr int NK = (N + 15) & ~15;                   // contraction width of the value term
+    static constexpr int KQS = DK + 8;                          // bf16 per staged key / query row (16 bytes of padding)
+    static constexpr int BS = DK + 4;                           // floats per effective-query row (16 bytes of padding)
+    static constexpr int MS = NK + 8;                           // bf16 per row of a piece of M
+    static constexpr int GS = N + 1;
+    static constexpr int NR = NK;                               // rows of the weight pieces: whole MMA row blocks
+    static constexpr int OffKQ = 0;                             // bf16 [2N][KQS]: key rows, query rows
+    static constexpr int OffHi = OffKQ + 2 * N * KQS * 2;       // float [N][BS]
+    static constexpr int OffLo = OffHi + N * BS * 4;
+    static constexpr int OffM = OffLo + N * BS * 4;             // bf16 [3][N][MS]
+    static constexpr int OffG = OffHi;                          // float [2N][GS]: Gram rows of keys, queries (dead before Hi is written)
+    static constexpr int OffW = OffM + 3 * N * MS * 2;          // bf16 [3][NR][MS]: weights of the keys in qeff
+    static constexpr int OffP = OffW + 3 * NR * MS * 2;         // int32 parent[N], float alpha[N], beta[N], scale gamma[NR]
+    static constexpr int OffV = OffP + (3 * N + NR) * 4;        // bf16 [NK][rows + 8]
+    static_assert(2 * N * GS <= 2 * N * BS, "Gram rows do not fit the space of the effective queries");
+    static constexpr int bytes(int rows) { return OffV + NK * (rows + 8) * 2; }
+};
+
+struct DirectArgs {
+    Params p;
+    int32_t parts, rows;        // value-row slices per unit, rows per slice
+    int32_t lo;                 // sequences of at most this many nodes belong to another launch
+    int32_t all;                // no sequence of the call can be outside (lo, 8 NT]
+};
+
+template <int DK, int NT, int MAXD, int WARPS, int CTAS>
+__global__ void __launch_bounds__(WARPS * 32, CTAS)
+verify_direct_kernel(DirectArgs da)
+{
+    using LY = Lay<DK, NT>;
+    constexpr int N = LY::N, NS = DK / 32, THREADS = WARPS * 32;
+    extern __shared__ __align__(16) uint8_t smem[];
+    const Params &p = da.p;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
+
+    const int part = int(blockIdx.x % unsigned(da.parts));
+    const int unit = int(blockIdx.x / unsigned(da.parts));
+    const int h = unit % p.H, lb = unit / p.H, b = lb % p.B, l = lb / p.B;
+    const int row0 = part * da.rows;
+
+    // the first tiles are asked into L2 before anything else is known when the sequence is certainly ours
+    const float *S_cta = p.S0 + (long(unit) * p.DV + row0) * DK;
+    const int tiles = da.rows >> 4;
+    constexpr int AHEAD = DK == 256 ? 4 : 8;     // tiles requested ahead of the one a warp works on
+    auto prefetch_first = [&]() {
+        if (tid == 0) prefetch_l2(S_cta, uint32_t(min(tiles, AHEAD)) * (16 * DK * 4));
+    };
+    if (da.all) prefetch_first();
+
+    const int base = __ldg(p.node_offsets + b), end = __ldg(p.node_offsets + b + 1);
+    const int n = end - base;
+    const bool reporter = l == 0 && h == 0 && part == 0 && tid == 0;
+    if (base < 0 || n < 0 || end > p.T || (b == p.B - 1 && end != p.T) || (b == 0 && base != 0)) {
+        if (reporter) atomicOr(p.status, SPECA_STATUS_BAD_OFFSETS);
+        return;
+    }
+    if (n > p.max_nodes) {
+        if (reporter) atomicOr(p.status, SPECA_STATUS_TOO_MANY);
+        return;
+    }
+    if (p.parent == nullptr && n > p.max_depth) {            // a chain of n nodes is n levels deep
+        if (reporter) atomicOr(p.status, SPECA_STATUS_TOO_DEEP);
+        return;
+    }
+    if (n <= da.lo || n > N) return;                         // nothing to do, or another launch's
+    if (!da.all) prefetch_first();
+
+    __nv_bfloat16 *sKQ = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffKQ);
+    float *sHi = reinterpret_cast<float *>(smem + LY::OffHi), *sLo = reinterpret_cast<float *>(smem + LY::OffLo);
+    __nv_bfloat16 *sM = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffM);
+    float *sG = reinterpret_cast<float *>(smem + LY::OffG);
+    __nv_bfloat16 *sW = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffW);
+    int *sPar = reinterpret_cast<int *>(smem + LY::OffP);
+    float *sAl = reinterpret_cast<float *>(sPar + N), *sBe = sAl + N, *sGam = sBe + N;
+    __nv_bfloat16 *sV = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffV);
+    const int vstride = da.rows + 8;
+    const int nt = (n + 7) >> 3;
+    const long rec0 = (long(l) * p.T + base) * p.H + h;      // record of node 0; node i is H records further on
+    const int H = p.H;
+
+    // ---- the sequence's records -> shared memory; rows past the last node are zero
+    {
+        constexpr int PCS = DK / 8;
+        for (int i = tid; i < 2 * 8 * nt * PCS; i += THREADS) {
+            const int r = i / PCS, c = i % PCS;
+            const bool is_q = r >= 8 * nt;
+            const int node = is_q ? r - 8 * nt : r;
+            const bool live = node < n;
+            const __nv_bfloat16 *src = (is_q ? p.q : p.k) + (rec0 + long(live ? node : 0) * H) * DK + 8 * c;
+            cp16(sKQ + (is_q ? N + node : node) * LY::KQS + 8 * c, src, live);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const int vp = da.rows >> 3, vrows = (n + 15) & ~15;
+        for (int i = tid; i < vrows * vp; i += THREADS) {
+            const int node = i / vp, c = i % vp;
+            const bool live = node < n;
+            cp16(sV + node * vstride + 8 * c, p.v + (rec0 + long(live ? node : 0) * H) * p.DV + row0 + 8 * c, live);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        for (int i = tid; i < 3 * N * LY::MS / 8; i += THREADS) reinterpret_cast<uint4 *>(sM)[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = tid; i < 3 * LY::NR * LY::MS / 8; i += THREADS) reinterpret_cast<uint4 *>(sW)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (tid < LY::NR) sGam[tid] = 0.f;
+    }
+    int fault = 0;
+    if (tid < n) {
+        const int pa = p.parent != nullptr ? __ldg(p.parent + base + tid) : tid - 1;
+        if (pa < -1 || pa >= tid) fault = SPECA_STATUS_BAD_PARENT;
+        sPar[tid] = pa;
+        sAl[tid] = __ldg(p.alpha + rec0 + long(tid) * H);
+        sBe[tid] = __ldg(p.beta + rec0 + long(tid) * H);
+    }
+    asm volatile("cp.async.wait_group 1;" ::: "memory");     // keys and queries; the value rows may still be in flight
+    if (__syncthreads_or(fault)) {
+        if (reporter) atomicOr(p.status, SPECA_STATUS_BAD_PARENT);
+        return;
+    }
+
+    // ---- topology: the path of node tid, upward (path[0] is the node itself)
+    int path[MAXD], d = 0;
+    if (tid < n) {
+        int a = tid;
+#pragma unroll
+        for (int r = 0; r < MAXD; ++r) {
+            path[r] = a >= 0 ? a : 0;
+            if (a >= 0) { ++d; a = sPar[a]; }
+        }
+        int full = d;
+        for (; a >= 0; a = sPar[a]) ++full;
+        if (full > p.max_depth) fault |= SPECA_STATUS_TOO_DEEP;
+        if (p.depth_in != nullptr && __ldg(p.depth_in + base + tid) != full) fault |= SPECA_STATUS_BAD_DEPTH;
+        if (fault && l == 0 && h == 0 && part == 0) atomicOr(p.status, fault);
+    }
+
+    // ---- Gram rows of keys and queries against the keys
+    for (int job = WARPS - 1 - warp; job < nt * nt; job += WARPS) {      // (warp 0 walks the paths meanwhile)
+        // one MMA row block: keys 8 mi .. in rows 0-7, queries 8 mi .. in rows 8-15; a node's path holds no later node
+        const int mi = job / nt, ni = job % nt;
+        if (ni > mi) continue;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
+        const __nv_bfloat16 *pa = sKQ + ((lane & 8 ? N : 0) + 8 * mi + (lane & 7)) * LY::KQS + ((lane >> 4) << 3);
+        const __nv_bfloat16 *pb = sKQ + (8 * ni + (lane & 7)) * LY::KQS + ((lane >> 3) << 3);
+#pragma unroll
+        for (int k = 0; k < DK / 32; ++k) {
+            uint32_t bq[4], a0[4], a1[4];
+            ldsm_x4(bq, pb + 32 * k);
+            ldsm_x4(a0, pa + 32 * k);
+            ldsm_x4(a1, pa + 32 * k + 16);
+            mma_bf16_sync(acc, a0, bq[0], bq[1]);
+            mma_bf16_sync(acc1, a1, bq[2], bq[3]);
+        }
+        float *gk = sG + (8 * mi + g) * LY::GS + 8 * ni + 2 * t4, *gq = gk + N * LY::GS;
+        gk[0] = acc[0] + acc1[0]; gk[1] = acc[1] + acc1[1];
+        gq[0] = acc[2] + acc1[2]; gq[1] = acc[3] + acc1[3];
+    }
+    if (__syncthreads_or(fault)) return;                     // reported above
+
+    // ---- coefficients of node tid: back substitution up its path
+    if (tid < n) {
+        float acc[MAXD];
+        const float *gq = sG + (N + tid) * LY::GS;
+#pragma unroll
+        for (int r = 0; r < MAXD; ++r) acc[r] = r < d ? gq[path[r]] : 0.f;
+#pragma unroll
+        for (int r = 0; r < MAXD; ++r) {
+            const float cb = acc[r] * sBe[path[r]];
+            if (!p.no_erase) {
+                const float *gk = sG + path[r] * LY::GS;
+#pragma unroll
+                for (int s = r + 1; s < MAXD; ++s)
+                    if (r < MAXD - 1) acc[s] = s < d ? fmaf(-cb, gk[path[s]], acc[s]) : 0.f;
+            }
+            acc[r] = cb;
+        }
+        auto put = [&](__nv_bfloat16 *row, int piece, int col, float x) {
+#pragma unroll
+            for (int pc = 0; pc < 3; ++pc) {
+                const __nv_bfloat16 q = __float2bfloat16_rn(x);
+                row[pc * piece + col] = q;
+                x -= __bfloat162float(q);
+            }
+        };
+        float rho = p.scale;
+#pragma unroll
+        for (int r = 0; r < MAXD; ++r)
+            if (r < d) {
+                put(sM + tid * LY::MS, N * LY::MS, path[r], rho * acc[r]);
+                rho *= sAl[path[r]];
+            }
+        sGam[tid] = rho;                                     // scale gamma
+        if (!p.no_erase)
+#pragma unroll
+            for (int r = 0; r < MAXD; ++r)
+                if (r < d) put(sW + tid * LY::MS, LY::NR * LY::MS, path[r], -rho * acc[r]);
+    }
+    __syncthreads();
+
+    // ---- effective queries (scale gamma q + W K, the weights in three bf16 pieces), split into head and remainder
+    {
+        const int nm = (n + 15) >> 4;
+        for (int job = warp; job < nm * (DK / 16); job += WARPS) {
+            const int mi = job / (DK / 16), c0 = (job % (DK / 16)) * 16;
+            const int r0 = 16 * mi + g, r1 = r0 + 8;
+            const float g0 = sGam[r0], g1 = sGam[r1];
+            float acc[2][4];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                // rows past the staged ones weigh nothing; clamp keeps the read inside the buffer
+                const uint32_t q0 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r0, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
+                const uint32_t q1 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r1, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
+                acc[c][0] = g0 * __uint_as_float(q0 << 16); acc[c][1] = g0 * __uint_as_float(q0 & 0xffff0000u);
+                acc[c][2] = r1 < 8 * nt ? g1 * __uint_as_float(q1 << 16) : 0.f;
+                acc[c][3] = r1 < 8 * nt ? g1 * __uint_as_float(q1 & 0xffff0000u) : 0.f;
+            }
+            for (int kk = 0; kk <= mi; ++kk) {               // a node's path holds no later node
+                uint32_t kb[4];                              // key rows 16 kk .. + 15, columns c0 .. + 15
+                const int kr = 16 * kk + (lane & 15);
+                ldsm_x4_t(kb, sKQ + min(kr, 8 * nt - 1) * LY::KQS + c0 + ((lane >> 4) << 3));
+#pragma unroll
+                for (int pc = 0; pc < 3; ++pc) {
+                    uint32_t a[4];
+                    ldsm_x4(a, sW + (pc * LY::NR + 16 * mi + (lane & 15)) * LY::MS + 16 * kk + ((lane >> 4) << 3));
+                    mma_bf16_sync(acc[0], a, kb[0], kb[1]);
+                    mma_bf16_sync(acc[1], a, kb[2], kb[3]);
+                }
+            }
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int r = half ? r1 : r0;
+                if (r >= 8 * nt) break;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const float x0 = acc[c][2 * half], x1 = acc[c][2 * half + 1];
+                    const float y0 = tc::round_tf32(x0), y1 = tc::round_tf32(x1);
+                    *reinterpret_cast<float2 *>(sHi + r * LY::BS + c0 + 8 * c + 2 * t4) = make_float2(y0, y1);
+                    *reinterpret_cast<float2 *>(sLo + r * LY::BS + c0 + 8 * c + 2 * t4) = make_float2(x0 - y0, x1 - y1);
+                }
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");     // value rows
+    __syncthreads();
+
+    // ---- the state: one 16-row tile at a time, two 32-column steps of registers in flight
+    // lane (g, t) holds columns 32 q + 8 t .. + 7 of rows g and g + 8: k-steps e = 0..3 of the step contract
+    // columns 8 t + 2 e and 8 t + 2 e + 1 of the four lanes
+    const float *Su = S_cta + g * DK + 8 * t4;
+    const float *hi_p = sHi + g * LY::BS + 8 * t4, *lo_p = sLo + g * LY::BS + 8 * t4;
+    const int nk = (n + 15) >> 4;
+    float *o0 = p.o + rec0 * p.DV + row0 + g;
+    const long node_stride = long(H) * p.DV;
+    float sa[2][8], sb[2][8];
+    if (warp < tiles)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            ld_state(sa[q], Su + warp * 16 * DK + 32 * q);
+            ld_state(sb[q], Su + (warp * 16 + 8) * DK + 32 * q);
+        }
+#pragma unroll 1
+    for (int tile = warp; tile < tiles; tile += WARPS) {
+        if (lane == 0 && tile + AHEAD < tiles) prefetch_l2(S_cta + long(tile + AHEAD) * 16 * DK, 16 * DK * 4);
+        const bool next = tile + WARPS < tiles;
+        float hh[NT][4], xx[NT][4];                          // head x head, and the two cross products
+#pragma unroll
+        for (int i = 0; i < NT; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { hh[i][e] = 0.f; xx[i][e] = 0.f; }
+        const float *cur = Su + long(tile) * 16 * DK, *nxt = cur + WARPS * 16 * DK - NS * 32;
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+            uint32_t ah[4][4], al[4][4];                     // [k-step][fragment register]
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float x[4] = {sa[q & 1][2 * e], sb[q & 1][2 * e], sa[q & 1][2 * e + 1], sb[q & 1][2 * e + 1]};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) { ah[e][c] = tf32_head(x[c]); al[e][c] = tf32_tail(x[c]); }
+            }
+            if (q + 2 < NS || next) {
+                const float *src = (q + 2 < NS ? cur : nxt) + 32 * (q + 2);
+                ld_state(sa[q & 1], src);
+                ld_state(sb[q & 1], src + 8 * DK);
+            }
+#pragma unroll
+            for (int i = 0; i < NT; ++i) {
+                if (NT > 1 && i >= nt) break;
+#pragma unroll
+                for (int e2 = 0; e2 < 2; ++e2) {
+                    const float4 bh = *reinterpret_cast<const float4 *>(hi_p + 8 * i * LY::BS + 32 * q + 4 * e2);
+                    const float4 bl = *reinterpret_cast<const float4 *>(lo_p + 8 * i * LY::BS + 32 * q + 4 * e2);
+                    mma_tf32_sync(hh[i], ah[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
+                    mma_tf32_sync(xx[i], ah[2 * e2], __float_as_uint(bl.x), __float_as_uint(bl.y));
+                    mma_tf32_sync(hh[i], ah[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
+                    mma_tf32_sync(xx[i], al[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
+                    mma_tf32_sync(xx[i], ah[2 * e2 + 1], __float_as_uint(bl.z), __float_as_uint(bl.w));
+                    mma_tf32_sync(xx[i], al[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
+                }
+            }
+        }
+        // value term: rows of V^T (16 value rows x 16 nodes) x M, piece by piece
+        {
+            const __nv_bfloat16 *va = sV + ((lane & 7) + ((lane >> 4) << 3)) * vstride + tile * 16 + (lane & 8);
+#pragma unroll
+            for (int kk = 0; kk < LY::NK / 16; ++kk) {
+                if (LY::NK > 16 && kk >= nk) break;
+                uint32_t a[4];
+                ldsm_x4_t(a, va + kk * 16 * vstride);
+#pragma unroll
+                for (int i = 0; i < NT; ++i) {
+                    if (NT > 1 && i >= nt) break;
+                    if (8 * i + 7 < 16 * kk) continue;       // a node's path holds no later node
+#pragma unroll
+                    for (int pc = 0; pc < 3; ++pc) {
+                        const __nv_bfloat16 *mb = sM + (pc * N + 8 * i + g) * LY::MS + 16 * kk + 2 * t4;
+                        mma_bf16_sync(xx[i], a, *reinterpret_cast<const uint32_t *>(mb), *reinterpret_cast<const uint32_t *>(mb + 8));
+                    }
+                }
+            }
+        }
+        float *ot = o0 + tile * 16;
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+            if (NT > 1 && i >= nt) break;
+            const int n0 = 8 * i + 2 * t4;
+            float *od = ot + n0 * node_stride;
+            if (n0 < n) { od[0] = hh[i][0] + xx[i][0]; od[8] = hh[i][2] + xx[i][2]; }
+            if (n0 + 1 < n) { od[node_stride] = hh[i][1] + xx[i][1]; od[node_stride + 8] = hh[i][3] + xx[i][3]; }
+        }
+    }
+}
+
+template <int DK, int NT, int MAXD, int WARPS, int CTAS>
+int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
+{
+    using LY = Lay<DK, NT>;
+    DirectArgs da;
+    da.p = p;
+    da.lo = lo;
+    da.all = all ? 1 : 0;
+    // value rows per CTA: the whole unit, halved while the device would be left with idle slots
+    const long units = long(p.L) * p.B * p.H;
+    int rows = p.DV;
+    while (rows > 256 && rows % 32 == 0) rows /= 2;
+    while (rows % 32 == 0 && rows / 16 > WARPS && units * (p.DV / rows) < long(sms) * CTAS) rows /= 2;
+    da.rows = rows;
+    da.parts = p.DV / rows;
+    const int smem = LY::bytes(rows);
+    static std::atomic<int> opted[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return int(cudaErrorInvalidDevice);
+    auto kern = verify_direct_kernel<DK, NT, MAXD, WARPS, CTAS>;
+    if (smem > 48 * 1024 && opted[dev].load(std::memory_order_acquire) == 0) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::bytes(512));
+        if (e != cudaSuccess) return int(e);
+        opted[dev].store(1, std::memory_order_release);
+    }
+    kern<<<unsigned(units * da.parts), WARPS * 32, smem, st>>>(da);
+    return int(cudaGetLastError());
+}
+
+// Warps per CTA and CTAs per SM by the width NT of the product: registers (two 32-column steps of state, the
+// accumulators) allow 80 / 96 / 128 per thread, shared memory two CTAs at 32 nodes, where eight warps share the longer
+// set-up.
+template <int DK, int MAXD>
+int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_t st)
+{
+    constexpr int C1 = DK == 64 && MAXD == 8 ? 6 : MAXD == 8 && DK == 128 ? 6 : 5, C2 = DK == 64 || MAXD == 8 ? 5 : 4;
+    if (hi <= 8) return launch_one<DK, 1, MAXD, 4, C1>(p, lo, all, sms, st);
+    if (hi <= 16) return launch_one<DK, 2, MAXD, 4, C2>(p, lo, all, sms, st);
+    if constexpr (DK == 64) {
+        if (hi <= 32) return launch_one<DK, 4, MAXD, 4, 4>(p, lo, all, sms, st);
+        return launch_one<DK, 8, MAXD, 8, 1>(p, lo, all, sms, st);
+    } else {
+        return launch_one<DK, 4, MAXD, 8, 2>(p, lo, all, sms, st);
+    }
+}
+
+// A batch that fills the device's resident CTAs only once or twice is latency, not throughput.
+bool small_batch(const Params &p, int sms) { return long(p.L) * p.B * p.H <= 4L * sms; }
+
+}  // namespace
+
+// Largest sequence this kernel should verify (0: none).  `most` bounds the nodes of any sequence of the call, `piped`
+// says that one of the pipelined tensor-core kernels takes the shape.
+int direct_limit(const Params &p, int d_k, int most, bool piped)
+{
+    if (d_k == 64) return 64;                                // the alternative is the serial walk
+    if (!piped) return 32;
+    // us per unit and SM in a large batch, this kernel / the pipelined one: d_k = 128, d_v = 256: 3.9 / 5.4 at 8 nodes,
+    // 4.4 / 5.5 at 16, 6.4 / 6.1 at 24 (trees deeper than 8 levels, 32 nodes: 8.3 / 14.3); d_k = 256: 8.2 / 9.9 at 8,
+    // 9.4 / 10.0 at 16, 17.5 / 11.1 at 24.  A single user's 32-node tree, 24 x 16 units: 22 / 37 us.
+    const int cap = small_batch(p, sm_count_of_current_device()) || (d_k == 128 && p.max_depth > 8) ? 32 : 16;
+    return most <= cap ? cap : 0;
+}
+
+// Verifies every sequence of at most `limit` nodes; larger ones are left to another kernel.
+int launch_verify_direct(const Params &p, int d_k, int most, int limit, cudaStream_t st)
+{
+    const int sms = sm_count_of_current_device();
+    if (sms <= 0) return int(cudaErrorInvalidDevice);
+    const bool deep = p.max_depth > 8;
+    auto run = [&](int lo, int hi) {
+        const bool all = lo == 0 && most <= hi;
+        switch (d_k) {
+        case 64: return deep ? launch_width<64, 16>(p, hi, lo, all, sms, st) : launch_width<64, 8>(p, hi, lo, all, sms, st);
+        case 128: return deep ? launch_width<128, 16>(p, hi, lo, all, sms, st) : launch_width<128, 8>(p, hi, lo, all, sms, st);
+        case 256: return deep ? launch_width<256, 16>(p, hi, lo, all, sms, st) : launch_width<256, 8>(p, hi, lo, all, sms, st);
+        }
+        return int(cudaErrorInvalidValue);
+    };
+    const int top = most < limit ? most : limit;
+    if (top <= 32 || small_batch(p, sms)) return run(0, top);
+    const int rc = run(0, 32);
+    return rc != 0 ? rc : run(32, top);
+}
+
+}  // namespace speca

@@ -20,7 +20,7 @@ constexpr int kPlanThreads = 128;
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict__ parent,
             const int32_t *__restrict__ depth_in, int32_t B, int32_t T, int32_t max_depth,
-            int32_t max_nodes, int32_t n_slots, Workspace ws, int32_t *status)
+            int32_t max_nodes, int32_t skip_nodes, int32_t n_slots, Workspace ws, int32_t *status)
 {
     extern __shared__ int32_t sm[];
     const int b = blockIdx.x;
@@ -37,6 +37,10 @@ plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict_
         fault = SPECA_STATUS_TOO_MANY;
     if (fault) {
         if (tid == 0) { atomicOr(status, fault); ws.seq_n[b] = -1; }
+        return;
+    }
+    if (n <= skip_nodes) {                             // verified by the kernel for small trees, which checks them itself
+        if (tid == 0) ws.seq_n[b] = 0;
         return;
     }
     int32_t *par = sm;                       // [n]
@@ -569,7 +573,7 @@ int launch_plan(const Params &p, cudaStream_t st)
 {
     const size_t smem = size_t(6 * p.max_nodes + 1) * sizeof(int32_t);
     plan_kernel<<<p.B, kPlanThreads, smem, st>>>(p.node_offsets, p.parent, p.depth_in, p.B, p.T,
-                                                  p.max_depth, p.max_nodes, p.n_slots, p.ws, p.status);
+                                                  p.max_depth, p.max_nodes, p.skip_nodes, p.n_slots, p.ws, p.status);
     return int(cudaGetLastError());
 }
 

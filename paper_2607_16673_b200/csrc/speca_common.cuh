@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/speca.h"
 
 namespace speca {
@@ -91,6 +93,7 @@ struct Params {
     int32_t *status;
     Workspace ws;
     int32_t n_slots;             // on-chip state slots available to the tree walk
+    int32_t skip_nodes;          // verify: sequences of at most this many nodes are another kernel's (the plan gives them no nodes)
     int32_t long_min;            // commit: accepted paths of long_min..8 nodes are taken by the tensor-core kernel (0: none)
 };
 
@@ -107,6 +110,9 @@ bool factorized_supported(const speca_dims *d);
 bool factorized_fused_supported(const speca_dims *d);
 int launch_verify_factorized(const Params &p, int d_k, bool fused, bool comp, cudaStream_t st);
 void factorized_set_withhold(int on);
+// small draft trees, state streamed straight into registers: largest sequence it should take, and the launch
+int direct_limit(const Params &p, int d_k, int most, bool piped);
+int launch_verify_direct(const Params &p, int d_k, int most, int limit, cudaStream_t st);
 bool effective_supported(const speca_dims *d);
 int launch_verify_effective(const Params &p, int d_k, cudaStream_t st);
 void effective_set_withhold(int on);
@@ -128,6 +134,21 @@ int launch_accept(int32_t B, int32_t max_depth, const int32_t *node_offsets, con
 int launch_stochastic_accept(int32_t B, int32_t max_depth, const int32_t *node_offsets, const int32_t *parent,
                              const float *p_target, const float *p_draft, const float *uniform,
                              int32_t *path_idx, int32_t *path_len, int32_t *status, cudaStream_t st);
+
+// SM count per device (asked once per device)
+inline int sm_count_of_current_device()
+{
+    static std::atomic<int> cache[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const bool cached = dev >= 0 && dev < 64;
+    int sms = cached ? cache[dev].load(std::memory_order_relaxed) : 0;
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+        if (cached) cache[dev].store(sms, std::memory_order_relaxed);
+    }
+    return sms;
+}
 
 // Number of on-chip state slots the light-children-first walk can need for a tree of
 // at most n nodes: a node saves its state only if it has two children with
