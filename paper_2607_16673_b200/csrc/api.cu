@@ -67,16 +67,18 @@ int verify_common(const speca_dims *dims, const float *S0, const uint16_t *q, co
     p.status = status_word;
     p.ws = carve_workspace(workspace, dims->batch, total_nodes);
     p.n_slots = tree_slots_needed(dims->max_nodes);
-    // AUTO: an fp32-grade tensor-core route where the shape fits -- the factorised kernel in its compensated form,
-    // or, for shapes it does not take (more than 32 nodes below 16 levels), the effective-query kernel -- else the
-    // serial walk.  The single-pass TF32 kernel runs only when asked for by name.
+    // AUTO and FACTORIZED: the effective-query kernel where the shape fits; with u requested the split-operand form of
+    // the factorised kernel (both come out of one walk there), except for shapes only the former takes (more than 32
+    // nodes at 9..16 levels).  AUTO falls back to the serial walk; the single-pass TF32 kernel runs only when asked for
+    // by name.
     const bool tf32 = dims->route == SPECA_ROUTE_TF32;
     if (tf32 && !factorized_supported(dims)) return SPECA_ERR_UNSUPPORTED;
     const bool tensor = dims->route == SPECA_ROUTE_AUTO || dims->route == SPECA_ROUTE_FACTORIZED;
-    const bool fact = tensor && factorized_supported(dims);
     if (dims->route == SPECA_ROUTE_EFFECTIVE && !effective_supported(dims)) return SPECA_ERR_UNSUPPORTED;
+    const bool fact = tensor && u != nullptr && factorized_supported(dims);
     const bool eff = dims->route == SPECA_ROUTE_EFFECTIVE || (tensor && !fact && effective_supported(dims));
     if (dims->route == SPECA_ROUTE_FACTORIZED && !fact && !eff) return SPECA_ERR_UNSUPPORTED;
+
     // Small trees go to the kernel that streams the state through registers (its loads are 32 bytes wide); it needs no
     // plan.  A chain longer than max_depth <= 16 is a fault that it reports itself.
     if (dims->route == SPECA_ROUTE_AUTO && u == nullptr && (reinterpret_cast<uintptr_t>(S0) & 31u) == 0) {

@@ -473,10 +473,10 @@ int direct_limit(const Params &p, int d_k, int most, bool piped)
 {
     if (d_k == 64) return 64;                                // the alternative is the serial walk
     if (!piped) return 32;
-    // us per unit and SM in a large batch, this kernel / the pipelined one: d_k = 128, d_v = 256: 3.9 / 5.4 at 8 nodes,
-    // 4.4 / 5.5 at 16, 6.4 / 6.1 at 24 (trees deeper than 8 levels, 32 nodes: 8.3 / 14.3); d_k = 256: 8.2 / 9.9 at 8,
-    // 9.4 / 10.0 at 16, 17.5 / 11.1 at 24.  A single user's 32-node tree, 24 x 16 units: 22 / 37 us.
-    const int cap = small_batch(p, sm_count_of_current_device()) || (d_k == 128 && p.max_depth > 8) ? 32 : 16;
+    // us per unit and SM in a large batch, this kernel / the pipelined one: d_k = 128, d_v = 256: 3.9 / 5.0 at 8 nodes,
+    // 4.4 / 5.0 at 16, 6.1 / 5.2 at 20..24; d_k = 256: 8.2 / 8.8 at 8, 9.4 / 8.8 at 16.  A single user's 32-node tree,
+    // 24 x 16 units: 22 / 33 us.
+    const int cap = small_batch(p, sm_count_of_current_device()) ? 32 : d_k == 128 ? 16 : 8;
     return most <= cap ? cap : 0;
 }
 

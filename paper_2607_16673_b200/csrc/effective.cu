@@ -1,53 +1,46 @@
-// Tree-masked verification with effective queries on the 5th-generation tensor cores
-// (tcgen05 + TMEM): the parallel route of Section 4.2 with every coefficient matrix moved to
-// the small side of ONE accumulation chain, at fp32 accuracy.
+// Tree-masked verification on the 5th-generation tensor cores (tcgen05 + TMEM): the parallel route of Section 4.2
+// with the triangular solve moved to coefficient rows, at fp32 accuracy.
 //
-// Mathematics.  With gamma_t the product of alpha over the root path of node t, a_0 .. a_{d-1}
-// that path (a_{d-1} = t) and rho_t[j] = gamma_t / gamma_{a_j}, the factorisation of Section 4.2
-// (A_tree = M_tree o K_b K_a^T, T = (I + A)^-1, O = Qhat S0^T - Attn (W S0^T) + Attn U) regroups as
-//        o_t = S0 qeff_t + sum_j Mq[t][a_j] v_{a_j} ,      u_t = -S0 weff_t + sum_j Mk[t][a_j] v_{a_j}
-// with, per node, two short coefficient rows taken from the gate-free triangular system
-// X = (I + Ahat)^-1, Ahat[t][i] = beta_t (k_t.k_i) over strict ancestors, and C = Phat X,
-// Phat[t][i] = q_t.k_i over the path:
-//        qeff_t = scale gamma_t ( q_t - sum_j C[t][j] beta_{a_j} k_{a_j} )   Mq[t][a_j] = scale rho_t[j] C[t][j] beta_{a_j}
-//        weff_t =       gamma_t   sum_j X[t][j] beta_{a_j} k_{a_j}           Mk[t][a_j] =       rho_t[j] X[t][j] beta_{a_j}
-// (W and Attn of the paper are these rows; the triangular solve is a back substitution along
-// ancestor paths, at most 15 steps).  Everything that depends on the state is then one dense
-// contraction of the state tile with N effective vectors, plus a small product with the value
-// rows; the epilogue only adds two accumulator columns and stores.
+// Mathematics.  With a_0 = t, a_1, ... the root path of node t taken upward, gamma_t the product of alpha over it
+// and rho_t[r] = alpha_{a_0} ... alpha_{a_{r-1}}, the factorisation of Section 4.2 (A_tree = M_tree o K_b K_a^T,
+// T = (I + A)^-1, O = Qhat S0^T - Attn (W S0^T) + Attn U) regroups as
+//        R = K S0^T ,  G = Q S0^T ,  x_a = v_a - gamma_a R_a                       (per node, over the value rows)
+//        o_t = scale gamma_t G_t + sum_r M[t][a_r] x_{a_r} ,     M[t][a_r] = scale rho_t[r] c_r beta_{a_r}
+// where c is a back substitution up the node's own path that needs Gram entries only,
+//        c_r = q_t.k_{a_r} - sum_{m<r} c_m beta_{a_m} (k_{a_m}.k_{a_r}) .
+// The corrected values u_t = sum_r M[t][a_r] x_{a_r} come out the same way with c_0 = 1, c_r = 0 on the right-hand
+// side and scale 1.  (Attn is M; the solve is at most 15 steps along a path.)  Per value tile that is one product of
+// the state with the raw rows of [K;Q], an element-wise step, and one product with M.
 //
-// Accuracy.  The tensor core reads fp32 operands as TF32 (top 19 bits).  Both operands are
-// therefore split: the state slice as landed (its TF32 head, free) and its exact remainder
-// S - tf32(S), rewritten in place by a CUDA-core role once the first pass has read the slice;
-// the effective vectors as a TF32-rounded head and the exact remainder.  First pass: S x head ->
-// accumulator columns [0,R); correction passes: S x tail and then (S - tf32(S)) x head -> columns
-// [R,2R).  The dropped term is 2^-22 of the result.  Mq / Mk are split into three bf16 pieces
-// (24 bits) and multiply the bf16 value rows exactly.
+// Accuracy.  Everything is split into bf16 pieces of 8 bits: the fp32 state and x into three each by truncation
+// (exact: 3 x 8 = 24 bits), M likewise; q, k, v are bf16 already.  S0 [K;Q]^T is three products of pieces, exact up
+// to the fp32 accumulation; x M^T keeps the six products down to 2^-16, the dropped ones are 2^-24 of the result.
 //
-// Mapping.  One persistent CTA per SM walks units (layer, sequence, head); 21 warps:
-//   warp 0        TMA producer: per unit the K-slices of the fp32 state (128-byte swizzle), slice by slice
-//                 over both value tiles, and, after the first slice pair, the unit's bf16 value rows --
-//                 all through one ring of 16 KiB slots;
-//   warps 1, 18   issue the first-pass tcgen05.mma of value tile 0 / 1 and the value-row product (an
-//                 instruction costs its issuer about 130 cycles and a unit needs about a hundred of
-//                 them, hence several issuers); warp 1 owns TMEM (two units of accumulators in flight)
-//                 and issues the Gram blocks;
-//   warps 19, 20  issue the correction passes of tile 0 / 1, each following two cursors (the tail
-//                 operand, ready as soon as the slice has landed; the rewritten slice, ready once the
-//                 split role is done with it) and releasing the ring slot;
-//   warps 2-5     solver: ancestor entries of the Gram block out of TMEM, the two back substitutions,
-//                 one record per operand row, the three bf16 pieces of M -- one unit ahead;
-//   warps 6-9     effective vectors from the records and the staged bf16 keys / queries, one K-slice
-//                 at a time into a ring of operand slices (so they never exist whole);
-//   warps 10-13   rewrite each state slice as its TF32 remainder between the passes;
-//   warps 14-17   epilogue: o (or u) = column t + column R + t, streamed out coalesced.
-// Every visit of a ring slot, state slice or value rows, completes the same four barriers in the
-// same order (landed, first pass read, rewritten, released), so that their phase parities stay in step.
-// Nodes keep their index order everywhere.  When u is requested a unit is walked twice (first the
-// o rows, then the u rows); the second walk finds the state tile in L2.  The order in which the
-// passes reach an accumulator column is not fixed, so two runs may differ in the last bit.
+// Why this form.  The staged bf16 rows of [K;Q], as TMA lands them, are the B operand: no fp32 operand is built, so
+// the state stream waits for no preparation, only the second product does, a tile later.  The pieces of the state go
+// into TMEM as the A operand, so a slice crosses shared memory twice (TMA write, one read) and its ring slot is free
+// as soon as it has been read; rewriting it in place between two TF32 passes took five crossings and three hand-overs.
+// A tile of 64 nodes takes 24 + 24 tcgen05 instructions.  The substitution over value rows, ~95 instructions per node
+// and warp in factorized.cu, is gone: what is left per element is a multiply-add on each side of the second product.
+//
+// Mapping.  One persistent CTA per SM walks units (layer, sequence, head) tile by tile (128 value rows); 20 warps:
+//   warp 0        TMA producer of the state slices (128 rows x 32 columns, 128-byte swizzle)
+//   warp 1        issues S0 [K;Q]^T; owns TMEM
+//   warp 2        issues the Gram blocks [K;Q] K^T (one unit ahead) and x M^T
+//   warp 3        TMA producer of the staged [K;Q] rows (two units) and the value rows (two tiles)
+//   warps 4-7     split: slice row per thread -> three bf16 pieces in TMEM (two buffers)
+//   warps 8-15    two epilogue groups, alternating tiles: R out of TMEM, x back into TMEM as three pieces; then
+//                 o = scale gamma G + (x M^T), coalesced
+//   warps 16-19   solver, one unit ahead: Gram entries of every row against its own path, back substitution (a thread
+//                 per node, registers), the pieces of M
+// TMEM: two tiles of accumulators (R | G, 128 columns; x M^T overwrites R), two A buffers of 48, x of 96, Gram of 64.
+// Ten roles take turns on four issue slots, so the kernel's size matters as much as its instruction count: loops stay
+// rolled where a role has slack.
+// With u requested a unit is walked twice (o rows, then u rows); the second walk finds the state tile in L2.
 // Every wait is bounded; on expiry the CTA raises SPECA_STATUS_TIMEOUT, drains and exits.
 #include <cuda.h>
+
+#include <type_traits>
 
 #include "speca_common.cuh"
 #include "tc_ptx.cuh"
@@ -60,70 +53,73 @@ using namespace tc;
 
 constexpr int kRows = 128;                      // value rows per tile (= TMEM lanes = MMA M)
 constexpr int kSliceBytes = kRows * 128;        // one ring slot: a K-slice of a tile (128 rows x 32 fp32)
-constexpr int kMaxD = 16;                       // tree depth taken
-constexpr int kAccCols = 128;                   // accumulator columns per tile: [head R | tail R], R <= 64
-constexpr int kPairCols = 2 * kAccCols;
-constexpr int kTmemCols = 512;
-constexpr int kThreads = 21 * 32;
-constexpr int kRecBytes = 112;                  // per operand row: count, 17 weights, 17 staging offsets
-constexpr int kRecW = 4, kRecOff = 72;
-constexpr int kRecBuf = 64 * kRecBytes;
+constexpr int kThreads = 20 * 32;
 constexpr int kWalkSeqs = 128;
-constexpr int kVBlock = 8192;                   // the two 64-value blocks of a staged value tile sit this far apart
+// TMEM columns
+constexpr int kTileCols = 128;                  // accumulators of a tile: R, then G
+constexpr int kAOff = 2 * kTileCols, kACols = 48;    // two buffers of three 16-column pieces (32 bf16 columns each)
+constexpr int kXOff = kAOff + 2 * kACols;       // x: three 32-column pieces (64 nodes), or two buffers of three 16-column pieces
+constexpr int kGramOff = kXOff + 96;
+constexpr int kTmemCols = 512;
+static_assert(kGramOff + 64 == kTmemCols, "TMEM columns");
 
 // shared-memory carve-up per instantiation
-template <int TP, int DK, int MAXN_> struct Lay {
+template <int DK, int MAXN_, int MAXD> struct Lay {
     static constexpr int MAXN = MAXN_;                          // nodes per sequence
     static constexpr int NC = DK / 32;                          // K-slices per tile
     static constexpr int SC = DK / 64;                          // 64-column regions of the staged bf16 rows
     static constexpr int SCB = 2 * MAXN * 128;                  // bytes per region: key rows, then query rows
     static constexpr int STAGE = SC * SCB;
-    static constexpr int BBUF = 2 * MAXN * 128;                 // one K-slice of the operand: head rows, tail rows
+    static constexpr int VBUF = MAXN * kRows * 2;               // value rows of a tile, [node][128] bf16
     static constexpr int MPIECE = MAXN * 128;                   // one bf16 piece of M: R rows x 64 columns
-    static constexpr int GS = kMaxD * kRows * 4;                // Gram entries of every row against its own path
-    static constexpr int NB = MAXN > 32 ? 3 : 4;                // operand slices in flight
-    static constexpr int kFixed = NB * BBUF + 2 * STAGE + 3 * MPIECE + GS + 2 * kRecBuf + 2 * 64 * 4 + 512 + 128 +
-                                  5 * kWalkSeqs;
-    static constexpr int kRoom = (227 * 1024 - kFixed - 1024) / kSliceBytes;
-    static constexpr int NS = kRoom > 8 ? 8 : kRoom;            // ring depth
-    static constexpr int OffRing = 0;
-    static constexpr int OffB = OffRing + NS * kSliceBytes;
-    static constexpr int OffStage = OffB + NB * BBUF;
+    static constexpr int MBUF2 = MAXN > 32 ? 32 * 128 : 3 * MPIECE;      // second buffer of M, for units of up to 32 nodes
+    static constexpr int GSTR = MAXD + 4;                       // floats per node of the Gram entries, by distance up the path
+    static constexpr int OffStage = 0;                          // two units
+    // (the Gram block's A operand spans 128 rows whatever MAXN: it reads on into the regions behind, rows nobody looks at)
     static constexpr int OffM = OffStage + 2 * STAGE;
-    static constexpr int OffGs = OffM + 3 * MPIECE;
-    static constexpr int OffRec = OffGs + GS;
-    static constexpr int OffAlpha = OffRec + 2 * kRecBuf;
-    static constexpr int OffBars = OffAlpha + 2 * 64 * 4;
-    static constexpr int OffMisc = OffBars + 512;               // abort flag, TMEM base, node depths
-    static constexpr int OffWalk = OffMisc + 128;
-    static constexpr int Bytes = OffWalk + 5 * kWalkSeqs;
+    static constexpr int OffV = OffM + (MAXN > 32 ? 3 : 6) * MPIECE;     // two tiles
+    static constexpr int OffRing = OffV + 2 * VBUF;
+    static constexpr int kSmall = 2 * MAXN * GSTR * 4 + 2 * 2 * MAXN * 4 + 2 * MAXN + 4 * 2 * MAXN * 4 + 5 * kWalkSeqs + 16 + 8 * 64;
+    static constexpr int kRoom = (227 * 1024 - OffRing - kSmall) / kSliceBytes;
+    static constexpr int NS = kRoom > 8 ? 8 : kRoom;            // ring depth
+    static constexpr int OffGk = OffRing + NS * kSliceBytes;    // [MAXN][GSTR] k_node . k_(ancestor at distance i + 1)
+    static constexpr int OffGq = OffGk + MAXN * GSTR * 4;       // [MAXN][GSTR] q_node . k_(ancestor at distance i)
+    static constexpr int OffAB = OffGq + MAXN * GSTR * 4;       // two units of float alpha, beta [MAXN]
+    static constexpr int OffGam = OffAB + 2 * 2 * MAXN * 4;     // four units of float gamma in x, factor of G [MAXN]
+    static constexpr int OffDepth = OffGam + 4 * 2 * MAXN * 4;  // two units of uint8 [MAXN]
+    static constexpr int OffWalk = OffDepth + 2 * MAXN;
+    static constexpr int OffMisc = OffWalk + 5 * kWalkSeqs;     // abort flag, TMEM base
+    static constexpr int OffBars = OffMisc + 16;
+    static constexpr int Bytes = OffBars + 8 * 64;
+    static_assert(Bytes - OffGk == kSmall, "small regions");
     static_assert(NS >= 4, "ring too shallow");
     static_assert(Bytes <= 227 * 1024, "shared memory budget");
 };
 
 constexpr int kMaxSlots = 8;
 enum Bar {
-    kFull = 0,                         // [8] TMA -> MMA (and split): slot landed
-    kEmpty = kFull + kMaxSlots,        // [8] MMA -> TMA: slot no longer read
-    kP1Done = kEmpty + kMaxSlots,      // [8] MMA -> split: first pass has read the slice
-    kLo = kP1Done + kMaxSlots,         // [8] split -> MMA: slice rewritten as its remainder
-    kKQFull = kLo + kMaxSlots,         // [2] TMA -> MMA, vector warps: staged bf16 key / query rows of a unit
-    kGramFull = kKQFull + 2,           // MMA -> solver: Gram block in TMEM
-    kGramDone,                         // solver -> MMA: Gram rows read, the columns may be overwritten
-    kBReady,                           // [4] vector warps -> MMA: operand slice written
-    kBFree = kBReady + 4,              // [4] MMA -> vector warps: operand slice no longer read
-    kMReady = kBFree + 4,              // solver -> MMA: pieces of M written
-    kMFree,                            // MMA -> solver: value term issued and done
-    kAccFull,                          // [2] MMA -> epilogue
-    kPairFree = kAccFull + 2,          // [2] epilogue -> MMA
-    kRecReady = kPairFree + 2,         // [2] solver -> vector warps: records of a unit written
-    kRecFree = kRecReady + 2,          // [2] vector warps -> solver
-    kSolveSync = kRecFree + 2,         // role-internal
-    kVecSync,
+    kFull = 0,                         // [8] TMA -> split: slice landed
+    kEmpty = kFull + kMaxSlots,        // [8] split -> TMA: slice read
+    kAReady = kEmpty + kMaxSlots,      // [2] split -> MMA: pieces of a slice in TMEM
+    kAFree = kAReady + 2,              // [2] MMA -> split
+    kKQFull = kAFree + 2,              // [2] TMA -> both issuers: staged rows of a unit
+    kKQFree = kKQFull + 2,             // [2] both issuers -> TMA
+    kVFull = kKQFree + 2,              // [2] TMA -> epilogue: value rows of a tile
+    kVFree = kVFull + 2,               // [2] epilogue -> TMA
+    kAccFull = kVFree + 2,             // [2] MMA -> epilogue: R and G of a tile
+    kAccFree = kAccFull + 2,           // [2] epilogue -> MMA
+    kXReady = kAccFree + 2,            // [2] epilogue -> MMA: x of a tile in TMEM, R read
+    kXFree = kXReady + 2,              // MMA -> epilogue
+    kOutFull,                          // [2] MMA -> epilogue: x M^T of a tile
+    kGramFull = kOutFull + 2,          // MMA -> solver
+    kGramFree,                         // solver -> MMA
+    kMReady,                           // [2] solver -> MMA, epilogue: M and gamma of a unit
+    kMFree = kMReady + 2,              // [2] MMA -> solver
+    kSync = kMFree + 2,                // solver, role-internal
     kDrain,
     kBarCount
 };
-static_assert(kBarCount * 8 <= 512, "barrier region too small");
+static_assert(kBarCount <= 64, "barrier region too small");
 
 struct EMaps { CUtensorMap k[4], q[4], v[4]; };       // one per box height: 16, 32, 48, 64 nodes
 
@@ -132,44 +128,49 @@ struct EParams {
     int32_t heads_per_group;
     int32_t withhold_first_load;     // failure-detection test: CTA 0 never requests its first state slice
     int32_t want_u;
-    long n_units;
+    int32_t gpl, dl, db, dg;         // groups of heads per (layer, sequence); a step of gridDim.x groups as (layers, sequences, groups)
 };
 
 // A unit is one (layer, sequence, head); with u requested it is walked twice (kind 0: o rows, kind 1: u rows).
-struct VUnit { int grp, hi, u, b, l, h, n, npad, base, kind; };
+// Units are taken in groups of HG consecutive heads of one (layer, sequence): group blockIdx.x, += gridDim.x, kept as
+// (layer, sequence, group of heads) and advanced by carries, not divisions: every role walks the list by itself, so
+// this code is there ten times.
+struct VUnit {
+    int l, b, h, u, n, npad, base, kind, hi;
+    int nl, nb, ng;                                              // the group after this one
+};
 struct Walk {
-    int HG, gpl, n_groups, H, B, grid, two;
+    int HG, gpl, L, B, H, dl, db, dg, two;                       // d*: a step of gridDim.x groups
     const int32_t *seq_n; const int32_t *offs;
     const uint8_t *tab;
 };
 
-__device__ __forceinline__ bool load_group(const Walk &w, int G, VUnit &x)
-{
-    for (; G < w.n_groups; G += w.grid) {
-        const int lb = G / w.gpl;
-        x.b = lb % w.B;
-        const bool in_tab = x.b < kWalkSeqs;
-        x.n = in_tab ? int(reinterpret_cast<const int8_t *>(w.tab + 4 * kWalkSeqs)[x.b]) : w.seq_n[x.b];
-        if (x.n > 0) {
-            x.grp = G; x.hi = 0; x.kind = 0;
-            x.l = lb / w.B;
-            x.h = (G - lb * w.gpl) * w.HG;
-            x.u = lb * w.H + x.h;
-            x.npad = (x.n + 15) & ~15;
-            x.base = in_tab ? reinterpret_cast<const int32_t *>(w.tab)[x.b] : __ldg(w.offs + x.b);
-            return true;
-        }
-    }
-    x.n = 0; x.grp = w.n_groups;
-    return false;
-}
-__device__ __forceinline__ bool first_unit(const Walk &w, VUnit &x) { return load_group(w, int(blockIdx.x), x); }
 __device__ __forceinline__ bool next_unit(const Walk &w, VUnit &x)
 {
     if (w.two && x.kind == 0) { x.kind = 1; return true; }
     x.kind = 0;
     if (++x.hi < w.HG) { ++x.h; ++x.u; return true; }
-    return load_group(w, x.grp + w.grid, x);
+    while (x.nl < w.L) {
+        x.l = x.nl; x.b = x.nb;
+        const int g = x.ng;
+        x.ng += w.dg; x.nb += w.db; x.nl += w.dl;
+        if (x.ng >= w.gpl) { x.ng -= w.gpl; ++x.nb; }
+        if (x.nb >= w.B) { x.nb -= w.B; ++x.nl; }
+        const bool in_tab = x.b < kWalkSeqs;
+        x.n = in_tab ? int(reinterpret_cast<const int8_t *>(w.tab + 4 * kWalkSeqs)[x.b]) : w.seq_n[x.b];
+        if (x.n > 0) {
+            x.hi = 0;
+            x.h = g * w.HG;
+            x.u = (x.l * w.B + x.b) * w.H + x.h;
+            x.npad = (x.n + 15) & ~15;
+            x.base = in_tab ? reinterpret_cast<const int32_t *>(w.tab)[x.b] : __ldg(w.offs + x.b);
+            return true;
+        }
+    }
+    x.n = 0;
+    x.hi = w.HG;
+    x.kind = 1;
+    return false;
 }
 
 // one arrival for the whole warp: every lane's earlier writes are ordered before it
@@ -179,10 +180,6 @@ __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane)
     if (lane == 0) mbar_arrive(bar);
 }
 
-__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-// what the tensor core's TF32 reading of x (low 13 mantissa bits dropped) leaves out; exact
-__device__ __forceinline__ float tf32_rest(float x) { return x - __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16])
 {
     uint32_t x[16];
@@ -193,6 +190,43 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16])
                  : "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) r[i] = __uint_as_float(x[i]);
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&x)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+        ::"r"(taddr), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7]), "r"(x[8]),
+          "r"(x[9]), "r"(x[10]), "r"(x[11]), "r"(x[12]), "r"(x[13]), "r"(x[14]), "r"(x[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&x)[8])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"r"(taddr), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// kind::f16 (bf16) with the A operand in TMEM: a 32-bit column holds two consecutive K elements, the even one low
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// Two fp32 values as three packed pairs of bf16 pieces (x0 in the low half), by truncation: a piece takes the top 8
+// bits of what is left, and three times 8 bits are all 24.
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &p1, uint32_t &p2, uint32_t &p3)
+{
+    const uint32_t a0 = __float_as_uint(x0), a1 = __float_as_uint(x1);
+    p1 = __byte_perm(a0, a1, 0x7632);
+    const float r0 = x0 - __uint_as_float(a0 & 0xffff0000u), r1 = x1 - __uint_as_float(a1 & 0xffff0000u);
+    const uint32_t b0 = __float_as_uint(r0), b1 = __float_as_uint(r1);
+    p2 = __byte_perm(b0, b1, 0x7632);
+    const float s0 = r0 - __uint_as_float(b0 & 0xffff0000u), s1 = r1 - __uint_as_float(b1 & 0xffff0000u);
+    p3 = __byte_perm(__float_as_uint(s0), __float_as_uint(s1), 0x7632);
 }
 
 // Optional self-profiling build (-DSPECA_PROF): cycles CTA 0 spends in each kind of wait, per warp,
@@ -224,19 +258,18 @@ __device__ __forceinline__ bool prof_wait(long long &acc, uint32_t bar, uint32_t
 #endif
 
 
-// TP = value tiles per unit (d_v / 128), DK = key width.
-//
-// Ring entries of a unit, in order: slices (c = 0; t = 0 .. TP-1), value tiles (t = 0 .. TP-1), then slices
-// (c = 1 .. NC-1; t).  For tile t the q-th entry (q = 0: slice 0, q = 1: value tile, q >= 2: slice q - 1) is
-// entry q * TP + t of the unit.
-template <int TP, int DK, int MAXN>
+// Units of up to 32 nodes use the x columns and the space of M as two buffers, so that a tile's second product does
+// not wait for the one before it.
+__device__ __forceinline__ uint32_t x_piece(bool small) { return small ? 16u : 32u; }
+__device__ __forceinline__ uint32_t x_off(bool small, uint32_t q) { return kXOff + ((small && (q & 1)) ? 48u : 0u); }
+
+// TP = value tiles per unit (d_v / 128), DK = key width, MAXN = nodes per sequence, MAXD = tree depth.
+template <int TP, int DK, int MAXN, int MAXD>
 __global__ void __launch_bounds__(kThreads, 1)
 verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid_constant__ EMaps maps, EParams ep)
 {
-    using LY = Lay<TP, DK, MAXN>;
-    constexpr int NS = LY::NS, NC = LY::NC, SC = LY::SC, SCB = LY::SCB, NB = LY::NB;
-    constexpr int NQ = NC + 1;                                    // ring entries per tile and unit
-    constexpr int NE = TP * NQ;                                   // ring entries per unit
+    using LY = Lay<DK, MAXN, MAXD>;
+    constexpr int NS = LY::NS, NC = LY::NC, SC = LY::SC, SCB = LY::SCB;
     extern __shared__ __align__(1024) uint8_t smem[];
     const Params &p = ep.p;
     const uint32_t sbase = smem_u32(smem);
@@ -248,35 +281,31 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
     auto bar = [&](int i) { return bars + 8u * uint32_t(i); };
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + LY::OffMisc);
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + LY::OffMisc + 8);
-    uint8_t *depth_s = smem + LY::OffMisc + 64;          // depth of every node of the unit in the solver's hands
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
-        for (int s = 0; s < kMaxSlots; ++s) {
-            mbar_init(bar(kFull + s), 1);
-            mbar_init(bar(kEmpty + s), 1);
-            mbar_init(bar(kP1Done + s), 2);
-            mbar_init(bar(kLo + s), 4);
-        }
+        for (int s = 0; s < kMaxSlots; ++s) { mbar_init(bar(kFull + s), 1); mbar_init(bar(kEmpty + s), 4); }
+#pragma unroll 1
         for (int i = 0; i < 2; ++i) {
+            mbar_init(bar(kAReady + i), 4);
+            mbar_init(bar(kAFree + i), 1);
             mbar_init(bar(kKQFull + i), 1);
-            mbar_init(bar(kAccFull + i), TP);
-            mbar_init(bar(kPairFree + i), 4);
-            mbar_init(bar(kRecReady + i), 4);
-            mbar_init(bar(kRecFree + i), 4);
+            mbar_init(bar(kKQFree + i), 2);
+            mbar_init(bar(kVFull + i), 1);
+            mbar_init(bar(kVFree + i), 4);
+            mbar_init(bar(kAccFull + i), 1);
+            mbar_init(bar(kAccFree + i), 4);
+            mbar_init(bar(kXReady + i), 4);
+            mbar_init(bar(kOutFull + i), 1);
+            mbar_init(bar(kMReady + i), 4);
+            mbar_init(bar(kMFree + i), 1);
         }
-        for (int i = 0; i < 4; ++i) {
-            mbar_init(bar(kBReady + i), 4);
-            mbar_init(bar(kBFree + i), TP);
-        }
+        mbar_init(bar(kXFree), 1);
         mbar_init(bar(kGramFull), 1);
-        mbar_init(bar(kGramDone), 4);
-        mbar_init(bar(kMReady), 4);
-        mbar_init(bar(kMFree), TP);
-        mbar_init(bar(kSolveSync), 4);
-        mbar_init(bar(kVecSync), 4);
-        mbar_init(bar(kDrain), 2 * TP);
+        mbar_init(bar(kGramFree), 4);
+        mbar_init(bar(kSync), 4);
+        mbar_init(bar(kDrain), 2);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int b = threadIdx.x; b < p.B && b < kWalkSeqs; b += blockDim.x) {
@@ -291,616 +320,448 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
     const uint32_t tmem_base = *tmem_slot;
 
     Walk walk;
-    walk.HG = ep.heads_per_group; walk.gpl = p.H / ep.heads_per_group;
-    walk.n_groups = int(ep.n_units / ep.heads_per_group);
-    walk.H = p.H; walk.B = p.B; walk.grid = int(gridDim.x);
+    walk.HG = ep.heads_per_group; walk.gpl = ep.gpl;
+    walk.L = p.L; walk.B = p.B; walk.H = p.H;
+    walk.dl = ep.dl; walk.db = ep.db; walk.dg = ep.dg;
     walk.two = ep.want_u;
     walk.seq_n = p.ws.seq_n; walk.offs = p.node_offsets;
     walk.tab = smem + LY::OffWalk;
+    VUnit x;                                                     // before the first unit
+    x.kind = 1; x.hi = walk.HG; x.n = 0;
+    x.ng = int(blockIdx.x) % ep.gpl; x.nb = int(blockIdx.x) / ep.gpl % p.B; x.nl = int(blockIdx.x) / ep.gpl / p.B;
+    bool ok = true;
 
     if (warp == 0) {
-        // ------------------------------------------------------------- TMA producer
+        // ------------------------------------------------------------- TMA producer: state slices
         uint32_t it = 0;
-        VUnit x;
-        bool ok = true;
         PROF_DECL
-        for (bool have = first_unit(walk, x); have && ok; have = next_unit(walk, x)) {
-            for (int e = 0; e < NE; ++e, ++it) {
+        while (ok && next_unit(walk, x)) {
+#pragma unroll 1
+            for (int e = 0; e < TP * NC; ++e, ++it) {
                 const int s = it % NS;
                 if (!(ok = WAIT(0, bar(kEmpty + s), ((it / NS) & 1) ^ 1))) break;
-                const uint32_t dst = sbase + LY::OffRing + s * kSliceBytes;
                 if (lane == 0 && !(ep.withhold_first_load && blockIdx.x == 0 && it == 0)) {
-                    if (e >= TP && e < 2 * TP) {
-                        // value rows of tile t: two blocks of 64 values, nodes down the rows
-                        const int t = e - TP;
-                        mbar_arrive_expect_tx(bar(kFull + s), uint32_t(2 * x.npad * 128));
-                        const CUtensorMap *vm = &maps.v[(x.npad >> 4) - 1];
-                        tma_load_3d(dst, vm, t * kRows, x.h, x.l * p.T + x.base, bar(kFull + s));
-                        tma_load_3d(dst + kVBlock, vm, t * kRows + 64, x.h, x.l * p.T + x.base, bar(kFull + s));
-                    } else {
-                        const int c = e < TP ? 0 : (e - TP) / TP, t = e % TP;
-                        mbar_arrive_expect_tx(bar(kFull + s), kSliceBytes);
-                        tma_load_3d(dst, &s0_map, c * 32, t * kRows, x.u, bar(kFull + s));
-                    }
+                    mbar_arrive_expect_tx(bar(kFull + s), kSliceBytes);
+                    tma_load_3d(sbase + LY::OffRing + s * kSliceBytes, &s0_map, (e % NC) * 32, (e / NC) * kRows, x.u, bar(kFull + s));
                 }
                 __syncwarp();
             }
         }
         PROF_STORE()
-        // let copies still in flight land before the CTA's shared memory goes away
-        if (*abort_flag) {
-            const uint64_t t0 = global_timer_ns();
-            while (global_timer_ns() - t0 < 200000ull) __nanosleep(1000);
-        }
-    } else if (warp == 1 || warp == 18) {
-        // ------------------------------------------------------------- first-pass MMA issuers, one warp per value tile
-        // Issuing a tcgen05 instruction costs its thread on the order of a hundred cycles and a unit needs about
-        // a hundred of them, so the work is spread over four warps that never wait for one another and write
-        // disjoint accumulator columns: per tile, this warp issues S x head -> columns [0,R) (kind::tf32, the
-        // slice as landed) and the value term, the second-pass warp the two correction products -> [R,2R).
-        // Warp 1 also issues the Gram blocks.
-        const int mt = warp == 1 ? 0 : 1;                        // tile of this warp
-        bool ok = mt < TP;
+    } else if (warp == 1) {
+        // ------------------------------------------------------------- MMA issuer: S0 [K;Q]^T
+        uint32_t it = 0, q = 0, useq = 0;                        // slices, tiles, units
         PROF_DECL
-        // Gram block of a unit: [K;Q] (128 rows) x K^T (npad columns) from the staged bf16 rows, parked in the
-        // unit's own accumulator columns (tile 0) until its state MMAs overwrite them.
-        auto issue_gram = [&](uint32_t seq, int npad) {
-            const int pr = seq & 1;
-            tc_fence_after();
-            if (lane == 0) {
-                const uint32_t idg = make_idesc_bf16(npad);
-                const uint32_t stage = sbase + LY::OffStage + pr * LY::STAGE;
-#pragma unroll
-                for (int c = 0; c < SC; ++c)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint64_t d = make_desc(stage + c * SCB + k * 32);
-                        mma_bf16(tmem_base + pr * kPairCols, d, d, idg, (c | k) != 0);
-                    }
-                mma_commit(bar(kGramFull));
-            }
-            __syncwarp();
-        };
-        auto gram_ready = [&](uint32_t seq) -> bool {
-            const int pr = seq & 1;
-            const bool a = mbar_test_wait(bar(kKQFull + pr), (seq >> 1) & 1);
-            const bool b = mbar_test_wait(bar(kPairFree + pr), ((seq >> 1) & 1) ^ 1);
-            return __all_sync(0xffffffffu, a && b);
-        };
-        auto gram_wait = [&](uint32_t seq) -> bool {
-            const int pr = seq & 1;
-            return WAIT(5, bar(kKQFull + pr), (seq >> 1) & 1) && WAIT(6, bar(kPairFree + pr), ((seq >> 1) & 1) ^ 1);
-        };
-        VUnit x, nx;
-        uint32_t useq = 0, gram_seq = 0;
-        bool have = ok && first_unit(walk, x);
-        while (have && ok) {
-            nx = x;
-            const bool have_next = next_unit(walk, nx);
-            const int R = x.npad;
-            const uint32_t acc = tmem_base + (useq & 1) * kPairCols + mt * kAccCols;
-            const uint32_t id1 = make_idesc(R);
-            if (mt == 0 && gram_seq == useq) {                   // first unit only: later ones are issued ahead
-                if (!(ok = gram_wait(gram_seq))) break;
-                issue_gram(gram_seq, R);
-                ++gram_seq;
-            }
-            for (int q = 0; q < NQ && ok; ++q) {
-                const uint32_t it = useq * NE + q * TP + mt;
-                const int s = it % NS;
-                const uint32_t ph = (it / NS) & 1;
-                const uint32_t sa = sbase + LY::OffRing + s * kSliceBytes;
-                if (mt == 0 && have_next && gram_seq == useq + 1 && q > 0) {
-                    // the next unit's Gram block: as soon as its rows are staged and its accumulators released, at
-                    // the latest before this unit's last slice, so that the preparation of that unit is never
-                    // queued behind a whole unit of state MMAs
-                    if (q == NQ - 1) {
-                        if (!(ok = gram_wait(gram_seq))) break;
-                        issue_gram(gram_seq, nx.npad);
-                        ++gram_seq;
-                    } else if (gram_ready(gram_seq)) {
-                        issue_gram(gram_seq, nx.npad);
-                        ++gram_seq;
-                    }
-                }
-                if (q == 1) {
-                    // value term: V^T (128 values x R nodes, as landed) x M^T, three bf16 pieces
-                    if (!(ok = WAIT(1, bar(kMReady), useq & 1))) break;
-                    if (!(ok = WAIT(0, bar(kFull + s), ph))) break;
+        for (; ok && next_unit(walk, x); ++useq) {
+            const int par = useq & 1;
+            const uint32_t idm = make_idesc_bf16(2 * x.npad);
+            const uint32_t stage = sbase + LY::OffStage + par * LY::STAGE;
+            if (!(ok = WAIT(0, bar(kKQFull + par), (useq >> 1) & 1))) break;
+#pragma unroll 1
+            for (int t = 0; t < TP && ok; ++t, ++q) {
+                const uint32_t acc = tmem_base + (q & 1) * kTileCols;
+                if (!(ok = WAIT(1, bar(kAccFree + (q & 1)), ((q >> 1) & 1) ^ 1))) break;
+#pragma unroll 1
+                for (int c = 0; c < NC; ++c, ++it) {
+                    const int ab = it & 1;
+                    if (!(ok = WAIT(2, bar(kAReady + ab), (it >> 1) & 1))) break;
                     tc_fence_after();
                     if (lane == 0) {
-                        const uint32_t idv = make_idesc_bf16_amn(R);
-                        const uint32_t mb = sbase + LY::OffM;
-                        for (int piece = 0; piece < 3; ++piece)
-                            for (int ks = 0; ks < R / 16; ++ks)
-                                mma_bf16(acc, make_desc_mn(sa + ks * 2048, kVBlock),
-                                         make_desc(mb + piece * LY::MPIECE + ks * 32), idv, 1);
-                        // every slot visit completes each of its four barriers once, in the same order as for a
-                        // slice (a slot must not come round again before every waiter has seen this visit)
-                        mma_commit(bar(kP1Done + s));
-                        mma_commit(bar(kP1Done + s));
-                        mma_commit(bar(kMFree));
-                    }
-                    __syncwarp();
-                } else {
-                    const int c = q == 0 ? 0 : q - 1;
-                    const uint32_t cc = useq * NC + c;
-                    if (q == 0) {
-                        // the accumulator pair must be released by the epilogue, and the Gram block parked in it read
-                        if (!(ok = WAIT(2, bar(kPairFree + (useq & 1)), ((useq >> 1) & 1) ^ 1))) break;
-                        // (tile 0 only: that is where it is parked, and only this warp keeps step with the solver)
-                        if (mt == 0 && !(ok = WAIT(3, bar(kGramDone), useq & 1))) break;
-                    }
-                    if (!(ok = WAIT(4, bar(kBReady + (cc % NB)), (cc / NB) & 1))) break;
-                    if (!(ok = WAIT(0, bar(kFull + s), ph))) break;
-                    tc_fence_after();
-                    if (lane == 0) {
-                        const uint32_t ba = sbase + LY::OffB + (cc % NB) * LY::BBUF;
+                        const uint32_t a = tmem_base + kAOff + ab * kACols;
+                        const uint64_t bd = make_desc(stage + (c >> 1) * SCB + (c & 1) * 64);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            mma_tf32(acc, make_desc(sa + k * 32), make_desc(ba + k * 32), id1, (c | k) != 0);
-                        mma_commit(bar(kP1Done + s));
+                        for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+                            for (int pc = 0; pc < 3; ++pc)       // (32 bytes further on: 2 in the descriptor's address field)
+                                mma_bf16_ts(acc, a + 16 * pc + 8 * ks, bd + 2 * ks, idm, (c | ks | pc) != 0);
+                        mma_commit(bar(kAFree + ab));
+                        if (c == NC - 1) {
+                            mma_commit(bar(kAccFull + (q & 1)));
+                            if (t == TP - 1) mma_commit(bar(kKQFree + par));
+                        }
                     }
                     __syncwarp();
                 }
             }
-            x = nx;
-            have = have_next;
+        }
+        PROF_STORE()
+    } else if (warp == 2) {
+        // ------------------------------------------------------------- MMA issuer: Gram blocks one unit ahead, x M^T
+        uint32_t q = 0, useq = 0, gseq = 0;
+        VUnit gx = x;
+        PROF_DECL
+        // pass s issues the Gram block of unit s, [K;Q] (128 rows) x K^T (R columns) from the staged rows, and the
+        // products of unit s - 1
+        for (bool first = true; ok; first = false) {
+            if (next_unit(walk, gx)) {
+                const int par = gseq & 1;
+                if (!(ok = WAIT(0, bar(kKQFull + par), (gseq >> 1) & 1))) break;
+                if (!(ok = WAIT(1, bar(kGramFree), (gseq & 1) ^ 1))) break;
+                tc_fence_after();
+                if (lane == 0) {
+                    const uint32_t idg = make_idesc_bf16(gx.npad);
+#pragma unroll 1
+                    for (int c = 0; c < SC; ++c) {
+                        const uint64_t d = make_desc(sbase + LY::OffStage + par * LY::STAGE + c * SCB);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) mma_bf16(tmem_base + kGramOff, d + 2 * k, d + 2 * k, idg, (c | k) != 0);
+                    }
+                    mma_commit(bar(kGramFull));
+                    mma_commit(bar(kKQFree + par));
+                }
+                __syncwarp();
+                ++gseq;
+            }
+            if (first) continue;
+            if (!next_unit(walk, x)) break;
+            const bool small = x.npad <= 32;
+            const int ksteps = x.npad >> 4, mbuf = useq & 1;
+            const uint32_t idx = make_idesc_bf16(x.npad), xps = x_piece(small);
+            if (!(ok = WAIT(2, bar(kMReady + mbuf), (useq >> 1) & 1))) break;
+#pragma unroll 1
+            for (int t = 0; t < TP; ++t, ++q) {
+                if (!(ok = WAIT(3, bar(kXReady + (q & 1)), (q >> 1) & 1))) break;
+                tc_fence_after();
+                if (lane == 0) {
+                    const uint32_t acc = tmem_base + (q & 1) * kTileCols, xa = tmem_base + x_off(small, q);
+                    const uint64_t md = make_desc(sbase + LY::OffM + (small && mbuf ? LY::MBUF2 : 0));
+                    uint32_t on = 0;
+#pragma unroll 1
+                    for (int ks = 0; ks < ksteps; ++ks)
+#pragma unroll
+                        for (int xp = 2; xp >= 0; --xp)           // small products first
+#pragma unroll
+                            for (int mp = 2 - xp; mp >= 0; --mp) {
+                                mma_bf16_ts(acc, xa + xps * xp + 8 * ks, md + uint64_t(mp * (LY::MPIECE >> 4) + 2 * ks), idx, on);
+                                on = 1;
+                            }
+                    mma_commit(bar(kOutFull + (q & 1)));
+                    mma_commit(bar(kXFree));
+                    if (t == TP - 1) mma_commit(bar(kMFree + mbuf));
+                }
+                __syncwarp();
+            }
             ++useq;
         }
         PROF_STORE()
-        // everything this warp issued must have completed before TMEM is released
-        if (mt < TP) {
-            if (lane == 0) mma_commit(bar(kDrain));
-            __syncwarp();
-            mbar_wait(bar(kDrain), 0, abort_flag);
-        }
-    } else if (warp == 19 || warp == 20) {
-        // ------------------------------------------------------------- correction MMA issuers, one warp per value tile
-        // Columns [R,2R) collect the two small products: S x tail while the slice is as landed, then
-        // (S - tf32(S)) x head once it has been rewritten in place.  Two cursors over the tile's slices: whichever
-        // product is ready is issued, so the rewrite of one slice is never waited for while another can go.
-        const int mt = warp - 19;
-        bool ok = mt < TP;
+    } else if (warp == 3) {
+        // ------------------------------------------------------------- TMA producer: staged [K;Q] rows, value rows
+        uint32_t kseq = 0, q = 0;
+        VUnit kx = x;
         PROF_DECL
-        struct Cur { VUnit x; uint32_t useq; int q; bool have; };
-        auto advance = [&](Cur &c, bool skip_values) {
-            if (++c.q == 1 && skip_values) ++c.q;                // value tiles have no product for this warp
-            if (c.q == NQ) { c.q = 0; ++c.useq; c.have = next_unit(walk, c.x); }
-        };
-        Cur f, g;
-        f.useq = 0; f.q = 0;
-        f.have = ok && first_unit(walk, f.x);
-        g = f;
-        uint64_t t0 = 0;
-        uint32_t spin = 0;
-        while (ok && (f.have || g.useq * NQ + g.q < f.useq * NQ + f.q)) {
-            bool prog = false;
-            if (g.useq * NQ + g.q < f.useq * NQ + f.q) {
-                const uint32_t it = g.useq * NE + g.q * TP + mt;
-                const int s = it % NS;
-                if (__all_sync(0xffffffffu, mbar_test_wait(bar(kLo + s), (it / NS) & 1))) {
-                    const int c = g.q == 0 ? 0 : g.q - 1;
-                    const uint32_t cc = g.useq * NC + c;
-                    tc_fence_after();
-                    if (g.q == 1) {
-                        // a value tile: its term has completed (the split warps saw that) and every waiter has seen
-                        // this visit of the slot, so it may come round again
-                        if (lane == 0) mbar_arrive(bar(kEmpty + s));
-                    } else if (lane == 0) {
-                        const int R = g.x.npad;
-                        const uint32_t acc = tmem_base + (g.useq & 1) * kPairCols + mt * kAccCols + R;
-                        const uint32_t sa = sbase + LY::OffRing + s * kSliceBytes;
-                        const uint32_t ba = sbase + LY::OffB + (cc % NB) * LY::BBUF;
-                        const uint32_t idc = make_idesc(R);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) mma_tf32(acc, make_desc(sa + k * 32), make_desc(ba + k * 32), idc, 1);
-                        mma_commit(bar(kEmpty + s));
-                        mma_commit(bar(kBFree + (cc % NB)));
-                        if (c == NC - 1) mma_commit(bar(kAccFull + (g.useq & 1)));
+        for (bool first = true; ok; first = false) {             // staged rows one unit ahead of the value rows
+            if (next_unit(walk, kx)) {
+                const int par = kseq & 1;
+                if (!(ok = WAIT(0, bar(kKQFree + par), ((kseq >> 1) & 1) ^ 1))) break;
+                if (lane == 0) {
+                    const int m = (kx.npad >> 4) - 1, z = kx.l * p.T + kx.base;
+                    const uint32_t stage = sbase + LY::OffStage + par * LY::STAGE;
+                    mbar_arrive_expect_tx(bar(kKQFull + par), uint32_t(4 * kx.npad * DK));
+#pragma unroll 1
+                    for (int c = 0; c < SC; ++c) {
+                        tma_load_3d(stage + c * SCB, &maps.k[m], c * 64, kx.h, z, bar(kKQFull + par));
+                        tma_load_3d(stage + c * SCB + kx.npad * 128, &maps.q[m], c * 64, kx.h, z, bar(kKQFull + par));
                     }
-                    __syncwarp();
-                    advance(g, false);
-                    prog = true;
                 }
+                __syncwarp();
+                ++kseq;
             }
-            if (f.have) {
-                const uint32_t it = f.useq * NE + f.q * TP + mt;
-                const int s = it % NS;
-                const int c = f.q == 0 ? 0 : f.q - 1;
-                const uint32_t cc = f.useq * NC + c;
-                const bool r0 = mbar_test_wait(bar(kFull + s), (it / NS) & 1);
-                const bool r1 = mbar_test_wait(bar(kBReady + (cc % NB)), (cc / NB) & 1);
-                // first slice of a unit: the accumulator pair must be released by the epilogue
-                const bool r2 = f.q != 0 || mbar_test_wait(bar(kPairFree + (f.useq & 1)), ((f.useq >> 1) & 1) ^ 1);
-                if (__all_sync(0xffffffffu, r0 && r1 && r2)) {
-                    tc_fence_after();
-                    if (lane == 0) {
-                        const int R = f.x.npad;
-                        const uint32_t acc = tmem_base + (f.useq & 1) * kPairCols + mt * kAccCols + R;
-                        const uint32_t sa = sbase + LY::OffRing + s * kSliceBytes;
-                        const uint32_t ba = sbase + LY::OffB + (cc % NB) * LY::BBUF + LY::MAXN * 128;
-                        const uint32_t idc = make_idesc(R);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            mma_tf32(acc, make_desc(sa + k * 32), make_desc(ba + k * 32), idc, (c | k) != 0);
-                        mma_commit(bar(kP1Done + s));
-                    }
-                    __syncwarp();
-                    advance(f, true);
-                    prog = true;
+            if (first) continue;
+            if (!next_unit(walk, x)) break;
+#pragma unroll 1
+            for (int t = 0; t < TP; ++t, ++q) {
+                const int vb = q & 1;
+                if (!(ok = WAIT(1, bar(kVFree + vb), ((q >> 1) & 1) ^ 1))) break;
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(bar(kVFull + vb), uint32_t(x.npad * kRows * 2));
+                    tma_load_3d(sbase + LY::OffV + vb * LY::VBUF, &maps.v[(x.npad >> 4) - 1], t * kRows, x.h, x.l * p.T + x.base,
+                                bar(kVFull + vb));
                 }
-            }
-            if (prog) {
-                spin = 0; t0 = 0;
-            } else {
-                // nothing to issue: sleep (up to 400 ns) on the barrier that is due next
-                if (g.useq * NQ + g.q < f.useq * NQ + f.q) {
-                    const uint32_t it = g.useq * NE + g.q * TP + mt;
-                    mbar_try_wait_for(bar(kLo + it % NS), (it / NS) & 1, 400);
-                } else if (f.have) {
-                    const uint32_t it = f.useq * NE + f.q * TP + mt;
-                    mbar_try_wait_for(bar(kFull + it % NS), (it / NS) & 1, 400);
-                }
-                if ((++spin & 255u) == 0u) {
-                    if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
-                    const uint64_t now = global_timer_ns();
-                    if (t0 == 0) t0 = now;
-                    if (__any_sync(0xffffffffu, now - t0 > kWaitLimitNs)) { *abort_flag = 1; ok = false; }
-                }
+                __syncwarp();
             }
         }
         PROF_STORE()
-        if (mt < TP) {
-            if (lane == 0) mma_commit(bar(kDrain));
-            __syncwarp();
-            mbar_wait(bar(kDrain), 0, abort_flag);
-        }
-    } else if (warp < 6) {
-        // ------------------------------------------------------------- solver: Gram block -> records and M
-        const int stid = threadIdx.x - 64;                       // 0..127
-        const int grow = 32 * (warp & 3) + lane;                 // Gram row (= TMEM lane) of this thread
-        const uint32_t lane_addr = uint32_t(32 * (warp & 3)) << 16;
-        float *Gs = reinterpret_cast<float *>(smem + LY::OffGs);    // [level][128 rows]: (row) . k_{a_level}
-        float *alpha_s = reinterpret_cast<float *>(smem + LY::OffAlpha);
-        float *beta_s = alpha_s + 64;
-        uint32_t ssync = 0, useq = 0;
+    } else if (warp < 8) {
+        // ------------------------------------------------------------- split: slice -> three bf16 pieces in TMEM
+        const int row = 32 * (warp & 3) + lane;                  // slice row = TMEM lane of this thread
+        const uint32_t abase = tmem_base + kAOff + (uint32_t(32 * (warp & 3)) << 16);
+        uint32_t it = 0;
         PROF_DECL
-        auto solve_sync = [&]() -> bool {
-            warp_arrive(bar(kSolveSync), lane);
-            const bool r = WAIT(0, bar(kSolveSync), ssync & 1);
-            ++ssync;
-            return r;
-        };
-        // per-thread topology and gates of a unit, fetched one unit ahead
-        int4 meta_n = make_int4(0, 0, 0, 0);
-        int meta2_n = 0;
-        float alpha_n = 0.f, beta_n = 0.f;
-        auto fetch_topo = [&](const VUnit &y) {
-            const int node = grow < y.npad ? grow : grow - y.npad;
-            const bool act = grow < 2 * y.npad && node < y.n;
-            meta_n = act ? __ldg(reinterpret_cast<const int4 *>(p.ws.anc) + y.base + node) : make_int4(0, 0, 0, 0);
-            meta2_n = act ? __ldg(p.ws.anc2 + 4 * (y.base + node)) : 0;
-            if (stid < y.n) {
-                const int r = (y.l * p.T + y.base + stid) * p.H + y.h;
-                alpha_n = __ldg(p.alpha + r);
-                beta_n = __ldg(p.beta + r);
+        while (ok && next_unit(walk, x)) {
+#pragma unroll 1
+            for (int e = 0; e < TP * NC; ++e, ++it) {
+                const int s = it % NS, ab = it & 1;
+                if (!(ok = WAIT(0, bar(kFull + s), (it / NS) & 1))) break;
+                const uint8_t *src = smem + LY::OffRing + s * kSliceBytes + row * 128;
+                uint32_t p1[16], p2[16], p3[16];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float4 v = *reinterpret_cast<const float4 *>(src + ((j ^ (row & 7)) << 4));
+                    split_pair(v.x, v.y, p1[2 * j], p2[2 * j], p3[2 * j]);
+                    split_pair(v.z, v.w, p1[2 * j + 1], p2[2 * j + 1], p3[2 * j + 1]);
+                }
+                warp_arrive(bar(kEmpty + s), lane);
+                if (!(ok = WAIT(1, bar(kAFree + ab), ((it >> 1) & 1) ^ 1))) break;
+                tc_fence_after();
+                const uint32_t dst = abase + ab * kACols;
+                tmem_st16(dst, p1);
+                tmem_st16(dst + 16, p2);
+                tmem_st16(dst + 32, p3);
+                tmem_st_wait();
+                tc_fence_before();
+                warp_arrive(bar(kAReady + ab), lane);
             }
-        };
-        VUnit x, nx;
-        bool ok = true;
-        bool have = first_unit(walk, x);
-        if (have) fetch_topo(x);
-        while (have && ok) {
-            const int par = useq & 1;
-            const int R = x.npad;
-            const int4 meta = meta_n;
-            const int meta2 = meta2_n;
-            const float my_alpha = alpha_n, my_beta = beta_n;
-            nx = x;
-            const bool have_next = next_unit(walk, nx);
-            if (have_next) fetch_topo(nx);
-            // ancestors by level, one byte each; the nodes of the path as a bit set
-            const unsigned long long anc_lo = (unsigned long long)(uint32_t(meta.y)) | ((unsigned long long)(uint32_t(meta.z)) << 32);
-            const unsigned long long anc_hi = (unsigned long long)(uint32_t(meta.w)) | ((unsigned long long)(uint32_t(meta2)) << 32);
-            const bool is_k = grow < R;
-            const int node = is_k ? grow : grow - R;
-            const bool in_rows = grow < 2 * R;
-            const bool active = in_rows && node < x.n;
-            const int d = active ? (meta.x & 0xff) : 0;
-            auto anc = [&](int j) -> int {
-                const int a = int(((j < 8 ? anc_lo : anc_hi) >> (8 * (j & 7))) & 0xffull);
-                return j < d - 1 ? a : node;
-            };
-            unsigned long long path = 0ull;
+        }
+        PROF_STORE()
+    } else if (warp < 16) {
+        // ------------------------------------------------------------- epilogue groups, alternating tiles
+        const int grp = (warp - 8) >> 2;
+        const int row = 32 * (warp & 3) + lane;
+        const uint32_t lane_addr = uint32_t(32 * (warp & 3)) << 16;
+        const uint32_t acc = tmem_base + grp * kTileCols + lane_addr;
+        const size_t stride = size_t(p.H) * p.DV;
+        uint32_t q = 0, useq = 0;
+        bool was_small = false;                                  // the tile before this one
+        PROF_DECL
+        for (; ok && next_unit(walk, x); ++useq) {
+            const int R = x.npad, n = x.n;
+            const bool small = R <= 32;
+            const uint32_t xps = x_piece(small), xb = tmem_base + x_off(small, grp) + lane_addr;
+            const float *gx = reinterpret_cast<const float *>(smem + LY::OffGam) + (useq & 3) * 2 * MAXN, *gf = gx + MAXN;
 #pragma unroll 1
-            for (int j = 0; j < d; ++j) path |= 1ull << anc(j);
-            // gates and depths of this unit's nodes (the previous unit's readers are behind the last sync)
-            if (stid < x.n) { alpha_s[stid] = my_alpha; beta_s[stid] = my_beta; }
-            if (is_k && active) depth_s[node] = uint8_t(d);
-            if (!(ok = solve_sync())) break;
-            if (!(ok = WAIT(4, bar(kGramFull), useq & 1))) break;
-            tc_fence_after();
-            {
+            for (int t = 0; t < TP; ++t, ++q) {
+                const bool shared_x = !(small && was_small);     // x columns shared with the tile before
+                was_small = small;
+                if (int(q & 1) != grp) continue;
+                const uint32_t ph = (q >> 1) & 1;
+                if (!(ok = WAIT(0, bar(kVFull + grp), ph))) break;
+                if (!(ok = WAIT(1, bar(kMReady + (useq & 1)), (useq >> 1) & 1))) break;
+                if (!(ok = WAIT(2, bar(kAccFull + grp), ph))) break;
+                if (shared_x && !(ok = WAIT(3, bar(kXFree), (q & 1) ^ 1))) break;
+                tc_fence_after();
+                {
+                    PROF_T0()
+                    const unsigned short *vt = reinterpret_cast<const unsigned short *>(smem + LY::OffV + grp * LY::VBUF) + row;
+#pragma unroll 1
+                    for (int c0 = 0; c0 < R; c0 += 16) {
+                        float r[16];
+                        tmem_ld16(acc + c0, r);
+                        uint32_t vv[16];
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) vv[i] = vt[(c0 + i) * kRows];
+                        tmem_ld_wait();
+                        uint32_t p1[8], p2[8], p3[8];
+#pragma unroll
+                        for (int i = 0; i < 16; i += 2) {
+                            const float2 gm = *reinterpret_cast<const float2 *>(gx + c0 + i);
+                            // rows past the last node belong to another sequence: they must not reach the product
+                            const float x0 = c0 + i < n ? fmaf(-gm.x, r[i], __uint_as_float(vv[i] << 16)) : 0.f;
+                            const float x1 = c0 + i + 1 < n ? fmaf(-gm.y, r[i + 1], __uint_as_float(vv[i + 1] << 16)) : 0.f;
+                            split_pair(x0, x1, p1[i >> 1], p2[i >> 1], p3[i >> 1]);
+                        }
+                        tmem_st8(xb + (c0 >> 1), p1);
+                        tmem_st8(xb + xps + (c0 >> 1), p2);
+                        tmem_st8(xb + 2 * xps + (c0 >> 1), p3);
+                    }
+                    tmem_st_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) { mbar_arrive(bar(kXReady + grp)); mbar_arrive(bar(kVFree + grp)); }
+                    PROF_ADD(6)
+                }
+                if (!(ok = WAIT(4, bar(kOutFull + grp), ph))) break;
+                tc_fence_after();
                 PROF_T0()
-                // Gram row of this thread, 16 columns at a time: keep the entries against the nodes of its own
-                // path, filed by the level of that node
-                const uint32_t gaddr = tmem_base + par * kPairCols + lane_addr;
+                const size_t rec0 = size_t((x.l * p.T + x.base) * p.H + x.h);
+                float *dst = (x.kind == 0 ? p.o : p.u) + rec0 * p.DV + t * kRows + row;
 #pragma unroll 1
-                for (int c0 = 0; c0 < R; c0 += 16) {
-                    float g16[16];
-                    tmem_ld16(gaddr + c0, g16);
-                    const uint4 dep = *reinterpret_cast<const uint4 *>(depth_s + c0);
+                for (int c0 = 0; c0 < n; c0 += 16) {
+                    float d[16], g[16];
+                    tmem_ld16(acc + c0, d);
+                    tmem_ld16(acc + R + c0, g);
                     tmem_ld_wait();
-                    const uint32_t dw[4] = {dep.x, dep.y, dep.z, dep.w};
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const int lev = int((dw[i >> 2] >> (8 * (i & 3))) & 0xffu) - 1;
-                        if ((path >> (c0 + i)) & 1ull) Gs[lev * kRows + grow] = g16[i];
+                        if (c0 + i < n) *dst = fmaf(gf[c0 + i], g[i], d[i]);
+                        dst += stride;
                     }
                 }
                 tc_fence_before();
-                warp_arrive(bar(kGramDone), lane);               // the state MMAs may now overwrite these columns
-                PROF_ADD(1)
-            }
-            if (!(ok = solve_sync())) break;                     // every row's entries visible
-
-            // Row of X = (I + Ahat)^-1 (key rows, right-hand side e_t) or of C = Phat X (query rows, right-hand
-            // side the row's own q.k entries) by back substitution along the path:
-            //     c_j = rhs_j - sum_{m > j} c_m beta_{a_m} (k_{a_m} . k_{a_j}).
-            // Then the record of operand row `node` (query-row threads on the o walk, key-row threads on the u
-            // walk): weight of k_{a_j} in the effective vector, -front gamma c_j beta_{a_j} (zero without the erase
-            // term), and the row of M: weight of v_{a_j} in the value term, front rho_j c_j beta_{a_j}, as three bf16
-            // pieces.
-            const bool mine = in_rows && (x.kind == 0 ? !is_k : is_k);
-            const float front = x.kind == 0 ? p.scale : 1.f;
-            uint8_t *rr = smem + LY::OffRec + par * kRecBuf + node * kRecBytes;
-            uint8_t *mrow = smem + LY::OffM + (node >> 3) * 1024 + (node & 7) * 128;
-            auto zero_mrow = [&]() {
-#pragma unroll
-                for (int pc = 0; pc < 3; ++pc)
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        *reinterpret_cast<uint4 *>(mrow + pc * LY::MPIECE + i * 16) = make_uint4(0u, 0u, 0u, 0u);
-            };
-            auto put_m = [&](int a, float mv) {
-                const uint32_t moff = uint32_t((((a >> 3) ^ (node & 7)) << 4) + (a & 7) * 2);
-#pragma unroll
-                for (int pc = 0; pc < 3; ++pc) {
-                    const __nv_bfloat16 bq = __float2bfloat16_rn(mv);
-                    *reinterpret_cast<__nv_bfloat16 *>(mrow + pc * LY::MPIECE + moff) = bq;
-                    mv -= __bfloat162float(bq);
-                }
-            };
-            auto put_rec = [&](int j, int a, float w) {
-                *reinterpret_cast<float *>(rr + kRecW + 4 * j) = w;
-                *reinterpret_cast<unsigned short *>(rr + kRecOff + 2 * j) = (unsigned short)((a >> 3) * 1024 + (a & 7) * 128);
-            };
-            float cf[kMaxD];
-            {
-                PROF_T0()
-                if (active) {
-#pragma unroll 1
-                    for (int j = d - 1; j >= 0; --j) {
-                        float acc = is_k ? (j == d - 1 ? 1.f : 0.f) : Gs[j * kRows + grow];
-                        if (!p.no_erase) {
-#pragma unroll 1
-                            for (int m = j + 1; m < d; ++m) {
-                                const int am = anc(m);
-                                acc = fmaf(-cf[m] * beta_s[am], Gs[j * kRows + am], acc);
-                            }
-                        }
-                        cf[j] = acc;
-                    }
-                }
+                warp_arrive(bar(kAccFree + grp), lane);
                 PROF_ADD(7)
-            }
-            if (!(ok = WAIT(3, bar(kRecFree + par), ((useq >> 1) & 1) ^ 1))) break;
-            float gamma = 1.f;
-            if (mine) {
-                int cnt = 0;
-                if (active) {
-#pragma unroll 1
-                    for (int j = 0; j < d; ++j) gamma *= alpha_s[anc(j)];
-#pragma unroll 1
-                    for (int j = 0; j < d; ++j) {
-                        const int a = anc(j);
-                        put_rec(j, a, p.no_erase ? 0.f : -front * gamma * cf[j] * beta_s[a]);
-                    }
-                    cnt = d;
-                    if (x.kind == 0) { put_rec(d, R + node, p.scale * gamma); cnt = d + 1; }
-                }
-                *reinterpret_cast<int *>(rr) = cnt;
-            }
-            warp_arrive(bar(kRecReady + par), lane);
-            if (!(ok = WAIT(5, bar(kMFree), (useq & 1) ^ 1))) break;
-            if (mine) {
-                zero_mrow();
-                if (active) {
-                    float rho = 1.f;
-#pragma unroll 1
-                    for (int j = d - 1; j >= 0; --j) {
-                        const int a = anc(j);
-                        put_m(a, front * rho * cf[j] * beta_s[a]);
-                        rho *= alpha_s[a];
-                    }
-                }
-            }
-            fence_proxy_async();
-            warp_arrive(bar(kMReady), lane);
-            if (!(ok = solve_sync())) break;                     // gates, depths and Gram entries of this unit are dead
-            x = nx;
-            have = have_next;
-            ++useq;
-        }
-        PROF_STORE()
-    } else if (warp < 10) {
-        // ------------------------------------------------------------- effective vectors, one K-slice at a time
-        const int vtid = threadIdx.x - 192;                      // 0..127
-        const int cg = vtid & 3;                                 // 8-column group of the slice
-        uint32_t useq = 0, cc = 0, vsync = 0;
-        PROF_DECL
-        auto load_kq = [&](const VUnit &y, int par) {           // one thread
-            const int m = (y.npad >> 4) - 1;
-            const int z = y.l * p.T + y.base;
-            const uint32_t stage = sbase + LY::OffStage + par * LY::STAGE;
-            mbar_arrive_expect_tx(bar(kKQFull + par), uint32_t(4 * y.npad * DK));
-#pragma unroll
-            for (int c = 0; c < SC; ++c) {
-                tma_load_3d(stage + c * SCB, &maps.k[m], c * 64, y.h, z, bar(kKQFull + par));
-                tma_load_3d(stage + c * SCB + y.npad * 128, &maps.q[m], c * 64, y.h, z, bar(kKQFull + par));
-            }
-        };
-        VUnit x, nx, nx2;
-        bool ok = true;
-        bool have = first_unit(walk, x);
-        if (have && vtid == 0) {
-            nx = x;
-            load_kq(x, 0);
-            if (next_unit(walk, nx)) load_kq(nx, 1);
-        }
-        const bool shallow = p.max_depth <= 8;                  // at most 9 terms per row: fully unrolled form
-        while (have && ok) {
-            const int par = useq & 1;
-            const int R = x.npad;
-            nx = x;
-            const bool have_next = next_unit(walk, nx);
-            nx2 = nx;
-            const bool have_next2 = have_next && next_unit(walk, nx2);
-            if (!(ok = WAIT(3, bar(kKQFull + par), (useq >> 1) & 1))) break;
-            if (!(ok = WAIT(4, bar(kRecReady + par), (useq >> 1) & 1))) break;
-            const uint8_t *stage = smem + LY::OffStage + par * LY::STAGE;
-            const uint8_t *rec = smem + LY::OffRec + par * kRecBuf;
-            for (int c = 0; c < NC; ++c, ++cc) {
-                const int bb = cc % NB;
-                if (!(ok = WAIT(6, bar(kBFree + bb), ((cc / NB) & 1) ^ 1))) break;
-                PROF_T0()
-                const uint8_t *region = stage + (c >> 1) * SCB;
-                const uint32_t slot = uint32_t((c & 1) * 4 + cg);
-                uint8_t *bbuf = smem + LY::OffB + bb * LY::BBUF;
-#pragma unroll 1
-                for (int crow = vtid >> 2; crow < R; crow += 32) {
-                    const uint8_t *rr = rec + crow * kRecBytes;
-                    const int cnt = *reinterpret_cast<const int *>(rr);
-                    float acc[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
-                    auto term = [&](float w, uint32_t off) {
-                        const uint4 raw = *reinterpret_cast<const uint4 *>(region + off + ((slot ^ ((off >> 7) & 7u)) << 4));
-                        acc[0] = fmaf(w, bf_lo(raw.x), acc[0]); acc[1] = fmaf(w, bf_hi(raw.x), acc[1]);
-                        acc[2] = fmaf(w, bf_lo(raw.y), acc[2]); acc[3] = fmaf(w, bf_hi(raw.y), acc[3]);
-                        acc[4] = fmaf(w, bf_lo(raw.z), acc[4]); acc[5] = fmaf(w, bf_hi(raw.z), acc[5]);
-                        acc[6] = fmaf(w, bf_lo(raw.w), acc[6]); acc[7] = fmaf(w, bf_hi(raw.w), acc[7]);
-                    };
-                    if (shallow) {
-                        // all nine loads in flight at once; terms past the end of the record weigh nothing
-#pragma unroll
-                        for (int j = 0; j < 9; ++j) {
-                            const float w = j < cnt ? *reinterpret_cast<const float *>(rr + kRecW + 4 * j) : 0.f;
-                            const uint32_t off = j < cnt ? *reinterpret_cast<const unsigned short *>(rr + kRecOff + 2 * j) : 0u;
-                            term(w, off);
-                        }
-                    } else {
-#pragma unroll 2
-                        for (int j = 0; j < cnt; ++j)
-                            term(*reinterpret_cast<const float *>(rr + kRecW + 4 * j),
-                                 *reinterpret_cast<const unsigned short *>(rr + kRecOff + 2 * j));
-                    }
-                    // head (TF32-rounded) and exact tail, one fp32 row each
-                    float hi[8], lo[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) { hi[i] = round_tf32(acc[i]); lo[i] = acc[i] - hi[i]; }
-                    const uint32_t sw = uint32_t(crow & 7);
-                    uint8_t *d0 = bbuf + (crow >> 3) * 1024 + (crow & 7) * 128;
-                    uint8_t *d1 = d0 + LY::MAXN * 128;
-                    *reinterpret_cast<float4 *>(d0 + (((2 * cg) ^ sw) << 4)) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-                    *reinterpret_cast<float4 *>(d0 + (((2 * cg + 1) ^ sw) << 4)) = make_float4(hi[4], hi[5], hi[6], hi[7]);
-                    *reinterpret_cast<float4 *>(d1 + (((2 * cg) ^ sw) << 4)) = make_float4(lo[0], lo[1], lo[2], lo[3]);
-                    *reinterpret_cast<float4 *>(d1 + (((2 * cg + 1) ^ sw) << 4)) = make_float4(lo[4], lo[5], lo[6], lo[7]);
-                }
-                fence_proxy_async();
-                warp_arrive(bar(kBReady + bb), lane);
-                PROF_ADD(7)
-            }
-            if (!ok) break;
-            warp_arrive(bar(kRecFree + par), lane);              // the records of this unit are dead
-            // every warp of the role has left the staged rows of this unit: request those of the unit after next
-            warp_arrive(bar(kVecSync), lane);
-            if (!(ok = WAIT(0, bar(kVecSync), vsync & 1))) break;
-            ++vsync;
-            if (vtid == 0 && have_next2) load_kq(nx2, par);
-            x = nx;
-            have = have_next;
-            ++useq;
-        }
-        PROF_STORE()
-    } else if (warp < 14) {
-        // ------------------------------------------------------------- TF32 remainder of every slice, in place
-        const int stid = threadIdx.x - 10 * 32;
-        uint32_t it = 0;
-        VUnit x;
-        bool ok = true;
-        PROF_DECL
-        for (bool have = first_unit(walk, x); have && ok; have = next_unit(walk, x)) {
-            for (int e = 0; e < NE; ++e, ++it) {
-                const int s = it % NS;
-                const uint32_t ph = (it / NS) & 1;
-                if (!(ok = WAIT(0, bar(kFull + s), ph))) break;
-                if (e >= TP && e < 2 * TP) {                     // value tiles are not split
-                    if (!(ok = WAIT(1, bar(kP1Done + s), ph))) break;
-                    warp_arrive(bar(kLo + s), lane);
-                    continue;
-                }
-                // the remainders are formed while the first products are still reading the slice; only the stores wait
-                float4 *sl = reinterpret_cast<float4 *>(smem + LY::OffRing + s * kSliceBytes);
-                float4 v[kSliceBytes / 16 / 128];
-#pragma unroll
-                for (int k = 0; k < kSliceBytes / 16 / 128; ++k) {
-                    v[k] = sl[stid + k * 128];
-                    v[k].x = tf32_rest(v[k].x); v[k].y = tf32_rest(v[k].y); v[k].z = tf32_rest(v[k].z); v[k].w = tf32_rest(v[k].w);
-                }
-                if (!(ok = WAIT(1, bar(kP1Done + s), ph))) break;
-#pragma unroll
-                for (int k = 0; k < kSliceBytes / 16 / 128; ++k) sl[stid + k * 128] = v[k];
-                fence_proxy_async();
-                warp_arrive(bar(kLo + s), lane);
             }
         }
         PROF_STORE()
     } else {
-        // ------------------------------------------------------------- epilogue
-        const int row = 32 * (warp & 3) + lane;
-        const uint32_t lane_addr = uint32_t(32 * (warp & 3)) << 16;
-        uint32_t useq = 0;
-        VUnit x;
-        bool ok = true;
+        // ------------------------------------------------------------- solver, one unit ahead
+        const int grow = 32 * (warp & 3) + lane;                 // Gram row (= TMEM lane) of this thread
+        const uint32_t gaddr = tmem_base + kGramOff + (uint32_t(32 * (warp & 3)) << 16);
+        float *Gk = reinterpret_cast<float *>(smem + LY::OffGk), *Gq = reinterpret_cast<float *>(smem + LY::OffGq);
+        constexpr int GSTR = LY::GSTR;
+        uint32_t useq = 0, nsync = 0;
+        bool was_small = false;
         PROF_DECL
-        for (bool have = first_unit(walk, x); have && ok; have = next_unit(walk, x), ++useq) {
-            const int pr = useq & 1;
-            if (!(ok = WAIT(0, bar(kAccFull + pr), (useq >> 1) & 1))) break;
-            tc_fence_after();
-            const int R = x.npad, n = x.n;
-            const size_t rec0 = size_t((x.l * p.T + x.base) * p.H + x.h);
-            float *dst = (x.kind == 0 ? p.o : p.u) + rec0 * p.DV + row;
-            const size_t stride = size_t(p.H) * p.DV;
-#pragma unroll
-            for (int t = 0; t < TP; ++t) {
-                const uint32_t acc = tmem_base + pr * kPairCols + t * kAccCols + lane_addr;
-#pragma unroll 1
-                for (int j0 = 0; j0 < n; j0 += 8) {
-                    float a[8], b[8];
-                    tmem_ld8(acc + j0, a);
-                    tmem_ld8(acc + R + j0, b);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (j0 + i < n) dst[(j0 + i) * stride + t * kRows] = a[i] + b[i];
+        auto role_sync = [&]() -> bool {
+            warp_arrive(bar(kSync), lane);
+            const bool r = WAIT(0, bar(kSync), nsync & 1);
+            ++nsync;
+            return r;
+        };
+        // topology and gates of the node this thread's row belongs to, fetched one unit ahead: its root path upward (one
+        // byte per step, zero past the end), the set of its nodes, its length
+        uint32_t up_n[4] = {0u, 0u, 0u, 0u}, lo_n = 0u, hi_n = 0u;
+        int d_n = 0;
+        float alpha_n = 1.f, beta_n = 0.f;
+        auto fetch_topo = [&](const VUnit &y) {
+            const int node = grow < y.npad ? grow : grow - y.npad;
+            d_n = 0;
+            if (node < y.n) {
+                const int i = y.base + node;
+                if (MAXD <= 8) {
+                    const int2 w = __ldg(reinterpret_cast<const int2 *>(p.ws.up) + 2 * i);
+                    up_n[0] = uint32_t(w.x); up_n[1] = uint32_t(w.y);
+                } else {
+                    const int4 w = __ldg(reinterpret_cast<const int4 *>(p.ws.up) + i);
+                    up_n[0] = uint32_t(w.x); up_n[1] = uint32_t(w.y); up_n[2] = uint32_t(w.z); up_n[3] = uint32_t(w.w);
                 }
+                const int2 s = __ldg(reinterpret_cast<const int2 *>(p.ws.set) + i);
+                lo_n = uint32_t(s.x); hi_n = uint32_t(s.y);
+                d_n = __ldg(p.ws.depth + i);
+                const int r = (y.l * p.T + i) * p.H + y.h;
+                alpha_n = __ldg(p.alpha + r);
+                beta_n = __ldg(p.beta + r);
             }
-            tc_fence_before();
-            warp_arrive(bar(kPairFree + pr), lane);
+        };
+        VUnit nx = x;
+        bool have = next_unit(walk, nx);
+        if (have) fetch_topo(nx);
+        for (; have && ok; ++useq) {
+            x = nx;
+            const int R = x.npad;
+            const bool is_k = grow < R, small = R <= 32;
+            const int node = is_k ? grow : grow - R;
+            const int d = grow < 2 * R ? d_n : 0;                // zero: a row without a node
+            uint32_t up[MAXD / 4];
+#pragma unroll
+            for (int i = 0; i < MAXD / 4; ++i) up[i] = up_n[i];
+            uint32_t set_lo = d > 0 ? lo_n : 0u, set_hi = d > 0 ? hi_n : 0u;
+            float *alpha_s = reinterpret_cast<float *>(smem + LY::OffAB) + (useq & 1) * 2 * MAXN, *beta_s = alpha_s + MAXN;
+            uint8_t *depth_s = smem + LY::OffDepth + (useq & 1) * MAXN;
+            if (is_k) {
+                depth_s[node] = uint8_t(d);
+                alpha_s[node] = alpha_n;
+                beta_s[node] = beta_n;
+                // (the key rows' own entry, distance 0, is not needed)
+                if (node < 32) set_lo &= ~(1u << node);
+                else set_hi &= ~(1u << (node & 31));
+            }
+            auto path = [&](int r) -> int { return int((up[r >> 2] >> (8 * (r & 3))) & 0xffu); };
+            have = next_unit(walk, nx);
+            if (have) fetch_topo(nx);
+            if (!(ok = role_sync())) break;                      // depths and gates visible; the last unit's entries are dead
+
+            // Gram row of this thread, 16 columns at a time: the entries against the nodes of its own path, filed by the
+            // distance up the path
+            if (!(ok = WAIT(1, bar(kGramFull), useq & 1))) break;
+            tc_fence_after();
+            {
+                PROF_T0()
+                float *G = (is_k ? Gk - 1 : Gq) + node * GSTR + d;
+#pragma unroll 1
+                for (int c0 = 0; c0 < R; c0 += 16) {
+                    float g[16];
+                    tmem_ld16(gaddr + c0, g);
+                    const uint4 dep = *reinterpret_cast<const uint4 *>(depth_s + c0);
+                    const uint32_t bits = (c0 & 32 ? set_hi : set_lo) >> (c0 & 16);
+                    tmem_ld_wait();
+                    const uint32_t dw[4] = {dep.x, dep.y, dep.z, dep.w};
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        if (bits & (1u << i)) G[-int((dw[i >> 2] >> (8 * (i & 3))) & 0xffu)] = g[i];
+                }
+                tc_fence_before();
+                warp_arrive(bar(kGramFree), lane);
+                PROF_ADD(5)
+            }
+            if (!(ok = role_sync())) break;                      // every row's entries visible
+
+            // back substitution up the node's own path (entries past its end only ever reach others past the end)
+            float c[MAXD];
+            if (is_k) {
+                PROF_T0()
+#pragma unroll
+                for (int i = 0; i < MAXD / 4; ++i) {
+                    float4 v = make_float4(i == 0 ? 1.f : 0.f, 0.f, 0.f, 0.f);
+                    if (x.kind == 0) v = *reinterpret_cast<const float4 *>(Gq + node * GSTR + 4 * i);
+                    c[4 * i] = v.x; c[4 * i + 1] = v.y; c[4 * i + 2] = v.z; c[4 * i + 3] = v.w;
+                }
+#pragma unroll
+                for (int r = 0; r < MAXD; ++r)
+                    if (r < d) {
+                        const int a = path(r);
+                        c[r] *= beta_s[a];
+                        if (!p.no_erase) {
+                            const float *gr = Gk + a * GSTR;
+#pragma unroll
+                            for (int i = 0; i < MAXD - 1 - r; i += 4) {
+                                const float4 v = *reinterpret_cast<const float4 *>(gr + i);
+                                const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    if (r + 1 + i + e < MAXD) c[r + 1 + i + e] = fmaf(-c[r], f[e], c[r + 1 + i + e]);
+                            }
+                        }
+                    }
+                PROF_ADD(6)
+            }
+            // the buffer of M: used by the unit two before this one, and, where one of them is large, by the last one
+            if (useq >= 2 && !(ok = WAIT(2, bar(kMFree + (useq & 1)), ((useq >> 1) & 1) ^ 1))) break;
+            if (useq >= 1 && !(small && was_small) && !(ok = WAIT(3, bar(kMFree + ((useq & 1) ^ 1)), ((useq - 1) >> 1) & 1))) break;
+            was_small = small;
+            if (is_k) {
+                PROF_T0()
+                // the node's row of M in three bf16 pieces, and its gamma
+                uint8_t *mrow = smem + LY::OffM + (small && (useq & 1) ? LY::MBUF2 : 0) + node * 128;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (8 * i < R)
+#pragma unroll
+                        for (int pc = 0; pc < 3; ++pc)
+                            *reinterpret_cast<uint4 *>(mrow + pc * LY::MPIECE + ((i ^ (node & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+                float rho = x.kind == 0 ? p.scale : 1.f, gam = 1.f;
+#pragma unroll
+                for (int r = 0; r < MAXD; ++r)
+                    if (r < d) {
+                        const int a = path(r);
+                        uint32_t p1, p2, p3;
+                        split_pair(rho * c[r], 0.f, p1, p2, p3);
+                        uint8_t *m = mrow + (((a >> 3) ^ (node & 7)) << 4) + (a & 7) * 2;
+                        *reinterpret_cast<unsigned short *>(m) = (unsigned short)(p1);
+                        *reinterpret_cast<unsigned short *>(m + LY::MPIECE) = (unsigned short)(p2);
+                        *reinterpret_cast<unsigned short *>(m + 2 * LY::MPIECE) = (unsigned short)(p3);
+                        rho *= alpha_s[a];
+                        gam *= alpha_s[a];
+                    }
+                float *gx = reinterpret_cast<float *>(smem + LY::OffGam) + (useq & 3) * 2 * MAXN;
+                gx[node] = p.no_erase ? 0.f : gam;
+                gx[MAXN + node] = x.kind == 0 ? p.scale * gam : 0.f;
+                fence_proxy_async();
+                PROF_ADD(7)
+            }
+            warp_arrive(bar(kMReady + (useq & 1)), lane);
         }
         PROF_STORE()
+    }
+    if (warp == 1 || warp == 2) {
+        // everything these warps issued must have completed before TMEM is released
+        if (lane == 0) mma_commit(bar(kDrain));
+        __syncwarp();
+        mbar_wait(bar(kDrain), 0, abort_flag);
+    }
+    if ((warp == 0 || warp == 3) && *abort_flag) {
+        // let copies still in flight land before the CTA's shared memory goes away
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 200000ull) __nanosleep(1000);
     }
 
     tc_fence_before();
@@ -912,6 +773,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
     }
 }
 
+template <int N> using Int = std::integral_constant<int, N>;
+
 struct DeviceInfo { int sm_count; bool attr_set; };
 DeviceInfo g_dev[64] = {};
 
@@ -921,7 +784,7 @@ bool effective_supported(const speca_dims *d)
 {
     if (d->d_k != 128 && d->d_k != 256) return false;
     if (d->d_v != kRows && d->d_v != 2 * kRows) return false;
-    if (d->max_depth > kMaxD) return false;
+    if (d->max_depth > 16) return false;
     return d->max_nodes <= (d->d_k == 128 ? 64 : 32);
 }
 
@@ -951,7 +814,7 @@ int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
         const cuuint64_t gs[2] = {cuuint64_t(d_k) * 2, cuuint64_t(p.H) * d_k * 2};
         const cuuint64_t vd[3] = {cuuint64_t(p.DV), cuuint64_t(p.H), cuuint64_t(p.L) * cuuint64_t(p.T)};
         const cuuint64_t vs[2] = {cuuint64_t(p.DV) * 2, cuuint64_t(p.H) * p.DV * 2};
-        for (int m = 0; m < 4; ++m) {
+        for (int m = 0; m < 4 && 16 * m < p.max_nodes; ++m) {    // box heights a sequence of this call can need
             const cuuint32_t bx[3] = {64, 1, cuuint32_t(16 * (m + 1))};
             CUresult r1 = encode(&em.k[m], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16 *>(p.k), gd, gs, bx,
                                  es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -959,8 +822,9 @@ int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
             CUresult r2 = encode(&em.q[m], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16 *>(p.q), gd, gs, bx,
                                  es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            CUresult r3 = encode(&em.v[m], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16 *>(p.v), vd, vs, bx,
-                                 es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            const cuuint32_t vx[3] = {kRows, 1, cuuint32_t(16 * (m + 1))};
+            CUresult r3 = encode(&em.v[m], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16 *>(p.v), vd, vs, vx,
+                                 es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS || r3 != CUDA_SUCCESS) return int(cudaErrorInvalidValue);
         }
@@ -979,18 +843,21 @@ int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
         auto opt_in = [&](const void *k, int bytes) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         };
-        opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, 128, 64>), Lay<1, 128, 64>::Bytes);
-        opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, 128, 64>), Lay<2, 128, 64>::Bytes);
-        opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, 128, 32>), Lay<1, 128, 32>::Bytes);
-        opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, 128, 32>), Lay<2, 128, 32>::Bytes);
-        opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, 256, 32>), Lay<1, 256, 32>::Bytes);
-        opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, 256, 32>), Lay<2, 256, 32>::Bytes);
+        auto all = [&](auto dk, auto mn) {
+            constexpr int DK = decltype(dk)::value, MN = decltype(mn)::value;
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, DK, MN, 8>), Lay<DK, MN, 8>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, DK, MN, 8>), Lay<DK, MN, 8>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, DK, MN, 16>), Lay<DK, MN, 16>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, DK, MN, 16>), Lay<DK, MN, 16>::Bytes);
+        };
+        all(Int<128>{}, Int<32>{});
+        all(Int<128>{}, Int<64>{});
+        all(Int<256>{}, Int<32>{});
         if (e != cudaSuccess) return int(e);
         di.attr_set = true;
     }
     EParams ep;
     ep.p = p;
-    ep.n_units = n_units;
     ep.want_u = p.u != nullptr ? 1 : 0;
     ep.withhold_first_load = g_withhold_first_load;
     // consecutive heads of one (layer, sequence) a CTA takes together: as many as divide H while every SM still gets a group
@@ -999,18 +866,22 @@ int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
         if (p.H % hg == 0 && n_units / hg >= di.sm_count) { ep.heads_per_group = hg; break; }
     const long n_groups = n_units / ep.heads_per_group;
     const int grid = int(n_groups < di.sm_count ? n_groups : di.sm_count);
+    ep.gpl = p.H / ep.heads_per_group;
+    ep.dg = grid % ep.gpl;
+    ep.db = grid / ep.gpl % p.B;
+    ep.dl = grid / ep.gpl / p.B;
     const bool one_tile = p.DV == kRows;
+    const bool deep = p.max_depth > 8;
+    auto go = [&](auto dk, auto mn, auto md) {
+        constexpr int DK = decltype(dk)::value, MN = decltype(mn)::value, MD = decltype(md)::value;
+        if (one_tile) verify_effective_kernel<1, DK, MN, MD><<<grid, kThreads, Lay<DK, MN, MD>::Bytes, st>>>(map, em, ep);
+        else verify_effective_kernel<2, DK, MN, MD><<<grid, kThreads, Lay<DK, MN, MD>::Bytes, st>>>(map, em, ep);
+    };
+    auto pick = [&](auto dk, auto mn) { deep ? go(dk, mn, Int<16>{}) : go(dk, mn, Int<8>{}); };
     // a smaller node budget leaves room for a deeper ring of state slices
-    if (d_k == 128 && p.max_nodes > 32) {
-        if (one_tile) verify_effective_kernel<1, 128, 64><<<grid, kThreads, Lay<1, 128, 64>::Bytes, st>>>(map, em, ep);
-        else verify_effective_kernel<2, 128, 64><<<grid, kThreads, Lay<2, 128, 64>::Bytes, st>>>(map, em, ep);
-    } else if (d_k == 128) {
-        if (one_tile) verify_effective_kernel<1, 128, 32><<<grid, kThreads, Lay<1, 128, 32>::Bytes, st>>>(map, em, ep);
-        else verify_effective_kernel<2, 128, 32><<<grid, kThreads, Lay<2, 128, 32>::Bytes, st>>>(map, em, ep);
-    } else {
-        if (one_tile) verify_effective_kernel<1, 256, 32><<<grid, kThreads, Lay<1, 256, 32>::Bytes, st>>>(map, em, ep);
-        else verify_effective_kernel<2, 256, 32><<<grid, kThreads, Lay<2, 256, 32>::Bytes, st>>>(map, em, ep);
-    }
+    if (d_k == 256) pick(Int<256>{}, Int<32>{});
+    else if (p.max_nodes <= 32) pick(Int<128>{}, Int<32>{});
+    else pick(Int<128>{}, Int<64>{});
     return int(cudaGetLastError());
 }
 

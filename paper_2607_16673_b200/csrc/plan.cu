@@ -137,6 +137,14 @@ plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict_
         rec2.y = rec2.z = rec2.w = 0;
         reinterpret_cast<int4 *>(ws.anc)[base + i] = rec;
         reinterpret_cast<int4 *>(ws.anc2)[base + i] = rec2;
+        uint32_t up[4] = {0u, 0u, 0u, 0u}, set[2] = {0u, 0u};
+        int r = 0;
+        for (int a = i; a >= 0; a = par[a], ++r) {
+            if (r < 16) up[r >> 2] |= (uint32_t(a) & 0xffu) << (8 * (r & 3));
+            if (a < 64) set[a >> 5] |= 1u << (a & 31);
+        }
+        reinterpret_cast<int4 *>(ws.up)[base + i] = make_int4(int(up[0]), int(up[1]), int(up[2]), int(up[3]));
+        reinterpret_cast<int2 *>(ws.set)[base + i] = make_int2(int(set[0]), int(set[1]));
     }
     __syncthreads();
     if (tid == 0) {
