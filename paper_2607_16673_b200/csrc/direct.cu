@@ -474,9 +474,11 @@ int direct_limit(const Params &p, int d_k, int most, bool piped)
     if (d_k == 64) return 64;                                // the alternative is the serial walk
     if (!piped) return 32;
     // us per unit and SM in a large batch, this kernel / the pipelined one: d_k = 128, d_v = 256: 3.9 / 5.0 at 8 nodes,
-    // 4.4 / 5.0 at 16, 6.1 / 5.2 at 20..24; d_k = 256: 8.2 / 8.8 at 8, 9.4 / 8.8 at 16.  A single user's 32-node tree,
-    // 24 x 16 units: 22 / 33 us.
-    const int cap = small_batch(p, sm_count_of_current_device()) ? 32 : d_k == 128 ? 16 : 8;
+    // 4.4 / 5.0 at 16, 6.1 / 5.2 at 20..24; d_k = 256: 8.2 / 8.8 at 8, 9.4 / 8.8 at 16.  A few users, us per call with the
+    // plan of the pipelined kernel: d_k = 128, 384 units of 32 nodes 22 / 28; d_k = 256, 192 units of 32 nodes 41 / 35,
+    // 384 units of 16 nodes 45 / 50.
+    const bool few = small_batch(p, sm_count_of_current_device());
+    const int cap = d_k == 128 ? (few ? 32 : 16) : (few ? 16 : 8);
     return most <= cap ? cap : 0;
 }
 
