@@ -92,6 +92,7 @@ int verify_common(const speca_dims *dims, const float *S0, const uint16_t *q, co
         }
     }
     if (!chain || fact || eff || tf32) {
+        p.plan_paths_only = eff;
         // with parent == NULL (chain entry point) the plan kernel assumes parent[i] = i - 1
         rc = cuda_rc(launch_plan(p, st));
         if (rc != SPECA_OK) return rc;

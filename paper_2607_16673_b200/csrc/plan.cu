@@ -20,7 +20,7 @@ constexpr int kPlanThreads = 128;
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict__ parent,
             const int32_t *__restrict__ depth_in, int32_t B, int32_t T, int32_t max_depth,
-            int32_t max_nodes, int32_t skip_nodes, int32_t n_slots, Workspace ws, int32_t *status)
+            int32_t max_nodes, int32_t skip_nodes, int32_t paths_only, int32_t n_slots, Workspace ws, int32_t *status)
 {
     extern __shared__ int32_t sm[];
     const int b = blockIdx.x;
@@ -62,6 +62,32 @@ plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict_
     __syncthreads();
     if (s_flag) {
         if (tid == 0) { atomicOr(status, s_flag); ws.seq_n[b] = -1; }
+        return;
+    }
+    if (paths_only) {
+        // all the effective-query kernel asks for (sequences of at most 64 nodes): the root path of every node, upward and
+        // as a set.  The schedule below takes three more passes over the tree: 11.6 us for 32 trees of 8..64 nodes, this
+        // one 3.5 us, in front of 0.5 ms of verification.
+        int flag = 0;
+        for (int i = tid; i < n; i += kPlanThreads) {
+            uint32_t up[4] = {0u, 0u, 0u, 0u}, lo = 0u, hi = 0u;
+            int d = 0;
+            for (int a = i; a >= 0; a = par[a], ++d) {
+                const uint32_t byte = uint32_t(a) << (8 * (d & 3));
+#pragma unroll
+                for (int w = 0; w < 4; ++w) up[w] |= (d >> 2) == w ? byte : 0u;
+                if (a < 32) lo |= 1u << a;
+                else hi |= 1u << (a - 32);
+            }
+            ws.depth[base + i] = d;
+            reinterpret_cast<int4 *>(ws.up)[base + i] = make_int4(int(up[0]), int(up[1]), int(up[2]), int(up[3]));
+            reinterpret_cast<int2 *>(ws.set)[base + i] = make_int2(int(lo), int(hi));
+            if (d > max_depth) flag |= SPECA_STATUS_TOO_DEEP;
+            if (depth_in != nullptr && depth_in[base + i] != d) flag |= SPECA_STATUS_BAD_DEPTH;
+        }
+        if (flag) atomicOr(status, flag);
+        const int bad = __syncthreads_or(flag);
+        if (tid == 0) ws.seq_n[b] = bad ? -1 : n;
         return;
     }
     // depth and subtree sizes: every node adds itself to all nodes on its root path
@@ -137,14 +163,6 @@ plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict_
         rec2.y = rec2.z = rec2.w = 0;
         reinterpret_cast<int4 *>(ws.anc)[base + i] = rec;
         reinterpret_cast<int4 *>(ws.anc2)[base + i] = rec2;
-        uint32_t up[4] = {0u, 0u, 0u, 0u}, set[2] = {0u, 0u};
-        int r = 0;
-        for (int a = i; a >= 0; a = par[a], ++r) {
-            if (r < 16) up[r >> 2] |= (uint32_t(a) & 0xffu) << (8 * (r & 3));
-            if (a < 64) set[a >> 5] |= 1u << (a & 31);
-        }
-        reinterpret_cast<int4 *>(ws.up)[base + i] = make_int4(int(up[0]), int(up[1]), int(up[2]), int(up[3]));
-        reinterpret_cast<int2 *>(ws.set)[base + i] = make_int2(int(set[0]), int(set[1]));
     }
     __syncthreads();
     if (tid == 0) {
@@ -227,8 +245,43 @@ stochastic_accept_kernel(int32_t B, int32_t max_depth, const int32_t *__restrict
     if (base < 0 || n < 0) fault = SPECA_STATUS_BAD_OFFSETS;
     if (n > 0x10000) fault |= SPECA_STATUS_TOO_MANY;
     auto passes = [&](int t) { return __fmul_rn(uniform[base + t], p_draft[base + t]) < p_target[base + t]; };
+    // Parents and verdicts of up to kStochNodes nodes are staged in shared memory: a walk that chases parents and lower
+    // siblings through global memory is a chain of loads of half a microsecond each (128 trees of 24..64 nodes: 15.0 us,
+    // staged 7.7 us).  Larger sequences are walked in place.
+    constexpr int kStochNodes = 256;
+    __shared__ int16_t s_par[4][kStochNodes];
+    __shared__ uint8_t s_pass[4][kStochNodes], s_chosen[4][kStochNodes];
+    int16_t *par = s_par[threadIdx.x >> 5];
+    uint8_t *ps = s_pass[threadIdx.x >> 5], *chosen = s_chosen[threadIdx.x >> 5];
     int best = -1;                     // (depth << 16) | (0xffff - index) of the deepest node whose root path is all chosen
-    if (!fault) {
+    if (!fault && n <= kStochNodes) {
+        for (int t = lane; t < n; t += 32) {
+            const int pa = parent[base + t];
+            const bool bad = pa < -1 || pa >= t;
+            par[t] = int16_t(bad ? -2 : pa);
+            ps[t] = passes(t);
+        }
+        __syncwarp();
+        // chosen: passing, with no passing sibling of lower index
+        for (int t = lane; t < n; t += 32) {
+            int ok = ps[t];
+            const int pa = par[t];
+            for (int s2 = pa + 1; s2 < t && ok && pa >= -1; ++s2) ok = !(par[s2] == pa && ps[s2]);
+            chosen[t] = uint8_t(ok);
+        }
+        __syncwarp();
+        for (int t = lane; t < n; t += 32) {
+            int d = 0, ok = 1;
+            for (int a = t; a >= 0;) {
+                const int pa = par[a];
+                if (pa < -1) { fault |= SPECA_STATUS_BAD_PARENT; ok = 0; break; }
+                if (!chosen[a]) { ok = 0; break; }
+                if (++d > max_depth) { fault |= SPECA_STATUS_TOO_DEEP; ok = 0; break; }
+                a = pa;
+            }
+            if (ok) best = max(best, (d << 16) | (0xffff - t));
+        }
+    } else if (!fault) {
         for (int t = lane; t < n; t += 32) {
             int d = 0, ok = 1;
             for (int a = t; a >= 0;) {
@@ -341,45 +394,62 @@ conv_commit_kernel(int32_t B, int32_t channels, int32_t W, int32_t T, int32_t ma
     }
 }
 
-// Proposal converter: tree attention mask -> parent array.  One CTA per sequence, thread i owns node i:
-// its parent is the strict ancestor with the most ancestors of its own.  The mask is checked to be the mask
+// Proposal converter: tree attention mask -> parent array.  One CTA per sequence, a warp per row of the mask: the
+// parent of a node is its strict ancestor with the most ancestors of its own.  The mask is checked to be the mask
 // of a tree in topological order (self bit set, no later node among the ancestors, parent exactly one
 // level up); otherwise the sequence gets STATUS_BAD_PARENT and its parents are left untouched.
+// Masks of up to kMaskStage bytes are brought into shared memory first, all loads in flight together: with a thread per
+// row reading global memory, or a warp per row twice over, the kernel is a chain of load latencies (128 masks of 64 x 64:
+// 10.1 us either way, staged 6.4 us).
+constexpr int kMaskStage = 16 * 1024;
 __global__ void __launch_bounds__(256)
 mask_to_parent_kernel(int32_t N, const uint8_t *__restrict__ mask, const int32_t *__restrict__ node_offsets,
                       int32_t *__restrict__ parent, int32_t *status)
 {
     extern __shared__ int32_t sm[];                     // [N] ancestors-or-self per node, [N] parent
-    __shared__ int32_t s_flag;
-    const int b = blockIdx.x;
+    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int base = node_offsets[b], n = node_offsets[b + 1] - base;
-    if (threadIdx.x == 0) s_flag = 0;
-    __syncthreads();
     if (n < 0 || n > N) {
         if (threadIdx.x == 0) atomicOr(status, n < 0 ? SPECA_STATUS_BAD_OFFSETS : SPECA_STATUS_TOO_MANY);
         return;
     }
     const uint8_t *m = mask + size_t(b) * N * N;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        int cnt = 0, bad = m[size_t(i) * N + i] == 0;
-        for (int j = 0; j < n; ++j) {
-            const int on = m[size_t(i) * N + j] != 0;
+    if (n * N <= kMaskStage) {
+        uint8_t *staged = reinterpret_cast<uint8_t *>(sm + 2 * N + ((2 * N) & 3 ? 4 - ((2 * N) & 3) : 0));
+        if ((N & 3) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15u) == 0)          // every mask starts on 16 bytes
+#pragma unroll 4
+            for (int i = threadIdx.x; i < n * N / 16 + (n * N % 16 != 0); i += 256)
+                reinterpret_cast<uint4 *>(staged)[i] = __ldg(reinterpret_cast<const uint4 *>(m) + i);
+        else
+#pragma unroll 8
+            for (int i = threadIdx.x; i < n * N; i += 256) staged[i] = m[i];
+        __syncthreads();
+        m = staged;
+    }
+    int bad = 0;
+    for (int i = warp; i < n; i += 8) {
+        int cnt = 0;
+        for (int j0 = 0; j0 < n; j0 += 32) {
+            const int j = j0 + lane;
+            const int on = j < n && m[size_t(i) * N + j] != 0;
             cnt += on;
-            bad |= on && j > i;
+            bad |= (on && j > i) || (j == i && !on);
         }
-        sm[i] = cnt;
-        if (bad) atomicOr(&s_flag, 1);
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) sm[i] = cnt;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        int best = -1;
-        for (int j = 0; j < n; ++j)
-            if (j != i && m[size_t(i) * N + j] != 0 && (best < 0 || sm[j] > sm[best])) best = j;
-        if (best >= 0 ? sm[best] != sm[i] - 1 : sm[i] != 1) atomicOr(&s_flag, 1);
-        sm[N + i] = best;
+    for (int i = warp; i < n; i += 8) {
+        int best = -1;                                  // (ancestors << 16) | (0xffff - index): the most, then the lowest index
+        for (int j0 = 0; j0 < n; j0 += 32) {
+            const int j = j0 + lane;
+            if (j < n && j != i && m[size_t(i) * N + j] != 0) best = max(best, (sm[j] << 16) | (0xffff - j));
+        }
+        best = __reduce_max_sync(0xffffffffu, best);
+        bad |= best >= 0 ? (best >> 16) != sm[i] - 1 : sm[i] != 1;
+        if (lane == 0) sm[N + i] = best < 0 ? -1 : 0xffff - (best & 0xffff);
     }
-    __syncthreads();
-    if (s_flag) {
+    if (__syncthreads_or(bad)) {
         if (threadIdx.x == 0) atomicOr(status, SPECA_STATUS_BAD_PARENT);
         return;
     }
@@ -441,95 +511,144 @@ chain_decompose_kernel(int32_t N, const int32_t *__restrict__ node_offsets, cons
     if (threadIdx.x == 0) n_chains[b] = s_count;
 }
 
-// Confidence-guided pruning, step 1: one CTA per sequence selects its nodes and writes them, already
-// re-indexed, at the sequence's INPUT offset; out_offsets[b + 1] receives the count.  Scores are
-// accumulated in fp32 in node order, which adds every path root first, exactly as the definition does.
+// Confidence-guided pruning, one CTA per sequence, run twice: first for the number of kept nodes, then for the
+// packed output.  Scores are accumulated in fp32 down the levels of the tree, which adds every path root first, exactly
+// as the definition does.
+//
+// The counts have to become offsets before anything can be written packed, and there is no scratch.  The first
+// run leaves ~count (negative) in out_offsets[b + 1]; in the second, sequence b adds up what it finds in entries
+// 1 .. b -- ~count, or the final offset if that sequence was quicker -- and replaces its own entry by the offset.
+// Every entry is either of the two whenever it is read, so the sum does not depend on who comes first.  (One CTA that
+// packed the sequences in turn took 86 us for 128 of them, its serial selection 15; both runs together 21 us.)
+constexpr int kPruneLevels = 16;
+
+// Calls step(i, parent of i) for every node with a parent, parents first: level by level, all threads of the CTA, for
+// the first kPruneLevels levels; what is deeper is a long chain, which one thread walks in index order.  done[] marks the
+// roots beforehand and everything afterwards.
+template <class Step>
+__device__ __forceinline__ void down_levels(int n, const int32_t *par, int32_t *done, Step step)
+{
+    int open = 1;
+    for (int level = 0; level < kPruneLevels && open; ++level) {
+        open = 0;
+        int ready = 0;                                  // bit k: the node of this thread's k-th turn is final after this level
+        for (int i = threadIdx.x, k = 0; i < n; i += 128, ++k)
+            if (!done[i]) {
+                if (done[par[i]]) { step(i, par[i]); ready |= 1 << k; }
+                else open = 1;
+            }
+        __syncthreads();
+        for (int i = threadIdx.x, k = 0; i < n; i += 128, ++k)
+            if ((ready >> k) & 1) done[i] = 1;
+        open = __syncthreads_or(open);
+    }
+    if (open) {
+        if (threadIdx.x == 0)
+            for (int i = 0; i < n; ++i)
+                if (!done[i]) { step(i, par[i]); done[i] = 1; }
+        __syncthreads();
+    }
+}
+
+template <bool WRITE>
 __global__ void __launch_bounds__(128)
-prune_select_kernel(int32_t N, float tau, int32_t budget, const int32_t *__restrict__ node_offsets,
-                    const int32_t *__restrict__ parent, const float *__restrict__ logp, int32_t *__restrict__ out_offsets,
-                    int32_t *__restrict__ out_parent, int32_t *__restrict__ out_index, int32_t *status)
+prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *__restrict__ node_offsets,
+             const int32_t *__restrict__ parent, const float *__restrict__ logp, int32_t *__restrict__ out_offsets,
+             int32_t *__restrict__ out_parent, int32_t *__restrict__ out_index, int32_t *status)
 {
     extern __shared__ int32_t sm[];
     float *q = reinterpret_cast<float *>(sm);           // [N]
-    int32_t *keep = sm + N, *newidx = sm + 2 * N;       // [N], [N]
-    __shared__ float s_thr;
-    __shared__ int32_t s_fault;
-    const int b = blockIdx.x;
+    int32_t *par = sm + N, *keep = sm + 2 * N, *newidx = sm + 3 * N, *done = sm + 4 * N;      // [N] each
+    __shared__ float s_max[4];
+    __shared__ int32_t s_cnt[4], s_dst;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int base = node_offsets[b], n = node_offsets[b + 1] - base;
-    if (threadIdx.x == 0) {
-        s_fault = 0;
-        if (n < 0 || base < 0) s_fault = SPECA_STATUS_BAD_OFFSETS;
-        else if (n > N) s_fault = SPECA_STATUS_TOO_MANY;
-        else {
-            float best = 0.f;
-            for (int i = 0; i < n; ++i) {
-                const int p = parent[base + i];
-                if (p < -1 || p >= i) { s_fault = SPECA_STATUS_BAD_PARENT; break; }
-                q[i] = (p >= 0 ? q[p] : 0.f) + logp[base + i];
-                best = (i == 0 || q[i] > best) ? q[i] : best;
-            }
-            s_thr = best - tau;
+
+    if (WRITE && warp == 0) {
+        int run = 0;
+        for (int i0 = 1; i0 <= b; i0 += 32) {
+            const int i = i0 + lane;
+            const int v = i <= b ? *reinterpret_cast<volatile int32_t *>(out_offsets + i) : ~0;
+            const unsigned fin = __ballot_sync(0xffffffffu, v >= 0);
+            const int last = 31 - __clz(int(fin));      // the last entry of these that is an offset already (-1: none)
+            const int sum = __reduce_add_sync(0xffffffffu, lane > last ? ~v : 0);
+            const int off = __shfl_sync(0xffffffffu, v, last < 0 ? 0 : last);
+            run = last < 0 ? run + sum : off + sum;
         }
+        if (lane == 0) s_dst = run;
     }
-    __syncthreads();
-    if (s_fault) {
-        if (threadIdx.x == 0) { atomicOr(status, s_fault); out_offsets[b + 1] = 0; }
+
+    int fault = 0;
+    if (n < 0 || base < 0) fault = SPECA_STATUS_BAD_OFFSETS;
+    else if (n > N) fault = SPECA_STATUS_TOO_MANY;
+    else
+        for (int i = tid; i < n; i += 128) {
+            const int p = parent[base + i];
+            if (p < -1 || p >= i) fault = SPECA_STATUS_BAD_PARENT;
+            par[i] = p;
+            q[i] = logp[base + i];
+            done[i] = p < 0;
+        }
+    const bool any_fault = __syncthreads_or(fault);
+    if (any_fault) {
+        if (!WRITE && fault != 0) atomicOr(status, fault);
+        if (tid == 0) *reinterpret_cast<volatile int32_t *>(out_offsets + b + 1) = WRITE ? s_dst : ~0;
+        if (WRITE && b == 0 && tid == 0) out_offsets[0] = 0;
         return;
     }
-    const float thr = s_thr;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    // scores: a node adds its parent's once that one is final
+    down_levels(n, par, done, [&](int i, int p) { q[i] = q[p] + q[i]; });
+    float best = -INFINITY;
+    for (int i = tid; i < n; i += 128) best = fmaxf(best, q[i]);
+    for (int off = 16; off; off >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, off));
+    if (lane == 0) s_max[warp] = best;
+    __syncthreads();
+    best = fmaxf(fmaxf(s_max[0], s_max[1]), fmaxf(s_max[2], s_max[3]));
+    if (n > 0 && q[0] != q[0]) best = q[0];             // a score that is no number in front keeps nothing
+    const float thr = best - tau;
+    for (int i = tid; i < n; i += 128) {
         const float qi = q[i];
         int rank = 0;
+#pragma unroll 4
         for (int j = 0; j < n; ++j) {
             const float qj = q[j];
             rank += (qj >= thr) && (qj > qi || (qj == qi && j < i));
         }
         keep[i] = (qi >= thr) && rank < budget;
+        done[i] = par[i] < 0;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int c = 0;
-        for (int i = 0; i < n; ++i) {
-            const int p = parent[base + i];
-            if (p >= 0 && !keep[p]) keep[i] = 0;
-            newidx[i] = c;
-            c += keep[i];
-        }
-        out_offsets[b + 1] = c;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x)
-        if (keep[i]) {
-            const int p = parent[base + i];
-            out_parent[base + newidx[i]] = p < 0 ? -1 : newidx[p];
-            out_index[base + newidx[i]] = i;
-        }
-}
-
-// Step 2: one CTA turns the counts into offsets and closes the gaps, sequence by sequence in order
-// (a sequence only ever moves toward the front, over space earlier sequences have already left).
-__global__ void __launch_bounds__(256)
-prune_pack_kernel(int32_t B, const int32_t *__restrict__ node_offsets, int32_t *__restrict__ out_offsets,
-                  int32_t *__restrict__ out_parent, int32_t *__restrict__ out_index)
-{
-    __shared__ int32_t s_out;
-    if (threadIdx.x == 0) { s_out = 0; out_offsets[0] = 0; }
-    __syncthreads();
-    for (int b = 0; b < B; ++b) {
-        const int base = node_offsets[b], cnt = out_offsets[b + 1], dst = s_out;
-        __syncthreads();                                 // everyone has read the count before it becomes an offset
-        if (dst != base)
-            for (int i0 = 0; i0 < cnt; i0 += blockDim.x) {
-                const int i = i0 + threadIdx.x;
-                int vp = 0, vi = 0;
-                if (i < cnt) { vp = out_parent[base + i]; vi = out_index[base + i]; }
-                __syncthreads();                         // dst < base: a slice is read before it can be overwritten
-                if (i < cnt) { out_parent[dst + i] = vp; out_index[dst + i] = vi; }
-                __syncthreads();
-            }
-        if (threadIdx.x == 0) { s_out = dst + cnt; out_offsets[b + 1] = dst + cnt; }
+    // a node goes with its parent
+    down_levels(n, par, done, [&](int i, int p) { keep[i] &= keep[p]; });
+    // new indices: kept nodes before this one
+    int count = 0;
+    for (int i0 = 0; i0 < n; i0 += 128) {
+        const int i = i0 + tid;
+        const int on = i < n && keep[i];
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (lane == 0) s_cnt[warp] = __popc(m);
+        __syncthreads();
+        int before = count;
+        for (int w = 0; w < warp; ++w) before += s_cnt[w];
+        if (i < n) newidx[i] = before + __popc(m & ((1u << lane) - 1u));
+        count += s_cnt[0] + s_cnt[1] + s_cnt[2] + s_cnt[3];
         __syncthreads();
     }
+    if (!WRITE) {
+        if (tid == 0) out_offsets[b + 1] = ~count;
+        return;
+    }
+    const int dst = s_dst;
+    if (tid == 0) {
+        *reinterpret_cast<volatile int32_t *>(out_offsets + b + 1) = dst + count;
+        if (b == 0) out_offsets[0] = 0;
+    }
+    for (int i = tid; i < n; i += 128)
+        if (keep[i]) {
+            const int p = par[i];
+            out_parent[dst + newidx[i]] = p < 0 ? -1 : newidx[p];
+            out_index[dst + newidx[i]] = i;
+        }
 }
 
 }  // namespace
@@ -537,7 +656,8 @@ prune_pack_kernel(int32_t B, const int32_t *__restrict__ node_offsets, int32_t *
 int launch_mask_to_parent(int32_t B, int32_t N, const uint8_t *mask, const int32_t *node_offsets, int32_t *parent,
                           int32_t *status, cudaStream_t st)
 {
-    mask_to_parent_kernel<<<B, 256, size_t(2 * N) * sizeof(int32_t), st>>>(N, mask, node_offsets, parent, status);
+    const size_t stage = size_t(N) * N <= kMaskStage ? size_t(N) * N : kMaskStage;
+    mask_to_parent_kernel<<<B, 256, size_t(2 * N) * sizeof(int32_t) + 32 + stage, st>>>(N, mask, node_offsets, parent, status);
     return int(cudaGetLastError());
 }
 
@@ -553,11 +673,13 @@ int launch_prune(int32_t B, int32_t N, float tau, int32_t budget, const int32_t 
                  const float *logp, int32_t *out_offsets, int32_t *out_parent, int32_t *out_index, int32_t *status,
                  cudaStream_t st)
 {
-    prune_select_kernel<<<B, 128, size_t(3 * N) * sizeof(int32_t), st>>>(N, tau, budget, node_offsets, parent, logp,
-                                                                        out_offsets, out_parent, out_index, status);
-    int e = int(cudaGetLastError());
+    const size_t smem = size_t(5 * N) * sizeof(int32_t);
+    prune_kernel<false><<<B, 128, smem, st>>>(N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent, out_index,
+                                              status);
+    const int e = int(cudaGetLastError());
     if (e != 0) return e;
-    prune_pack_kernel<<<1, 256, 0, st>>>(B, node_offsets, out_offsets, out_parent, out_index);
+    prune_kernel<true><<<B, 128, smem, st>>>(N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent, out_index,
+                                             status);
     return int(cudaGetLastError());
 }
 
@@ -581,7 +703,8 @@ int launch_plan(const Params &p, cudaStream_t st)
 {
     const size_t smem = size_t(6 * p.max_nodes + 1) * sizeof(int32_t);
     plan_kernel<<<p.B, kPlanThreads, smem, st>>>(p.node_offsets, p.parent, p.depth_in, p.B, p.T,
-                                                  p.max_depth, p.max_nodes, p.skip_nodes, p.n_slots, p.ws, p.status);
+                                                  p.max_depth, p.max_nodes, p.skip_nodes, p.plan_paths_only,
+                                                  p.n_slots, p.ws, p.status);
     return int(cudaGetLastError());
 }
 

@@ -36,8 +36,8 @@ struct Workspace {
     int32_t *depth;     // [T]   depth computed from parent[]
     int32_t *anc;       // [T][4] per node: depth | position << 8, ancestor node indices of levels 1..12 (one byte each)
     int32_t *anc2;      // [T][4] per node: ancestor node indices of levels 13..15, spare
-    int32_t *up;        // [T][4] per node: its root path upward, itself first, one byte per step (the first 16), zero past the end
-    int32_t *set;       // [T][2] per node: the nodes of its root path as a set (those below 64)
+    int32_t *up;        // (plan_paths_only) [T][4] per node: its root path upward, itself first, one byte per step (the first 16), zero past the end
+    int32_t *set;       // (plan_paths_only) [T][2] per node: the nodes of its root path as a set (those below 64)
     int32_t *pend;      // [B][kPendWords] pending accepted path (fused commit-and-verify only)
 };
 
@@ -98,6 +98,7 @@ struct Params {
     Workspace ws;
     int32_t n_slots;             // on-chip state slots available to the tree walk
     int32_t skip_nodes;          // verify: sequences of at most this many nodes are another kernel's (the plan gives them no nodes)
+    int32_t plan_paths_only;     // plan: root paths upward and as sets instead of the processing order and what goes with it
     int32_t long_min;            // commit: accepted paths of long_min..8 nodes are taken by the tensor-core kernel (0: none)
 };
 

@@ -159,3 +159,39 @@ def test_chain_decompose_matches_the_definition():
     torch.cuda.synchronize()
     assert int(status.item()) & speca.STATUS_BAD_PARENT
     assert cnt.cpu().tolist() == [1, 0, 2] and head.cpu().tolist() == [0, 0, 0, -7, -7, 0, 0, 2]
+
+
+@pytest.mark.parametrize("n_max", [3, 40, 65, 130, 300])
+def test_larger_sequences_and_odd_mask_widths(n_max):
+    """Mask widths that are no multiple of four or too large to stage, sequences beyond a warp's or a CTA's stride, and a
+    chain deeper than the levels the pruning walks together: converter, pruning and stochastic acceptance bit-exact."""
+    rng = np.random.default_rng(70 + n_max)
+    parents = [synth.chain_parent(n_max), np.zeros(0, np.int32)] + \
+              [synth.random_tree_parent(int(n), 12, 4, rng) for n in rng.integers(1, n_max + 1, 6)]
+    offs = np.concatenate([[0], np.cumsum([len(p) for p in parents])]).astype(np.int32)
+    parent, T = np.concatenate(parents).astype(np.int32), int(offs[-1])
+    mask = np.zeros((len(parents), n_max, n_max), np.uint8)
+    for b, p in enumerate(parents):
+        for i, a in enumerate(p):
+            if a >= 0:
+                mask[b, i] = mask[b, a]
+            mask[b, i, i] = 1
+    i32 = dict(dtype=torch.int32, device="cuda")
+    status, got = torch.zeros(1, **i32), torch.full((T,), -7, **i32)
+    speca.tree_mask_to_parent(t(mask), t(offs), got, status)
+    assert np.array_equal(got.cpu().numpy(), parent)
+    logp = np.log(rng.uniform(0.02, 1.0, T)).astype(np.float32)
+    for tau, budget in ((4.0, n_max // 2), (1e4, n_max - 1)):
+        oo, op, oi = torch.zeros(len(parents) + 1, **i32), torch.full((T,), -7, **i32), torch.full((T,), -7, **i32)
+        speca.prune_tree(n_max, tau, budget, t(offs), t(parent), t(logp), oo, op, oi, status)
+        ro, rp, ri = oracle.prune_tree(offs, parent, logp, tau, budget)
+        n = int(ro[-1])
+        assert np.array_equal(oo.cpu().numpy(), ro)
+        assert np.array_equal(op.cpu().numpy()[:n], rp) and np.array_equal(oi.cpu().numpy()[:n], ri)
+    u, pd = rng.random(T).astype(np.float32), rng.uniform(0.1, 1, T).astype(np.float32)
+    pt = (pd * rng.uniform(0.2, 1.0, T)).astype(np.float32)
+    pidx, plen = torch.full((len(parents), 16), -7, **i32), torch.full((len(parents),), -7, **i32)
+    speca.stochastic_accept(len(parents), 16, t(offs), t(parent), t(pt), t(pd), t(u), pidx, plen, status)
+    pi, pl = oracle.stochastic_accept(offs, parent, pt, pd, u, 16)
+    assert np.array_equal(pidx.cpu().numpy(), pi) and np.array_equal(plen.cpu().numpy(), pl)
+    assert int(status.item()) == 0
