@@ -5,10 +5,16 @@ for q, k, v; int32 for topology), checks shapes and dtypes, and passes raw devic
 pointers plus the current CUDA stream to the entry point of the same name.  Nothing
 is computed here and there is no fallback: if ``libspeca.so`` has not been built
 (``python -m paper_2607_16673_b200.build``) every call raises.
+
+The marshalling itself is native (``csrc/marshal.cpp``).  It answers None where an argument is not plainly what the
+entry point wants; the Python code below each call then checks the arguments one by one, to say which one is wrong or to
+convert it.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -17,6 +23,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libspeca.so")
+MARSHAL_PATH = os.path.join(_HERE, "speca_marshal.so")
 
 OK = 0
 STATUS_BAD_PARENT, STATUS_BAD_OFFSETS, STATUS_BAD_PATH, STATUS_TOO_DEEP = 1, 2, 4, 8
@@ -103,6 +110,23 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native = None
+
+
+def _load_native():
+    """The native marshalling, bound to the entry points of libspeca.so."""
+    global _native
+    L = lib()
+    if not os.path.exists(MARSHAL_PATH):
+        raise SpecaError(f"{MARSHAL_PATH} is missing: build it with `python -m paper_2607_16673_b200.build`")
+    loader = importlib.machinery.ExtensionFileLoader("speca_marshal", MARSHAL_PATH)
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("speca_marshal", loader))
+    loader.exec_module(mod)
+    mod.bind({name[len("speca_"):]: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in EXPORTS})
+    _native = mod
+    return mod
+
+
 def _check(rc: int, what: str) -> None:
     if rc != OK:
         raise SpecaError(f"{what}: {lib().speca_strerror(rc).decode()} (code {rc})")
@@ -136,6 +160,9 @@ def alloc_workspace(dims: Dims, total_nodes: int, device="cuda") -> torch.Tensor
 
 
 def decode_step(dims: Dims, S, q, k, v, alpha, beta, o) -> None:
+    rc = (_native or _load_native()).decode_step(dims, S, q, k, v, alpha, beta, o)
+    if rc is not None:
+        return _check(rc, "speca_decode_step")
     L, B, H, dk, dv = dims.n_layers, dims.batch, dims.heads, dims.d_k, dims.d_v
     d = dims.c()
     rc = lib().speca_decode_step(
@@ -156,6 +183,10 @@ def _verify_args(dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes, o, u
 
 
 def verify_chain(dims: Dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes, o, u, workspace, status) -> None:
+    rc = (_native or _load_native()).verify_chain(dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes, o, u,
+                                                  workspace, status)
+    if rc is not None:
+        return _check(rc, "speca_verify_chain")
     ins, outs = _verify_args(dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes, o, u)
     d = dims.c()
     rc = lib().speca_verify_chain(ctypes.byref(d), *ins, int(total_nodes), *outs,
@@ -166,6 +197,10 @@ def verify_chain(dims: Dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes
 
 def verify_tree(dims: Dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes, parent, depth, o, u,
                 workspace, status) -> None:
+    rc = (_native or _load_native()).verify_tree(dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes, parent,
+                                                 depth, o, u, workspace, status)
+    if rc is not None:
+        return _check(rc, "speca_verify_tree")
     ins, outs = _verify_args(dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes, o, u)
     T = int(total_nodes)
     d = dims.c()
@@ -182,6 +217,10 @@ def verify_tree_noalloc(dims: Dims, S0, q, k, v, alpha, beta, node_offsets, tota
     memory: the scratch is a fixed array inside the library (batch <= NOALLOC_MAX_BATCH,
     total_nodes <= NOALLOC_MAX_NODES).  Calls on one device share that array, so calls that
     could overlap on the GPU must be ordered by the caller."""
+    rc = (_native or _load_native()).verify_tree_noalloc(dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes,
+                                                         parent, depth, o, u, status)
+    if rc is not None:
+        return _check(rc, "speca_verify_tree_noalloc")
     ins, outs = _verify_args(dims, S0, q, k, v, alpha, beta, node_offsets, total_nodes, o, u)
     T = int(total_nodes)
     d = dims.c()
@@ -193,6 +232,10 @@ def verify_tree_noalloc(dims: Dims, S0, q, k, v, alpha, beta, node_offsets, tota
 
 def greedy_accept(batch: int, max_depth: int, node_offsets, parent, draft_tok, target_tok, root_target_tok,
                   path_idx, path_len, next_tok, status) -> None:
+    rc = (_native or _load_native()).greedy_accept(batch, max_depth, node_offsets, parent, draft_tok, target_tok,
+                                                   root_target_tok, path_idx, path_len, next_tok, status)
+    if rc is not None:
+        return _check(rc, "speca_greedy_accept")
     i32 = torch.int32
     rc = lib().speca_greedy_accept(
         int(batch), int(max_depth), _ptr(node_offsets, i32, (batch + 1,), "node_offsets"),
@@ -207,6 +250,10 @@ def greedy_accept(batch: int, max_depth: int, node_offsets, parent, draft_tok, t
 def stochastic_accept(batch: int, max_depth: int, node_offsets, parent, p_target, p_draft, uniform,
                       path_idx, path_len, status) -> None:
     """speca_stochastic_accept: the walk over first passing children (uniform * p_draft < p_target)."""
+    rc = (_native or _load_native()).stochastic_accept(batch, max_depth, node_offsets, parent, p_target, p_draft,
+                                                       uniform, path_idx, path_len, status)
+    if rc is not None:
+        return _check(rc, "speca_stochastic_accept")
     i32, f32 = torch.int32, torch.float32
     shape = tuple(parent.shape)
     rc = lib().speca_stochastic_accept(
@@ -219,6 +266,10 @@ def stochastic_accept(batch: int, max_depth: int, node_offsets, parent, p_target
 
 
 def commit(dims: Dims, S, k, v, alpha, beta, node_offsets, total_nodes, parent, path_idx, path_len, status) -> None:
+    rc = (_native or _load_native()).commit(dims, S, k, v, alpha, beta, node_offsets, total_nodes, parent, path_idx,
+                                            path_len, status)
+    if rc is not None:
+        return _check(rc, "speca_commit")
     L, B, H, dk, dv, T = dims.n_layers, dims.batch, dims.heads, dims.d_k, dims.d_v, int(total_nodes)
     i32 = torch.int32
     d = dims.c()
@@ -238,6 +289,11 @@ def commit_verify_tree(dims: Dims, S, prev, path_idx, path_len, q, k, v, alpha, 
     new draft from the committed state.  ``prev`` is None (nothing pending) or a dict with the
     previous draft's ``k, v, alpha, beta`` records, ``u`` (what its verification wrote, or None),
     ``node_offsets``, ``total_nodes`` and ``parent`` (or None)."""
+    rc = (_native or _load_native()).commit_verify_tree(dims, S, prev, path_idx, path_len, q, k, v, alpha, beta,
+                                                        node_offsets, total_nodes, parent, depth, o, u, workspace,
+                                                        status)
+    if rc is not None:
+        return _check(rc, "speca_commit_verify_tree")
     L, B, H, dk, dv, T = dims.n_layers, dims.batch, dims.heads, dims.d_k, dims.d_v, int(total_nodes)
     i32 = torch.int32
     if prev is None:
@@ -269,6 +325,9 @@ def commit_verify_tree(dims: Dims, S, prev, path_idx, path_len, q, k, v, alpha, 
 def commit_conv(C, x, node_offsets, total_nodes, path_idx, path_len, status) -> None:
     """speca_commit_conv: shift the inputs of the accepted nodes into the convolution state.
     C bf16 [L,B,W,channels] (in place), x bf16 [L,T,channels]."""
+    rc = (_native or _load_native()).commit_conv(C, x, node_offsets, total_nodes, path_idx, path_len, status)
+    if rc is not None:
+        return _check(rc, "speca_commit_conv")
     L, B, W, ch = C.shape
     T = int(total_nodes)
     i32 = torch.int32
@@ -282,6 +341,9 @@ def commit_conv(C, x, node_offsets, total_nodes, path_idx, path_len, status) -> 
 
 def tree_mask_to_parent(mask, node_offsets, parent, status) -> None:
     """speca_tree_mask_to_parent: mask uint8 [B,N,N] -> parent int32 [T] (written in place)."""
+    rc = (_native or _load_native()).tree_mask_to_parent(mask, node_offsets, parent, status)
+    if rc is not None:
+        return _check(rc, "speca_tree_mask_to_parent")
     B, N, N2 = mask.shape
     assert N == N2
     rc = lib().speca_tree_mask_to_parent(int(B), int(N), _ptr(mask, torch.uint8, (B, N, N), "mask"),
@@ -295,6 +357,10 @@ def prune_tree(max_nodes: int, tau: float, budget: int, node_offsets, parent, lo
                out_index, status) -> None:
     """speca_prune_tree: keep the nodes within tau of the best cumulative log-probability, at most
     `budget` per sequence; packed outputs."""
+    rc = (_native or _load_native()).prune_tree(max_nodes, tau, budget, node_offsets, parent, logp, out_offsets,
+                                                out_parent, out_index, status)
+    if rc is not None:
+        return _check(rc, "speca_prune_tree")
     i32 = torch.int32
     B = node_offsets.numel() - 1
     T = parent.numel()
@@ -308,6 +374,9 @@ def prune_tree(max_nodes: int, tau: float, budget: int, node_offsets, parent, lo
 
 def chain_decompose(max_nodes: int, node_offsets, parent, chain_head, n_chains, status) -> None:
     """speca_chain_decompose: heavy-light chains; chain_head[t] = first node of t's chain, n_chains per sequence."""
+    rc = (_native or _load_native()).chain_decompose(max_nodes, node_offsets, parent, chain_head, n_chains, status)
+    if rc is not None:
+        return _check(rc, "speca_chain_decompose")
     i32 = torch.int32
     B = node_offsets.numel() - 1
     T = parent.numel()

@@ -1,7 +1,8 @@
-"""Compile libspeca.so (the CUDA library behind the C ABI) for sm_100a with nvcc.
+"""Compile libspeca.so (the CUDA library behind the C ABI) for sm_100a with nvcc, and speca_marshal.so (the binding's
+argument marshalling, against torch's headers) with the host compiler.
 
-Run as ``python -m paper_2607_16673_b200.build``.  The shared object is written
-next to this file, so it travels with the source tree.  nvcc cross-compiles without a GPU.
+Run as ``python -m paper_2607_16673_b200.build``.  The shared objects are written
+next to this file, so they travel with the source tree.  nvcc cross-compiles without a GPU.
 """
 from __future__ import annotations
 
@@ -13,6 +14,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libspeca.so")
+MARSHAL = os.path.join(HERE, "speca_marshal.so")
 SOURCES = ["api.cu", "plan.cu", "serial.cu", "commit_mma.cu", "direct.cu", "factorized.cu", "effective.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 
@@ -30,10 +32,25 @@ def _newest_source_mtime() -> float:
     return max(os.path.getmtime(d) for d in deps)
 
 
+def _start_marshal(tmp: str) -> subprocess.Popen:
+    import sysconfig
+
+    from torch.utils import cpp_extension
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    inc = [sysconfig.get_paths()["include"], *cpp_extension.include_paths(), os.path.join(cuda, "include")]
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-DUSE_CUDA", *[f"-I{d}" for d in inc],
+           os.path.join(CSRC, "marshal.cpp"), "-o", tmp, *[f"-L{d}" for d in cpp_extension.library_paths()],
+           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
+    newest = _newest_source_mtime()
+    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= newest for f in (LIB, MARSHAL)):
         return LIB
     nvcc = _nvcc()
+    marshal_tmp = MARSHAL + f".tmp{os.getpid()}"
+    marshal = _start_marshal(marshal_tmp)
     objdir = os.path.join(HERE, "build")
     os.makedirs(objdir, exist_ok=True)
     # no --use_fast_math: IEEE fp32 arithmetic everywhere, parity is judged on it
@@ -49,15 +66,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
         procs.append((src, subprocess.Popen([nvcc, *flags, "-c", os.path.join(CSRC, src), "-o", obj],
                                             stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
-    for src, pr in procs:
+    for src, pr in procs + [("marshal.cpp", marshal)]:
         out, _ = pr.communicate()
         if out.strip():
             print(f"--- {src}\n{out}", file=sys.stderr)
         failed |= pr.returncode != 0
     if failed:
-        raise RuntimeError("nvcc failed")
+        raise RuntimeError("compilation failed")
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.run([nvcc, "-shared", *ARCH, "-o", tmp, *objs, "-lcudart"], check=True)
+    os.replace(marshal_tmp, MARSHAL)
     os.replace(tmp, LIB)
     return LIB
 
