@@ -23,14 +23,14 @@
 //
 // A CTA takes one unit (layer, sequence, head) or a slice of its value rows and checks the topology of its sequence
 // itself (one parent walk per node), so no plan kernel runs in front of it.  It asks the first rows of its tile into L2
-// with one bulk prefetch before it knows anything else, so that the set-up runs under the latency of HBM and the loop
+// with one bulk prefetch, so that the set-up runs under the latency of HBM and the loop
 // over 16-row tiles needs two 32-column steps of registers in flight, not whole tiles: 24 warps fit an SM.  Holding
 // whole tiles in registers through the set-up (16 warps) took 5.1 us per 8-node unit and SM instead of 3.9, at 16
 // nodes 8.0 instead of 4.4.
-// Measured (d_k = 128, d_v = 256, 12288 units): 8 nodes 322 us = 5.6 TB/s (pipelined kernel 448 us), 16 nodes 361 us =
-// 5.6 TB/s (457); d_k = d_v = 64, 24576 units of 8 / 16 / 32 nodes: 154 / 212 / 342 us (serial walk 343 / 645 / 1364).
-// What bounds it: the state stream up to 8 nodes (87 % of the copy rate), above that also the shared-memory reads of the
-// vectors (two 16-byte loads per six MMAs and lane) and, at 32 nodes, two CTAs' worth of warps to hide a longer set-up.
+// Measured (d_k = 128, d_v = 256, 12288 units): 8 nodes 301 us = 6.0 TB/s (pipelined kernel 411 us), 16 nodes 337 us =
+// 6.0 TB/s (417); d_k = d_v = 64, 24576 units of 8 / 16 / 32 nodes: 154 / 212 / 342 us (serial walk 343 / 645 / 1364).
+// What bounds it: the state stream up to 16 nodes (93 % of the copy rate), above that the set-up (a chain of about ten
+// latencies, 6-9 us of a CTA's life) and at 32 nodes the MMAs.  For a few users, 384 chains of 8: 10.4 us.
 #include <atomic>
 
 #include "speca_common.cuh"
@@ -85,7 +85,7 @@ __device__ __forceinline__ void cp16(void *dst, const void *src, bool live)
 }
 
 // Shared memory of one CTA (bytes); N = 8 NT nodes at most, `rows` value rows.
-template <int DK, int NT> struct Lay {
+template <int DK, int NT, int MAXD> struct Lay {
     static constexpr int N = 8 * NT;
     static constexpr int NK = (N + 15) & ~15;                   // contraction width of the value term
     static constexpr int KQS = DK + 8;                          // bf16 per staged key / query row (16 bytes of padding)
@@ -100,7 +100,13 @@ template <int DK, int NT> struct Lay {
     static constexpr int OffG = OffHi;                          // float [2N][GS]: Gram rows of keys, queries (dead before Hi is written)
     static constexpr int OffW = OffM + 3 * N * MS * 2;          // bf16 [3][NR][MS]: weights of the keys in qeff
     static constexpr int OffP = OffW + 3 * NR * MS * 2;         // int32 parent[N], float alpha[N], beta[N], scale gamma[NR]
-    static constexpr int OffV = OffP + (3 * N + NR) * 4;        // bf16 [NK][rows + 8]
+    // rows of the back substitution: float c beta [N][MAXD], float rho [N][MAXD], uint8 path [N][MAXD]; behind the Gram
+    // rows where those leave room, and as dead as they are afterwards
+    static constexpr int GEnd = (OffG + 2 * N * GS * 4 + 15) & ~15, CBytes = 9 * N * MAXD;
+    static constexpr bool kFits = GEnd + CBytes <= OffHi + 2 * N * BS * 4;
+    static constexpr int POwn = OffP + (3 * N + NR) * 4;
+    static constexpr int OffC = kFits ? GEnd : POwn;
+    static constexpr int OffV = kFits ? POwn : POwn + CBytes;   // bf16 [NK][rows + 8]
     static_assert(2 * N * GS <= 2 * N * BS, "Gram rows do not fit the space of the effective queries");
     static constexpr int bytes(int rows) { return OffV + NK * (rows + 8) * 2; }
 };
@@ -109,14 +115,14 @@ struct DirectArgs {
     Params p;
     int32_t parts, rows;        // value-row slices per unit, rows per slice
     int32_t lo;                 // sequences of at most this many nodes belong to another launch
-    int32_t all;                // no sequence of the call can be outside (lo, 8 NT]
+    int32_t early;              // ask for the state before the records: see launch_one
 };
 
 template <int DK, int NT, int MAXD, int WARPS, int CTAS>
 __global__ void __launch_bounds__(WARPS * 32, CTAS)
 verify_direct_kernel(DirectArgs da)
 {
-    using LY = Lay<DK, NT>;
+    using LY = Lay<DK, NT, MAXD>;
     constexpr int N = LY::N, NS = DK / 32, THREADS = WARPS * 32;
     extern __shared__ __align__(16) uint8_t smem[];
     const Params &p = da.p;
@@ -134,7 +140,7 @@ verify_direct_kernel(DirectArgs da)
     auto prefetch_first = [&]() {
         if (tid == 0) prefetch_l2(S_cta, uint32_t(min(tiles, AHEAD)) * (16 * DK * 4));
     };
-    if (da.all) prefetch_first();
+    if (da.early) prefetch_first();
 
     const int base = __ldg(p.node_offsets + b), end = __ldg(p.node_offsets + b + 1);
     const int n = end - base;
@@ -152,8 +158,6 @@ verify_direct_kernel(DirectArgs da)
         return;
     }
     if (n <= da.lo || n > N) return;                         // nothing to do, or another launch's
-    if (!da.all) prefetch_first();
-
     __nv_bfloat16 *sKQ = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffKQ);
     float *sHi = reinterpret_cast<float *>(smem + LY::OffHi), *sLo = reinterpret_cast<float *>(smem + LY::OffLo);
     __nv_bfloat16 *sM = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffM);
@@ -161,6 +165,8 @@ verify_direct_kernel(DirectArgs da)
     __nv_bfloat16 *sW = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffW);
     int *sPar = reinterpret_cast<int *>(smem + LY::OffP);
     float *sAl = reinterpret_cast<float *>(sPar + N), *sBe = sAl + N, *sGam = sBe + N;
+    float *sC = reinterpret_cast<float *>(smem + LY::OffC);
+    uint8_t *sPath = smem + LY::OffC + 8 * N * MAXD;
     __nv_bfloat16 *sV = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffV);
     const int vstride = da.rows + 8;
     const int nt = (n + 7) >> 3;
@@ -168,6 +174,13 @@ verify_direct_kernel(DirectArgs da)
     const int H = p.H;
 
     // ---- the sequence's records -> shared memory; rows past the last node are zero
+    int pa = -1, fault = 0;
+    float al = 1.f, be = 0.f;
+    if (tid < n) {
+        pa = p.parent != nullptr ? __ldg(p.parent + base + tid) : tid - 1;
+        al = __ldg(p.alpha + rec0 + long(tid) * H);
+        be = __ldg(p.beta + rec0 + long(tid) * H);
+    }
     {
         constexpr int PCS = DK / 8;
         for (int i = tid; i < 2 * 8 * nt * PCS; i += THREADS) {
@@ -186,17 +199,16 @@ verify_direct_kernel(DirectArgs da)
             cp16(sV + node * vstride + 8 * c, p.v + (rec0 + long(live ? node : 0) * H) * p.DV + row0 + 8 * c, live);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
+        if (!da.early) prefetch_first();
         for (int i = tid; i < 3 * N * LY::MS / 8; i += THREADS) reinterpret_cast<uint4 *>(sM)[i] = make_uint4(0u, 0u, 0u, 0u);
         for (int i = tid; i < 3 * LY::NR * LY::MS / 8; i += THREADS) reinterpret_cast<uint4 *>(sW)[i] = make_uint4(0u, 0u, 0u, 0u);
         if (tid < LY::NR) sGam[tid] = 0.f;
     }
-    int fault = 0;
     if (tid < n) {
-        const int pa = p.parent != nullptr ? __ldg(p.parent + base + tid) : tid - 1;
         if (pa < -1 || pa >= tid) fault = SPECA_STATUS_BAD_PARENT;
         sPar[tid] = pa;
-        sAl[tid] = __ldg(p.alpha + rec0 + long(tid) * H);
-        sBe[tid] = __ldg(p.beta + rec0 + long(tid) * H);
+        sAl[tid] = al;
+        sBe[tid] = be;
     }
     asm volatile("cp.async.wait_group 1;" ::: "memory");     // keys and queries; the value rows may still be in flight
     if (__syncthreads_or(fault)) {
@@ -260,28 +272,47 @@ verify_direct_kernel(DirectArgs da)
             }
             acc[r] = cb;
         }
-        auto put = [&](__nv_bfloat16 *row, int piece, int col, float x) {
-#pragma unroll
-            for (int pc = 0; pc < 3; ++pc) {
-                const __nv_bfloat16 q = __float2bfloat16_rn(x);
-                row[pc * piece + col] = q;
-                x -= __bfloat162float(q);
-            }
-        };
         float rho = p.scale;
+        float *cb = sC + tid * MAXD, *ro = cb + N * MAXD;
 #pragma unroll
-        for (int r = 0; r < MAXD; ++r)
-            if (r < d) {
-                put(sM + tid * LY::MS, N * LY::MS, path[r], rho * acc[r]);
-                rho *= sAl[path[r]];
-            }
+        for (int r = 0; r < MAXD; ++r) {
+            cb[r] = acc[r];
+            ro[r] = rho;
+            sPath[tid * MAXD + r] = uint8_t(r < d ? path[r] : 0xff);
+            rho *= r < d ? sAl[path[r]] : 1.f;
+        }
         sGam[tid] = rho;                                     // scale gamma
-        if (!p.no_erase)
-#pragma unroll
-            for (int r = 0; r < MAXD; ++r)
-                if (r < d) put(sW + tid * LY::MS, LY::NR * LY::MS, path[r], -rho * acc[r]);
     }
     __syncthreads();
+    // the weights of value rows (M) and keys (W) in three bf16 pieces: every thread of the CTA takes its share, one node
+    // and step up the path at a time (left to the thread of each node this was two thirds of the phase)
+    for (int i = tid; i < n * MAXD; i += THREADS) {
+        const int a = sPath[i];
+        if (a == 0xff) continue;
+        const int node = i / MAXD;
+        const float cb = sC[i];
+        float m = sC[N * MAXD + i] * cb, w = p.no_erase ? 0.f : -sGam[node] * cb;
+        __nv_bfloat16 *md = sM + node * LY::MS + a, *wd = sW + node * LY::MS + a;
+#pragma unroll
+        for (int pc = 0; pc < 3; ++pc) {
+            const __nv_bfloat16 mq = __float2bfloat16_rn(m), wq = __float2bfloat16_rn(w);
+            md[pc * N * LY::MS] = mq;
+            wd[pc * LY::NR * LY::MS] = wq;
+            m -= __bfloat162float(mq);
+            w -= __bfloat162float(wq);
+        }
+    }
+    __syncthreads();
+
+    // the first two steps of this warp's first tile, requested a phase ahead of their use
+    const float *Su = S_cta + g * DK + 8 * t4;
+    float sa[2][8], sb[2][8];
+    if (warp < tiles)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            ld_state(sa[q], Su + warp * 16 * DK + 32 * q);
+            ld_state(sb[q], Su + (warp * 16 + 8) * DK + 32 * q);
+        }
 
     // ---- effective queries (scale gamma q + W K, the weights in three bf16 pieces), split into head and remainder
     {
@@ -332,18 +363,10 @@ verify_direct_kernel(DirectArgs da)
     // ---- the state: one 16-row tile at a time, two 32-column steps of registers in flight
     // lane (g, t) holds columns 32 q + 8 t .. + 7 of rows g and g + 8: k-steps e = 0..3 of the step contract
     // columns 8 t + 2 e and 8 t + 2 e + 1 of the four lanes
-    const float *Su = S_cta + g * DK + 8 * t4;
     const float *hi_p = sHi + g * LY::BS + 8 * t4, *lo_p = sLo + g * LY::BS + 8 * t4;
     const int nk = (n + 15) >> 4;
     float *o0 = p.o + rec0 * p.DV + row0 + g;
     const long node_stride = long(H) * p.DV;
-    float sa[2][8], sb[2][8];
-    if (warp < tiles)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            ld_state(sa[q], Su + warp * 16 * DK + 32 * q);
-            ld_state(sb[q], Su + (warp * 16 + 8) * DK + 32 * q);
-        }
 #pragma unroll 1
     for (int tile = warp; tile < tiles; tile += WARPS) {
         if (lane == 0 && tile + AHEAD < tiles) prefetch_l2(S_cta + long(tile + AHEAD) * 16 * DK, 16 * DK * 4);
@@ -416,14 +439,21 @@ verify_direct_kernel(DirectArgs da)
     }
 }
 
+// A batch that fills the device's resident CTAs only once or twice is latency, not throughput.
+bool small_batch(const Params &p, int sms) { return long(p.L) * p.B * p.H <= 4L * sms; }
+
 template <int DK, int NT, int MAXD, int WARPS, int CTAS>
 int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
 {
-    using LY = Lay<DK, NT>;
+    using LY = Lay<DK, NT, MAXD>;
     DirectArgs da;
     da.p = p;
     da.lo = lo;
-    da.all = all ? 1 : 0;
+    // Asking for the state before anything else is known keeps HBM busy in a large batch (12288 units of 8 nodes, d_k = 128,
+    // d_v = 256: 301 us, after the records 320).  Where all CTAs start at once, or a tile is small, the records then
+    // queue behind the state, and the set-up waits for them (384 chains of 8: 11.8 us, after the records 10.4; 4608
+    // units of 32 nodes at d_k = d_v = 64: 67.8 / 65.8).
+    da.early = all && DK > 64 && !small_batch(p, sms);
     // value rows per CTA: the whole unit, halved while the device would be left with idle slots
     const long units = long(p.L) * p.B * p.H;
     int rows = p.DV;
@@ -461,9 +491,6 @@ int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_
         return launch_one<DK, 4, MAXD, 8, 2>(p, lo, all, sms, st);
     }
 }
-
-// A batch that fills the device's resident CTAs only once or twice is latency, not throughput.
-bool small_batch(const Params &p, int sms) { return long(p.L) * p.B * p.H <= 4L * sms; }
 
 }  // namespace
 
