@@ -29,8 +29,8 @@
 //   warp 2        issues the Gram blocks [K;Q] K^T (one unit ahead) and x M^T
 //   warp 3        TMA producer of the staged [K;Q] rows (two units) and the value rows (two tiles)
 //   warps 4-7     split: slice row per thread -> three bf16 pieces in TMEM (two buffers)
-//   warps 8-15    two epilogue groups, alternating tiles: R out of TMEM, x back into TMEM as three pieces; then
-//                 o = scale gamma G + (x M^T), coalesced
+//   warps 8-15    epilogue, two warps per TMEM lane quarter that share a tile's columns: R out of TMEM, x back into TMEM
+//                 as three pieces; then, while the next tile's product runs, o = scale gamma G + (x M^T), coalesced
 //   warps 16-19   solver, one unit ahead: Gram entries of every row against its own path, back substitution (a thread
 //                 per node, registers), the pieces of M
 // TMEM: two tiles of accumulators (R | G, 128 columns; x M^T overwrites R), two A buffers of 48, x of 96, Gram of 64.
@@ -58,7 +58,7 @@ constexpr int kWalkSeqs = 128;
 // TMEM columns
 constexpr int kTileCols = 128;                  // accumulators of a tile: R, then G
 constexpr int kAOff = 2 * kTileCols, kACols = 48;    // two buffers of three 16-column pieces (32 bf16 columns each)
-constexpr int kXOff = kAOff + 2 * kACols;       // x: three 32-column pieces (64 nodes), or two buffers of three 16-column pieces
+constexpr int kXOff = kAOff + 2 * kACols;       // x: three 32-column pieces (64 nodes)
 constexpr int kGramOff = kXOff + 96;
 constexpr int kTmemCols = 512;
 static_assert(kGramOff + 64 == kTmemCols, "TMEM columns");
@@ -108,12 +108,12 @@ enum Bar {
     kVFree = kVFull + 2,               // [2] epilogue -> TMA
     kAccFull = kVFree + 2,             // [2] MMA -> epilogue: R and G of a tile
     kAccFree = kAccFull + 2,           // [2] epilogue -> MMA
-    kXReady = kAccFree + 2,            // [2] epilogue -> MMA: x of a tile in TMEM, R read
-    kXFree = kXReady + 2,              // MMA -> epilogue
-    kOutFull,                          // [2] MMA -> epilogue: x M^T of a tile
+    kXReady = kAccFree + 2,            // epilogue -> MMA: x of a tile in TMEM, R read
+    kOutFull,                          // [2] MMA -> epilogue: x M^T of a tile complete, its x no longer read
     kGramFull = kOutFull + 2,          // MMA -> solver
     kGramFree,                         // solver -> MMA
-    kMReady,                           // [2] solver -> MMA, epilogue: M and gamma of a unit
+    kGamReady,                         // [2] solver -> epilogue: gamma of a unit
+    kMReady = kGamReady + 2,           // [2] solver -> MMA: M of a unit
     kMFree = kMReady + 2,              // [2] MMA -> solver
     kSync = kMFree + 2,                // solver, role-internal
     kDrain,
@@ -199,10 +199,9 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&x)[16
           "r"(x[9]), "r"(x[10]), "r"(x[11]), "r"(x[12]), "r"(x[13]), "r"(x[14]), "r"(x[15])
         : "memory");
 }
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&x)[8])
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&x)[4])
 {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                 ::"r"(taddr), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7])
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3])
                  : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -220,13 +219,13 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
 // bits of what is left, and three times 8 bits are all 24.
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &p1, uint32_t &p2, uint32_t &p3)
 {
-    const uint32_t a0 = __float_as_uint(x0), a1 = __float_as_uint(x1);
-    p1 = __byte_perm(a0, a1, 0x7632);
-    const float r0 = x0 - __uint_as_float(a0 & 0xffff0000u), r1 = x1 - __uint_as_float(a1 & 0xffff0000u);
-    const uint32_t b0 = __float_as_uint(r0), b1 = __float_as_uint(r1);
-    p2 = __byte_perm(b0, b1, 0x7632);
-    const float s0 = r0 - __uint_as_float(b0 & 0xffff0000u), s1 = r1 - __uint_as_float(b1 & 0xffff0000u);
-    p3 = __byte_perm(__float_as_uint(s0), __float_as_uint(s1), 0x7632);
+    auto rest = [](float2 x) {                          // x minus its top 16 bits, exact
+        const float2 t = make_float2(__uint_as_float(__float_as_uint(x.x) & 0xffff0000u), __uint_as_float(__float_as_uint(x.y) & 0xffff0000u));
+        return __ffma2_rn(t, make_float2(-1.f, -1.f), x);
+    };
+    auto pack = [](float2 x) { return __byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x7632); };
+    const float2 a = make_float2(x0, x1), b = rest(a), c = rest(b);
+    p1 = pack(a); p2 = pack(b); p3 = pack(c);
 }
 
 // Optional self-profiling build (-DSPECA_PROF): cycles CTA 0 spends in each kind of wait, per warp,
@@ -258,11 +257,6 @@ __device__ __forceinline__ bool prof_wait(long long &acc, uint32_t bar, uint32_t
 #endif
 
 
-// Units of up to 32 nodes use the x columns and the space of M as two buffers, so that a tile's second product does
-// not wait for the one before it.
-__device__ __forceinline__ uint32_t x_piece(bool small) { return small ? 16u : 32u; }
-__device__ __forceinline__ uint32_t x_off(bool small, uint32_t q) { return kXOff + ((small && (q & 1)) ? 48u : 0u); }
-
 // TP = value tiles per unit (d_v / 128), DK = key width, MAXN = nodes per sequence, MAXD = tree depth.
 template <int TP, int DK, int MAXN, int MAXD>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -293,15 +287,15 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             mbar_init(bar(kKQFull + i), 1);
             mbar_init(bar(kKQFree + i), 2);
             mbar_init(bar(kVFull + i), 1);
-            mbar_init(bar(kVFree + i), 4);
+            mbar_init(bar(kVFree + i), 8);
             mbar_init(bar(kAccFull + i), 1);
-            mbar_init(bar(kAccFree + i), 4);
-            mbar_init(bar(kXReady + i), 4);
+            mbar_init(bar(kAccFree + i), 8);
+            mbar_init(bar(kGamReady + i), 4);
             mbar_init(bar(kOutFull + i), 1);
             mbar_init(bar(kMReady + i), 4);
             mbar_init(bar(kMFree + i), 1);
         }
-        mbar_init(bar(kXFree), 1);
+        mbar_init(bar(kXReady), 8);
         mbar_init(bar(kGramFull), 1);
         mbar_init(bar(kGramFree), 4);
         mbar_init(bar(kSync), 4);
@@ -416,14 +410,14 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             if (!next_unit(walk, x)) break;
             const bool small = x.npad <= 32;
             const int ksteps = x.npad >> 4, mbuf = useq & 1;
-            const uint32_t idx = make_idesc_bf16(x.npad), xps = x_piece(small);
+            const uint32_t idx = make_idesc_bf16(x.npad);
             if (!(ok = WAIT(2, bar(kMReady + mbuf), (useq >> 1) & 1))) break;
 #pragma unroll 1
             for (int t = 0; t < TP; ++t, ++q) {
-                if (!(ok = WAIT(3, bar(kXReady + (q & 1)), (q >> 1) & 1))) break;
+                if (!(ok = WAIT(3, bar(kXReady), q & 1))) break;
                 tc_fence_after();
                 if (lane == 0) {
-                    const uint32_t acc = tmem_base + (q & 1) * kTileCols, xa = tmem_base + x_off(small, q);
+                    const uint32_t acc = tmem_base + (q & 1) * kTileCols, xa = tmem_base + kXOff;
                     const uint64_t md = make_desc(sbase + LY::OffM + (small && mbuf ? LY::MBUF2 : 0));
                     uint32_t on = 0;
 #pragma unroll 1
@@ -432,11 +426,10 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                         for (int xp = 2; xp >= 0; --xp)           // small products first
 #pragma unroll
                             for (int mp = 2 - xp; mp >= 0; --mp) {
-                                mma_bf16_ts(acc, xa + xps * xp + 8 * ks, md + uint64_t(mp * (LY::MPIECE >> 4) + 2 * ks), idx, on);
+                                mma_bf16_ts(acc, xa + 32 * xp + 8 * ks, md + uint64_t(mp * (LY::MPIECE >> 4) + 2 * ks), idx, on);
                                 on = 1;
                             }
                     mma_commit(bar(kOutFull + (q & 1)));
-                    mma_commit(bar(kXFree));
                     if (t == TP - 1) mma_commit(bar(kMFree + mbuf));
                 }
                 __syncwarp();
@@ -500,6 +493,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                     split_pair(v.x, v.y, p1[2 * j], p2[2 * j], p3[2 * j]);
                     split_pair(v.z, v.w, p1[2 * j + 1], p2[2 * j + 1], p3[2 * j + 1]);
                 }
+                // the loads must have been performed, not only issued, before the copy engine may write the slot again
+                fence_proxy_async();
                 warp_arrive(bar(kEmpty + s), lane);
                 if (!(ok = WAIT(1, bar(kAFree + ab), ((it >> 1) & 1) ^ 1))) break;
                 tc_fence_after();
@@ -514,82 +509,99 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         }
         PROF_STORE()
     } else if (warp < 16) {
-        // ------------------------------------------------------------- epilogue groups, alternating tiles
+        // ------------------------------------------------------------- epilogue
+        // Step s takes tile s - 1 from x M^T to o, which frees its accumulators, and then tile s from R to x: the state product
+        // of a tile runs under the second product of the one before it and under both of these.  (The other way round the
+        // accumulators came free a whole state product later: 8-node units 4.9 us instead of 4.6.)  Columns go in chunks of
+        // 8 nodes, alternately to the two warps of a lane quarter.
         const int grp = (warp - 8) >> 2;
         const int row = 32 * (warp & 3) + lane;
         const uint32_t lane_addr = uint32_t(32 * (warp & 3)) << 16;
-        const uint32_t acc = tmem_base + grp * kTileCols + lane_addr;
+        const uint32_t xb = tmem_base + kXOff + lane_addr;
         const size_t stride = size_t(p.H) * p.DV;
-        uint32_t q = 0, useq = 0;
-        bool was_small = false;                                  // the tile before this one
+        uint32_t q = 0, useq = 0xffffffffu;
+        int t = TP - 1, pn = 0, pR = 0;                          // tile of the unit; nodes and rows of the last tile's unit (0: none)
+        const float *pgf = nullptr;
+        float *pdst = nullptr;
+        bool more = true;
         PROF_DECL
-        for (; ok && next_unit(walk, x); ++useq) {
-            const int R = x.npad, n = x.n;
-            const bool small = R <= 32;
-            const uint32_t xps = x_piece(small), xb = tmem_base + x_off(small, grp) + lane_addr;
-            const float *gx = reinterpret_cast<const float *>(smem + LY::OffGam) + (useq & 3) * 2 * MAXN, *gf = gx + MAXN;
-#pragma unroll 1
-            for (int t = 0; t < TP; ++t, ++q) {
-                const bool shared_x = !(small && was_small);     // x columns shared with the tile before
-                was_small = small;
-                if (int(q & 1) != grp) continue;
-                const uint32_t ph = (q >> 1) & 1;
-                if (!(ok = WAIT(0, bar(kVFull + grp), ph))) break;
-                if (!(ok = WAIT(1, bar(kMReady + (useq & 1)), (useq >> 1) & 1))) break;
-                if (!(ok = WAIT(2, bar(kAccFull + grp), ph))) break;
-                if (shared_x && !(ok = WAIT(3, bar(kXFree), (q & 1) ^ 1))) break;
-                tc_fence_after();
-                {
-                    PROF_T0()
-                    const unsigned short *vt = reinterpret_cast<const unsigned short *>(smem + LY::OffV + grp * LY::VBUF) + row;
-#pragma unroll 1
-                    for (int c0 = 0; c0 < R; c0 += 16) {
-                        float r[16];
-                        tmem_ld16(acc + c0, r);
-                        uint32_t vv[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) vv[i] = vt[(c0 + i) * kRows];
-                        tmem_ld_wait();
-                        uint32_t p1[8], p2[8], p3[8];
-#pragma unroll
-                        for (int i = 0; i < 16; i += 2) {
-                            const float2 gm = *reinterpret_cast<const float2 *>(gx + c0 + i);
-                            // rows past the last node belong to another sequence: they must not reach the product
-                            const float x0 = c0 + i < n ? fmaf(-gm.x, r[i], __uint_as_float(vv[i] << 16)) : 0.f;
-                            const float x1 = c0 + i + 1 < n ? fmaf(-gm.y, r[i + 1], __uint_as_float(vv[i + 1] << 16)) : 0.f;
-                            split_pair(x0, x1, p1[i >> 1], p2[i >> 1], p3[i >> 1]);
-                        }
-                        tmem_st8(xb + (c0 >> 1), p1);
-                        tmem_st8(xb + xps + (c0 >> 1), p2);
-                        tmem_st8(xb + 2 * xps + (c0 >> 1), p3);
-                    }
-                    tmem_st_wait();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) { mbar_arrive(bar(kXReady + grp)); mbar_arrive(bar(kVFree + grp)); }
-                    PROF_ADD(6)
-                }
-                if (!(ok = WAIT(4, bar(kOutFull + grp), ph))) break;
+        while (ok) {
+            if (more && ++t == TP) {
+                t = 0;
+                ++useq;
+                more = next_unit(walk, x);
+            }
+            if (pn == 0 && !more) break;
+            const uint32_t slot = q & 1, ps = slot ^ 1;
+            if (pn > 0 && !(ok = WAIT(4, bar(kOutFull + ps), ((q - 1) >> 1) & 1))) break;
+            const float *gx = reinterpret_cast<const float *>(smem + LY::OffGam) + (useq & 3) * 2 * MAXN;
+            if (pn > 0) {
                 tc_fence_after();
                 PROF_T0()
-                const size_t rec0 = size_t((x.l * p.T + x.base) * p.H + x.h);
-                float *dst = (x.kind == 0 ? p.o : p.u) + rec0 * p.DV + t * kRows + row;
+                const uint32_t acc = tmem_base + ps * kTileCols + lane_addr;
+                float *dst = pdst + size_t(8 * grp) * stride;
 #pragma unroll 1
-                for (int c0 = 0; c0 < n; c0 += 16) {
-                    float d[16], g[16];
-                    tmem_ld16(acc + c0, d);
-                    tmem_ld16(acc + R + c0, g);
+                for (int c0 = 8 * grp; c0 < pn; c0 += 16, dst += 8 * stride) {
+                    float d[8], g[8], gf[8];
+                    tmem_ld8(acc + c0, d);
+                    tmem_ld8(acc + pR + c0, g);
+                    *reinterpret_cast<float4 *>(gf) = *reinterpret_cast<const float4 *>(pgf + c0);
+                    *reinterpret_cast<float4 *>(gf + 4) = *reinterpret_cast<const float4 *>(pgf + c0 + 4);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        if (c0 + i < n) *dst = fmaf(gf[c0 + i], g[i], d[i]);
+                    for (int i = 0; i < 8; ++i) {
+                        if (c0 + i < pn) *dst = fmaf(gf[i], g[i], d[i]);
                         dst += stride;
                     }
                 }
                 tc_fence_before();
-                warp_arrive(bar(kAccFree + grp), lane);
+                warp_arrive(bar(kAccFree + ps), lane);
                 PROF_ADD(7)
             }
+            if (more) {
+                if (!(ok = WAIT(0, bar(kVFull + slot), (q >> 1) & 1))) break;
+                if (!(ok = WAIT(1, bar(kGamReady + (useq & 1)), (useq >> 1) & 1))) break;
+                if (!(ok = WAIT(2, bar(kAccFull + slot), (q >> 1) & 1))) break;
+                tc_fence_after();
+                PROF_T0()
+                const uint32_t acc = tmem_base + slot * kTileCols + lane_addr;
+                const unsigned short *vt = reinterpret_cast<const unsigned short *>(smem + LY::OffV + slot * LY::VBUF) + row;
+#pragma unroll 1
+                for (int c0 = 8 * grp; c0 < x.npad; c0 += 16) {
+                    float r[8];
+                    tmem_ld8(acc + c0, r);
+                    uint32_t vv[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) vv[i] = vt[(c0 + i) * kRows];
+                    float gm[8];
+                    *reinterpret_cast<float4 *>(gm) = *reinterpret_cast<const float4 *>(gx + c0);
+                    *reinterpret_cast<float4 *>(gm + 4) = *reinterpret_cast<const float4 *>(gx + c0 + 4);
+                    tmem_ld_wait();
+                    uint32_t p1[4], p2[4], p3[4];
+#pragma unroll
+                    for (int i = 0; i < 8; i += 2) {
+                        // rows past the last node belong to another sequence: they must not reach the product
+                        const float x0 = c0 + i < x.n ? fmaf(-gm[i], r[i], __uint_as_float(vv[i] << 16)) : 0.f;
+                        const float x1 = c0 + i + 1 < x.n ? fmaf(-gm[i + 1], r[i + 1], __uint_as_float(vv[i + 1] << 16)) : 0.f;
+                        split_pair(x0, x1, p1[i >> 1], p2[i >> 1], p3[i >> 1]);
+                    }
+                    tmem_st4(xb + (c0 >> 1), p1);
+                    tmem_st4(xb + 32 + (c0 >> 1), p2);
+                    tmem_st4(xb + 64 + (c0 >> 1), p3);
+                }
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) { mbar_arrive(bar(kXReady)); mbar_arrive(bar(kVFree + slot)); }
+                PROF_ADD(6)
+            }
+            pn = 0;
+            if (more) {
+                pn = x.n; pR = x.npad;
+                pgf = gx + MAXN;
+                pdst = (x.kind == 0 ? p.o : p.u) + size_t((x.l * p.T + x.base) * p.H + x.h) * p.DV + t * kRows + row;
+            }
+            ++q;
         }
         PROF_STORE()
     } else {
@@ -714,8 +726,23 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                     }
                 PROF_ADD(6)
             }
-            // the buffer of M: used by the unit two before this one, and, where one of them is large, by the last one
+            // gamma, which the epilogue needs a product earlier than M, once the unit two before this one is done with (its
+            // readers have then seen every phase of these barriers so far, and left the buffer of four units ago)
             if (useq >= 2 && !(ok = WAIT(2, bar(kMFree + (useq & 1)), ((useq >> 1) & 1) ^ 1))) break;
+            if (is_k) {
+                float gam = 1.f;
+                const float front = x.kind == 0 ? p.scale : 1.f;
+#pragma unroll
+                for (int r = 0; r < MAXD; ++r) {
+                    c[r] *= front * gam;                         // M[t][a_r]
+                    if (r < d) gam *= alpha_s[path(r)];
+                }
+                float *gx = reinterpret_cast<float *>(smem + LY::OffGam) + (useq & 3) * 2 * MAXN;
+                gx[node] = p.no_erase ? 0.f : gam;
+                gx[MAXN + node] = x.kind == 0 ? p.scale * gam : 0.f;
+            }
+            warp_arrive(bar(kGamReady + (useq & 1)), lane);
+            // the buffer of M: used by the unit two before this one, and, where one of them is large, by the last one
             if (useq >= 1 && !(small && was_small) && !(ok = WAIT(3, bar(kMFree + ((useq & 1) ^ 1)), ((useq - 1) >> 1) & 1))) break;
             was_small = small;
             if (is_k) {
@@ -728,23 +755,17 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
 #pragma unroll
                         for (int pc = 0; pc < 3; ++pc)
                             *reinterpret_cast<uint4 *>(mrow + pc * LY::MPIECE + ((i ^ (node & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
-                float rho = x.kind == 0 ? p.scale : 1.f, gam = 1.f;
 #pragma unroll
                 for (int r = 0; r < MAXD; ++r)
                     if (r < d) {
                         const int a = path(r);
                         uint32_t p1, p2, p3;
-                        split_pair(rho * c[r], 0.f, p1, p2, p3);
+                        split_pair(c[r], 0.f, p1, p2, p3);
                         uint8_t *m = mrow + (((a >> 3) ^ (node & 7)) << 4) + (a & 7) * 2;
                         *reinterpret_cast<unsigned short *>(m) = (unsigned short)(p1);
                         *reinterpret_cast<unsigned short *>(m + LY::MPIECE) = (unsigned short)(p2);
                         *reinterpret_cast<unsigned short *>(m + 2 * LY::MPIECE) = (unsigned short)(p3);
-                        rho *= alpha_s[a];
-                        gam *= alpha_s[a];
                     }
-                float *gx = reinterpret_cast<float *>(smem + LY::OffGam) + (useq & 3) * 2 * MAXN;
-                gx[node] = p.no_erase ? 0.f : gam;
-                gx[MAXN + node] = x.kind == 0 ? p.scale * gam : 0.f;
                 fence_proxy_async();
                 PROF_ADD(7)
             }

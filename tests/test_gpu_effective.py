@@ -49,3 +49,20 @@ def test_rule_without_erase():
     finally:
         oracle.set_rule(speca.RULE_GATED_DELTA)
     assert rel_err(dp.o.cpu().numpy(), ref) <= TOL_FP32
+
+
+@pytest.mark.parametrize("d_v", [128, 256])
+def test_ring_slots_are_read_before_they_are_refilled(d_v):
+    """Many units per CTA from a state that L2 holds (the second walk of a unit with u requested reads it there): a ring slot
+    comes round again as fast as it can.  Every repetition must give the first one's bits."""
+    rng = np.random.default_rng(830)
+    sizes = [64, 1, 32, 33, 8, 16, 64, 17, 48, 49, 31, 15, 2]
+    prob = synth.make_problem(831, 4, 3, 128, d_v, [tree(n, 8, rng) for n in sizes * 4], state_std=0.3)
+    dp = DevProblem(prob, route=speca.ROUTE_EFFECTIVE, want_u=True, max_nodes=64)
+    dp.verify_tree()
+    assert dp.status_value() == 0 and rel_err(dp.o.cpu().numpy(), oracle_verify(prob)) <= TOL_FP32
+    o, u = dp.o.clone(), dp.u.clone()
+    for _ in range(40):
+        dp.o.zero_(); dp.u.zero_()
+        dp.verify_tree()
+        assert bool((dp.o == o).all()) and bool((dp.u == u).all())
