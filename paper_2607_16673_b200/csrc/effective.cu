@@ -206,13 +206,15 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&x)[4])
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // kind::f16 (bf16) with the A operand in TMEM: a 32-bit column holds two consecutive K elements, the even one low
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate,
+                                            uint32_t lead)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
 }
 // Two fp32 values as three packed pairs of bf16 pieces (x0 in the low half), by truncation: a piece takes the top 8
@@ -325,6 +327,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
     x.ng = int(blockIdx.x) % ep.gpl; x.nb = int(blockIdx.x) / ep.gpl % p.B; x.nl = int(blockIdx.x) / ep.gpl / p.B;
     bool ok = true;
 
+    const uint32_t lead = elect_one();                           // the thread that issues this warp's tcgen05 instructions
+
     if (warp == 0) {
         // ------------------------------------------------------------- TMA producer: state slices
         uint32_t it = 0;
@@ -360,21 +364,18 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                     const int ab = it & 1;
                     if (!(ok = WAIT(2, bar(kAReady + ab), (it >> 1) & 1))) break;
                     tc_fence_after();
-                    if (lane == 0) {
-                        const uint32_t a = tmem_base + kAOff + ab * kACols;
-                        const uint64_t bd = make_desc(stage + (c >> 1) * SCB + (c & 1) * 64);
+                    const uint32_t a = tmem_base + kAOff + ab * kACols;
+                    const uint64_t bd = make_desc(stage + (c >> 1) * SCB + (c & 1) * 64);
 #pragma unroll
-                        for (int ks = 0; ks < 2; ++ks)
+                    for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
-                            for (int pc = 0; pc < 3; ++pc)       // (32 bytes further on: 2 in the descriptor's address field)
-                                mma_bf16_ts(acc, a + 16 * pc + 8 * ks, bd + 2 * ks, idm, (c | ks | pc) != 0);
-                        mma_commit(bar(kAFree + ab));
-                        if (c == NC - 1) {
-                            mma_commit(bar(kAccFull + (q & 1)));
-                            if (t == TP - 1) mma_commit(bar(kKQFree + par));
-                        }
+                        for (int pc = 0; pc < 3; ++pc)           // (32 bytes further on: 2 in the descriptor's address field)
+                            mma_bf16_ts(acc, a + 16 * pc + 8 * ks, bd + 2 * ks, idm, (c | ks | pc) != 0, lead);
+                    mma_commit(bar(kAFree + ab), lead);
+                    if (c == NC - 1) {
+                        mma_commit(bar(kAccFull + (q & 1)), lead);
+                        if (t == TP - 1) mma_commit(bar(kKQFree + par), lead);
                     }
-                    __syncwarp();
                 }
             }
         }
@@ -392,18 +393,15 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 if (!(ok = WAIT(0, bar(kKQFull + par), (gseq >> 1) & 1))) break;
                 if (!(ok = WAIT(1, bar(kGramFree), (gseq & 1) ^ 1))) break;
                 tc_fence_after();
-                if (lane == 0) {
-                    const uint32_t idg = make_idesc_bf16(gx.npad);
+                const uint32_t idg = make_idesc_bf16(gx.npad);
 #pragma unroll 1
-                    for (int c = 0; c < SC; ++c) {
-                        const uint64_t d = make_desc(sbase + LY::OffStage + par * LY::STAGE + c * SCB);
+                for (int c = 0; c < SC; ++c) {
+                    const uint64_t d = make_desc(sbase + LY::OffStage + par * LY::STAGE + c * SCB);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) mma_bf16(tmem_base + kGramOff, d + 2 * k, d + 2 * k, idg, (c | k) != 0);
-                    }
-                    mma_commit(bar(kGramFull));
-                    mma_commit(bar(kKQFree + par));
+                    for (int k = 0; k < 4; ++k) mma_bf16(tmem_base + kGramOff, d + 2 * k, d + 2 * k, idg, (c | k) != 0, lead);
                 }
-                __syncwarp();
+                mma_commit(bar(kGramFull), lead);
+                mma_commit(bar(kKQFree + par), lead);
                 ++gseq;
             }
             if (first) continue;
@@ -416,23 +414,18 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             for (int t = 0; t < TP; ++t, ++q) {
                 if (!(ok = WAIT(3, bar(kXReady), q & 1))) break;
                 tc_fence_after();
-                if (lane == 0) {
-                    const uint32_t acc = tmem_base + (q & 1) * kTileCols, xa = tmem_base + kXOff;
-                    const uint64_t md = make_desc(sbase + LY::OffM + (small && mbuf ? LY::MBUF2 : 0));
-                    uint32_t on = 0;
+                const uint32_t acc = tmem_base + (q & 1) * kTileCols, xa = tmem_base + kXOff;
+                const uint64_t md = make_desc(sbase + LY::OffM + (small && mbuf ? LY::MBUF2 : 0));
 #pragma unroll 1
-                    for (int ks = 0; ks < ksteps; ++ks)
+                for (int ks = 0; ks < ksteps; ++ks)
 #pragma unroll
-                        for (int xp = 2; xp >= 0; --xp)           // small products first
+                    for (int xp = 2; xp >= 0; --xp)               // small products first
 #pragma unroll
-                            for (int mp = 2 - xp; mp >= 0; --mp) {
-                                mma_bf16_ts(acc, xa + 32 * xp + 8 * ks, md + uint64_t(mp * (LY::MPIECE >> 4) + 2 * ks), idx, on);
-                                on = 1;
-                            }
-                    mma_commit(bar(kOutFull + (q & 1)));
-                    if (t == TP - 1) mma_commit(bar(kMFree + mbuf));
-                }
-                __syncwarp();
+                        for (int mp = 2 - xp; mp >= 0; --mp)
+                            mma_bf16_ts(acc, xa + 32 * xp + 8 * ks, md + uint64_t(mp * (LY::MPIECE >> 4) + 2 * ks), idx,
+                                        (ks | (2 - xp)) != 0, lead);
+                mma_commit(bar(kOutFull + (q & 1)), lead);
+                if (t == TP - 1) mma_commit(bar(kMFree + mbuf), lead);
             }
             ++useq;
         }
@@ -775,8 +768,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
     }
     if (warp == 1 || warp == 2) {
         // everything these warps issued must have completed before TMEM is released
-        if (lane == 0) mma_commit(bar(kDrain));
-        __syncwarp();
+        mma_commit(bar(kDrain), lead);
         mbar_wait(bar(kDrain), 0, abort_flag);
     }
     if ((warp == 0 || warp == 3) && *abort_flag) {

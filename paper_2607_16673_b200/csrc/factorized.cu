@@ -438,6 +438,8 @@ verify_factorized_kernel(const __grid_constant__ CUtensorMap s0_map, const __gri
     walk.pend = FUSED ? p.ws.pend : nullptr;
     walk.tab = smem + kOffWalk;
 
+    const uint32_t lead = elect_one();                           // the thread that issues this warp's tcgen05 instructions
+
     if (warp == 0 && FUSED) {
         // ------------------------------------------------------------- TMA producer of the fused kernel
         // Besides loading state slices it sends the advanced slices back: a TMA store needs a good
@@ -608,18 +610,17 @@ verify_factorized_kernel(const __grid_constant__ CUtensorMap s0_map, const __gri
             if (!wait_fast(bar(kBarStageReady), seq & 1, abort_flag)) return false;
             if (!wait_fast(bar(kBarPairFree + pr), ((seq >> 1) & 1) ^ 1, abort_flag)) return false;
             tc_fence_after();
-            if (lane == 0) {
+            {
                 const uint32_t idg = make_idesc_bf16(npad);
 #pragma unroll
                 for (int c = 0; c < SC; ++c)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const uint64_t d = make_desc(stage + c * SCB + k * 32);
-                        mma_bf16(tmem_base + pr * kPairCols, d, d, idg, (c | k) != 0);
+                        mma_bf16(tmem_base + pr * kPairCols, d, d, idg, (c | k) != 0, lead);
                     }
-                mma_commit(bar(kBarGramFull));
+                mma_commit(bar(kBarGramFull), lead);
             }
-            __syncwarp();
             return true;
         };
         bool have = ok && first_unit(walk, x);
@@ -644,41 +645,38 @@ verify_factorized_kernel(const __grid_constant__ CUtensorMap s0_map, const __gri
                     const uint32_t ph = (it / NS) & 1;
                     if (!(ok = WAIT(2, bar(kBarFull + s), ph))) break;
                     tc_fence_after();
-                    if (lane == 0) {
+                    {
                         const uint32_t sa = sbase + kOffRing + s * kStageBytes;
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            mma_tf32(acc, make_desc(sa + k * 32), make_desc(bop + c * BCB + k * 32), idm, (c | k) != 0);
-                        mma_commit(bar(kBarP1Done + s));
+                            mma_tf32(acc, make_desc(sa + k * 32), make_desc(bop + c * BCB + k * 32), idm, (c | k) != 0, lead);
+                        mma_commit(bar(kBarP1Done + s), lead);
                     }
-                    __syncwarp();
                     if (ps >= 0) {
                         if (!(ok = WAIT(3, bar(kBarLo + ps), pph))) break;
                         tc_fence_after();
-                        if (lane == 0) {
+                        {
                             const uint32_t sa = sbase + kOffRing + ps * kStageBytes;
 #pragma unroll
                             for (int k = 0; k < 4; ++k)
-                                mma_tf32(acc, make_desc(sa + k * 32), make_desc(bop + (c - 1) * BCB + k * 32), idm, 1);
-                            mma_commit(bar(kBarEmpty + ps));
+                                mma_tf32(acc, make_desc(sa + k * 32), make_desc(bop + (c - 1) * BCB + k * 32), idm, 1, lead);
+                            mma_commit(bar(kBarEmpty + ps), lead);
                         }
-                        __syncwarp();
                     }
                     ps = s; pph = ph;
                 } else {
                     // the last slice's second pass closes the tile
                     if (!(ok = WAIT(3, bar(kBarLo + ps), pph))) break;
                     tc_fence_after();
-                    if (lane == 0) {
+                    {
                         const uint32_t sa = sbase + kOffRing + ps * kStageBytes;
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            mma_tf32(acc, make_desc(sa + k * 32), make_desc(bop + (NC - 1) * BCB + k * 32), idm, 1);
-                        mma_commit(bar(kBarEmpty + ps));
-                        mma_commit(bar(kBarAccFull + pr));
-                        mma_commit(bar(kBarBFree));
+                            mma_tf32(acc, make_desc(sa + k * 32), make_desc(bop + (NC - 1) * BCB + k * 32), idm, 1, lead);
+                        mma_commit(bar(kBarEmpty + ps), lead);
+                        mma_commit(bar(kBarAccFull + pr), lead);
+                        mma_commit(bar(kBarBFree), lead);
                     }
-                    __syncwarp();
                 }
             }
             if (!ok) break;
@@ -689,8 +687,7 @@ verify_factorized_kernel(const __grid_constant__ CUtensorMap s0_map, const __gri
         PROF_STORE()
         // everything this warp issued must have completed before TMEM is released
         if (mt < TP) {
-            if (lane == 0) mma_commit(bar(kBarDrain));
-            __syncwarp();
+            mma_commit(bar(kBarDrain), lead);
             mbar_wait(bar(kBarDrain), 0, abort_flag);
         }
     } else if (COMP && warp >= 15) {
@@ -740,18 +737,17 @@ verify_factorized_kernel(const __grid_constant__ CUtensorMap s0_map, const __gri
             // the epilogue group must have released this pair of accumulators (unit seq - 2)
             if (!WAIT(1, bar(kBarPairFree + pr), ((seq >> 1) & 1) ^ 1)) return false;
             tc_fence_after();
-            if (lane == 0) {
+            {
                 const uint32_t idg = make_idesc_bf16(npad);
 #pragma unroll
                 for (int c = 0; c < SC; ++c)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const uint64_t d = make_desc(stage + c * SCB + k * 32);
-                        mma_bf16(tmem_base + pr * kPairCols, d, d, idg, (c | k) != 0);
+                        mma_bf16(tmem_base + pr * kPairCols, d, d, idg, (c | k) != 0, lead);
                     }
-                mma_commit(bar(kBarGramFull));
+                mma_commit(bar(kBarGramFull), lead);
             }
-            __syncwarp();
             return true;
         };
         bool have = first_unit(walk, x);
@@ -769,28 +765,26 @@ verify_factorized_kernel(const __grid_constant__ CUtensorMap s0_map, const __gri
                     const uint32_t ph = (it / NS) & 1;
                     if (!(ok = WAIT(4, bar((FUSED ? kBarUpd : kBarFull) + s), ph))) break;
                     tc_fence_after();
-                    if (lane == 0) {
+                    {
                         const uint32_t sa = sbase + kOffRing + s * kStageBytes;
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
                             mma_tf32(acc + t * kAccCols, make_desc(sa + k * 32),
-                                     make_desc(bop + c * BCB + k * 32), idm, (c | k) != 0);
-                        mma_commit(bar(kBarEmpty + s));
+                                     make_desc(bop + c * BCB + k * 32), idm, (c | k) != 0, lead);
+                        mma_commit(bar(kBarEmpty + s), lead);
                     }
-                    __syncwarp();
                 }
             }
             if (!ok) break;
-            if (lane == 0) { mma_commit(bar(kBarAccFull + pr)); mma_commit(bar(kBarBFree)); }
-            __syncwarp();
+            mma_commit(bar(kBarAccFull + pr), lead);
+            mma_commit(bar(kBarBFree), lead);
             ++unit_seq;
             have = next_unit(walk, x);
             if (have) ok = issue_gram(unit_seq, x.npad);
         }
         PROF_STORE()
         // everything this warp issued must have completed before TMEM is released
-        if (lane == 0) mma_commit(bar(kBarDrain));
-        __syncwarp();
+        mma_commit(bar(kBarDrain), lead);
         mbar_wait(bar(kBarDrain), 0, abort_flag);
     } else if (warp < 6) {
         // ------------------------------------------------------------- operand + coefficient preparation

@@ -154,19 +154,35 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols)
 {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
+// tcgen05 instructions are issued by one thread.  The whole warp runs up to them and the instruction itself is predicated
+// on `lead` (elect_one, taken once per warp: a commit covers what its own thread issued), so that addresses and
+// descriptors stay in uniform registers.  Inside a branch of one lane every operand is moved there anew: six products
+// and a commit took 556 cycles, predicated 258 (N = 32; the tensor core's own rate is 46 a product).
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t lead;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(lead));
+    return lead;
+}
 __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate)
+                                         uint32_t accumulate, uint32_t lead)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint32_t bar)
+__device__ __forceinline__ void mma_commit(uint32_t bar, uint32_t lead)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+        ::"r"(bar), "r"(lead)
+        : "memory");
 }
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&r)[8])
 {
@@ -221,36 +237,17 @@ __device__ __forceinline__ uint32_t make_idesc_bf16(int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(n >> 3) << 17) | (uint32_t(128 >> 4) << 24);
 }
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate)
+                                         uint32_t accumulate, uint32_t lead)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
 }
 
-// MN-major operand with the 128-byte swizzle: the operand sits in shared memory with its M (or N) extent
-// contiguous, as a row-major [K][MN] tile of 16-bit elements.  A row of 128 bytes holds 64 consecutive MN
-// elements of one K index, 8 K indices form a 1024-byte group (stride byte offset), and the next 64 MN
-// elements start `mn_block_bytes` further on (leading byte offset).  The instruction descriptor must mark
-// the operand as MN-major (make_idesc_bf16_amn).
-__device__ __forceinline__ uint64_t make_desc_mn(uint32_t smem_addr, uint32_t mn_block_bytes)
-{
-    uint64_t d = 0;
-    d |= uint64_t((smem_addr >> 4) & 0x3fffu);
-    d |= uint64_t((mn_block_bytes >> 4) & 0x3fffu) << 16;
-    d |= uint64_t(1024 >> 4) << 32;
-    d |= uint64_t(1) << 46;
-    d |= uint64_t(2) << 61;
-    return d;
-}
-// kind::f16, bf16 operands, fp32 accumulate, A MN-major (bit 15), B K-major, M = 128
-__device__ __forceinline__ uint32_t make_idesc_bf16_amn(int n)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (uint32_t(n >> 3) << 17) | (uint32_t(128 >> 4) << 24);
-}
 // round an fp32 value to TF32 (nearest); the result is an fp32 bit pattern with the low 13 mantissa bits clear
 __device__ __forceinline__ float round_tf32(float x)
 {
