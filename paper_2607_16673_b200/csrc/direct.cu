@@ -500,12 +500,12 @@ int direct_limit(const Params &p, int d_k, int most, bool piped)
 {
     if (d_k == 64) return 64;                                // the alternative is the serial walk
     if (!piped) return 32;
-    // us per unit and SM in a large batch, this kernel / the pipelined one: d_k = 128, d_v = 256: 3.9 / 5.0 at 8 nodes,
-    // 4.4 / 5.0 at 16, 6.1 / 5.2 at 20..24; d_k = 256: 8.2 / 8.8 at 8, 9.4 / 8.8 at 16.  A few users, us per call with the
-    // plan of the pipelined kernel: d_k = 128, 384 units of 32 nodes 22 / 28; d_k = 256, 192 units of 32 nodes 41 / 35,
-    // 384 units of 16 nodes 45 / 50.
+    // us per unit and SM in a large batch, this kernel / the pipelined one: d_k = 128, d_v = 256: 3.6 / 4.0 at 8 nodes,
+    // 4.05 / 4.1 at 16, 6.1 / 5.0 at 20..24; d_k = 256: 8.2 / 6.6 at 8.  A few users, us per call with the plan of the
+    // pipelined kernel: d_k = 128, d_v = 128, 384 units of 8 / 16 / 32 nodes 10.7 / 16.0 / 19.5, 22.7 / 21.5 / 22.7;
+    // d_k = 256, 384 units of 8 nodes 30 / 37, 192 units of 16 nodes 25.4 / 24.7.
     const bool few = small_batch(p, sm_count_of_current_device());
-    const int cap = d_k == 128 ? (few ? 32 : 16) : (few ? 16 : 8);
+    const int cap = d_k == 128 ? (few ? 32 : 16) : (few ? 8 : 0);
     return most <= cap ? cap : 0;
 }
 

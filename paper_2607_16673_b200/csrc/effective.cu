@@ -23,17 +23,22 @@
 // A tile of 64 nodes takes 24 + 24 tcgen05 instructions.  The substitution over value rows, ~95 instructions per node
 // and warp in factorized.cu, is gone: what is left per element is a multiply-add on each side of the second product.
 //
-// Mapping.  One persistent CTA per SM walks units (layer, sequence, head) tile by tile (128 value rows); 20 warps:
+// Mapping.  One persistent CTA per SM walks units (layer, sequence, head) tile by tile (128 value rows); 24 warps:
 //   warp 0        TMA producer of the state slices (128 rows x 32 columns, 128-byte swizzle)
 //   warp 1        issues S0 [K;Q]^T; owns TMEM
 //   warp 2        issues the Gram blocks [K;Q] K^T (one unit ahead) and x M^T
 //   warp 3        TMA producer of the staged [K;Q] rows (two units) and the value rows (two tiles)
-//   warps 4-7     split: slice row per thread -> three bf16 pieces in TMEM (two buffers)
-//   warps 8-15    epilogue, two warps per TMEM lane quarter that share a tile's columns: R out of TMEM, x back into TMEM
+//   warps 4-11    split: slice row per thread -> three bf16 pieces in TMEM; two groups alternate slices, a buffer each
+//   warps 12-19   epilogue, two warps per TMEM lane quarter that share a tile's columns: R out of TMEM, x back into TMEM
 //                 as three pieces; then, while the next tile's product runs, o = scale gamma G + (x M^T), coalesced
-//   warps 16-19   solver, one unit ahead: Gram entries of every row against its own path, back substitution (a thread
+//   warps 20-23   solver, one unit ahead: Gram entries of every row against its own path, back substitution (a thread
 //                 per node, registers), the pieces of M
 // TMEM: two tiles of accumulators (R | G, 128 columns; x M^T overwrites R), two A buffers of 48, x of 96, Gram of 64.
+// Measured in large batches, us per unit and SM (share of the copy rate): d_k = 128, d_v = 256: 8 nodes 4.0 (85 %), 16
+// nodes 4.1 (92 %), 32 nodes 5.3 (85 %), 64 nodes 7.2 (83 %), 64 nodes at 16 levels 8.2; d_k = d_v = 256: 8 nodes 6.6
+// (97 %), 32 nodes 8.1 (97 %).  One split group instead of two: 4.75, 4.8, 5.1, 7.4, 7.9; 8.9, 9.4: a group needs
+// about 750 cycles a slice, the tensor core 280.  What bounds it: HBM at d_k = 256; at d_k = 128 the solver and the epilogue of
+// a unit, which come round twice as often.
 // Ten roles take turns on four issue slots, so the kernel's size matters as much as its instruction count: loops stay
 // rolled where a role has slack.
 // With u requested a unit is walked twice (o rows, then u rows); the second walk finds the state tile in L2.
@@ -53,7 +58,7 @@ using namespace tc;
 
 constexpr int kRows = 128;                      // value rows per tile (= TMEM lanes = MMA M)
 constexpr int kSliceBytes = kRows * 128;        // one ring slot: a K-slice of a tile (128 rows x 32 fp32)
-constexpr int kThreads = 20 * 32;
+constexpr int kThreads = 24 * 32;
 constexpr int kWalkSeqs = 128;
 // TMEM columns
 constexpr int kTileCols = 128;                  // accumulators of a tile: R, then G
@@ -81,7 +86,7 @@ template <int DK, int MAXN_, int MAXD> struct Lay {
     static constexpr int OffRing = OffV + 2 * VBUF;
     static constexpr int kSmall = 2 * MAXN * GSTR * 4 + 2 * 2 * MAXN * 4 + 2 * MAXN + 4 * 2 * MAXN * 4 + 5 * kWalkSeqs + 16 + 8 * 64;
     static constexpr int kRoom = (227 * 1024 - OffRing - kSmall) / kSliceBytes;
-    static constexpr int NS = kRoom > 8 ? 8 : kRoom;            // ring depth
+    static constexpr int NS = kRoom > 8 ? 8 : kRoom & ~1;       // ring depth: even, so that a slot is always the same split group's
     static constexpr int OffGk = OffRing + NS * kSliceBytes;    // [MAXN][GSTR] k_node . k_(ancestor at distance i + 1)
     static constexpr int OffGq = OffGk + MAXN * GSTR * 4;       // [MAXN][GSTR] q_node . k_(ancestor at distance i)
     static constexpr int OffAB = OffGq + MAXN * GSTR * 4;       // two units of float alpha, beta [MAXN]
@@ -467,9 +472,10 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             }
         }
         PROF_STORE()
-    } else if (warp < 8) {
+    } else if (warp < 12) {
         // ------------------------------------------------------------- split: slice -> three bf16 pieces in TMEM
         const int row = 32 * (warp & 3) + lane;                  // slice row = TMEM lane of this thread
+        const int sgrp = (warp - 4) >> 2;                   // two groups, alternating slices
         const uint32_t abase = tmem_base + kAOff + (uint32_t(32 * (warp & 3)) << 16);
         uint32_t it = 0;
         PROF_DECL
@@ -477,6 +483,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
 #pragma unroll 1
             for (int e = 0; e < TP * NC; ++e, ++it) {
                 const int s = it % NS, ab = it & 1;
+                if (ab != sgrp) continue;
                 if (!(ok = WAIT(0, bar(kFull + s), (it / NS) & 1))) break;
                 const uint8_t *src = smem + LY::OffRing + s * kSliceBytes + row * 128;
                 uint32_t p1[16], p2[16], p3[16];
@@ -501,13 +508,13 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             }
         }
         PROF_STORE()
-    } else if (warp < 16) {
+    } else if (warp < 20) {
         // ------------------------------------------------------------- epilogue
         // Step s takes tile s - 1 from x M^T to o, which frees its accumulators, and then tile s from R to x: the state product
         // of a tile runs under the second product of the one before it and under both of these.  (The other way round the
         // accumulators came free a whole state product later: 8-node units 4.9 us instead of 4.6.)  Columns go in chunks of
         // 8 nodes, alternately to the two warps of a lane quarter.
-        const int grp = (warp - 8) >> 2;
+        const int grp = (warp - 12) >> 2;
         const int row = 32 * (warp & 3) + lane;
         const uint32_t lane_addr = uint32_t(32 * (warp & 3)) << 16;
         const uint32_t xb = tmem_base + kXOff + lane_addr;
