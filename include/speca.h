@@ -196,7 +196,7 @@ int speca_stochastic_accept(int32_t batch, int32_t max_depth,
  * the sequence's state bitwise untouched (it is neither read nor written).  If
  * parent_or_null is given the path is checked to be a chain of parent links starting at
  * a child of the committed state; an invalid path skips the sequence.
- * The state is advanced token by token; in large batches (d_k <= 128) paths of four to
+ * The state is advanced token by token; in large batches (d_k <= 128) paths of six to
  * eight nodes are advanced in the unrolled form of Section 4.2 instead (one product of the
  * state tile with all keys of the path, the recurrence per row, one rank-A update, on
  * tensor cores with every fp32 operand split into a TF32 head and its exact remainder).

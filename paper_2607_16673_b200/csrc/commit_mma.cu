@@ -2,8 +2,8 @@
 // Section 5.2 immediate update).
 //
 // The token-by-token commit costs three fp32 FMAs per state element and accepted node, each node's
-// update waiting for the previous one's row reduction: beyond about four nodes the arithmetic, not
-// HBM, sets its speed.  For a path of A nodes (4 <= A <= 8) the same result is, per state row r,
+// update waiting for the previous one's row reduction: beyond about five nodes the arithmetic, not
+// HBM, sets its speed.  For a path of A nodes (6 <= A <= 8) the same result is, per state row r,
 //        R[r][i] = S0[r,:] . k_i                                          (one product with all keys)
 //        u_i[r]  = beta_i v_i[r] - beta_i gamma_i R[r][i] - sum_{j<i} beta_i (gamma_i/gamma_j) (k_j.k_i) u_j[r]
 //        S_A     = gamma_A S0 + sum_j (gamma_A/gamma_j) u_j k_j^T         (one rank-A update)
@@ -254,9 +254,8 @@ commit_long_kernel(Params p)
     }
 }
 
-// Batch size from which the second launch pays: its tail (about 25 us) against what the long paths save (about a
-// seventh of their own time, for the third or so of the sequences that accept four nodes or more), i.e. from about
-// half a millisecond of commit on -- 128 16-row tiles per resident warp.
+// Batch size from which the second launch pays: its tail (about 25 us) against what the long paths save (6 % of their own
+// time at six nodes, 22 % at eight), i.e. from about half a millisecond of commit on -- 128 16-row tiles per resident warp.
 constexpr int kMinTilesPerWarp = 128;
 std::atomic<int> g_min_tiles_per_warp{kMinTilesPerWarp};
 

@@ -204,16 +204,25 @@ verify_serial_kernel(Params p)
 // ---------------------------------------------------------------------------
 // commit: advance S in place over the accepted factor records
 // ---------------------------------------------------------------------------
-template <int DK, int RS, int WARPS>
+// A CTA advances TILES consecutive tiles of one unit over the same path.  The path is found, checked and staged
+// once; the second tile is asked into L2 when the first is loaded, so that HBM stays busy while the path is staged and
+// walked.  Paths of three nodes, 12288 units of d_k = 128, d_v = 256: a tile a CTA 562 us = 5.8 TB/s, two 490 us = 6.6
+// TB/s, which is the copy rate; four 568 (fewer CTAs start than end).
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+template <int DK, int RS, int WARPS, int TILES>
 __global__ void __launch_bounds__(WARPS * 32, 2048 / (WARPS * 32) / 2)
 commit_kernel(Params p)
 {
-    constexpr int G = Map<DK>::G, RPS = Map<DK>::RPS, ROWS = WARPS * RS * RPS;
-    const int tiles = p.DV / ROWS;
-    const long unit = blockIdx.x / tiles;
+    constexpr int G = Map<DK>::G, RPS = Map<DK>::RPS, ROWS = WARPS * RS * RPS, part_rows = ROWS * TILES;
+    const int parts = p.DV / part_rows;
+    const long unit = blockIdx.x / parts;
+    const int part = blockIdx.x % parts;
     const int h = int(unit % p.H), b = int((unit / p.H) % p.B), l = int(unit / (long(p.H) * p.B));
     const int lane = threadIdx.x & 31, g = lane % G, sub = lane / G;
-    const int row0 = (blockIdx.x % tiles) * ROWS + (threadIdx.x >> 5) * RS * RPS;
 
     // path_len == 0: the sequence's state is neither read nor written
     const int len = __ldg(p.path_len + b);
@@ -223,22 +232,24 @@ commit_kernel(Params p)
     // paths the tensor-core commit takes (it validates them itself)
     if (p.long_min > 0 && len >= p.long_min && len <= 8 && len <= p.max_depth) return;
 
-    // Start streaming the state tile right away; the accepted path is validated in the
+    // Start streaming the state right away; the accepted path is validated in the
     // shadow of these loads (one thread per path step), and nothing is stored if it is bad.
-    float *Su = p.S + unit * p.DV * DK;
+    float *S_part = p.S + (unit * p.DV + long(part) * part_rows) * DK;
+    const int tile_row = (threadIdx.x >> 5) * RS * RPS + sub;        // row inside a tile (row set 0)
     float2 s[RS][8];
     const bool len_ok = len > 0 && len <= p.max_depth;
     if (len_ok) {
+        if (TILES > 1 && threadIdx.x == 0) prefetch_l2(S_part + long(ROWS) * DK, (TILES - 1) * ROWS * DK * 4);
 #pragma unroll
-        for (int r = 0; r < RS; ++r) load_row<G>(Su + long(row0 + r * RPS + sub) * DK, g, s[r]);
+        for (int r = 0; r < RS; ++r) load_row<G>(S_part + long(tile_row + r * RPS) * DK, g, s[r]);
     }
-    // The factor records of the whole accepted path (k rows, alpha, beta, the tile's v values)
+    // The factor records of the whole accepted path (k rows, alpha, beta, the part's v values)
     // are staged in shared memory while the state tile is in flight, so that the token-by-token
     // recurrence below never waits on global memory.
     __shared__ int s_path[16];
     __shared__ __align__(16) __nv_bfloat16 s_k[16][DK];
     __shared__ float s_alpha[16], s_beta[16];
-    __shared__ __nv_bfloat16 s_v[16][ROWS];
+    __shared__ __nv_bfloat16 s_v[16][part_rows];
     int fault = 0;
     if (!len_ok) fault = SPECA_STATUS_TOO_DEEP;
     else if (base < 0 || n < 0 || base + n > p.T) fault = SPECA_STATUS_BAD_OFFSETS;
@@ -257,7 +268,6 @@ commit_kernel(Params p)
             }
         }
         constexpr int PIECES = DK / 8;                       // 16-byte pieces per k row
-        const int row_base = (blockIdx.x % tiles) * ROWS;
         for (int idx = threadIdx.x; idx < len * PIECES; idx += WARPS * 32) {
             const int d = idx / PIECES, piece = idx % PIECES;
             const int t = __ldg(p.path_idx + b * p.max_depth + d);
@@ -268,12 +278,12 @@ commit_kernel(Params p)
                              : "memory");
             }
         }
-        for (int idx = threadIdx.x; idx < len * ROWS; idx += WARPS * 32) {
-            const int d = idx / ROWS, r = idx % ROWS;
+        for (int idx = threadIdx.x; idx < len * part_rows; idx += WARPS * 32) {
+            const int d = idx / part_rows, r = idx % part_rows;
             const int t = __ldg(p.path_idx + b * p.max_depth + d);
             if (t >= 0 && t < n) {
                 const long rec = (long(l) * p.T + base + t) * p.H + h;
-                s_v[d][r] = p.v[rec * p.DV + row_base + r];
+                s_v[d][r] = p.v[rec * p.DV + part * part_rows + r];
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
@@ -281,33 +291,39 @@ commit_kernel(Params p)
     fault = __syncthreads_or(fault);
     if (fault) {
         // report one of the faults seen by the CTA (BAD_PATH is the only per-thread one)
-        if (threadIdx.x == 0 && blockIdx.x % tiles == 0 && h == 0 && l == 0)
+        if (threadIdx.x == 0 && part == 0 && h == 0 && l == 0)
             atomicOr(p.status, !len_ok ? SPECA_STATUS_TOO_DEEP
                                        : ((base < 0 || n < 0 || base + n > p.T) ? SPECA_STATUS_BAD_OFFSETS
                                                                                 : SPECA_STATUS_BAD_PATH));
         return;
     }
 
-    const int tile_row = (threadIdx.x >> 5) * RS * RPS + sub;        // row inside the CTA's tile (row set 0)
-    for (int d = 0; d < len; ++d) {
-        float2 kx[8];
+#pragma unroll 1
+    for (int tile = 0; tile < TILES; ++tile) {
+        float *S_tile = S_part + long(tile) * ROWS * DK;
+        if (tile > 0)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint2 raw = *(reinterpret_cast<const uint2 *>(&s_k[d][0]) + g + G * c);
-            kx[2 * c + 0] = make_float2(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u));
-            kx[2 * c + 1] = make_float2(__uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
-        }
-        const float alpha = s_alpha[d], beta = s_beta[d];
+            for (int r = 0; r < RS; ++r) load_row<G>(S_tile + long(tile_row + r * RPS) * DK, g, s[r]);
+        for (int d = 0; d < len; ++d) {
+            float2 kx[8];
 #pragma unroll
-        for (int r = 0; r < RS; ++r) {
-            const float sk = group_sum<G>(dot16(s[r], kx));
-            const float vv = __bfloat162float(s_v[d][tile_row + r * RPS]);
-            const float u = p.no_erase ? beta * vv : beta * (vv - alpha * sk);
-            axpy16(s[r], kx, alpha, u);
+            for (int c = 0; c < 4; ++c) {
+                const uint2 raw = *(reinterpret_cast<const uint2 *>(&s_k[d][0]) + g + G * c);
+                kx[2 * c + 0] = make_float2(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u));
+                kx[2 * c + 1] = make_float2(__uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
+            }
+            const float alpha = s_alpha[d], beta = s_beta[d];
+#pragma unroll
+            for (int r = 0; r < RS; ++r) {
+                const float sk = group_sum<G>(dot16(s[r], kx));
+                const float vv = __bfloat162float(s_v[d][tile * ROWS + tile_row + r * RPS]);
+                const float u = p.no_erase ? beta * vv : beta * (vv - alpha * sk);
+                axpy16(s[r], kx, alpha, u);
+            }
         }
+#pragma unroll
+        for (int r = 0; r < RS; ++r) store_row<G>(S_tile + long(tile_row + r * RPS) * DK, g, s[r]);
     }
-#pragma unroll
-    for (int r = 0; r < RS; ++r) store_row<G>(Su + long(row0 + r * RPS + sub) * DK, g, s[r]);
 }
 
 // Rows covered by one CTA for a given d_k: the largest of {32,16,8,4,2} rows (RS in
@@ -339,8 +355,16 @@ template <int DK, int RS, int WARPS> struct LaunchDecode {
 template <int DK, int RS, int WARPS> struct LaunchCommit {
     static int run(const Params &p, cudaStream_t st)
     {
-        const long blocks = n_units(p) * (p.DV / rows_per_cta<DK, RS, WARPS>());
-        commit_kernel<DK, RS, WARPS><<<unsigned(blocks), WARPS * 32, 0, st>>>(p);
+        constexpr int ROWS = rows_per_cta<DK, RS, WARPS>();
+        const long tiles = n_units(p) * (p.DV / ROWS);
+        // Two tiles a CTA from four rounds of such CTAs on (d_k = 128, d_v = 256, 1536 units: 74.8 -> 72.0 us); below that
+        // twice the CTAs serve the device better, and a 64-wide tile is done before its second is there (24576 units of
+        // d_k = d_v = 64: 162 us, two tiles 166).
+        const long round = long(sm_count_of_current_device()) * (2048 / (WARPS * 32) / 2);
+        if (DK > 64 && p.DV % (2 * ROWS) == 0 && tiles >= 8 * round)
+            commit_kernel<DK, RS, WARPS, 2><<<unsigned(tiles / 2), WARPS * 32, 0, st>>>(p);
+        else
+            commit_kernel<DK, RS, WARPS, 1><<<unsigned(tiles), WARPS * 32, 0, st>>>(p);
         return int(cudaGetLastError());
     }
 };
@@ -394,8 +418,9 @@ int launch_decode(const Params &p, int d_k, cudaStream_t st)
 }
 
 // Accepted paths of kCommitLongMin nodes or more go to the tensor-core kernel where it takes the shape: from there
-// on the token-by-token form is bound by its arithmetic, not by HBM.
-constexpr int kCommitLongMin = 4;
+// on the token-by-token form is bound by its arithmetic, not by HBM (49152 units of d_k = 128, d_v = 256, ms, token by token /
+// tensor cores: 4 nodes 1.99 / 2.23, 6 nodes 2.37 / 2.24, 8 nodes 2.91 / 2.25).
+constexpr int kCommitLongMin = 6;
 
 int launch_commit(const Params &p_in, int d_k, cudaStream_t st)
 {
