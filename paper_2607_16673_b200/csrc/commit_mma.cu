@@ -42,6 +42,7 @@ template <int DK>
 __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm)
 commit_long_kernel(Params p)
 {
+    after_previous_kernel();
     constexpr int NME = DK / 8;              // permuted k-steps of the first product = column blocks of the second
     constexpr int NM = DK / 16;              // 16-byte chunks of a row per lane
     __shared__ uint16_t s_long[kListCap];
@@ -278,8 +279,8 @@ int launch_commit_long(const Params &p, int d_k, cudaStream_t st)
     const int sms = sm_count_of_current_device();
     if (sms <= 0) return int(cudaErrorInvalidDevice);
     const int grid = sms * kCtasPerSm;
-    if (d_k == 64) commit_long_kernel<64><<<grid, kWarps * 32, 0, st>>>(p);
-    else commit_long_kernel<128><<<grid, kWarps * 32, 0, st>>>(p);
+    if (d_k == 64) launch(commit_long_kernel<64>, grid, kWarps * 32, 0, st, p);
+    else launch(commit_long_kernel<128>, grid, kWarps * 32, 0, st, p);
     return int(cudaGetLastError());
 }
 

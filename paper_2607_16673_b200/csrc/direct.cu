@@ -122,6 +122,7 @@ template <int DK, int NT, int MAXD, int WARPS, int CTAS>
 __global__ void __launch_bounds__(WARPS * 32, CTAS)
 verify_direct_kernel(DirectArgs da)
 {
+    after_previous_kernel();
     using LY = Lay<DK, NT, MAXD>;
     constexpr int N = LY::N, NS = DK / 32, THREADS = WARPS * 32;
     extern __shared__ __align__(16) uint8_t smem[];
@@ -471,7 +472,7 @@ int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
         if (e != cudaSuccess) return int(e);
         opted[dev].store(1, std::memory_order_release);
     }
-    kern<<<unsigned(units * da.parts), WARPS * 32, smem, st>>>(da);
+    launch(kern, unsigned(units * da.parts), WARPS * 32, smem, st, da);
     return int(cudaGetLastError());
 }
 

@@ -269,6 +269,7 @@ template <int TP, int DK, int MAXN, int MAXD>
 __global__ void __launch_bounds__(kThreads, 1)
 verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid_constant__ EMaps maps, EParams ep)
 {
+    after_previous_kernel();
     using LY = Lay<DK, MAXN, MAXD>;
     constexpr int NS = LY::NS, NC = LY::NC, SC = LY::SC, SCB = LY::SCB;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -894,8 +895,8 @@ int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
     const bool deep = p.max_depth > 8;
     auto go = [&](auto dk, auto mn, auto md) {
         constexpr int DK = decltype(dk)::value, MN = decltype(mn)::value, MD = decltype(md)::value;
-        if (one_tile) verify_effective_kernel<1, DK, MN, MD><<<grid, kThreads, Lay<DK, MN, MD>::Bytes, st>>>(map, em, ep);
-        else verify_effective_kernel<2, DK, MN, MD><<<grid, kThreads, Lay<DK, MN, MD>::Bytes, st>>>(map, em, ep);
+        if (one_tile) launch(verify_effective_kernel<1, DK, MN, MD>, grid, kThreads, Lay<DK, MN, MD>::Bytes, st, map, em, ep);
+        else launch(verify_effective_kernel<2, DK, MN, MD>, grid, kThreads, Lay<DK, MN, MD>::Bytes, st, map, em, ep);
     };
     auto pick = [&](auto dk, auto mn) { deep ? go(dk, mn, Int<16>{}) : go(dk, mn, Int<8>{}); };
     // a smaller node budget leaves room for a deeper ring of state slices

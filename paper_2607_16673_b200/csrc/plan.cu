@@ -22,6 +22,7 @@ plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict_
             const int32_t *__restrict__ depth_in, int32_t B, int32_t T, int32_t max_depth,
             int32_t max_nodes, int32_t skip_nodes, int32_t paths_only, int32_t n_slots, Workspace ws, int32_t *status)
 {
+    after_previous_kernel();
     extern __shared__ int32_t sm[];
     const int b = blockIdx.x;
     const int tid = threadIdx.x;
@@ -180,6 +181,7 @@ accept_kernel(int32_t B, int32_t max_depth, const int32_t *__restrict__ node_off
               int32_t *__restrict__ path_idx, int32_t *__restrict__ path_len,
               int32_t *__restrict__ next_tok, int32_t *status)
 {
+    after_previous_kernel();
     const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (b >= B) return;
@@ -236,6 +238,7 @@ stochastic_accept_kernel(int32_t B, int32_t max_depth, const int32_t *__restrict
                          const float *__restrict__ p_draft, const float *__restrict__ uniform,
                          int32_t *__restrict__ path_idx, int32_t *__restrict__ path_len, int32_t *status)
 {
+    after_previous_kernel();
     const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (b >= B) return;
@@ -328,6 +331,7 @@ pending_check_kernel(int32_t B, int32_t Tp, int32_t max_depth, int32_t max_len, 
                      const int32_t *__restrict__ path_idx, const int32_t *__restrict__ path_len,
                      int32_t *__restrict__ pend, int32_t *status)
 {
+    after_previous_kernel();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
     int32_t *rec = pend + b * kPendWords;
@@ -360,6 +364,7 @@ conv_commit_kernel(int32_t B, int32_t channels, int32_t W, int32_t T, int32_t ma
                    const uint4 *__restrict__ x, const int32_t *__restrict__ node_offsets,
                    const int32_t *__restrict__ path_idx, const int32_t *__restrict__ path_len, int32_t *status)
 {
+    after_previous_kernel();
     const int l = blockIdx.x / B, b = blockIdx.x % B;
     const int A = path_len[b];
     if (A == 0) return;
@@ -406,6 +411,7 @@ __global__ void __launch_bounds__(256)
 mask_to_parent_kernel(int32_t N, const uint8_t *__restrict__ mask, const int32_t *__restrict__ node_offsets,
                       int32_t *__restrict__ parent, int32_t *status)
 {
+    after_previous_kernel();
     extern __shared__ int32_t sm[];                     // [N] ancestors-or-self per node, [N] parent
     const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int base = node_offsets[b], n = node_offsets[b + 1] - base;
@@ -465,6 +471,7 @@ __global__ void __launch_bounds__(256)
 chain_decompose_kernel(int32_t N, const int32_t *__restrict__ node_offsets, const int32_t *__restrict__ parent,
                        int32_t *__restrict__ chain_head, int32_t *__restrict__ n_chains, int32_t *status)
 {
+    after_previous_kernel();
     extern __shared__ int32_t sm[];                     // [N] subtree size, [N] key of the heavy child
     __shared__ int32_t s_flag, s_count;
     const int b = blockIdx.x;
@@ -556,6 +563,7 @@ prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *__restrict__ n
              const int32_t *__restrict__ parent, const float *__restrict__ logp, int32_t *__restrict__ out_offsets,
              int32_t *__restrict__ out_parent, int32_t *__restrict__ out_index, int32_t *status)
 {
+    after_previous_kernel();
     extern __shared__ int32_t sm[];
     float *q = reinterpret_cast<float *>(sm);           // [N]
     int32_t *par = sm + N, *keep = sm + 2 * N, *newidx = sm + 3 * N, *done = sm + 4 * N;      // [N] each
@@ -657,14 +665,14 @@ int launch_mask_to_parent(int32_t B, int32_t N, const uint8_t *mask, const int32
                           int32_t *status, cudaStream_t st)
 {
     const size_t stage = size_t(N) * N <= kMaskStage ? size_t(N) * N : kMaskStage;
-    mask_to_parent_kernel<<<B, 256, size_t(2 * N) * sizeof(int32_t) + 32 + stage, st>>>(N, mask, node_offsets, parent, status);
+    launch(mask_to_parent_kernel, B, 256, size_t(2 * N) * sizeof(int32_t) + 32 + stage, st, N, mask, node_offsets, parent, status);
     return int(cudaGetLastError());
 }
 
 int launch_chain_decompose(int32_t B, int32_t N, const int32_t *node_offsets, const int32_t *parent,
                            int32_t *chain_head, int32_t *n_chains, int32_t *status, cudaStream_t st)
 {
-    chain_decompose_kernel<<<B, 256, size_t(2 * N) * sizeof(int32_t), st>>>(N, node_offsets, parent, chain_head, n_chains,
+    launch(chain_decompose_kernel, B, 256, size_t(2 * N) * sizeof(int32_t), st, N, node_offsets, parent, chain_head, n_chains,
                                                                          status);
     return int(cudaGetLastError());
 }
@@ -674,11 +682,11 @@ int launch_prune(int32_t B, int32_t N, float tau, int32_t budget, const int32_t 
                  cudaStream_t st)
 {
     const size_t smem = size_t(5 * N) * sizeof(int32_t);
-    prune_kernel<false><<<B, 128, smem, st>>>(N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent, out_index,
+    launch(prune_kernel<false>, B, 128, smem, st, N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent, out_index,
                                               status);
     const int e = int(cudaGetLastError());
     if (e != 0) return e;
-    prune_kernel<true><<<B, 128, smem, st>>>(N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent, out_index,
+    launch(prune_kernel<true>, B, 128, smem, st, N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent, out_index,
                                              status);
     return int(cudaGetLastError());
 }
@@ -687,14 +695,14 @@ int launch_conv_commit(int32_t L, int32_t B, int32_t channels, int32_t W, int32_
                        const void *x, const int32_t *node_offsets, const int32_t *path_idx, const int32_t *path_len,
                        int32_t *status, cudaStream_t st)
 {
-    conv_commit_kernel<<<L * B, 256, 0, st>>>(B, channels, W, T, max_depth, static_cast<uint4 *>(C),
+    launch(conv_commit_kernel, L * B, 256, 0, st, B, channels, W, T, max_depth, static_cast<uint4 *>(C),
                                               static_cast<const uint4 *>(x), node_offsets, path_idx, path_len, status);
     return int(cudaGetLastError());
 }
 
 int launch_pending_check(const Params &p, int max_len, cudaStream_t st)
 {
-    pending_check_kernel<<<(p.B + 127) / 128, 128, 0, st>>>(p.B, p.Tp, p.max_depth, max_len, p.max_nodes, p.pnode_offsets,
+    launch(pending_check_kernel, (p.B + 127) / 128, 128, 0, st, p.B, p.Tp, p.max_depth, max_len, p.max_nodes, p.pnode_offsets,
                                                             p.pparent, p.path_idx, p.path_len, p.ws.pend, p.status);
     return int(cudaGetLastError());
 }
@@ -702,7 +710,7 @@ int launch_pending_check(const Params &p, int max_len, cudaStream_t st)
 int launch_plan(const Params &p, cudaStream_t st)
 {
     const size_t smem = size_t(6 * p.max_nodes + 1) * sizeof(int32_t);
-    plan_kernel<<<p.B, kPlanThreads, smem, st>>>(p.node_offsets, p.parent, p.depth_in, p.B, p.T,
+    launch(plan_kernel, p.B, kPlanThreads, smem, st, p.node_offsets, p.parent, p.depth_in, p.B, p.T,
                                                   p.max_depth, p.max_nodes, p.skip_nodes, p.plan_paths_only,
                                                   p.n_slots, p.ws, p.status);
     return int(cudaGetLastError());
@@ -714,8 +722,7 @@ int launch_accept(int32_t B, int32_t max_depth, const int32_t *node_offsets, con
                   cudaStream_t st)
 {
     const int warps = 4;
-    accept_kernel<<<(B + warps - 1) / warps, warps * 32, 0, st>>>(
-        B, max_depth, node_offsets, parent, draft_tok, target_tok, root_target_tok, path_idx, path_len,
+    launch(accept_kernel, (B + warps - 1) / warps, warps * 32, 0, st, B, max_depth, node_offsets, parent, draft_tok, target_tok, root_target_tok, path_idx, path_len,
         next_tok, status);
     return int(cudaGetLastError());
 }
@@ -725,8 +732,7 @@ int launch_stochastic_accept(int32_t B, int32_t max_depth, const int32_t *node_o
                              int32_t *path_idx, int32_t *path_len, int32_t *status, cudaStream_t st)
 {
     const int warps = 4;
-    stochastic_accept_kernel<<<(B + warps - 1) / warps, warps * 32, 0, st>>>(
-        B, max_depth, node_offsets, parent, p_target, p_draft, uniform, path_idx, path_len, status);
+    launch(stochastic_accept_kernel, (B + warps - 1) / warps, warps * 32, 0, st, B, max_depth, node_offsets, parent, p_target, p_draft, uniform, path_idx, path_len, status);
     return int(cudaGetLastError());
 }
 

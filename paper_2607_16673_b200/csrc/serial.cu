@@ -89,6 +89,7 @@ template <int DK, int RS, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32)
 decode_kernel(Params p)
 {
+    after_previous_kernel();
     constexpr int G = Map<DK>::G, RPS = Map<DK>::RPS, ROWS = WARPS * RS * RPS;
     const int tiles = p.DV / ROWS;
     const long unit = blockIdx.x / tiles;                       // (l*B + b)*H + h == record index (T == B)
@@ -124,6 +125,7 @@ template <int DK, int RS, int WARPS, bool CHAIN>
 __global__ void __launch_bounds__(WARPS * 32)
 verify_serial_kernel(Params p)
 {
+    after_previous_kernel();
     constexpr int G = Map<DK>::G, RPS = Map<DK>::RPS, ROWS = WARPS * RS * RPS;
     extern __shared__ float4 slot_mem[];                         // [n_slots][ROWS][DK] floats
     const int tiles = p.DV / ROWS;
@@ -217,6 +219,7 @@ template <int DK, int RS, int WARPS, int TILES>
 __global__ void __launch_bounds__(WARPS * 32, 2048 / (WARPS * 32) / 2)
 commit_kernel(Params p)
 {
+    after_previous_kernel();
     constexpr int G = Map<DK>::G, RPS = Map<DK>::RPS, ROWS = WARPS * RS * RPS, part_rows = ROWS * TILES;
     const int parts = p.DV / part_rows;
     const long unit = blockIdx.x / parts;
@@ -347,7 +350,7 @@ template <int DK, int RS, int WARPS> struct LaunchDecode {
     static int run(const Params &p, cudaStream_t st)
     {
         const long blocks = n_units(p) * (p.DV / rows_per_cta<DK, RS, WARPS>());
-        decode_kernel<DK, RS, WARPS><<<unsigned(blocks), WARPS * 32, 0, st>>>(p);
+        launch(decode_kernel<DK, RS, WARPS>, unsigned(blocks), WARPS * 32, 0, st, p);
         return int(cudaGetLastError());
     }
 };
@@ -362,9 +365,9 @@ template <int DK, int RS, int WARPS> struct LaunchCommit {
         // d_k = d_v = 64: 162 us, two tiles 166).
         const long round = long(sm_count_of_current_device()) * (2048 / (WARPS * 32) / 2);
         if (DK > 64 && p.DV % (2 * ROWS) == 0 && tiles >= 8 * round)
-            commit_kernel<DK, RS, WARPS, 2><<<unsigned(tiles / 2), WARPS * 32, 0, st>>>(p);
+            launch(commit_kernel<DK, RS, WARPS, 2>, unsigned(tiles / 2), WARPS * 32, 0, st, p);
         else
-            commit_kernel<DK, RS, WARPS, 1><<<unsigned(tiles), WARPS * 32, 0, st>>>(p);
+            launch(commit_kernel<DK, RS, WARPS, 1>, unsigned(tiles), WARPS * 32, 0, st, p);
         return int(cudaGetLastError());
     }
 };
@@ -373,7 +376,7 @@ template <int DK, int RS, int WARPS> struct LaunchChain {
     static int run(const Params &p, cudaStream_t st)
     {
         const long blocks = n_units(p) * (p.DV / rows_per_cta<DK, RS, WARPS>());
-        verify_serial_kernel<DK, RS, WARPS, true><<<unsigned(blocks), WARPS * 32, 0, st>>>(p);
+        launch(verify_serial_kernel<DK, RS, WARPS, true>, unsigned(blocks), WARPS * 32, 0, st, p);
         return int(cudaGetLastError());
     }
 };
@@ -389,7 +392,7 @@ template <int DK, int RS, int WARPS> struct LaunchTree {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
             if (e != cudaSuccess) return int(e);
         }
-        kern<<<unsigned(blocks), WARPS * 32, smem, st>>>(p);
+        launch(kern, unsigned(blocks), WARPS * 32, smem, st, p);
         return int(cudaGetLastError());
     }
 };

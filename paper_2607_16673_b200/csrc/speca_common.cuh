@@ -155,6 +155,36 @@ inline int sm_count_of_current_device()
     return sms;
 }
 
+// ---------------------------------------------------------------------------
+// Overlapped launches (programmatic dependent launch).  A round is a handful of kernels on one stream, and between two of
+// them the device used to sit idle while one drained and the next was set up.  Every kernel here first waits until the
+// kernel in front of it has completed and its writes are visible, and only then lets the one behind it be set up, beside
+// its own last wave of blocks.  The order matters: the next kernel's blocks start with clean L1 lines only after
+// everything before this kernel has been written, so that its read-only loads are as safe as after a plain launch.
+// Kernels that are not launched this way, the caller's own among them, are waited for and wait as ever.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void after_previous_kernel()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+inline cudaError_t launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, const A &...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Number of on-chip state slots the light-children-first walk can need for a tree of
 // at most n nodes: a node saves its state only if it has two children with
 // children of their own (subtree >= 5 nodes) and every live slot at least halves
