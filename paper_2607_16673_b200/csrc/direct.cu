@@ -93,21 +93,24 @@ template <int DK, int NT, int MAXD> struct Lay {
     static constexpr int MS = NK + 8;                           // bf16 per row of a piece of M
     static constexpr int GS = N + 1;
     static constexpr int NR = NK;                               // rows of the weight pieces: whole MMA row blocks
+    // a node's path holds no later node, so row block m of the weights ends with column 16 m + 15
+    __host__ __device__ static constexpr int w_row(int r) { return 128 * (r >> 4) * ((r >> 4) + 2) + (r & 15) * (16 * (r >> 4) + 24); }
+    static constexpr int WP = w_row(NR);                        // bf16 per piece
     static constexpr int OffKQ = 0;                             // bf16 [2N][KQS]: key rows, query rows
     static constexpr int OffHi = OffKQ + 2 * N * KQS * 2;       // float [N][BS]
     static constexpr int OffLo = OffHi + N * BS * 4;
     static constexpr int OffM = OffLo + N * BS * 4;             // bf16 [3][N][MS]
     static constexpr int OffG = OffHi;                          // float [2N][GS]: Gram rows of keys, queries (dead before Hi is written)
-    static constexpr int OffW = OffM + 3 * N * MS * 2;          // bf16 [3][NR][MS]: weights of the keys in qeff
-    static constexpr int OffP = OffW + 3 * NR * MS * 2;         // int32 parent[N], float alpha[N], beta[N], scale gamma[NR]
+    static constexpr int OffW = OffM + 3 * N * MS * 2;          // bf16 [3][WP]: weights of the keys in qeff
+    static constexpr int OffP = OffW + 3 * WP * 2;         // int32 parent[N], float alpha[N], beta[N], scale gamma[NR]
     // rows of the back substitution: float c beta [N][MAXD], float rho [N][MAXD], uint8 path [N][MAXD]; behind the Gram
-    // rows where those leave room, and as dead as they are afterwards
+    // rows where those leave room, else over them (one barrier more), and as dead as they are afterwards
     static constexpr int GEnd = (OffG + 2 * N * GS * 4 + 15) & ~15, CBytes = 9 * N * MAXD;
-    static constexpr bool kFits = GEnd + CBytes <= OffHi + 2 * N * BS * 4;
-    static constexpr int POwn = OffP + (3 * N + NR) * 4;
-    static constexpr int OffC = kFits ? GEnd : POwn;
-    static constexpr int OffV = kFits ? POwn : POwn + CBytes;   // bf16 [NK][rows + 8]
+    static constexpr bool kOver = GEnd + CBytes > OffHi + 2 * N * BS * 4;
+    static constexpr int OffC = kOver ? OffG : GEnd;
+    static constexpr int OffV = OffP + (3 * N + NR) * 4;        // bf16 [NK][rows + 8]
     static_assert(2 * N * GS <= 2 * N * BS, "Gram rows do not fit the space of the effective queries");
+    static_assert(OffG + CBytes <= GEnd || !kOver, "rows of the back substitution do not fit the space of the Gram rows");
     static constexpr int bytes(int rows) { return OffV + NK * (rows + 8) * 2; }
 };
 
@@ -125,6 +128,8 @@ verify_direct_kernel(DirectArgs da)
     after_previous_kernel();
     using LY = Lay<DK, NT, MAXD>;
     constexpr int N = LY::N, NS = DK / 32, THREADS = WARPS * 32;
+    // a product wider than four column tiles is split between the warps: tile by tile, PARTS warps beside each other
+    constexpr int NTP = NT > 4 ? 4 : NT, PARTS = NT / NTP, STRIDE = WARPS / PARTS;
     extern __shared__ __align__(16) uint8_t smem[];
     const Params &p = da.p;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
@@ -202,7 +207,7 @@ verify_direct_kernel(DirectArgs da)
         asm volatile("cp.async.commit_group;" ::: "memory");
         if (!da.early) prefetch_first();
         for (int i = tid; i < 3 * N * LY::MS / 8; i += THREADS) reinterpret_cast<uint4 *>(sM)[i] = make_uint4(0u, 0u, 0u, 0u);
-        for (int i = tid; i < 3 * LY::NR * LY::MS / 8; i += THREADS) reinterpret_cast<uint4 *>(sW)[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = tid; i < 3 * LY::WP / 8; i += THREADS) reinterpret_cast<uint4 *>(sW)[i] = make_uint4(0u, 0u, 0u, 0u);
         if (tid < LY::NR) sGam[tid] = 0.f;
     }
     if (tid < n) {
@@ -257,8 +262,8 @@ verify_direct_kernel(DirectArgs da)
     if (__syncthreads_or(fault)) return;                     // reported above
 
     // ---- coefficients of node tid: back substitution up its path
+    float acc[MAXD];
     if (tid < n) {
-        float acc[MAXD];
         const float *gq = sG + (N + tid) * LY::GS;
 #pragma unroll
         for (int r = 0; r < MAXD; ++r) acc[r] = r < d ? gq[path[r]] : 0.f;
@@ -273,6 +278,9 @@ verify_direct_kernel(DirectArgs da)
             }
             acc[r] = cb;
         }
+    }
+    if (LY::kOver) __syncthreads();
+    if (tid < n) {
         float rho = p.scale;
         float *cb = sC + tid * MAXD, *ro = cb + N * MAXD;
 #pragma unroll
@@ -293,12 +301,12 @@ verify_direct_kernel(DirectArgs da)
         const int node = i / MAXD;
         const float cb = sC[i];
         float m = sC[N * MAXD + i] * cb, w = p.no_erase ? 0.f : -sGam[node] * cb;
-        __nv_bfloat16 *md = sM + node * LY::MS + a, *wd = sW + node * LY::MS + a;
+        __nv_bfloat16 *md = sM + node * LY::MS + a, *wd = sW + LY::w_row(node) + a;
 #pragma unroll
         for (int pc = 0; pc < 3; ++pc) {
             const __nv_bfloat16 mq = __float2bfloat16_rn(m), wq = __float2bfloat16_rn(w);
             md[pc * N * LY::MS] = mq;
-            wd[pc * LY::NR * LY::MS] = wq;
+            wd[pc * LY::WP] = wq;
             m -= __bfloat162float(mq);
             w -= __bfloat162float(wq);
         }
@@ -308,11 +316,11 @@ verify_direct_kernel(DirectArgs da)
     // the first two steps of this warp's first tile, requested a phase ahead of their use
     const float *Su = S_cta + g * DK + 8 * t4;
     float sa[2][8], sb[2][8];
-    if (warp < tiles)
+    if (warp / PARTS < tiles)
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            ld_state(sa[q], Su + warp * 16 * DK + 32 * q);
-            ld_state(sb[q], Su + (warp * 16 + 8) * DK + 32 * q);
+            ld_state(sa[q], Su + warp / PARTS * 16 * DK + 32 * q);
+            ld_state(sb[q], Su + (warp / PARTS * 16 + 8) * DK + 32 * q);
         }
 
     // ---- effective queries (scale gamma q + W K, the weights in three bf16 pieces), split into head and remainder
@@ -339,7 +347,7 @@ verify_direct_kernel(DirectArgs da)
 #pragma unroll
                 for (int pc = 0; pc < 3; ++pc) {
                     uint32_t a[4];
-                    ldsm_x4(a, sW + (pc * LY::NR + 16 * mi + (lane & 15)) * LY::MS + 16 * kk + ((lane >> 4) << 3));
+                    ldsm_x4(a, sW + pc * LY::WP + LY::w_row(16 * mi + (lane & 15)) + 16 * kk + ((lane >> 4) << 3));
                     mma_bf16_sync(acc[0], a, kb[0], kb[1]);
                     mma_bf16_sync(acc[1], a, kb[2], kb[3]);
                 }
@@ -364,20 +372,22 @@ verify_direct_kernel(DirectArgs da)
     // ---- the state: one 16-row tile at a time, two 32-column steps of registers in flight
     // lane (g, t) holds columns 32 q + 8 t .. + 7 of rows g and g + 8: k-steps e = 0..3 of the step contract
     // columns 8 t + 2 e and 8 t + 2 e + 1 of the four lanes
-    const float *hi_p = sHi + g * LY::BS + 8 * t4, *lo_p = sLo + g * LY::BS + 8 * t4;
-    const int nk = (n + 15) >> 4;
+    const int half = PARTS == 1 ? 0 : warp % PARTS, i0 = half * NTP;         // this warp's column tiles: i0 ..
+    const float *hi_p = sHi + (8 * i0 + g) * LY::BS + 8 * t4, *lo_p = sLo + (8 * i0 + g) * LY::BS + 8 * t4;
+    const int nk = (n + 15) >> 4, ntp = nt - i0;
+    if (PARTS > 1 && ntp <= 0) return;
     float *o0 = p.o + rec0 * p.DV + row0 + g;
     const long node_stride = long(H) * p.DV;
 #pragma unroll 1
-    for (int tile = warp; tile < tiles; tile += WARPS) {
-        if (lane == 0 && tile + AHEAD < tiles) prefetch_l2(S_cta + long(tile + AHEAD) * 16 * DK, 16 * DK * 4);
-        const bool next = tile + WARPS < tiles;
-        float hh[NT][4], xx[NT][4];                          // head x head, and the two cross products
+    for (int tile = warp / PARTS; tile < tiles; tile += STRIDE) {
+        if (lane == 0 && half == 0 && tile + AHEAD < tiles) prefetch_l2(S_cta + long(tile + AHEAD) * 16 * DK, 16 * DK * 4);
+        const bool next = tile + STRIDE < tiles;
+        float hh[NTP][4], xx[NTP][4];                         // head x head, and the two cross products
 #pragma unroll
-        for (int i = 0; i < NT; ++i)
+        for (int i = 0; i < NTP; ++i)
 #pragma unroll
             for (int e = 0; e < 4; ++e) { hh[i][e] = 0.f; xx[i][e] = 0.f; }
-        const float *cur = Su + long(tile) * 16 * DK, *nxt = cur + WARPS * 16 * DK - NS * 32;
+        const float *cur = Su + long(tile) * 16 * DK, *nxt = cur + STRIDE * 16 * DK - NS * 32;
 #pragma unroll
         for (int q = 0; q < NS; ++q) {
             uint32_t ah[4][4], al[4][4];                     // [k-step][fragment register]
@@ -393,8 +403,8 @@ verify_direct_kernel(DirectArgs da)
                 ld_state(sb[q & 1], src + 8 * DK);
             }
 #pragma unroll
-            for (int i = 0; i < NT; ++i) {
-                if (NT > 1 && i >= nt) break;
+            for (int i = 0; i < NTP; ++i) {
+                if (NTP > 1 && i >= ntp) break;
 #pragma unroll
                 for (int e2 = 0; e2 < 2; ++e2) {
                     const float4 bh = *reinterpret_cast<const float4 *>(hi_p + 8 * i * LY::BS + 32 * q + 4 * e2);
@@ -417,12 +427,12 @@ verify_direct_kernel(DirectArgs da)
                 uint32_t a[4];
                 ldsm_x4_t(a, va + kk * 16 * vstride);
 #pragma unroll
-                for (int i = 0; i < NT; ++i) {
-                    if (NT > 1 && i >= nt) break;
-                    if (8 * i + 7 < 16 * kk) continue;       // a node's path holds no later node
+                for (int i = 0; i < NTP; ++i) {
+                    if (NTP > 1 && i >= ntp) break;
+                    if (8 * (i0 + i) + 7 < 16 * kk) continue;       // a node's path holds no later node
 #pragma unroll
                     for (int pc = 0; pc < 3; ++pc) {
-                        const __nv_bfloat16 *mb = sM + (pc * N + 8 * i + g) * LY::MS + 16 * kk + 2 * t4;
+                        const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
                         mma_bf16_sync(xx[i], a, *reinterpret_cast<const uint32_t *>(mb), *reinterpret_cast<const uint32_t *>(mb + 8));
                     }
                 }
@@ -430,9 +440,9 @@ verify_direct_kernel(DirectArgs da)
         }
         float *ot = o0 + tile * 16;
 #pragma unroll
-        for (int i = 0; i < NT; ++i) {
-            if (NT > 1 && i >= nt) break;
-            const int n0 = 8 * i + 2 * t4;
+        for (int i = 0; i < NTP; ++i) {
+            if (NTP > 1 && i >= ntp) break;
+            const int n0 = 8 * (i0 + i) + 2 * t4;
             float *od = ot + n0 * node_stride;
             if (n0 < n) { od[0] = hh[i][0] + xx[i][0]; od[8] = hh[i][2] + xx[i][2]; }
             if (n0 + 1 < n) { od[node_stride] = hh[i][1] + xx[i][1]; od[node_stride + 8] = hh[i][3] + xx[i][3]; }
@@ -478,7 +488,9 @@ int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
 
 // Warps per CTA and CTAs per SM by the width NT of the product: registers (two 32-column steps of state, the
 // accumulators) allow 80 / 96 / 128 per thread, shared memory two CTAs at 32 nodes, where eight warps share the longer
-// set-up.
+// set-up, and at 64.  There two warps share a state tile, 32 nodes each: a whole 64-node product per warp took 198
+// registers and left four of the eight warps of a 64-row unit without a tile (1060 units of 33..40 nodes beside 3548
+// smaller ones, d_k = d_v = 64: one round of calls 137 us with one CTA per SM, 112 with two).
 template <int DK, int MAXD>
 int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_t st)
 {
@@ -487,7 +499,7 @@ int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_
     if (hi <= 16) return launch_one<DK, 2, MAXD, 4, C2>(p, lo, all, sms, st);
     if constexpr (DK == 64) {
         if (hi <= 32) return launch_one<DK, 4, MAXD, 4, 4>(p, lo, all, sms, st);
-        return launch_one<DK, 8, MAXD, 8, 1>(p, lo, all, sms, st);
+        return launch_one<DK, 8, MAXD, 8, 2>(p, lo, all, sms, st);
     } else {
         return launch_one<DK, 4, MAXD, 8, 2>(p, lo, all, sms, st);
     }
