@@ -465,11 +465,18 @@ int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
     // queue behind the state, and the set-up waits for them (384 chains of 8: 11.8 us, after the records 10.4; 4608
     // units of 32 nodes at d_k = d_v = 64: 67.8 / 65.8).
     da.early = all && DK > 64 && !small_batch(p, sms);
-    // value rows per CTA: the whole unit, halved while the device would be left with idle slots
-    const long units = long(p.L) * p.B * p.H;
+    // Value rows per CTA: the whole unit, halved as long as all halves start at once: a second wave of set-ups costs more
+    // than the idle slots (us, whole / halved: 384 units at d_k = d_v = 128 of 16 nodes 20.5 / 22.5, 12 nodes 18.4 / 22.5; d_v
+    // = 256, 8 nodes 20.5 / 24.6; 384 units at d_k = 256 of 8 nodes 36.9 / 41.0).  Only where a warp has two 16 KB
+    // tiles left is the halving worth the second wave (192 units at d_k = 256 of 8 nodes 24.6 / 22.5).
+    const long units = long(p.L) * p.B * p.H, slots = long(sms) * CTAS;
     int rows = p.DV;
     while (rows > 256 && rows % 32 == 0) rows /= 2;
-    while (rows % 32 == 0 && rows / 16 > WARPS && units * (p.DV / rows) < long(sms) * CTAS) rows /= 2;
+    while (rows % 32 == 0 && rows / 16 > WARPS) {
+        const long ctas = units * (p.DV / rows);
+        if (ctas * 2 > slots && !(DK == 256 && rows <= 32 * WARPS && ctas < slots)) break;
+        rows /= 2;
+    }
     da.rows = rows;
     da.parts = p.DV / rows;
     const int smem = LY::bytes(rows);
@@ -488,9 +495,7 @@ int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
 
 // Warps per CTA and CTAs per SM by the width NT of the product: registers (two 32-column steps of state, the
 // accumulators) allow 80 / 96 / 128 per thread, shared memory two CTAs at 32 nodes, where eight warps share the longer
-// set-up, and at 64.  There two warps share a state tile, 32 nodes each: a whole 64-node product per warp took 198
-// registers and left four of the eight warps of a 64-row unit without a tile (1060 units of 33..40 nodes beside 3548
-// smaller ones, d_k = d_v = 64: one round of calls 137 us with one CTA per SM, 112 with two).
+// set-up.
 template <int DK, int MAXD>
 int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_t st)
 {
@@ -501,6 +506,12 @@ int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_
         if (hi <= 32) return launch_one<DK, 4, MAXD, 4, 4>(p, lo, all, sms, st);
         return launch_one<DK, 8, MAXD, 8, 2>(p, lo, all, sms, st);
     } else {
+        // between two and three units per SM one wave of smaller CTAs beats two of the others (d_k = d_v = 128, 32 nodes: 384
+        // units 24.6 us, with eight warps 26.6; 432 units the same; 576 units take two waves either way); at d_v > 128 three
+        // do not fit in shared memory
+        const long units = long(p.L) * p.B * p.H;
+        if constexpr (DK == 128)
+            if (p.DV <= 128 && units > 2 * sms && units <= 3 * sms) return launch_one<DK, 4, MAXD, 4, 3>(p, lo, all, sms, st);
         return launch_one<DK, 4, MAXD, 8, 2>(p, lo, all, sms, st);
     }
 }

@@ -43,6 +43,15 @@ def test_chain_entry_point(n):
     check(prob, 16, chain=True)
 
 
+@pytest.mark.parametrize("L,B,d_k,d_v", [(3, 12, 128, 128), (3, 12, 128, 32), (3, 12, 256, 256), (2, 6, 256, 256)])
+def test_batches_around_one_wave(L, B, d_k, d_v):
+    """Between two and three units per SM (smaller CTAs), and unit counts whose value rows are split or not."""
+    rng = np.random.default_rng(705 + d_v)
+    top = 32 if d_k == 128 else 8
+    parents = [tree(int(n), 6, rng) for n in np.linspace(1, top, B).round()]
+    check(synth.make_problem(706 + d_v, L, 12, d_k, d_v, parents), top)
+
+
 @pytest.mark.parametrize("d_k,B", [(64, 12), (128, 40)])
 def test_ragged_batch_crosses_the_launch_boundaries(d_k, B):
     """Large enough for several launches by size; empty sequences, forests and every size class in one batch."""
