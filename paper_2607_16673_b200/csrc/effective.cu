@@ -130,22 +130,22 @@ struct EMaps { CUtensorMap k[4], q[4], v[4]; };       // one per box height: 16,
 
 struct EParams {
     Params p;
-    int32_t heads_per_group;
+    int32_t share;                   // log2 of the units that share a head's keys and queries: see launch_verify_effective
     int32_t withhold_first_load;     // failure-detection test: CTA 0 never requests its first state slice
     int32_t want_u;
-    int32_t gpl, dl, db, dg;         // groups of heads per (layer, sequence); a step of gridDim.x groups as (layers, sequences, groups)
+    int32_t dl, db, dh;              // a step of gridDim.x units as (layers, sequences, heads)
 };
 
 // A unit is one (layer, sequence, head); with u requested it is walked twice (kind 0: o rows, kind 1: u rows).
-// Units are taken in groups of HG consecutive heads of one (layer, sequence): group blockIdx.x, += gridDim.x, kept as
-// (layer, sequence, group of heads) and advanced by carries, not divisions: every role walks the list by itself, so
-// this code is there ten times.
+// Units go round the CTAs one by one: unit blockIdx.x, += gridDim.x, kept as (layer, sequence, head) and advanced by
+// carries, not divisions: every role walks the list by itself, so this code is there ten times.  (Four consecutive heads
+// at a time left some CTAs four units more than others: 16 sequences of 40..64 nodes, a round 626 us, one by one 614.)
 struct VUnit {
-    int l, b, h, u, n, npad, base, kind, hi;
-    int nl, nb, ng;                                              // the group after this one
+    int l, b, h, u, n, npad, base, kind;
+    int nl, nb, nh;                                              // the unit after this one
 };
 struct Walk {
-    int HG, gpl, L, B, H, dl, db, dg, two;                       // d*: a step of gridDim.x groups
+    int L, B, H, dl, db, dh, two;                                // d*: a step of gridDim.x units
     const int32_t *seq_n; const int32_t *offs;
     const uint8_t *tab;
 };
@@ -154,18 +154,14 @@ __device__ __forceinline__ bool next_unit(const Walk &w, VUnit &x)
 {
     if (w.two && x.kind == 0) { x.kind = 1; return true; }
     x.kind = 0;
-    if (++x.hi < w.HG) { ++x.h; ++x.u; return true; }
     while (x.nl < w.L) {
-        x.l = x.nl; x.b = x.nb;
-        const int g = x.ng;
-        x.ng += w.dg; x.nb += w.db; x.nl += w.dl;
-        if (x.ng >= w.gpl) { x.ng -= w.gpl; ++x.nb; }
+        x.l = x.nl; x.b = x.nb; x.h = x.nh;
+        x.nh += w.dh; x.nb += w.db; x.nl += w.dl;
+        if (x.nh >= w.H) { x.nh -= w.H; ++x.nb; }
         if (x.nb >= w.B) { x.nb -= w.B; ++x.nl; }
         const bool in_tab = x.b < kWalkSeqs;
         x.n = in_tab ? int(reinterpret_cast<const int8_t *>(w.tab + 4 * kWalkSeqs)[x.b]) : w.seq_n[x.b];
         if (x.n > 0) {
-            x.hi = 0;
-            x.h = g * w.HG;
             x.u = (x.l * w.B + x.b) * w.H + x.h;
             x.npad = (x.n + 15) & ~15;
             x.base = in_tab ? reinterpret_cast<const int32_t *>(w.tab)[x.b] : __ldg(w.offs + x.b);
@@ -173,11 +169,14 @@ __device__ __forceinline__ bool next_unit(const Walk &w, VUnit &x)
         }
     }
     x.n = 0;
-    x.hi = w.HG;
     x.kind = 1;
     return false;
 }
 
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 // one arrival for the whole warp: every lane's earlier writes are ordered before it
 __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane)
 {
@@ -269,7 +268,6 @@ template <int TP, int DK, int MAXN, int MAXD>
 __global__ void __launch_bounds__(kThreads, 1)
 verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid_constant__ EMaps maps, EParams ep)
 {
-    after_previous_kernel();
     using LY = Lay<DK, MAXN, MAXD>;
     constexpr int NS = LY::NS, NC = LY::NC, SC = LY::SC, SCB = LY::SCB;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -310,27 +308,31 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         mbar_init(bar(kDrain), 2);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), kTmemCols);
+    // The plan kernel runs just before this one and writes none of the state: the first tile of the first unit is on its
+    // way into L2 while the plan is made.
+    if (threadIdx.x == 0 && (blockIdx.x < unsigned(p.L * p.B * p.H)))
+        prefetch_l2(p.S0 + size_t(blockIdx.x) * p.DV * DK, uint32_t(kRows * DK * 4));
+    after_previous_kernel();
     for (int b = threadIdx.x; b < p.B && b < kWalkSeqs; b += blockDim.x) {
         const int n = p.ws.seq_n[b];
         reinterpret_cast<int32_t *>(smem + LY::OffWalk)[b] = p.node_offsets[b];
         reinterpret_cast<int8_t *>(smem + LY::OffWalk + 4 * kWalkSeqs)[b] = int8_t(n < 0 ? -1 : n);
     }
-    if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
     Walk walk;
-    walk.HG = ep.heads_per_group; walk.gpl = ep.gpl;
     walk.L = p.L; walk.B = p.B; walk.H = p.H;
-    walk.dl = ep.dl; walk.db = ep.db; walk.dg = ep.dg;
+    walk.dl = ep.dl; walk.db = ep.db; walk.dh = ep.dh;
     walk.two = ep.want_u;
     walk.seq_n = p.ws.seq_n; walk.offs = p.node_offsets;
     walk.tab = smem + LY::OffWalk;
     VUnit x;                                                     // before the first unit
-    x.kind = 1; x.hi = walk.HG; x.n = 0;
-    x.ng = int(blockIdx.x) % ep.gpl; x.nb = int(blockIdx.x) / ep.gpl % p.B; x.nl = int(blockIdx.x) / ep.gpl / p.B;
+    x.kind = 1; x.n = 0;
+    x.nh = int(blockIdx.x) % p.H; x.nb = int(blockIdx.x) / p.H % p.B; x.nl = int(blockIdx.x) / p.H / p.B;
     bool ok = true;
 
     const uint32_t lead = elect_one();                           // the thread that issues this warp's tcgen05 instructions
@@ -451,8 +453,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                     mbar_arrive_expect_tx(bar(kKQFull + par), uint32_t(4 * kx.npad * DK));
 #pragma unroll 1
                     for (int c = 0; c < SC; ++c) {
-                        tma_load_3d(stage + c * SCB, &maps.k[m], c * 64, kx.h, z, bar(kKQFull + par));
-                        tma_load_3d(stage + c * SCB + kx.npad * 128, &maps.q[m], c * 64, kx.h, z, bar(kKQFull + par));
+                        tma_load_3d(stage + c * SCB, &maps.k[m], c * 64, kx.h >> ep.share, z, bar(kKQFull + par));
+                        tma_load_3d(stage + c * SCB + kx.npad * 128, &maps.q[m], c * 64, kx.h >> ep.share, z, bar(kKQFull + par));
                     }
                 }
                 __syncwarp();
@@ -640,7 +642,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 const int2 s = __ldg(reinterpret_cast<const int2 *>(p.ws.set) + i);
                 lo_n = uint32_t(s.x); hi_n = uint32_t(s.y);
                 d_n = __ldg(p.ws.depth + i);
-                const int r = (y.l * p.T + i) * p.H + y.h;
+                const int r = ((y.l * p.T + i) * p.H + y.h) >> ep.share;
                 alpha_n = __ldg(p.alpha + r);
                 beta_n = __ldg(p.beta + r);
             }
@@ -812,11 +814,30 @@ bool effective_supported(const speca_dims *d)
 static int g_withhold_first_load = 0;
 void effective_set_withhold(int on) { g_withhold_first_load = on; }
 
-int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
+int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
 {
     if (d_k != 128 && d_k != 256) return int(cudaErrorInvalidValue);
     EncodeTiledFn encode = encode_tiled_fn();
     if (encode == nullptr) return int(cudaErrorNotSupported);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return int(cudaErrorInvalidDevice);
+    DeviceInfo &di = g_dev[dev];
+    if (di.sm_count == 0) {
+        int n = 0;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        di.sm_count = n > 0 ? n : 148;
+    }
+    // Few units leave SMs idle, or with one unit while others work on two.  A head of two value tiles then counts as two
+    // heads of one tile that share keys, queries and gates: states, value rows and outputs already lie that way.  The
+    // coefficients are made twice, and a unit's solve takes as long whatever its value rows, so this pays while every half has an SM
+    // of its own (48 units, d_k = 128, 64 nodes: verification 17.4 us, whole units 19.5) and, for up to 8 levels, where
+    // the busiest SM walks fewer tiles of few (192 units: 27.7, whole 29.7; at 16 levels 35.8 / 33.8).
+    Params p = call;
+    const int heads = p.H;
+    const long sms = di.sm_count, whole = (long(p.L) * p.B * p.H + sms - 1) / sms, halves = (2L * p.L * p.B * p.H + sms - 1) / sms;
+    const int share = p.DV == 2 * kRows && (halves == 1 || (p.max_depth <= 8 && halves < 2 * whole && whole <= 4)) ? 1 : 0;
+    p.H <<= share;
+    p.DV >>= share;
     const long n_units = long(p.L) * p.B * p.H;
     const cuuint32_t es[3] = {1, 1, 1};
     CUtensorMap map;
@@ -831,8 +852,8 @@ int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
     }
     EMaps em;
     {
-        const cuuint64_t gd[3] = {cuuint64_t(d_k), cuuint64_t(p.H), cuuint64_t(p.L) * cuuint64_t(p.T)};
-        const cuuint64_t gs[2] = {cuuint64_t(d_k) * 2, cuuint64_t(p.H) * d_k * 2};
+        const cuuint64_t gd[3] = {cuuint64_t(d_k), cuuint64_t(heads), cuuint64_t(p.L) * cuuint64_t(p.T)};
+        const cuuint64_t gs[2] = {cuuint64_t(d_k) * 2, cuuint64_t(heads) * d_k * 2};
         const cuuint64_t vd[3] = {cuuint64_t(p.DV), cuuint64_t(p.H), cuuint64_t(p.L) * cuuint64_t(p.T)};
         const cuuint64_t vs[2] = {cuuint64_t(p.DV) * 2, cuuint64_t(p.H) * p.DV * 2};
         for (int m = 0; m < 4 && 16 * m < p.max_nodes; ++m) {    // box heights a sequence of this call can need
@@ -851,14 +872,6 @@ int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
         }
     }
 
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return int(cudaErrorInvalidDevice);
-    DeviceInfo &di = g_dev[dev];
-    if (di.sm_count == 0) {
-        int n = 0;
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        di.sm_count = n > 0 ? n : 148;
-    }
     if (!di.attr_set) {
         cudaError_t e = cudaSuccess;
         auto opt_in = [&](const void *k, int bytes) {
@@ -881,16 +894,11 @@ int launch_verify_effective(const Params &p, int d_k, cudaStream_t st)
     ep.p = p;
     ep.want_u = p.u != nullptr ? 1 : 0;
     ep.withhold_first_load = g_withhold_first_load;
-    // consecutive heads of one (layer, sequence) a CTA takes together: as many as divide H while every SM still gets a group
-    ep.heads_per_group = 1;
-    for (int hg = 4; hg > 1; hg >>= 1)
-        if (p.H % hg == 0 && n_units / hg >= di.sm_count) { ep.heads_per_group = hg; break; }
-    const long n_groups = n_units / ep.heads_per_group;
-    const int grid = int(n_groups < di.sm_count ? n_groups : di.sm_count);
-    ep.gpl = p.H / ep.heads_per_group;
-    ep.dg = grid % ep.gpl;
-    ep.db = grid / ep.gpl % p.B;
-    ep.dl = grid / ep.gpl / p.B;
+    ep.share = share;
+    const int grid = int(n_units < di.sm_count ? n_units : di.sm_count);
+    ep.dh = grid % p.H;
+    ep.db = grid / p.H % p.B;
+    ep.dl = grid / p.H / p.B;
     const bool one_tile = p.DV == kRows;
     const bool deep = p.max_depth > 8;
     auto go = [&](auto dk, auto mn, auto md) {

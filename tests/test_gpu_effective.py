@@ -37,6 +37,25 @@ def test_small_and_large_units_in_turn(d_k, d_v, depth, want_u):
         assert rel_err(dp.u.cpu().numpy(), ds.u.cpu().numpy()) <= TOL_FP32
 
 
+@pytest.mark.parametrize("want_u", [False, True])
+@pytest.mark.parametrize("d_k", [128, 256])
+@pytest.mark.parametrize("L,B,H", [(1, 1, 1), (2, 7, 5), (3, 21, 3), (1, 37, 4), (4, 10, 5)])
+def test_heads_split_by_value_tile(L, B, H, d_k, want_u):
+    """Unit counts on both sides of every bound at which a head of two value tiles counts as two units."""
+    rng = np.random.default_rng(840 + B)
+    top = 64 if d_k == 128 else 32
+    parents = [tree(int(n), 8, rng) for n in np.linspace(top, 1, B).round()]
+    prob = synth.make_problem(841 + B, L, H, d_k, 256, parents, max_depth=8, state_std=0.3)
+    dp = DevProblem(prob, route=speca.ROUTE_EFFECTIVE, want_u=want_u, max_nodes=top)
+    dp.verify_tree()
+    assert dp.status_value() == 0
+    assert rel_err(dp.o.cpu().numpy(), oracle_verify(prob)) <= TOL_FP32
+    if want_u:
+        ds = DevProblem(prob, route=speca.ROUTE_SERIAL, want_u=True, max_nodes=top)
+        ds.verify_tree()
+        assert rel_err(dp.u.cpu().numpy(), ds.u.cpu().numpy()) <= TOL_FP32
+
+
 def test_rule_without_erase():
     rng = np.random.default_rng(820)
     prob = synth.make_problem(821, 2, 4, 128, 256, [tree(n, 8, rng) for n in (40, 7, 64)])
