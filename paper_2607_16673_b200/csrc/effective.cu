@@ -133,19 +133,20 @@ struct EParams {
     int32_t share;                   // log2 of the units that share a head's keys and queries: see launch_verify_effective
     int32_t withhold_first_load;     // failure-detection test: CTA 0 never requests its first state slice
     int32_t want_u;
-    int32_t dl, db, dh;              // a step of gridDim.x units as (layers, sequences, heads)
+    int32_t heads_per_group;
+    int32_t gpl, dl, db, dg;         // groups of heads per (layer, sequence); a step of gridDim.x groups as (layers, sequences, groups)
 };
 
 // A unit is one (layer, sequence, head); with u requested it is walked twice (kind 0: o rows, kind 1: u rows).
-// Units go round the CTAs one by one: unit blockIdx.x, += gridDim.x, kept as (layer, sequence, head) and advanced by
-// carries, not divisions: every role walks the list by itself, so this code is there ten times.  (Four consecutive heads
-// at a time left some CTAs four units more than others: 16 sequences of 40..64 nodes, a round 626 us, one by one 614.)
+// Units are taken in groups of HG consecutive heads of one (layer, sequence): group blockIdx.x, += gridDim.x, kept as
+// (layer, sequence, group of heads) and advanced by carries, not divisions: every role walks the list by itself, so
+// this code is there ten times.
 struct VUnit {
-    int l, b, h, u, n, npad, base, kind;
-    int nl, nb, nh;                                              // the unit after this one
+    int l, b, h, u, n, npad, base, kind, hi;
+    int nl, nb, ng;                                              // the group after this one
 };
 struct Walk {
-    int L, B, H, dl, db, dh, two;                                // d*: a step of gridDim.x units
+    int HG, gpl, L, B, H, dl, db, dg, two;                       // d*: a step of gridDim.x groups
     const int32_t *seq_n; const int32_t *offs;
     const uint8_t *tab;
 };
@@ -154,14 +155,18 @@ __device__ __forceinline__ bool next_unit(const Walk &w, VUnit &x)
 {
     if (w.two && x.kind == 0) { x.kind = 1; return true; }
     x.kind = 0;
+    if (++x.hi < w.HG) { ++x.h; ++x.u; return true; }
     while (x.nl < w.L) {
-        x.l = x.nl; x.b = x.nb; x.h = x.nh;
-        x.nh += w.dh; x.nb += w.db; x.nl += w.dl;
-        if (x.nh >= w.H) { x.nh -= w.H; ++x.nb; }
+        x.l = x.nl; x.b = x.nb;
+        const int g = x.ng;
+        x.ng += w.dg; x.nb += w.db; x.nl += w.dl;
+        if (x.ng >= w.gpl) { x.ng -= w.gpl; ++x.nb; }
         if (x.nb >= w.B) { x.nb -= w.B; ++x.nl; }
         const bool in_tab = x.b < kWalkSeqs;
         x.n = in_tab ? int(reinterpret_cast<const int8_t *>(w.tab + 4 * kWalkSeqs)[x.b]) : w.seq_n[x.b];
         if (x.n > 0) {
+            x.hi = 0;
+            x.h = g * w.HG;
             x.u = (x.l * w.B + x.b) * w.H + x.h;
             x.npad = (x.n + 15) & ~15;
             x.base = in_tab ? reinterpret_cast<const int32_t *>(w.tab)[x.b] : __ldg(w.offs + x.b);
@@ -169,6 +174,7 @@ __device__ __forceinline__ bool next_unit(const Walk &w, VUnit &x)
         }
     }
     x.n = 0;
+    x.hi = w.HG;
     x.kind = 1;
     return false;
 }
@@ -264,7 +270,9 @@ __device__ __forceinline__ bool prof_wait(long long &acc, uint32_t bar, uint32_t
 
 
 // TP = value tiles per unit (d_v / 128), DK = key width, MAXN = nodes per sequence, MAXD = tree depth.
-template <int TP, int DK, int MAXN, int MAXD>
+// FEW = a call of a few units per SM: launched beside the plan kernel, value tiles of a head on two SMs.  (In a long call
+// every instruction of the ten roles counts, and the plain form is 1 to 2 % faster.)
+template <int TP, int DK, int MAXN, int MAXD, bool FEW>
 __global__ void __launch_bounds__(kThreads, 1)
 verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid_constant__ EMaps maps, EParams ep)
 {
@@ -308,32 +316,36 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         mbar_init(bar(kDrain), 2);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), kTmemCols);
-    // The plan kernel runs just before this one and writes none of the state: the first tile of the first unit is on its
-    // way into L2 while the plan is made.
-    if (threadIdx.x == 0 && (blockIdx.x < unsigned(p.L * p.B * p.H)))
-        prefetch_l2(p.S0 + size_t(blockIdx.x) * p.DV * DK, uint32_t(kRows * DK * 4));
-    after_previous_kernel();
+    if constexpr (FEW) {
+        // The plan kernel runs just before this one and writes none of the state: the first tile of the first unit is on
+        // its way into L2 while the plan is made.
+        if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), kTmemCols);
+        if (threadIdx.x == 0) prefetch_l2(p.S0 + size_t(blockIdx.x) * p.DV * DK, uint32_t(kRows * DK * 4));
+        wait_for_previous_kernel();
+    }
     for (int b = threadIdx.x; b < p.B && b < kWalkSeqs; b += blockDim.x) {
         const int n = p.ws.seq_n[b];
         reinterpret_cast<int32_t *>(smem + LY::OffWalk)[b] = p.node_offsets[b];
         reinterpret_cast<int8_t *>(smem + LY::OffWalk + 4 * kWalkSeqs)[b] = int8_t(n < 0 ? -1 : n);
     }
+    if (!FEW && warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
     Walk walk;
+    walk.HG = ep.heads_per_group; walk.gpl = ep.gpl;
     walk.L = p.L; walk.B = p.B; walk.H = p.H;
-    walk.dl = ep.dl; walk.db = ep.db; walk.dh = ep.dh;
+    walk.dl = ep.dl; walk.db = ep.db; walk.dg = ep.dg;
     walk.two = ep.want_u;
     walk.seq_n = p.ws.seq_n; walk.offs = p.node_offsets;
     walk.tab = smem + LY::OffWalk;
     VUnit x;                                                     // before the first unit
-    x.kind = 1; x.n = 0;
-    x.nh = int(blockIdx.x) % p.H; x.nb = int(blockIdx.x) / p.H % p.B; x.nl = int(blockIdx.x) / p.H / p.B;
+    x.kind = 1; x.hi = walk.HG; x.n = 0;
+    x.ng = int(blockIdx.x) % ep.gpl; x.nb = int(blockIdx.x) / ep.gpl % p.B; x.nl = int(blockIdx.x) / ep.gpl / p.B;
     bool ok = true;
+    auto head_of = [&](const VUnit &y) { return FEW ? y.h >> ep.share : y.h; };
 
     const uint32_t lead = elect_one();                           // the thread that issues this warp's tcgen05 instructions
 
@@ -453,8 +465,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                     mbar_arrive_expect_tx(bar(kKQFull + par), uint32_t(4 * kx.npad * DK));
 #pragma unroll 1
                     for (int c = 0; c < SC; ++c) {
-                        tma_load_3d(stage + c * SCB, &maps.k[m], c * 64, kx.h >> ep.share, z, bar(kKQFull + par));
-                        tma_load_3d(stage + c * SCB + kx.npad * 128, &maps.q[m], c * 64, kx.h >> ep.share, z, bar(kKQFull + par));
+                        tma_load_3d(stage + c * SCB, &maps.k[m], c * 64, head_of(kx), z, bar(kKQFull + par));
+                        tma_load_3d(stage + c * SCB + kx.npad * 128, &maps.q[m], c * 64, head_of(kx), z, bar(kKQFull + par));
                     }
                 }
                 __syncwarp();
@@ -642,7 +654,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 const int2 s = __ldg(reinterpret_cast<const int2 *>(p.ws.set) + i);
                 lo_n = uint32_t(s.x); hi_n = uint32_t(s.y);
                 d_n = __ldg(p.ws.depth + i);
-                const int r = ((y.l * p.T + i) * p.H + y.h) >> ep.share;
+                const int r = FEW ? ((y.l * p.T + i) * p.H + y.h) >> ep.share : (y.l * p.T + i) * p.H + y.h;
                 alpha_n = __ldg(p.alpha + r);
                 beta_n = __ldg(p.beta + r);
             }
@@ -776,6 +788,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         }
         PROF_STORE()
     }
+    if (FEW && warp == 0) let_next_kernel_in();
     if (warp == 1 || warp == 2) {
         // everything these warps issued must have completed before TMEM is released
         mma_commit(bar(kDrain), lead);
@@ -879,10 +892,14 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
         };
         auto all = [&](auto dk, auto mn) {
             constexpr int DK = decltype(dk)::value, MN = decltype(mn)::value;
-            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, DK, MN, 8>), Lay<DK, MN, 8>::Bytes);
-            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, DK, MN, 8>), Lay<DK, MN, 8>::Bytes);
-            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, DK, MN, 16>), Lay<DK, MN, 16>::Bytes);
-            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, DK, MN, 16>), Lay<DK, MN, 16>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, DK, MN, 8, false>), Lay<DK, MN, 8>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, DK, MN, 8, true>), Lay<DK, MN, 8>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, DK, MN, 8, false>), Lay<DK, MN, 8>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, DK, MN, 8, true>), Lay<DK, MN, 8>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, DK, MN, 16, false>), Lay<DK, MN, 16>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<1, DK, MN, 16, true>), Lay<DK, MN, 16>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, DK, MN, 16, false>), Lay<DK, MN, 16>::Bytes);
+            opt_in(reinterpret_cast<const void *>(verify_effective_kernel<2, DK, MN, 16, true>), Lay<DK, MN, 16>::Bytes);
         };
         all(Int<128>{}, Int<32>{});
         all(Int<128>{}, Int<64>{});
@@ -895,18 +912,32 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     ep.want_u = p.u != nullptr ? 1 : 0;
     ep.withhold_first_load = g_withhold_first_load;
     ep.share = share;
-    const int grid = int(n_units < di.sm_count ? n_units : di.sm_count);
-    ep.dh = grid % p.H;
-    ep.db = grid / p.H % p.B;
-    ep.dl = grid / p.H / p.B;
+    // Consecutive heads of one (layer, sequence) that a CTA takes together.  The next head of a group costs a role two
+    // additions, the next group some hundred cycles of a chain that short units wait for; but whole groups leave some CTAs
+    // longer lists than others.  Verification in us with groups of 4 / single heads: 128 sequences, half 64-node trees,
+    // 332 units per CTA 1753 / 1807; 32 ragged ones, 83 units 455 / 439; 16 of 40..64 nodes, 41 units 341 / 323.
+    ep.heads_per_group = p.H % 4 == 0 && n_units / 4 >= 32 * sms ? 4 : 1;
+    const long n_groups = n_units / ep.heads_per_group;
+    const int grid = int(n_groups < di.sm_count ? n_groups : di.sm_count);
+    ep.gpl = p.H / ep.heads_per_group;
+    ep.dg = grid % ep.gpl;
+    ep.db = grid / ep.gpl % p.B;
+    ep.dl = grid / ep.gpl / p.B;
     const bool one_tile = p.DV == kRows;
     const bool deep = p.max_depth > 8;
-    auto go = [&](auto dk, auto mn, auto md) {
-        constexpr int DK = decltype(dk)::value, MN = decltype(mn)::value, MD = decltype(md)::value;
-        if (one_tile) launch(verify_effective_kernel<1, DK, MN, MD>, grid, kThreads, Lay<DK, MN, MD>::Bytes, st, map, em, ep);
-        else launch(verify_effective_kernel<2, DK, MN, MD>, grid, kThreads, Lay<DK, MN, MD>::Bytes, st, map, em, ep);
+    // Launched beside the plan kernel where that is a part of the whole that counts (384 units of 64 nodes 37.9 -> 35.8 us,
+    // 12288 units not measurable).
+    const bool few = share != 0 || n_units < 8 * sms;
+    auto go = [&](auto tp, auto dk, auto mn, auto md) {
+        constexpr int TP = decltype(tp)::value, DK = decltype(dk)::value, MN = decltype(mn)::value, MD = decltype(md)::value;
+        constexpr int bytes = Lay<DK, MN, MD>::Bytes;
+        if (few) launch(verify_effective_kernel<TP, DK, MN, MD, true>, grid, kThreads, bytes, st, map, em, ep);
+        else verify_effective_kernel<TP, DK, MN, MD, false><<<grid, kThreads, bytes, st>>>(map, em, ep);
     };
-    auto pick = [&](auto dk, auto mn) { deep ? go(dk, mn, Int<16>{}) : go(dk, mn, Int<8>{}); };
+    auto pick = [&](auto dk, auto mn) {
+        if (one_tile) deep ? go(Int<1>{}, dk, mn, Int<16>{}) : go(Int<1>{}, dk, mn, Int<8>{});
+        else deep ? go(Int<2>{}, dk, mn, Int<16>{}) : go(Int<2>{}, dk, mn, Int<8>{});
+    };
     // a smaller node budget leaves room for a deeper ring of state slices
     if (d_k == 256) pick(Int<256>{}, Int<32>{});
     else if (p.max_nodes <= 32) pick(Int<128>{}, Int<32>{});

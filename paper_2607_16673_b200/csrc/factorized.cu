@@ -346,7 +346,6 @@ template <int TP, bool FUSED, int DK = kDK, bool DEEP = false, bool COMP = false
 __global__ void __launch_bounds__(FUSED ? kThreadsFused : (COMP ? kThreadsComp : kThreads), 1)
 verify_factorized_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid_constant__ KQMaps kq, FParams fp)
 {
-    after_previous_kernel();
     // The swizzled operand regions need 1024-byte alignment.  The array is declared with that
     // alignment and used directly, so every access below stays a shared-memory access for the
     // compiler (address space known, no aliasing with the global output pointers).
@@ -1328,11 +1327,11 @@ void launch_one(bool one_tile, int d_k, int grid, cudaStream_t st, const CUtenso
 {
     constexpr int threads = FUSED ? kThreadsFused : (COMP ? kThreadsComp : kThreads);
     if (d_k == kDK) {
-        if (one_tile) launch(verify_factorized_kernel<1, FUSED, 128, DEEP, COMP>, grid, threads, kSmemBytes, st, map, kq, fp);
-        else launch(verify_factorized_kernel<2, FUSED, 128, DEEP, COMP>, grid, threads, kSmemBytes, st, map, kq, fp);
+        if (one_tile) verify_factorized_kernel<1, FUSED, 128, DEEP, COMP><<<grid, threads, kSmemBytes, st>>>(map, kq, fp);
+        else verify_factorized_kernel<2, FUSED, 128, DEEP, COMP><<<grid, threads, kSmemBytes, st>>>(map, kq, fp);
     } else {
-        if (one_tile) launch(verify_factorized_kernel<1, FUSED, 256, DEEP, COMP>, grid, threads, kSmemBytes, st, map, kq, fp);
-        else launch(verify_factorized_kernel<2, FUSED, 256, DEEP, COMP>, grid, threads, kSmemBytes, st, map, kq, fp);
+        if (one_tile) verify_factorized_kernel<1, FUSED, 256, DEEP, COMP><<<grid, threads, kSmemBytes, st>>>(map, kq, fp);
+        else verify_factorized_kernel<2, FUSED, 256, DEEP, COMP><<<grid, threads, kSmemBytes, st>>>(map, kq, fp);
     }
 }
 
