@@ -1038,11 +1038,10 @@ def run_sweep(args):
             return
         L = args.layers or 4
         S = synth.device_state(1, L, B, H, dk, dv, 0.02, dev)
-        roles = {0: {0: "TMA producer", 1: "MMA issuer, tile 0", 14: "MMA issuer, tile 1", 2: "preparation", 6: "epilogue group 0",
-                     10: "epilogue group 1", 15: "split"},
-                 3: {0: "TMA producer", 1: "MMA issuer", 2: "preparation", 6: "epilogue group 0", 10: "epilogue group 1"},
-                 4: {0: "TMA producer", 1: "first pass, tile 0", 18: "first pass, tile 1", 19: "correction, tile 0",
-                     20: "correction, tile 1", 2: "solver", 6: "vector", 10: "split", 14: "epilogue"}}
+        effective = {0: "state TMA", 1: "state product issuer", 2: "Gram and second product issuer", 3: "records TMA",
+                     4: "split group 0", 8: "split group 1", 12: "epilogue, even chunks", 16: "epilogue, odd chunks", 20: "solver"}
+        roles = {0: effective, 4: effective,
+                 3: {0: "TMA producer", 1: "MMA issuer", 2: "preparation", 6: "epilogue group 0", 10: "epilogue group 1"}}
         sm = torch.cuda.get_device_properties(dev).multi_processor_count
         for wl in ("chains8", "trees64", "cfg5"):
             hi = host_round_inputs(wl, B, 5000)

@@ -90,10 +90,11 @@ extern "C" {
 #define SPECA_ROUTE_TF32        3   /* the same factorisation with the state read once as TF32 (single pass)  */
 #define SPECA_ROUTE_EFFECTIVE   4   /* effective-query form of the factorisation, fp32-grade (trees up to 16 levels) */
 /* SPECA_ROUTE_FACTORIZED takes d_v in {128, 256}, max_depth <= 16 and max_nodes <= 64 (d_k = 128) or <= 32
- * (d_k = 256).  Both tensor-core operands are split into a TF32 head and its exact remainder, so outputs
- * carry fp32 accuracy whatever the magnitude of the state.  AUTO uses it whenever it applies and the serial
- * route otherwise, except that small trees (up to 64 nodes at d_k = 64, 16 or 32 at wider keys, any d_v) without u go
- * to a kernel of their own at the same accuracy; asking for it explicitly outside these shapes is SPECA_ERR_UNSUPPORTED.
+ * (d_k = 256).  Everything the tensor core multiplies is split into exact pieces, so outputs carry fp32 accuracy
+ * whatever the magnitude of the state.  AUTO uses it whenever it applies and the serial route otherwise; asking for
+ * it explicitly outside these shapes is SPECA_ERR_UNSUPPORTED.  Without u both run the effective-query kernel, and AUTO
+ * sends small trees (up to 64 nodes at d_k = 64, 16 or 32 at wider keys, any d_v) to a kernel of their own at the same
+ * accuracy; the substitution kernel serves the calls that ask for u.
  * SPECA_ROUTE_TF32 is never picked by AUTO: it reads the fp32 state through a single TF32 pass (10 mantissa
  * bits, truncated), which leaves errors of about 2^-11 of the output's scale, growing with the state; it takes
  * max_depth <= 8 with max_nodes <= 64 (d_k = 128) or <= 32 (d_k = 256), or max_depth <= 16 with max_nodes <=

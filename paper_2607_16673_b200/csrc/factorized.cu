@@ -1,5 +1,6 @@
 // Tree-masked factorised verification on the 5th-generation tensor cores (tcgen05 + TMEM),
-// the B200 form of the parallel route of Section 4.2.
+// the B200 form of the parallel route of Section 4.2.  It serves the single-pass TF32 route, the one-pass fused round and
+// calls that ask for u; without u the fp32-grade routes run effective.cu, 1.3 to 1.5 times as fast.
 //
 // Mathematics.  With gamma_t the product of alpha over the root path of node t, the rule
 // S_t = alpha_t S_p + u_t k_t^T unrolls to
