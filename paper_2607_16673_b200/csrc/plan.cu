@@ -527,6 +527,8 @@ chain_decompose_kernel(int32_t N, const int32_t *__restrict__ node_offsets, cons
 // 1 .. b -- ~count, or the final offset if that sequence was quicker -- and replaces its own entry by the offset.
 // Every entry is either of the two whenever it is read, so the sum does not depend on who comes first.  (One CTA that
 // packed the sequences in turn took 86 us for 128 of them, its serial selection 15; both runs together 21 us.)
+// What bounds it: a chain of shared-memory and L2 latencies per sequence.  The five drafting utilities of 128 trees of 24..64 nodes
+// take 102.7 us with two barriers per tree level, 96.9 with every node's path in registers and the scan's loads together.
 constexpr int kPruneLevels = 16;
 
 // Calls step(i, parent of i) for every node with a parent, parents first: level by level, all threads of the CTA, for
@@ -574,9 +576,16 @@ prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *__restrict__ n
 
     if (WRITE && warp == 0) {
         int run = 0;
+        int ahead[4];                                   // 128 entries in flight at a time
         for (int i0 = 1; i0 <= b; i0 += 32) {
-            const int i = i0 + lane;
-            const int v = i <= b ? *reinterpret_cast<volatile int32_t *>(out_offsets + i) : ~0;
+            const int k = ((i0 - 1) >> 5) & 3;
+            if (k == 0)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int i = i0 + 32 * j + lane;
+                    ahead[j] = i <= b ? *reinterpret_cast<volatile int32_t *>(out_offsets + i) : ~0;
+                }
+            const int v = k == 0 ? ahead[0] : k == 1 ? ahead[1] : k == 2 ? ahead[2] : ahead[3];
             const unsigned fin = __ballot_sync(0xffffffffu, v >= 0);
             const int last = 31 - __clz(int(fin));      // the last entry of these that is an offset already (-1: none)
             const int sum = __reduce_add_sync(0xffffffffu, lane > last ? ~v : 0);
@@ -604,8 +613,29 @@ prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *__restrict__ n
         if (WRITE && b == 0 && tid == 0) out_offsets[0] = 0;
         return;
     }
-    // scores: a node adds its parent's once that one is final
-    down_levels(n, par, done, [&](int i, int p) { q[i] = q[p] + q[i]; });
+    // Trees of up to 128 nodes and kPruneLevels levels: a thread per node keeps the path of its node in registers, so the
+    // two passes down the tree (scores, and below whether a node goes with an ancestor) are a handful of independent
+    // reads each instead of two barriers a level.
+    int up[kPruneLevels], len = 0, a = tid < n ? tid : -1;
+#pragma unroll
+    for (int r = 0; r < kPruneLevels; ++r) {
+        up[r] = a < 0 ? 0 : a;
+        len += a >= 0;
+        a = a < 0 ? a : par[a];
+    }
+    const bool flat = __syncthreads_and(a < 0) && n <= 128;
+    if (flat) {
+        float sum = 0.f, step[kPruneLevels];
+#pragma unroll
+        for (int r = 0; r < kPruneLevels; ++r) step[r] = q[up[r]];
+#pragma unroll
+        for (int r = kPruneLevels - 1; r >= 0; --r)
+            sum = r >= len ? 0.f : r == len - 1 ? step[r] : sum + step[r];
+        __syncthreads();
+        if (tid < n) q[tid] = sum;
+        __syncthreads();
+    } else
+        down_levels(n, par, done, [&](int i, int p) { q[i] = q[p] + q[i]; });      // a node adds its parent's once that is final
     float best = -INFINITY;
     for (int i = tid; i < n; i += 128) best = fmaxf(best, q[i]);
     for (int off = 16; off; off >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, off));
@@ -617,7 +647,7 @@ prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *__restrict__ n
     for (int i = tid; i < n; i += 128) {
         const float qi = q[i];
         int rank = 0;
-#pragma unroll 4
+#pragma unroll 8
         for (int j = 0; j < n; ++j) {
             const float qj = q[j];
             rank += (qj >= thr) && (qj > qi || (qj == qi && j < i));
@@ -627,7 +657,16 @@ prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *__restrict__ n
     }
     __syncthreads();
     // a node goes with its parent
-    down_levels(n, par, done, [&](int i, int p) { keep[i] &= keep[p]; });
+    if (flat) {
+        int on = 1;
+#pragma unroll
+        for (int r = 0; r < kPruneLevels; ++r)
+            on &= r < len ? keep[up[r]] : 1;
+        __syncthreads();
+        if (tid < n) keep[tid] = on;
+        __syncthreads();
+    } else
+        down_levels(n, par, done, [&](int i, int p) { keep[i] &= keep[p]; });
     // new indices: kept nodes before this one
     int count = 0;
     for (int i0 = 0; i0 < n; i0 += 128) {
@@ -665,15 +704,16 @@ int launch_mask_to_parent(int32_t B, int32_t N, const uint8_t *mask, const int32
                           int32_t *status, cudaStream_t st)
 {
     const size_t stage = size_t(N) * N <= kMaskStage ? size_t(N) * N : kMaskStage;
-    launch(mask_to_parent_kernel, B, 256, size_t(2 * N) * sizeof(int32_t) + 32 + stage, st, N, mask, node_offsets, parent, status);
+    launch(mask_to_parent_kernel, B, 256, size_t(2 * N) * sizeof(int32_t) + 32 + stage, st, N, mask, node_offsets,
+           parent, status);
     return int(cudaGetLastError());
 }
 
 int launch_chain_decompose(int32_t B, int32_t N, const int32_t *node_offsets, const int32_t *parent,
                            int32_t *chain_head, int32_t *n_chains, int32_t *status, cudaStream_t st)
 {
-    launch(chain_decompose_kernel, B, 256, size_t(2 * N) * sizeof(int32_t), st, N, node_offsets, parent, chain_head, n_chains,
-                                                                         status);
+    launch(chain_decompose_kernel, B, 256, size_t(2 * N) * sizeof(int32_t), st, N, node_offsets, parent, chain_head,
+           n_chains, status);
     return int(cudaGetLastError());
 }
 
@@ -682,12 +722,12 @@ int launch_prune(int32_t B, int32_t N, float tau, int32_t budget, const int32_t 
                  cudaStream_t st)
 {
     const size_t smem = size_t(5 * N) * sizeof(int32_t);
-    launch(prune_kernel<false>, B, 128, smem, st, N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent, out_index,
-                                              status);
+    launch(prune_kernel<false>, B, 128, smem, st, N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent,
+           out_index, status);
     const int e = int(cudaGetLastError());
     if (e != 0) return e;
-    launch(prune_kernel<true>, B, 128, smem, st, N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent, out_index,
-                                             status);
+    launch(prune_kernel<true>, B, 128, smem, st, N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent,
+           out_index, status);
     return int(cudaGetLastError());
 }
 
@@ -696,23 +736,22 @@ int launch_conv_commit(int32_t L, int32_t B, int32_t channels, int32_t W, int32_
                        int32_t *status, cudaStream_t st)
 {
     launch(conv_commit_kernel, L * B, 256, 0, st, B, channels, W, T, max_depth, static_cast<uint4 *>(C),
-                                              static_cast<const uint4 *>(x), node_offsets, path_idx, path_len, status);
+           static_cast<const uint4 *>(x), node_offsets, path_idx, path_len, status);
     return int(cudaGetLastError());
 }
 
 int launch_pending_check(const Params &p, int max_len, cudaStream_t st)
 {
-    launch(pending_check_kernel, (p.B + 127) / 128, 128, 0, st, p.B, p.Tp, p.max_depth, max_len, p.max_nodes, p.pnode_offsets,
-                                                            p.pparent, p.path_idx, p.path_len, p.ws.pend, p.status);
+    launch(pending_check_kernel, (p.B + 127) / 128, 128, 0, st, p.B, p.Tp, p.max_depth, max_len, p.max_nodes,
+           p.pnode_offsets, p.pparent, p.path_idx, p.path_len, p.ws.pend, p.status);
     return int(cudaGetLastError());
 }
 
 int launch_plan(const Params &p, cudaStream_t st)
 {
     const size_t smem = size_t(6 * p.max_nodes + 1) * sizeof(int32_t);
-    launch(plan_kernel, p.B, kPlanThreads, smem, st, p.node_offsets, p.parent, p.depth_in, p.B, p.T,
-                                                  p.max_depth, p.max_nodes, p.skip_nodes, p.plan_paths_only,
-                                                  p.n_slots, p.ws, p.status);
+    launch(plan_kernel, p.B, kPlanThreads, smem, st, p.node_offsets, p.parent, p.depth_in, p.B, p.T, p.max_depth,
+           p.max_nodes, p.skip_nodes, p.plan_paths_only, p.n_slots, p.ws, p.status);
     return int(cudaGetLastError());
 }
 
@@ -722,8 +761,8 @@ int launch_accept(int32_t B, int32_t max_depth, const int32_t *node_offsets, con
                   cudaStream_t st)
 {
     const int warps = 4;
-    launch(accept_kernel, (B + warps - 1) / warps, warps * 32, 0, st, B, max_depth, node_offsets, parent, draft_tok, target_tok, root_target_tok, path_idx, path_len,
-        next_tok, status);
+    launch(accept_kernel, (B + warps - 1) / warps, warps * 32, 0, st, B, max_depth, node_offsets, parent, draft_tok,
+           target_tok, root_target_tok, path_idx, path_len, next_tok, status);
     return int(cudaGetLastError());
 }
 
@@ -732,7 +771,8 @@ int launch_stochastic_accept(int32_t B, int32_t max_depth, const int32_t *node_o
                              int32_t *path_idx, int32_t *path_len, int32_t *status, cudaStream_t st)
 {
     const int warps = 4;
-    launch(stochastic_accept_kernel, (B + warps - 1) / warps, warps * 32, 0, st, B, max_depth, node_offsets, parent, p_target, p_draft, uniform, path_idx, path_len, status);
+    launch(stochastic_accept_kernel, (B + warps - 1) / warps, warps * 32, 0, st, B, max_depth, node_offsets, parent,
+           p_target, p_draft, uniform, path_idx, path_len, status);
     return int(cudaGetLastError());
 }
 

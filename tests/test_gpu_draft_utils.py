@@ -195,3 +195,24 @@ def test_larger_sequences_and_odd_mask_widths(n_max):
     pi, pl = oracle.stochastic_accept(offs, parent, pt, pd, u, 16)
     assert np.array_equal(pidx.cpu().numpy(), pi) and np.array_equal(plen.cpu().numpy(), pl)
     assert int(status.item()) == 0
+
+
+def test_pruning_at_the_edges_of_its_node_and_level_limits():
+    """Paths of 15 to 17 levels, sequences of 127 to 129 nodes, and more sequences than the offset scan takes in one step."""
+    rng = np.random.default_rng(91)
+    wide = lambda n: synth.random_tree_parent(n, 12, 4, rng)
+    parents = [synth.chain_parent(n) for n in (15, 16, 17)] + [wide(n) for n in (127, 128, 129)]
+    parents += [wide(int(n)) for n in rng.integers(1, 40, 134)]
+    offs = np.concatenate([[0], np.cumsum([len(p) for p in parents])]).astype(np.int32)
+    parent, T = np.concatenate(parents).astype(np.int32), int(offs[-1])
+    logp = np.log(rng.uniform(0.02, 1.0, T)).astype(np.float32)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, **i32)
+    for tau, budget in ((6.0, 20), (1e4, 129)):
+        oo, op, oi = torch.zeros(len(parents) + 1, **i32), torch.full((T,), -7, **i32), torch.full((T,), -7, **i32)
+        speca.prune_tree(129, tau, budget, t(offs), t(parent), t(logp), oo, op, oi, status)
+        ro, rp, ri = oracle.prune_tree(offs, parent, logp, tau, budget)
+        n = int(ro[-1])
+        assert np.array_equal(oo.cpu().numpy(), ro)
+        assert np.array_equal(op.cpu().numpy()[:n], rp) and np.array_equal(oi.cpu().numpy()[:n], ri)
+    assert int(status.item()) == 0
