@@ -149,7 +149,9 @@ int speca_verify_chain(const speca_dims *dims, const float *S0,
 /* Tree verification (Sections 4.2-4.3).  Node t sees the state obtained by applying
  * the rule along its own ancestor path root..t starting from S0; siblings never
  * influence each other and shared prefixes are computed once.  Same outputs as
- * speca_verify_chain; `depth_or_null` is optional. */
+ * speca_verify_chain; `depth_or_null` is optional.  Without u a key or value that is not
+ * finite reaches the nodes that have it on their path and no others (AUTO, SERIAL and
+ * EFFECTIVE; their outputs are Inf or NaN, which of the two differs between routes). */
 int speca_verify_tree(const speca_dims *dims, const float *S0,
                       const uint16_t *q, const uint16_t *k, const uint16_t *v,
                       const float *alpha, const float *beta,

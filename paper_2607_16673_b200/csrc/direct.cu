@@ -21,6 +21,12 @@
 // dropped one is 2^-22 of the result); M is split into three bf16 pieces and multiplies the bf16 value rows
 // exactly.
 //
+// The products run over all nodes of a block with zero weights off the path, and zero times a value that is not finite
+// is no zero.  So where an output is not finite the CTA looks for such records (repair), takes them out of the products and
+// goes over its rows once more: a node with the key on its path still gets it through its Gram entries, the value elements
+// are put back at the end for the nodes that have them on their path, and the rest of the draft stays clean.  (Looking
+// before the first pass took 2 to 12 % of a small unit.)
+//
 // A CTA takes one unit (layer, sequence, head) or a slice of its value rows and checks the topology of its sequence
 // itself (one parent walk per node), so no plan kernel runs in front of it.  It asks the first rows of its tile into L2
 // with one bulk prefetch, so that the set-up runs under the latency of HBM and the loop
@@ -73,6 +79,12 @@ __device__ __forceinline__ void ld_state(float (&x)[8], const float *p)
     asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7]) : "l"(p));
 }
+__device__ __forceinline__ bool finite(float x) { return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u; }
+// the two bf16 of a word with those that are not finite replaced by zero
+__device__ __forceinline__ uint32_t finite_pair(uint32_t w)
+{
+    return ((w & 0x7f80u) == 0x7f80u ? 0u : w & 0xffffu) | ((w & 0x7f800000u) == 0x7f800000u ? 0u : w & 0xffff0000u);
+}
 __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
 {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -121,9 +133,49 @@ struct DirectArgs {
     int32_t early;              // ask for the state before the records: see launch_one
 };
 
+// After a pass with an output that is not finite.  First pass: keys and value elements that are not finite are replaced by
+// zero in shared memory; true if there were any.  Second pass: the value elements are added for the nodes that have them on
+// their path.
+template <int DK, int NT, int MAXD, int THREADS>
+__device__ __forceinline__ bool repair(const DirectArgs &da, uint8_t *smem, int pass)
+{
+    using LY = Lay<DK, NT, MAXD>;
+    constexpr int N = LY::N;
+    const Params &p = da.p;
+    const int part = int(blockIdx.x % unsigned(da.parts)), unit = int(blockIdx.x / unsigned(da.parts)), rows = da.rows;
+    const int h = unit % p.H, lb = unit / p.H, b = lb % p.B, l = lb / p.B;
+    const int base = p.node_offsets[b], n = p.node_offsets[b + 1] - base;
+    const long rec0 = (long(l) * p.T + base) * p.H + h;
+    if (pass == 0) {
+        int odd = 0;
+        auto clean = [&](uint32_t *word) {
+            const uint32_t w = finite_pair(*word);
+            if (w != *word) { *word = w; odd = 1; }
+        };
+        for (int i = threadIdx.x; i < n * (DK / 2); i += THREADS)
+            clean(reinterpret_cast<uint32_t *>(smem + LY::OffKQ) + i / (DK / 2) * (LY::KQS / 2) + i % (DK / 2));
+        for (int i = threadIdx.x; i < n * (rows >> 1); i += THREADS)
+            clean(reinterpret_cast<uint32_t *>(smem + LY::OffV) + i / (rows >> 1) * ((rows + 8) >> 1) + i % (rows >> 1));
+        return __syncthreads_or(odd);
+    }
+    const int *par = reinterpret_cast<const int *>(smem + LY::OffP);
+    for (int i = threadIdx.x; i < n * rows; i += THREADS) {
+        const int t = i / rows, r = part * rows + i % rows;
+        float sum = 0.f;
+        for (int a = t; a >= 0; a = par[a]) {
+            const float v = __bfloat162float(p.v[(rec0 + long(a) * p.H) * p.DV + r]);
+            const __nv_bfloat16 *m = reinterpret_cast<const __nv_bfloat16 *>(smem + LY::OffM) + t * LY::MS + a;
+            if (!finite(v))
+                sum += v * (__bfloat162float(m[0]) + __bfloat162float(m[N * LY::MS]) + __bfloat162float(m[2 * N * LY::MS]));
+        }
+        if (sum != 0.f) p.o[(rec0 + long(t) * p.H) * p.DV + r] += sum;
+    }
+    return false;
+}
+
 template <int DK, int NT, int MAXD, int WARPS, int CTAS>
 __global__ void __launch_bounds__(WARPS * 32, CTAS)
-verify_direct_kernel(DirectArgs da)
+verify_direct_kernel(const __grid_constant__ DirectArgs da)
 {
     after_previous_kernel();
     using LY = Lay<DK, NT, MAXD>;
@@ -313,140 +365,150 @@ verify_direct_kernel(DirectArgs da)
     }
     __syncthreads();
 
-    // the first two steps of this warp's first tile, requested a phase ahead of their use
-    const float *Su = S_cta + g * DK + 8 * t4;
-    float sa[2][8], sb[2][8];
-    if (warp / PARTS < tiles)
+    for (int pass = 0;; ++pass) {                            // (the second one only after a repair)
+        // the first two steps of this warp's first tile, requested a phase ahead of their use
+        const float *Su = S_cta + g * DK + 8 * t4;
+        float sa[2][8], sb[2][8];
+        if (warp / PARTS < tiles)
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            ld_state(sa[q], Su + warp / PARTS * 16 * DK + 32 * q);
-            ld_state(sb[q], Su + (warp / PARTS * 16 + 8) * DK + 32 * q);
-        }
+            for (int q = 0; q < 2; ++q) {
+                ld_state(sa[q], Su + warp / PARTS * 16 * DK + 32 * q);
+                ld_state(sb[q], Su + (warp / PARTS * 16 + 8) * DK + 32 * q);
+            }
 
-    // ---- effective queries (scale gamma q + W K, the weights in three bf16 pieces), split into head and remainder
-    {
-        const int nm = (n + 15) >> 4;
-        for (int job = warp; job < nm * (DK / 16); job += WARPS) {
-            const int mi = job / (DK / 16), c0 = (job % (DK / 16)) * 16;
-            const int r0 = 16 * mi + g, r1 = r0 + 8;
-            const float g0 = sGam[r0], g1 = sGam[r1];
-            float acc[2][4];
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                // rows past the staged ones weigh nothing; clamp keeps the read inside the buffer
-                const uint32_t q0 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r0, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
-                const uint32_t q1 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r1, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
-                acc[c][0] = g0 * __uint_as_float(q0 << 16); acc[c][1] = g0 * __uint_as_float(q0 & 0xffff0000u);
-                acc[c][2] = r1 < 8 * nt ? g1 * __uint_as_float(q1 << 16) : 0.f;
-                acc[c][3] = r1 < 8 * nt ? g1 * __uint_as_float(q1 & 0xffff0000u) : 0.f;
-            }
-            for (int kk = 0; kk <= mi; ++kk) {               // a node's path holds no later node
-                uint32_t kb[4];                              // key rows 16 kk .. + 15, columns c0 .. + 15
-                const int kr = 16 * kk + (lane & 15);
-                ldsm_x4_t(kb, sKQ + min(kr, 8 * nt - 1) * LY::KQS + c0 + ((lane >> 4) << 3));
-#pragma unroll
-                for (int pc = 0; pc < 3; ++pc) {
-                    uint32_t a[4];
-                    ldsm_x4(a, sW + pc * LY::WP + LY::w_row(16 * mi + (lane & 15)) + 16 * kk + ((lane >> 4) << 3));
-                    mma_bf16_sync(acc[0], a, kb[0], kb[1]);
-                    mma_bf16_sync(acc[1], a, kb[2], kb[3]);
-                }
-            }
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int r = half ? r1 : r0;
-                if (r >= 8 * nt) break;
+        // ---- effective queries (scale gamma q + W K, the weights in three bf16 pieces), split into head and remainder
+        {
+            const int nm = (n + 15) >> 4;
+            for (int job = warp; job < nm * (DK / 16); job += WARPS) {
+                const int mi = job / (DK / 16), c0 = (job % (DK / 16)) * 16;
+                const int r0 = 16 * mi + g, r1 = r0 + 8;
+                const float g0 = sGam[r0], g1 = sGam[r1];
+                float acc[2][4];
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                    const float x0 = acc[c][2 * half], x1 = acc[c][2 * half + 1];
-                    const float y0 = tc::round_tf32(x0), y1 = tc::round_tf32(x1);
-                    *reinterpret_cast<float2 *>(sHi + r * LY::BS + c0 + 8 * c + 2 * t4) = make_float2(y0, y1);
-                    *reinterpret_cast<float2 *>(sLo + r * LY::BS + c0 + 8 * c + 2 * t4) = make_float2(x0 - y0, x1 - y1);
+                    // rows past the staged ones weigh nothing; clamp keeps the read inside the buffer
+                    const uint32_t q0 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r0, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
+                    const uint32_t q1 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r1, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
+                    acc[c][0] = g0 * __uint_as_float(q0 << 16); acc[c][1] = g0 * __uint_as_float(q0 & 0xffff0000u);
+                    acc[c][2] = r1 < 8 * nt ? g1 * __uint_as_float(q1 << 16) : 0.f;
+                    acc[c][3] = r1 < 8 * nt ? g1 * __uint_as_float(q1 & 0xffff0000u) : 0.f;
                 }
-            }
-        }
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");     // value rows
-    __syncthreads();
-
-    // ---- the state: one 16-row tile at a time, two 32-column steps of registers in flight
-    // lane (g, t) holds columns 32 q + 8 t .. + 7 of rows g and g + 8: k-steps e = 0..3 of the step contract
-    // columns 8 t + 2 e and 8 t + 2 e + 1 of the four lanes
-    const int half = PARTS == 1 ? 0 : warp % PARTS, i0 = half * NTP;         // this warp's column tiles: i0 ..
-    const float *hi_p = sHi + (8 * i0 + g) * LY::BS + 8 * t4, *lo_p = sLo + (8 * i0 + g) * LY::BS + 8 * t4;
-    const int nk = (n + 15) >> 4, ntp = nt - i0;
-    if (PARTS > 1 && ntp <= 0) return;
-    float *o0 = p.o + rec0 * p.DV + row0 + g;
-    const long node_stride = long(H) * p.DV;
-#pragma unroll 1
-    for (int tile = warp / PARTS; tile < tiles; tile += STRIDE) {
-        if (lane == 0 && half == 0 && tile + AHEAD < tiles) prefetch_l2(S_cta + long(tile + AHEAD) * 16 * DK, 16 * DK * 4);
-        const bool next = tile + STRIDE < tiles;
-        float hh[NTP][4], xx[NTP][4];                         // head x head, and the two cross products
-#pragma unroll
-        for (int i = 0; i < NTP; ++i)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { hh[i][e] = 0.f; xx[i][e] = 0.f; }
-        const float *cur = Su + long(tile) * 16 * DK, *nxt = cur + STRIDE * 16 * DK - NS * 32;
-#pragma unroll
-        for (int q = 0; q < NS; ++q) {
-            uint32_t ah[4][4], al[4][4];                     // [k-step][fragment register]
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float x[4] = {sa[q & 1][2 * e], sb[q & 1][2 * e], sa[q & 1][2 * e + 1], sb[q & 1][2 * e + 1]};
-#pragma unroll
-                for (int c = 0; c < 4; ++c) { ah[e][c] = tf32_head(x[c]); al[e][c] = tf32_tail(x[c]); }
-            }
-            if (q + 2 < NS || next) {
-                const float *src = (q + 2 < NS ? cur : nxt) + 32 * (q + 2);
-                ld_state(sa[q & 1], src);
-                ld_state(sb[q & 1], src + 8 * DK);
-            }
-#pragma unroll
-            for (int i = 0; i < NTP; ++i) {
-                if (NTP > 1 && i >= ntp) break;
-#pragma unroll
-                for (int e2 = 0; e2 < 2; ++e2) {
-                    const float4 bh = *reinterpret_cast<const float4 *>(hi_p + 8 * i * LY::BS + 32 * q + 4 * e2);
-                    const float4 bl = *reinterpret_cast<const float4 *>(lo_p + 8 * i * LY::BS + 32 * q + 4 * e2);
-                    mma_tf32_sync(hh[i], ah[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
-                    mma_tf32_sync(xx[i], ah[2 * e2], __float_as_uint(bl.x), __float_as_uint(bl.y));
-                    mma_tf32_sync(hh[i], ah[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
-                    mma_tf32_sync(xx[i], al[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
-                    mma_tf32_sync(xx[i], ah[2 * e2 + 1], __float_as_uint(bl.z), __float_as_uint(bl.w));
-                    mma_tf32_sync(xx[i], al[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
-                }
-            }
-        }
-        // value term: rows of V^T (16 value rows x 16 nodes) x M, piece by piece
-        {
-            const __nv_bfloat16 *va = sV + ((lane & 7) + ((lane >> 4) << 3)) * vstride + tile * 16 + (lane & 8);
-#pragma unroll
-            for (int kk = 0; kk < LY::NK / 16; ++kk) {
-                if (LY::NK > 16 && kk >= nk) break;
-                uint32_t a[4];
-                ldsm_x4_t(a, va + kk * 16 * vstride);
-#pragma unroll
-                for (int i = 0; i < NTP; ++i) {
-                    if (NTP > 1 && i >= ntp) break;
-                    if (8 * (i0 + i) + 7 < 16 * kk) continue;       // a node's path holds no later node
+                for (int kk = 0; kk <= mi; ++kk) {               // a node's path holds no later node
+                    uint32_t kb[4];                              // key rows 16 kk .. + 15, columns c0 .. + 15
+                    const int kr = 16 * kk + (lane & 15);
+                    ldsm_x4_t(kb, sKQ + min(kr, 8 * nt - 1) * LY::KQS + c0 + ((lane >> 4) << 3));
 #pragma unroll
                     for (int pc = 0; pc < 3; ++pc) {
-                        const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
-                        mma_bf16_sync(xx[i], a, *reinterpret_cast<const uint32_t *>(mb), *reinterpret_cast<const uint32_t *>(mb + 8));
+                        uint32_t a[4];
+                        ldsm_x4(a, sW + pc * LY::WP + LY::w_row(16 * mi + (lane & 15)) + 16 * kk + ((lane >> 4) << 3));
+                        mma_bf16_sync(acc[0], a, kb[0], kb[1]);
+                        mma_bf16_sync(acc[1], a, kb[2], kb[3]);
+                    }
+                }
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    const int r = half ? r1 : r0;
+                    if (r >= 8 * nt) break;
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const float x0 = acc[c][2 * half], x1 = acc[c][2 * half + 1];
+                        const float y0 = tc::round_tf32(x0), y1 = tc::round_tf32(x1);
+                        *reinterpret_cast<float2 *>(sHi + r * LY::BS + c0 + 8 * c + 2 * t4) = make_float2(y0, y1);
+                        *reinterpret_cast<float2 *>(sLo + r * LY::BS + c0 + 8 * c + 2 * t4) = make_float2(x0 - y0, x1 - y1);
                     }
                 }
             }
         }
-        float *ot = o0 + tile * 16;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");     // value rows
+        __syncthreads();
+
+        // ---- the state: one 16-row tile at a time, two 32-column steps of registers in flight
+        // lane (g, t) holds columns 32 q + 8 t .. + 7 of rows g and g + 8: k-steps e = 0..3 of the step contract
+        // columns 8 t + 2 e and 8 t + 2 e + 1 of the four lanes
+        const int half = PARTS == 1 ? 0 : warp % PARTS, i0 = half * NTP;         // this warp's column tiles: i0 ..
+        const float *hi_p = sHi + (8 * i0 + g) * LY::BS + 8 * t4, *lo_p = sLo + (8 * i0 + g) * LY::BS + 8 * t4;
+        const int nk = (n + 15) >> 4, ntp = nt - i0;
+        const int tile_end = PARTS > 1 && ntp <= 0 ? 0 : tiles;
+        float *o0 = p.o + rec0 * p.DV + row0 + g;
+        const long node_stride = long(H) * p.DV;
+        float zero = 0.f;                                        // the sum of the outputs times zero
+#pragma unroll 1
+        for (int tile = warp / PARTS; tile < tile_end; tile += STRIDE) {
+            if (lane == 0 && half == 0 && tile + AHEAD < tiles) prefetch_l2(S_cta + long(tile + AHEAD) * 16 * DK, 16 * DK * 4);
+            const bool next = tile + STRIDE < tiles;
+            float hh[NTP][4], xx[NTP][4];                         // head x head, and the two cross products
 #pragma unroll
-        for (int i = 0; i < NTP; ++i) {
-            if (NTP > 1 && i >= ntp) break;
-            const int n0 = 8 * (i0 + i) + 2 * t4;
-            float *od = ot + n0 * node_stride;
-            if (n0 < n) { od[0] = hh[i][0] + xx[i][0]; od[8] = hh[i][2] + xx[i][2]; }
-            if (n0 + 1 < n) { od[node_stride] = hh[i][1] + xx[i][1]; od[node_stride + 8] = hh[i][3] + xx[i][3]; }
+            for (int i = 0; i < NTP; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { hh[i][e] = 0.f; xx[i][e] = 0.f; }
+            const float *cur = Su + long(tile) * 16 * DK, *nxt = cur + STRIDE * 16 * DK - NS * 32;
+#pragma unroll
+            for (int q = 0; q < NS; ++q) {
+                uint32_t ah[4][4], al[4][4];                     // [k-step][fragment register]
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float x[4] = {sa[q & 1][2 * e], sb[q & 1][2 * e], sa[q & 1][2 * e + 1], sb[q & 1][2 * e + 1]};
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) { ah[e][c] = tf32_head(x[c]); al[e][c] = tf32_tail(x[c]); }
+                }
+                if (q + 2 < NS || next) {
+                    const float *src = (q + 2 < NS ? cur : nxt) + 32 * (q + 2);
+                    ld_state(sa[q & 1], src);
+                    ld_state(sb[q & 1], src + 8 * DK);
+                }
+#pragma unroll
+                for (int i = 0; i < NTP; ++i) {
+                    if (NTP > 1 && i >= ntp) break;
+#pragma unroll
+                    for (int e2 = 0; e2 < 2; ++e2) {
+                        const float4 bh = *reinterpret_cast<const float4 *>(hi_p + 8 * i * LY::BS + 32 * q + 4 * e2);
+                        const float4 bl = *reinterpret_cast<const float4 *>(lo_p + 8 * i * LY::BS + 32 * q + 4 * e2);
+                        mma_tf32_sync(hh[i], ah[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
+                        mma_tf32_sync(xx[i], ah[2 * e2], __float_as_uint(bl.x), __float_as_uint(bl.y));
+                        mma_tf32_sync(hh[i], ah[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
+                        mma_tf32_sync(xx[i], al[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
+                        mma_tf32_sync(xx[i], ah[2 * e2 + 1], __float_as_uint(bl.z), __float_as_uint(bl.w));
+                        mma_tf32_sync(xx[i], al[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
+                    }
+                }
+            }
+            // value term: rows of V^T (16 value rows x 16 nodes) x M, piece by piece
+            {
+                const __nv_bfloat16 *va = sV + ((lane & 7) + ((lane >> 4) << 3)) * vstride + tile * 16 + (lane & 8);
+#pragma unroll
+                for (int kk = 0; kk < LY::NK / 16; ++kk) {
+                    if (LY::NK > 16 && kk >= nk) break;
+                    uint32_t a[4];
+                    ldsm_x4_t(a, va + kk * 16 * vstride);
+#pragma unroll
+                    for (int i = 0; i < NTP; ++i) {
+                        if (NTP > 1 && i >= ntp) break;
+                        if (8 * (i0 + i) + 7 < 16 * kk) continue;       // a node's path holds no later node
+#pragma unroll
+                        for (int pc = 0; pc < 3; ++pc) {
+                            const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
+                            mma_bf16_sync(xx[i], a, *reinterpret_cast<const uint32_t *>(mb), *reinterpret_cast<const uint32_t *>(mb + 8));
+                        }
+                    }
+                }
+            }
+            float *ot = o0 + tile * 16;
+#pragma unroll
+            for (int i = 0; i < NTP; ++i) {
+                if (NTP > 1 && i >= ntp) break;
+                const int n0 = 8 * (i0 + i) + 2 * t4;
+                float *od = ot + n0 * node_stride;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    hh[i][e] += xx[i][e];
+                    zero = fmaf(hh[i][e], 0.f, zero);
+                }
+                if (n0 < n) { od[0] = hh[i][0]; od[8] = hh[i][2]; }
+                if (n0 + 1 < n) { od[node_stride] = hh[i][1]; od[node_stride + 8] = hh[i][3]; }
+            }
         }
+        const bool odd = __syncthreads_or(!(zero == 0.f));
+        if (!(odd || pass > 0) || !repair<DK, NT, MAXD, THREADS>(da, smem, pass)) break;
     }
 }
 

@@ -41,6 +41,9 @@
 // a unit, which come round twice as often.
 // Ten roles take turns on four issue slots, so the kernel's size matters as much as its instruction count: loops stay
 // rolled where a role has slack.
+// x M^T runs over all nodes with zeros in M off the path, and zero times a value that is not finite is no zero: where an
+// epilogue warp meets such an x it leaves it out of the product and makes G of the nodes that have it on their path not
+// finite instead.
 // With u requested a unit is walked twice (o rows, then u rows); the second walk finds the state tile in L2.
 // Every wait is bounded; on expiry the CTA raises SPECA_STATUS_TIMEOUT, drains and exits.
 #include <cuda.h>
@@ -213,6 +216,17 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&x)[4])
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3])
                  : "memory");
+}
+__device__ __forceinline__ float tmem_ld1(uint32_t taddr)
+{
+    uint32_t x;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(x) : "r"(taddr) : "memory");
+    tmem_ld_wait();
+    return __uint_as_float(x);
+}
+__device__ __forceinline__ void tmem_st1(uint32_t taddr, float x)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(__float_as_uint(x)) : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // kind::f16 (bf16) with the A operand in TMEM: a 32-bit column holds two consecutive K elements, the even one low
@@ -581,8 +595,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 PROF_T0()
                 const uint32_t acc = tmem_base + slot * kTileCols + lane_addr;
                 const unsigned short *vt = reinterpret_cast<const unsigned short *>(smem + LY::OffV + slot * LY::VBUF) + row;
-#pragma unroll 1
-                for (int c0 = 8 * grp; c0 < x.npad; c0 += 16) {
+                // x of 8 nodes (clean: those that are not finite as zero), its sum times zero, the set of those not finite
+                auto make_x = [&](int c0, bool clean, float2 &zero, uint32_t &odd) {
                     float r[8];
                     tmem_ld8(acc + c0, r);
                     uint32_t vv[8];
@@ -596,13 +610,41 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
 #pragma unroll
                     for (int i = 0; i < 8; i += 2) {
                         // rows past the last node belong to another sequence: they must not reach the product
-                        const float x0 = c0 + i < x.n ? fmaf(-gm[i], r[i], __uint_as_float(vv[i] << 16)) : 0.f;
-                        const float x1 = c0 + i + 1 < x.n ? fmaf(-gm[i + 1], r[i + 1], __uint_as_float(vv[i + 1] << 16)) : 0.f;
+                        float x0 = c0 + i < x.n ? fmaf(-gm[i], r[i], __uint_as_float(vv[i] << 16)) : 0.f;
+                        float x1 = c0 + i + 1 < x.n ? fmaf(-gm[i + 1], r[i + 1], __uint_as_float(vv[i + 1] << 16)) : 0.f;
+                        zero = __ffma2_rn(make_float2(x0, x1), make_float2(0.f, 0.f), zero);
+                        if (clean) {
+                            if (!(fabsf(x0) < INFINITY)) { odd |= 1u << i; x0 = 0.f; }
+                            if (!(fabsf(x1) < INFINITY)) { odd |= 2u << i; x1 = 0.f; }
+                        }
                         split_pair(x0, x1, p1[i >> 1], p2[i >> 1], p3[i >> 1]);
                     }
+                    if (clean && ((c0 >> 3) & 1) != grp) return;         // the other warp's chunk
                     tmem_st4(xb + (c0 >> 1), p1);
                     tmem_st4(xb + 32 + (c0 >> 1), p2);
                     tmem_st4(xb + 64 + (c0 >> 1), p3);
+                };
+                float2 zero = make_float2(0.f, 0.f);
+                uint32_t none = 0u;
+#pragma unroll 1
+                for (int c0 = 8 * grp; c0 < x.npad; c0 += 16) make_x(c0, false, zero, none);
+                if (__any_sync(0xffffffffu, !(zero.x + zero.y == 0.f))) {
+                    // Both warps of the lane quarter may come here: each looks at all nodes, so that both write the same G.
+                    // (R stays until all epilogue warps have arrived below.)
+                    uint32_t odd_lo = 0u, odd_hi = 0u;
+#pragma unroll 1
+                    for (int c0 = 0; c0 < x.npad; c0 += 8) {
+                        uint32_t odd = 0u;
+                        make_x(c0, true, zero, odd);
+                        if (c0 < 32) odd_lo |= odd << c0;
+                        else odd_hi |= odd << (c0 - 32);
+                    }
+#pragma unroll 1
+                    for (int i = 0; i < x.n; ++i) {
+                        const int2 set = reinterpret_cast<const int2 *>(p.ws.set)[x.base + i];
+                        const float g = tmem_ld1(acc + x.npad + i);
+                        tmem_st1(acc + x.npad + i, ((uint32_t(set.x) & odd_lo) | (uint32_t(set.y) & odd_hi)) != 0u ? NAN : g);
+                    }
                 }
                 tmem_st_wait();
                 tc_fence_before();
