@@ -17,9 +17,17 @@
 // state; while one CTA builds its coefficients the other resident CTAs stream.  The pipelined tcgen05 kernel
 // spends most of a small unit on hand-overs between its roles instead.
 //
-// fp32 accuracy: both operands are split into a TF32 head and the exact remainder (three products; the
-// dropped one is 2^-22 of the result); M is split into three bf16 pieces and multiplies the bf16 value rows
-// exactly.
+// fp32 accuracy: both operands are split into a TF32 head and the remainder (three products; the dropped one is 2^-22 of
+// the result); M and the weights of the keys are split into three bf16 pieces and multiply bf16 rows exactly.  The tensor
+// core truncates where it adds, relative to the largest term, accumulator included; a long chain of products in one
+// accumulator loses a bit or two toward zero.  So the large sums (Gram entries, leading pieces, 32-column steps of the
+// state product) start from zero and are added up in fp32 proper.  Error against 64 bits, 2-norm of the difference over
+// that of the outputs, x 10^-8, chained / now / the route that takes the shape without this kernel: d_k = d_v = 64 (serial
+// walk): chains of 8 15.0 / 7.2 / 7.2, of 16 15.0 / 7.9 / 7.1, trees of 30 15.0 / 6.9 / 7.2; 128 x 64 (serial walk): chains
+// of 8 17.7 / 7.7 / 7.6, trees of 30 17.6 / 7.4 / 7.7; 128 x 256 (substitution kernel): chains of 8 17.6 / 7.7 / 15.4, trees
+// of 30 17.6 / 7.3 / 14.1; 256 x 256, chains of 8 24.2 / 8.7 / 30.3.  (Of the part that comes from the state alone 14, the
+// serial walk 7.6, the substitution kernel 90.)  It costs 2 to 6 % of a unit: 24576 units of 8 / 30 nodes at 64 x 64 142 /
+// 326 us chained, 148 / 336 now, 12288 units of 16 nodes at 128 x 256 388 and 394.
 //
 // The products run over all nodes of a block with zero weights off the path, and zero times a value that is not finite
 // is no zero.  So where an output is not finite the CTA looks for such records (repair), takes them out of the products and
@@ -46,7 +54,8 @@ namespace speca {
 
 namespace {
 
-__device__ __forceinline__ uint32_t tf32_head(float x) { return __float_as_uint(x) & 0xffffe000u; }
+// (rounded: the remainder then fits TF32 but for its last bit; a value that is not finite stays one)
+__device__ __forceinline__ uint32_t tf32_head(float x) { return (__float_as_uint(x) + 0x1000u) & 0xffffe000u; }
 __device__ __forceinline__ uint32_t tf32_tail(float x) { return __float_as_uint(x - __uint_as_float(tf32_head(x))); }
 
 // (not volatile: the compiler may interleave independent products)
@@ -62,6 +71,14 @@ __device__ __forceinline__ void mma_bf16_sync(float (&d)[4], const uint32_t (&a)
                  "{%0, %1, %2, %3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// the product alone (C = 0)
+__device__ __forceinline__ void mma_bf16_first(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%10, %10, %10, %10};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void *p)
 {
@@ -304,8 +321,11 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
             ldsm_x4(bq, pb + 32 * k);
             ldsm_x4(a0, pa + 32 * k);
             ldsm_x4(a1, pa + 32 * k + 16);
-            mma_bf16_sync(acc, a0, bq[0], bq[1]);
-            mma_bf16_sync(acc1, a1, bq[2], bq[3]);
+            float part0[4], part1[4];
+            mma_bf16_first(part0, a0, bq[0], bq[1]);
+            mma_bf16_first(part1, a1, bq[2], bq[3]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { acc[e] += part0[e]; acc1[e] += part1[e]; }
         }
         float *gk = sG + (8 * mi + g) * LY::GS + 8 * ni + 2 * t4, *gq = gk + N * LY::GS;
         gk[0] = acc[0] + acc1[0]; gk[1] = acc[1] + acc1[1];
@@ -397,13 +417,22 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                     uint32_t kb[4];                              // key rows 16 kk .. + 15, columns c0 .. + 15
                     const int kr = 16 * kk + (lane & 15);
                     ldsm_x4_t(kb, sKQ + min(kr, 8 * nt - 1) * LY::KQS + c0 + ((lane >> 4) << 3));
+                    float lo[2][4], hi[2][4];
 #pragma unroll
-                    for (int pc = 0; pc < 3; ++pc) {
+                    for (int pc = 2; pc >= 0; --pc) {
                         uint32_t a[4];
                         ldsm_x4(a, sW + pc * LY::WP + LY::w_row(16 * mi + (lane & 15)) + 16 * kk + ((lane >> 4) << 3));
-                        mma_bf16_sync(acc[0], a, kb[0], kb[1]);
-                        mma_bf16_sync(acc[1], a, kb[2], kb[3]);
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            if (pc == 2) mma_bf16_first(lo[c], a, kb[2 * c], kb[2 * c + 1]);
+                            else if (pc == 1) mma_bf16_sync(lo[c], a, kb[2 * c], kb[2 * c + 1]);
+                            else mma_bf16_first(hi[c], a, kb[2 * c], kb[2 * c + 1]);
+                        }
                     }
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) acc[c][e] += hi[c][e] + lo[c][e];
                 }
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
@@ -459,17 +488,20 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
 #pragma unroll
                 for (int i = 0; i < NTP; ++i) {
                     if (NTP > 1 && i >= ntp) break;
+                    float part[4] = {0.f, 0.f, 0.f, 0.f};    // of this step
 #pragma unroll
                     for (int e2 = 0; e2 < 2; ++e2) {
                         const float4 bh = *reinterpret_cast<const float4 *>(hi_p + 8 * i * LY::BS + 32 * q + 4 * e2);
                         const float4 bl = *reinterpret_cast<const float4 *>(lo_p + 8 * i * LY::BS + 32 * q + 4 * e2);
-                        mma_tf32_sync(hh[i], ah[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
+                        mma_tf32_sync(part, ah[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
                         mma_tf32_sync(xx[i], ah[2 * e2], __float_as_uint(bl.x), __float_as_uint(bl.y));
-                        mma_tf32_sync(hh[i], ah[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
+                        mma_tf32_sync(part, ah[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
                         mma_tf32_sync(xx[i], al[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
                         mma_tf32_sync(xx[i], ah[2 * e2 + 1], __float_as_uint(bl.z), __float_as_uint(bl.w));
                         mma_tf32_sync(xx[i], al[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
                     }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) hh[i][e] += part[e];
                 }
             }
             // value term: rows of V^T (16 value rows x 16 nodes) x M, piece by piece
@@ -484,11 +516,17 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                     for (int i = 0; i < NTP; ++i) {
                         if (NTP > 1 && i >= ntp) break;
                         if (8 * (i0 + i) + 7 < 16 * kk) continue;       // a node's path holds no later node
+                        float lo[4], hi[4];
 #pragma unroll
-                        for (int pc = 0; pc < 3; ++pc) {
+                        for (int pc = 2; pc >= 0; --pc) {
                             const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
-                            mma_bf16_sync(xx[i], a, *reinterpret_cast<const uint32_t *>(mb), *reinterpret_cast<const uint32_t *>(mb + 8));
+                            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(mb), b1 = *reinterpret_cast<const uint32_t *>(mb + 8);
+                            if (pc == 2) mma_bf16_first(lo, a, b0, b1);
+                            else if (pc == 1) mma_bf16_sync(lo, a, b0, b1);
+                            else mma_bf16_first(hi, a, b0, b1);
                         }
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) { hh[i][e] += hi[e]; xx[i][e] += lo[e]; }
                     }
                 }
             }

@@ -5,8 +5,9 @@
 // costs about a microsecond on top of its kernel launches.
 //
 // Every function returns the C entry point's code, or None if an argument is not plainly what the entry point wants (a
-// wrong dtype, shape, device or layout, or a number that is no Python int): the binding then runs its own checks, which
-// name the argument, or converts it.  Nothing is kept between calls but the addresses of the entry points.
+// wrong dtype, shape, device or layout, or a number that is no integer): the binding then runs its own checks, which
+// name the argument, or converts it.  So does whatever torch throws on the way (a tensor without strides or without
+// storage, no device to take a stream of): see guarded().  Nothing is kept between calls but the addresses of the entry points.
 #include <Python.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <c10/cuda/CUDAStream.h>
@@ -47,9 +48,12 @@ struct Reader {
 
     int integer(PyObject *o)
     {
-        if (!ok || o == nullptr || !PyLong_Check(o)) { ok = false; return 0; }
-        const long v = PyLong_AsLong(o);
-        if ((v == -1 && PyErr_Occurred()) || v != long(int(v))) { PyErr_Clear(); ok = false; }
+        if (!ok || o == nullptr) { ok = false; return 0; }
+        // (numpy's integers among them; a tensor's value would have to be fetched, which int() does in the binding)
+        PyObject *i = PyLong_Check(o) ? Py_NewRef(o) : PyIndex_Check(o) && !THPVariable_Check(o) ? PyNumber_Index(o) : nullptr;
+        const long v = i != nullptr ? PyLong_AsLong(i) : -1;
+        Py_XDECREF(i);
+        if (i == nullptr || (v == -1 && PyErr_Occurred()) || v != long(int(v))) { PyErr_Clear(); ok = false; }
         return int(v);
     }
     int attr(PyObject *o, Name n)
@@ -90,6 +94,13 @@ struct Reader {
     float *f32(PyObject *o, std::initializer_list<int64_t> s) { return static_cast<float *>(ptr(o, ScalarType::Float, s)); }
     int32_t *i32(PyObject *o, std::initializer_list<int64_t> s) { return static_cast<int32_t *>(ptr(o, ScalarType::Int, s)); }
     uint16_t *bf16(PyObject *o, std::initializer_list<int64_t> s) { return static_cast<uint16_t *>(ptr(o, ScalarType::BFloat16, s)); }
+    // bytes of any shape
+    struct Bytes { void *ptr; size_t size; };
+    Bytes bytes(PyObject *o)
+    {
+        const at::Tensor *t = tensor(o, ScalarType::Byte);
+        return t != nullptr ? Bytes{t->data_ptr(), size_t(t->numel())} : Bytes{nullptr, 0};
+    }
     // a tensor whose shape the others are checked against
     const at::Tensor *any(PyObject *o, ScalarType type, int64_t ndim)
     {
@@ -99,10 +110,11 @@ struct Reader {
     }
 };
 
+// `f` runs without the interpreter lock and must not throw: addresses are taken before.
 template <class F> PyObject *call(const Reader &r, F f)
 {
     if (!r.ok) Py_RETURN_NONE;
-    int rc;
+    int rc = 0;
     void *st = c10::cuda::getCurrentCUDAStream().stream();
     Py_BEGIN_ALLOW_THREADS
     rc = f(st);
@@ -150,10 +162,10 @@ PyObject *verify_chain(PyObject *, PyObject *const *a, Py_ssize_t n)
     const speca_dims d = r.dims(a[0]);
     const Draft x(r, d, a[1], a + 2);
     float *o = r.f32(a[9], {d.n_layers, x.T, d.heads, d.d_v}), *u = r.f32(a[10], {d.n_layers, x.T, d.heads, d.d_v});
-    const at::Tensor *ws = r.tensor(a[11], ScalarType::Byte);
+    const Reader::Bytes ws = r.bytes(a[11]);
     int32_t *status = r.i32(a[12], {1});
     return call(r, [&](void *st) {
-        return g_api.verify_chain(&d, x.S, x.q, x.k, x.v, x.alpha, x.beta, x.offs, x.T, o, u, ws->data_ptr(), size_t(ws->numel()), status, st);
+        return g_api.verify_chain(&d, x.S, x.q, x.k, x.v, x.alpha, x.beta, x.offs, x.T, o, u, ws.ptr, ws.size, status, st);
     });
 }
 
@@ -165,11 +177,11 @@ PyObject *verify_tree(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Draft x(r, d, a[1], a + 2);
     int32_t *parent = r.i32(a[9], {x.T}), *depth = r.i32(a[10], {x.T});
     float *o = r.f32(a[11], {d.n_layers, x.T, d.heads, d.d_v}), *u = r.f32(a[12], {d.n_layers, x.T, d.heads, d.d_v});
-    const at::Tensor *ws = r.tensor(a[13], ScalarType::Byte);
+    const Reader::Bytes ws = r.bytes(a[13]);
     int32_t *status = r.i32(a[14], {1});
     return call(r, [&](void *st) {
-        return g_api.verify_tree(&d, x.S, x.q, x.k, x.v, x.alpha, x.beta, x.offs, x.T, parent, depth, o, u, ws->data_ptr(),
-                                 size_t(ws->numel()), status, st);
+        return g_api.verify_tree(&d, x.S, x.q, x.k, x.v, x.alpha, x.beta, x.offs, x.T, parent, depth, o, u, ws.ptr,
+                                 ws.size, status, st);
     });
 }
 
@@ -192,12 +204,14 @@ PyObject *greedy_accept(PyObject *, PyObject *const *a, Py_ssize_t n)
     Reader r(n, 11);
     if (!r.ok) Py_RETURN_NONE;
     const int B = r.integer(a[0]), D = r.integer(a[1]);
-    const at::Tensor *par = r.any(a[3], ScalarType::Int, 1);
-    const int64_t T = par != nullptr ? par->numel() : 0;
+    const at::Tensor *par_t = r.any(a[3], ScalarType::Int, 1);
+    if (!r.ok) Py_RETURN_NONE;
+    const int64_t T = par_t->numel();
+    const int32_t *par = par_t->const_data_ptr<int32_t>();
     int32_t *offs = r.i32(a[2], {B + 1}), *draft = r.i32(a[4], {T}), *target = r.i32(a[5], {T}), *root = r.i32(a[6], {B}),
             *idx = r.i32(a[7], {B, D}), *len = r.i32(a[8], {B}), *next = r.i32(a[9], {B}), *status = r.i32(a[10], {1});
     return call(r, [&](void *st) {
-        return g_api.greedy_accept(B, D, offs, par->const_data_ptr<int32_t>(), draft, target, root, idx, len, next, status, st);
+        return g_api.greedy_accept(B, D, offs, par, draft, target, root, idx, len, next, status, st);
     });
 }
 
@@ -206,13 +220,15 @@ PyObject *stochastic_accept(PyObject *, PyObject *const *a, Py_ssize_t n)
     Reader r(n, 10);
     if (!r.ok) Py_RETURN_NONE;
     const int B = r.integer(a[0]), D = r.integer(a[1]);
-    const at::Tensor *par = r.any(a[3], ScalarType::Int, 1);
-    const int64_t T = par != nullptr ? par->numel() : 0;
+    const at::Tensor *par_t = r.any(a[3], ScalarType::Int, 1);
+    if (!r.ok) Py_RETURN_NONE;
+    const int64_t T = par_t->numel();
+    const int32_t *par = par_t->const_data_ptr<int32_t>();
     int32_t *offs = r.i32(a[2], {B + 1});
     float *pt = r.f32(a[4], {T}), *pd = r.f32(a[5], {T}), *un = r.f32(a[6], {T});
     int32_t *idx = r.i32(a[7], {B, D}), *len = r.i32(a[8], {B}), *status = r.i32(a[9], {1});
     return call(r, [&](void *st) {
-        return g_api.stochastic_accept(B, D, offs, par->const_data_ptr<int32_t>(), pt, pd, un, idx, len, status, st);
+        return g_api.stochastic_accept(B, D, offs, par, pt, pd, un, idx, len, status, st);
     });
 }
 
@@ -266,11 +282,11 @@ PyObject *commit_verify_tree(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Draft x(r, d, a[1], a + 5);
     int32_t *parent = r.i32(a[12], {x.T}), *depth = r.i32(a[13], {x.T});
     float *o = r.f32(a[14], {L, x.T, H, dv}), *u = r.f32(a[15], {L, x.T, H, dv});
-    const at::Tensor *ws = r.tensor(a[16], ScalarType::Byte);
+    const Reader::Bytes ws = r.bytes(a[16]);
     int32_t *status = r.i32(a[17], {1});
     return call(r, [&](void *st) {
         return g_api.commit_verify_tree(&d, x.S, pk, pv, pa, pb, pu, po, Tp, pp, idx, len, x.q, x.k, x.v, x.alpha, x.beta, x.offs, x.T,
-                                        parent, depth, o, u, ws->data_ptr(), size_t(ws->numel()), status, st);
+                                        parent, depth, o, u, ws.ptr, ws.size, status, st);
     });
 }
 
@@ -285,9 +301,11 @@ PyObject *commit_conv(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (idx->size(0) != B || L > INT32_MAX || B > INT32_MAX || W > INT32_MAX || ch > INT32_MAX || D > INT32_MAX) Py_RETURN_NONE;
     uint16_t *x = r.bf16(a[1], {L, T, ch});
     int32_t *offs = r.i32(a[2], {B + 1}), *len = r.i32(a[5], {B}), *status = r.i32(a[6], {1});
+    uint16_t *c_ptr = static_cast<uint16_t *>(C->data_ptr());
+    const int32_t *idx_ptr = idx->const_data_ptr<int32_t>();
     return call(r, [&](void *st) {
-        return g_api.commit_conv(int(L), int(B), int(ch), int(W), int(D), static_cast<uint16_t *>(C->data_ptr()), x, offs, T,
-                                 idx->const_data_ptr<int32_t>(), len, status, st);
+        return g_api.commit_conv(int(L), int(B), int(ch), int(W), int(D), c_ptr, x, offs, T,
+                                 idx_ptr, len, status, st);
     });
 }
 
@@ -297,28 +315,30 @@ PyObject *tree_mask_to_parent(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (!r.ok) Py_RETURN_NONE;
     const at::Tensor *mask = r.any(a[0], ScalarType::Byte, 3), *par = r.any(a[2], ScalarType::Int, 1);
     if (!r.ok || mask->size(1) != mask->size(2) || mask->size(0) > INT32_MAX || mask->size(1) > INT32_MAX) Py_RETURN_NONE;
-    const int64_t B = mask->size(0);
+    const int64_t B = mask->size(0), N = mask->size(1);
     int32_t *offs = r.i32(a[1], {B + 1}), *status = r.i32(a[3], {1});
+    const uint8_t *mask_ptr = mask->const_data_ptr<uint8_t>();
+    int32_t *par_ptr = static_cast<int32_t *>(par->data_ptr());
     return call(r, [&](void *st) {
-        return g_api.tree_mask_to_parent(int(B), int(mask->size(1)), mask->const_data_ptr<uint8_t>(), offs,
-                                         static_cast<int32_t *>(par->data_ptr()), status, st);
+        return g_api.tree_mask_to_parent(int(B), int(N), mask_ptr, offs, par_ptr, status, st);
     });
 }
 
 PyObject *prune_tree(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     Reader r(n, 10);
-    if (!r.ok || !PyFloat_Check(a[1])) Py_RETURN_NONE;
+    if (!r.ok || !(PyFloat_Check(a[1]) || PyLong_Check(a[1]))) Py_RETURN_NONE;
     const int N = r.integer(a[0]), budget = r.integer(a[2]);
-    const float tau = float(PyFloat_AS_DOUBLE(a[1]));
-    const at::Tensor *offs = r.any(a[3], ScalarType::Int, 1), *par = r.any(a[4], ScalarType::Int, 1);
-    if (!r.ok || offs->numel() < 1 || offs->numel() > INT32_MAX) Py_RETURN_NONE;
-    const int64_t B = offs->numel() - 1, T = par->numel();
+    const float tau = float(PyFloat_AsDouble(a[1]));
+    if (PyErr_Occurred()) { PyErr_Clear(); Py_RETURN_NONE; }     // an integer beyond every double
+    const at::Tensor *offs_t = r.any(a[3], ScalarType::Int, 1), *par_t = r.any(a[4], ScalarType::Int, 1);
+    if (!r.ok || offs_t->numel() < 1 || offs_t->numel() > INT32_MAX) Py_RETURN_NONE;
+    const int64_t B = offs_t->numel() - 1, T = par_t->numel();
+    const int32_t *offs = offs_t->const_data_ptr<int32_t>(), *par = par_t->const_data_ptr<int32_t>();
     float *logp = r.f32(a[5], {T});
     int32_t *oo = r.i32(a[6], {B + 1}), *op = r.i32(a[7], {T}), *oi = r.i32(a[8], {T}), *status = r.i32(a[9], {1});
     return call(r, [&](void *st) {
-        return g_api.prune_tree(int(B), N, tau, budget, offs->const_data_ptr<int32_t>(), par->const_data_ptr<int32_t>(), logp, oo, op,
-                                oi, status, st);
+        return g_api.prune_tree(int(B), N, tau, budget, offs, par, logp, oo, op, oi, status, st);
     });
 }
 
@@ -327,12 +347,13 @@ PyObject *chain_decompose(PyObject *, PyObject *const *a, Py_ssize_t n)
     Reader r(n, 6);
     if (!r.ok) Py_RETURN_NONE;
     const int N = r.integer(a[0]);
-    const at::Tensor *offs = r.any(a[1], ScalarType::Int, 1), *par = r.any(a[2], ScalarType::Int, 1);
-    if (!r.ok || offs->numel() < 1 || offs->numel() > INT32_MAX) Py_RETURN_NONE;
-    const int64_t B = offs->numel() - 1, T = par->numel();
+    const at::Tensor *offs_t = r.any(a[1], ScalarType::Int, 1), *par_t = r.any(a[2], ScalarType::Int, 1);
+    if (!r.ok || offs_t->numel() < 1 || offs_t->numel() > INT32_MAX) Py_RETURN_NONE;
+    const int64_t B = offs_t->numel() - 1, T = par_t->numel();
+    const int32_t *offs = offs_t->const_data_ptr<int32_t>(), *par = par_t->const_data_ptr<int32_t>();
     int32_t *head = r.i32(a[3], {T}), *count = r.i32(a[4], {B}), *status = r.i32(a[5], {1});
     return call(r, [&](void *st) {
-        return g_api.chain_decompose(int(B), N, offs->const_data_ptr<int32_t>(), par->const_data_ptr<int32_t>(), head, count, status, st);
+        return g_api.chain_decompose(int(B), N, offs, par, head, count, status, st);
     });
 }
 
@@ -365,7 +386,18 @@ PyObject *bind(PyObject *, PyObject *table)
     Py_RETURN_NONE;
 }
 
-#define FAST(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void *>(f)), METH_FASTCALL, nullptr}
+// An exception must not leave a C function: to the interpreter it would be std::terminate.
+template <PyObject *(*F)(PyObject *, PyObject *const *, Py_ssize_t)>
+PyObject *guarded(PyObject *self, PyObject *const *a, Py_ssize_t n)
+{
+    try {
+        return F(self, a, n);
+    } catch (...) {
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
+}
+#define FAST(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void *>(&guarded<f>)), METH_FASTCALL, nullptr}
 PyMethodDef kMethods[] = {
     FAST(decode_step), FAST(verify_chain), FAST(verify_tree), FAST(verify_tree_noalloc), FAST(greedy_accept),
     FAST(stochastic_accept), FAST(commit), FAST(commit_verify_tree), FAST(commit_conv), FAST(tree_mask_to_parent),

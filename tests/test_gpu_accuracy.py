@@ -110,3 +110,31 @@ def test_single_pass_route_degrades_with_the_state_and_is_never_the_default():
     e_fast, e_auto = rel_err(cpu(fast.o), ref), rel_err(cpu(auto.o), ref)
     print(f"single pass {e_fast:.3e}, default {e_auto:.3e}")
     assert e_auto <= TOL_FP32 and e_fast > 10 * e_auto
+
+
+@pytest.mark.parametrize("d_k,d_v,nodes,depth,chain,before,margin", [
+    (64, 64, 8, 8, True, speca.ROUTE_SERIAL, 1.1), (64, 64, 16, 16, True, speca.ROUTE_SERIAL, 1.2),
+    (64, 64, 30, 8, False, speca.ROUTE_SERIAL, 1.0), (64, 128, 60, 16, False, speca.ROUTE_SERIAL, 1.0),
+    (128, 96, 8, 8, True, speca.ROUTE_SERIAL, 1.2), (128, 64, 30, 8, False, speca.ROUTE_SERIAL, 1.0),
+    (256, 64, 8, 8, True, speca.ROUTE_SERIAL, 1.2), (256, 32, 30, 8, False, speca.ROUTE_SERIAL, 1.1),
+    (128, 128, 8, 8, True, speca.ROUTE_FACTORIZED, 1.0), (128, 256, 30, 16, False, speca.ROUTE_FACTORIZED, 1.0),
+    (256, 256, 8, 8, True, speca.ROUTE_FACTORIZED, 1.0)])
+def test_the_default_route_is_no_further_off_than_the_one_it_replaced(d_k, d_v, nodes, depth, chain, before, margin):
+    """Error against the oracle (2-norm of the difference) of the register-streaming kernel and of the route that would
+    take the same shape without it (FACTORIZED with u is the substitution kernel).  `margin` is for the few per cent by
+    which two fp32 computations that round in another order differ; sums left to the tensor core's truncating adder are
+    a factor of 1.2 to 3 off."""
+    rng = np.random.default_rng(nodes + d_k)
+    parents = [synth.chain_parent(nodes) if chain else synth.random_tree_parent(nodes, depth, 4, rng) for _ in range(6)]
+    prob = synth.make_problem(4600 + d_k + nodes, 2, 4, d_k, d_v, parents, max_depth=depth)
+    ref = oracle_verify(prob)
+
+    def error(route, want_u):
+        dp = DevProblem(prob, route=route, want_u=want_u)
+        (dp.verify_chain if chain else dp.verify_tree)()
+        assert dp.status_value() == 0
+        return float(np.linalg.norm(cpu(dp.o).astype(np.float64) - ref) / np.linalg.norm(ref))
+
+    now, then = error(speca.ROUTE_AUTO, False), error(before, before == speca.ROUTE_FACTORIZED)
+    print(f"{d_k} x {d_v}, {nodes} nodes: {now:.3e}, before {then:.3e}")
+    assert now <= margin * then
