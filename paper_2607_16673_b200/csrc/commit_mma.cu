@@ -58,7 +58,7 @@ commit_long_kernel(Params p)
         int count = 0;
         for (int b0 = 0; b0 < p.B; b0 += 32) {
             const int b = b0 + lane;
-            const int len = b < p.B ? __ldg(p.path_len + b) : 0;
+            const int len = b < p.B ? p.path_len[b] : 0;
             const bool take = len >= p.long_min && len <= kLongMax && len <= p.max_depth;
             const unsigned m = __ballot_sync(0xffffffffu, take);
             if (take) s_long[count + __popc(m & ((1u << lane) - 1u))] = uint16_t(b);
@@ -85,19 +85,19 @@ commit_long_kernel(Params p)
         const int h = int(rest % p.H); rest /= p.H;
         const int l = int(rest % p.L);
         const int b = s_long[rest / p.L];
-        const int len = __ldg(p.path_len + b);
-        const int base = __ldg(p.node_offsets + b);
-        const int n = __ldg(p.node_offsets + b + 1) - base;
+        const int len = p.path_len[b];
+        const int base = p.node_offsets[b];
+        const int n = p.node_offsets[b + 1] - base;
 
         // validate the path as the token-by-token kernel does; a bad path leaves the state untouched
         int fault = 0;
         long rec = 0;
         if (base < 0 || n < 0 || base + n > p.T) fault = SPECA_STATUS_BAD_OFFSETS;
         else if (lane < len) {
-            const int node = __ldg(p.path_idx + b * p.max_depth + lane);
-            const int prev = lane > 0 ? __ldg(p.path_idx + b * p.max_depth + lane - 1) : -1;
+            const int node = p.path_idx[b * p.max_depth + lane];
+            const int prev = lane > 0 ? p.path_idx[b * p.max_depth + lane - 1] : -1;
             if (node < 0 || node >= n) fault = SPECA_STATUS_BAD_PATH;
-            else if (p.parent != nullptr && __ldg(p.parent + base + node) != prev) fault = SPECA_STATUS_BAD_PATH;
+            else if (p.parent != nullptr && p.parent[base + node] != prev) fault = SPECA_STATUS_BAD_PATH;
             rec = (long(l) * p.T + base + node) * p.H + h;
         }
         const unsigned bad = __ballot_sync(0xffffffffu, fault != 0);
@@ -105,8 +105,8 @@ commit_long_kernel(Params p)
             if (l == 0 && h == 0 && part == 0 && lane == __ffs(bad) - 1) atomicOr(p.status, fault);
             continue;
         }
-        const float alpha = lane < len ? __ldg(p.alpha + rec) : 1.f;
-        const float beta = lane < len ? __ldg(p.beta + rec) : 0.f;
+        const float alpha = lane < len ? p.alpha[rec] : 1.f;
+        const float beta = lane < len ? p.beta[rec] : 0.f;
 
         // key fragments in the permuted order, and the Gram block of the keys from the same values
         const long rec_g = __shfl_sync(0xffffffffu, rec, g);
@@ -117,14 +117,14 @@ commit_long_kernel(Params p)
         for (int me = 0; me < NME; ++me) {
             const int m = me >> 1, e = me & 1;
             uint32_t w = 0;
-            if (g < len) w = __ldg(reinterpret_cast<const uint32_t *>(p.k + rec_g * DK + 4 * (t + 4 * m) + 2 * e));
+            if (g < len) w = *reinterpret_cast<const uint32_t *>(p.k + rec_g * DK + 4 * (t + 4 * m) + 2 * e);
             const uint32_t b0 = w << 16, b1 = w & 0xffff0000u;
             tab1[me][lane] = make_float2(__uint_as_float(b0), __uint_as_float(b1));
             const uint32_t a[4] = {b0, 0u, b1, 0u};
             mma_tf32_sync(gram, a, b0, b1);
             const int col2 = 4 * ((g >> 1) + 4 * m) + 2 * e + (g & 1);
-            const unsigned short x0 = t < len ? __ldg(reinterpret_cast<const unsigned short *>(p.k + rec_t * DK + col2)) : 0;
-            const unsigned short x1 = t + 4 < len ? __ldg(reinterpret_cast<const unsigned short *>(p.k + rec_t4 * DK + col2)) : 0;
+            const unsigned short x0 = t < len ? *reinterpret_cast<const unsigned short *>(p.k + rec_t * DK + col2) : 0;
+            const unsigned short x1 = t + 4 < len ? *reinterpret_cast<const unsigned short *>(p.k + rec_t4 * DK + col2) : 0;
             tab2[me][lane] = make_float2(__uint_as_float(uint32_t(x0) << 16), __uint_as_float(uint32_t(x1) << 16));
         }
         // coefficient rows: lane i (< 8) builds row i from the Gram entries k_j . k_i, which sit in lanes
@@ -176,7 +176,7 @@ commit_long_kernel(Params p)
 #pragma unroll
             for (int i = 0; i < kLongMax; ++i) {
                 const long rec_i = __shfl_sync(0xffffffffu, rec, i);
-                vv[i] = i < len ? __uint_as_float(uint32_t(__ldg(reinterpret_cast<const unsigned short *>(p.v + rec_i * p.DV + my_row))) << 16)
+                vv[i] = i < len ? __uint_as_float(uint32_t(*reinterpret_cast<const unsigned short *>(p.v + rec_i * p.DV + my_row)) << 16)
                                 : 0.f;
             }
             // R = S0 K^T

@@ -217,7 +217,7 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
     };
     if (da.early) prefetch_first();
 
-    const int base = __ldg(p.node_offsets + b), end = __ldg(p.node_offsets + b + 1);
+    const int base = p.node_offsets[b], end = p.node_offsets[b + 1];
     const int n = end - base;
     const bool reporter = l == 0 && h == 0 && part == 0 && tid == 0;
     if (base < 0 || n < 0 || end > p.T || (b == p.B - 1 && end != p.T) || (b == 0 && base != 0)) {
@@ -252,9 +252,9 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
     int pa = -1, fault = 0;
     float al = 1.f, be = 0.f;
     if (tid < n) {
-        pa = p.parent != nullptr ? __ldg(p.parent + base + tid) : tid - 1;
-        al = __ldg(p.alpha + rec0 + long(tid) * H);
-        be = __ldg(p.beta + rec0 + long(tid) * H);
+        pa = p.parent != nullptr ? p.parent[base + tid] : tid - 1;
+        al = p.alpha[rec0 + long(tid) * H];
+        be = p.beta[rec0 + long(tid) * H];
     }
     {
         constexpr int PCS = DK / 8;
@@ -303,7 +303,7 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
         int full = d;
         for (; a >= 0; a = sPar[a]) ++full;
         if (full > p.max_depth) fault |= SPECA_STATUS_TOO_DEEP;
-        if (p.depth_in != nullptr && __ldg(p.depth_in + base + tid) != full) fault |= SPECA_STATUS_BAD_DEPTH;
+        if (p.depth_in != nullptr && p.depth_in[base + tid] != full) fault |= SPECA_STATUS_BAD_DEPTH;
         if (fault && l == 0 && h == 0 && part == 0) atomicOr(p.status, fault);
     }
 

@@ -172,7 +172,7 @@ __device__ __forceinline__ bool next_unit(const Walk &w, VUnit &x)
             x.h = g * w.HG;
             x.u = (x.l * w.B + x.b) * w.H + x.h;
             x.npad = (x.n + 15) & ~15;
-            x.base = in_tab ? reinterpret_cast<const int32_t *>(w.tab)[x.b] : __ldg(w.offs + x.b);
+            x.base = in_tab ? reinterpret_cast<const int32_t *>(w.tab)[x.b] : w.offs[x.b];
             return true;
         }
     }
@@ -687,18 +687,18 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             if (node < y.n) {
                 const int i = y.base + node;
                 if (MAXD <= 8) {
-                    const int2 w = __ldg(reinterpret_cast<const int2 *>(p.ws.up) + 2 * i);
+                    const int2 w = reinterpret_cast<const int2 *>(p.ws.up)[2 * i];
                     up_n[0] = uint32_t(w.x); up_n[1] = uint32_t(w.y);
                 } else {
-                    const int4 w = __ldg(reinterpret_cast<const int4 *>(p.ws.up) + i);
+                    const int4 w = reinterpret_cast<const int4 *>(p.ws.up)[i];
                     up_n[0] = uint32_t(w.x); up_n[1] = uint32_t(w.y); up_n[2] = uint32_t(w.z); up_n[3] = uint32_t(w.w);
                 }
-                const int2 s = __ldg(reinterpret_cast<const int2 *>(p.ws.set) + i);
+                const int2 s = reinterpret_cast<const int2 *>(p.ws.set)[i];
                 lo_n = uint32_t(s.x); hi_n = uint32_t(s.y);
-                d_n = __ldg(p.ws.depth + i);
+                d_n = p.ws.depth[i];
                 const int r = FEW ? ((y.l * p.T + i) * p.H + y.h) >> ep.share : (y.l * p.T + i) * p.H + y.h;
-                alpha_n = __ldg(p.alpha + r);
-                beta_n = __ldg(p.beta + r);
+                alpha_n = p.alpha[r];
+                beta_n = p.beta[r];
             }
         };
         VUnit nx = x;

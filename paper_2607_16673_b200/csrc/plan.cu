@@ -18,8 +18,8 @@ constexpr int kPlanThreads = 128;
 
 // One CTA per sequence.  Dynamic smem: 6 int32 arrays of max_nodes (+1).
 __global__ void __launch_bounds__(kPlanThreads)
-plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict__ parent,
-            const int32_t *__restrict__ depth_in, int32_t B, int32_t T, int32_t max_depth,
+plan_kernel(const int32_t *node_offsets, const int32_t *parent,
+            const int32_t *depth_in, int32_t B, int32_t T, int32_t max_depth,
             int32_t max_nodes, int32_t skip_nodes, int32_t paths_only, int32_t n_slots, Workspace ws, int32_t *status)
 {
     after_previous_kernel();
@@ -175,9 +175,9 @@ plan_kernel(const int32_t *__restrict__ node_offsets, const int32_t *__restrict_
 // One warp per sequence.  Each lane takes nodes t = lane, lane+32, ... and walks t's
 // root path checking every token against the prediction made at its parent.
 __global__ void __launch_bounds__(128)
-accept_kernel(int32_t B, int32_t max_depth, const int32_t *__restrict__ node_offsets,
-              const int32_t *__restrict__ parent, const int32_t *__restrict__ draft_tok,
-              const int32_t *__restrict__ target_tok, const int32_t *__restrict__ root_target_tok,
+accept_kernel(int32_t B, int32_t max_depth, const int32_t *node_offsets,
+              const int32_t *parent, const int32_t *draft_tok,
+              const int32_t *target_tok, const int32_t *root_target_tok,
               int32_t *__restrict__ path_idx, int32_t *__restrict__ path_len,
               int32_t *__restrict__ next_tok, int32_t *status)
 {
@@ -233,9 +233,9 @@ accept_kernel(int32_t B, int32_t max_depth, const int32_t *__restrict__ node_off
 // passes, and stops when none does.  A node is therefore on the accepted path iff it and all
 // its ancestors are "chosen": passing, with no passing sibling of lower index.
 __global__ void __launch_bounds__(128)
-stochastic_accept_kernel(int32_t B, int32_t max_depth, const int32_t *__restrict__ node_offsets,
-                         const int32_t *__restrict__ parent, const float *__restrict__ p_target,
-                         const float *__restrict__ p_draft, const float *__restrict__ uniform,
+stochastic_accept_kernel(int32_t B, int32_t max_depth, const int32_t *node_offsets,
+                         const int32_t *parent, const float *p_target,
+                         const float *p_draft, const float *uniform,
                          int32_t *__restrict__ path_idx, int32_t *__restrict__ path_len, int32_t *status)
 {
     after_previous_kernel();
@@ -327,8 +327,8 @@ stochastic_accept_kernel(int32_t B, int32_t max_depth, const int32_t *__restrict
 // arrays (word 9).
 __global__ void __launch_bounds__(128)
 pending_check_kernel(int32_t B, int32_t Tp, int32_t max_depth, int32_t max_len, int32_t max_nodes,
-                     const int32_t *__restrict__ pnode_offsets, const int32_t *__restrict__ pparent,
-                     const int32_t *__restrict__ path_idx, const int32_t *__restrict__ path_len,
+                     const int32_t *pnode_offsets, const int32_t *pparent,
+                     const int32_t *path_idx, const int32_t *path_len,
                      int32_t *__restrict__ pend, int32_t *status)
 {
     after_previous_kernel();
@@ -361,8 +361,8 @@ pending_check_kernel(int32_t B, int32_t Tp, int32_t max_depth, int32_t max_len, 
 constexpr int kConvMaxWidth = 8;
 __global__ void __launch_bounds__(256)
 conv_commit_kernel(int32_t B, int32_t channels, int32_t W, int32_t T, int32_t max_depth, uint4 *__restrict__ C,
-                   const uint4 *__restrict__ x, const int32_t *__restrict__ node_offsets,
-                   const int32_t *__restrict__ path_idx, const int32_t *__restrict__ path_len, int32_t *status)
+                   const uint4 *x, const int32_t *node_offsets,
+                   const int32_t *path_idx, const int32_t *path_len, int32_t *status)
 {
     after_previous_kernel();
     const int l = blockIdx.x / B, b = blockIdx.x % B;
@@ -390,7 +390,7 @@ conv_commit_kernel(int32_t B, int32_t channels, int32_t W, int32_t T, int32_t ma
             if (w < W) {
                 const int s = A + w;                    // index in (old rows, accepted rows); the last W are kept
                 if (s < W) row[w] = Cb[s * vec + c];
-                else row[w] = __ldg(x + (size_t(l) * T + base + path_idx[b * max_depth + (s - W)]) * vec + c);
+                else row[w] = x[(size_t(l) * T + base + path_idx[b * max_depth + (s - W)]) * vec + c];
             }
         }
 #pragma unroll
@@ -408,7 +408,7 @@ conv_commit_kernel(int32_t B, int32_t channels, int32_t W, int32_t T, int32_t ma
 // 10.1 us either way, staged 6.4 us).
 constexpr int kMaskStage = 16 * 1024;
 __global__ void __launch_bounds__(256)
-mask_to_parent_kernel(int32_t N, const uint8_t *__restrict__ mask, const int32_t *__restrict__ node_offsets,
+mask_to_parent_kernel(int32_t N, const uint8_t *mask, const int32_t *node_offsets,
                       int32_t *__restrict__ parent, int32_t *status)
 {
     after_previous_kernel();
@@ -425,7 +425,7 @@ mask_to_parent_kernel(int32_t N, const uint8_t *__restrict__ mask, const int32_t
         if ((N & 3) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15u) == 0)          // every mask starts on 16 bytes
 #pragma unroll 4
             for (int i = threadIdx.x; i < n * N / 16 + (n * N % 16 != 0); i += 256)
-                reinterpret_cast<uint4 *>(staged)[i] = __ldg(reinterpret_cast<const uint4 *>(m) + i);
+                reinterpret_cast<uint4 *>(staged)[i] = reinterpret_cast<const uint4 *>(m)[i];
         else
 #pragma unroll 8
             for (int i = threadIdx.x; i < n * N; i += 256) staged[i] = m[i];
@@ -468,7 +468,7 @@ mask_to_parent_kernel(int32_t N, const uint8_t *__restrict__ mask, const int32_t
 // of the committed state).  Subtree sizes are integer sums over ancestor walks, the heavy child an
 // integer maximum: both are exact whatever the order of the atomics.
 __global__ void __launch_bounds__(256)
-chain_decompose_kernel(int32_t N, const int32_t *__restrict__ node_offsets, const int32_t *__restrict__ parent,
+chain_decompose_kernel(int32_t N, const int32_t *node_offsets, const int32_t *parent,
                        int32_t *__restrict__ chain_head, int32_t *__restrict__ n_chains, int32_t *status)
 {
     after_previous_kernel();
@@ -561,8 +561,8 @@ __device__ __forceinline__ void down_levels(int n, const int32_t *par, int32_t *
 
 template <bool WRITE>
 __global__ void __launch_bounds__(128)
-prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *__restrict__ node_offsets,
-             const int32_t *__restrict__ parent, const float *__restrict__ logp, int32_t *__restrict__ out_offsets,
+prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *node_offsets,
+             const int32_t *parent, const float *logp, int32_t *__restrict__ out_offsets,
              int32_t *__restrict__ out_parent, int32_t *__restrict__ out_index, int32_t *status)
 {
     after_previous_kernel();

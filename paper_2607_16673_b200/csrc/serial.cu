@@ -36,7 +36,7 @@ template <int G> __device__ __forceinline__ void load_vec(const __nv_bfloat16 *p
 {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(p) + g + G * c);
+        const uint2 raw = reinterpret_cast<const uint2 *>(p)[g + G * c];
         x[2 * c + 0] = make_float2(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u));
         x[2 * c + 1] = make_float2(__uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
     }
@@ -79,14 +79,14 @@ __device__ __forceinline__ void axpy16(float2 (&s)[8], const float2 (&k)[8], flo
 
 __device__ __forceinline__ float bf16_to_float(const __nv_bfloat16 *p)
 {
-    return __uint_as_float(uint32_t(__ldg(reinterpret_cast<const unsigned short *>(p))) << 16);
+    return __uint_as_float(uint32_t(*reinterpret_cast<const unsigned short *>(p)) << 16);
 }
 
 // ---------------------------------------------------------------------------
 // decode step: S in place, one token per sequence
 // ---------------------------------------------------------------------------
 template <int DK, int RS, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32)
+__global__ void __launch_bounds__(WARPS * 32, 2048 / (WARPS * 32) / 2)
 decode_kernel(Params p)
 {
     after_previous_kernel();
@@ -103,7 +103,7 @@ decode_kernel(Params p)
     float2 kx[8], qx[8];
     load_vec<G>(p.k + unit * DK, g, kx);
     load_vec<G>(p.q + unit * DK, g, qx);
-    const float alpha = __ldg(p.alpha + unit), beta = __ldg(p.beta + unit);
+    const float alpha = p.alpha[unit], beta = p.beta[unit];
     const float kq = group_sum<G>(dot16(kx, qx));
 #pragma unroll
     for (int r = 0; r < RS; ++r) {
@@ -134,10 +134,10 @@ verify_serial_kernel(Params p)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane % G, sub = lane / G;
     const int row0 = (blockIdx.x % tiles) * ROWS + warp * RS * RPS;
 
-    const int base = __ldg(p.node_offsets + b);
+    const int base = p.node_offsets[b];
     int n;
     if (CHAIN) {
-        n = __ldg(p.node_offsets + b + 1) - base;
+        n = p.node_offsets[b + 1] - base;
         int fault = 0;
         if (base < 0 || n < 0 || base + n > p.T) fault = SPECA_STATUS_BAD_OFFSETS;
         else if (n > p.max_nodes) fault = SPECA_STATUS_TOO_MANY;
@@ -162,7 +162,7 @@ verify_serial_kernel(Params p)
         int t = j, load = 0, save = 0;
         bool leaf = (j == n - 1);
         if (!CHAIN) {
-            const int e = __ldg(p.ws.plan + base + j);
+            const int e = p.ws.plan[base + j];
             t = e & 0xffff;
             load = (e >> kPlanLoadShift) & 15;
             save = (e >> kPlanSaveShift) & 15;
@@ -180,7 +180,7 @@ verify_serial_kernel(Params p)
         float2 kx[8], qx[8];
         load_vec<G>(p.k + rec * DK, g, kx);
         load_vec<G>(p.q + rec * DK, g, qx);
-        const float alpha = __ldg(p.alpha + rec), beta = __ldg(p.beta + rec);
+        const float alpha = p.alpha[rec], beta = p.beta[rec];
         const float kq = group_sum<G>(dot16(kx, qx));
 #pragma unroll
         for (int r = 0; r < RS; ++r) {
@@ -228,9 +228,9 @@ commit_kernel(Params p)
     const int lane = threadIdx.x & 31, g = lane % G, sub = lane / G;
 
     // path_len == 0: the sequence's state is neither read nor written
-    const int len = __ldg(p.path_len + b);
-    const int base = __ldg(p.node_offsets + b);
-    const int n = __ldg(p.node_offsets + b + 1) - base;
+    const int len = p.path_len[b];
+    const int base = p.node_offsets[b];
+    const int n = p.node_offsets[b + 1] - base;
     if (len == 0) return;
     // paths the tensor-core commit takes (it validates them itself)
     if (p.long_min > 0 && len >= p.long_min && len <= 8 && len <= p.max_depth) return;
@@ -259,21 +259,21 @@ commit_kernel(Params p)
     else {
         if (int(threadIdx.x) < len) {
             const int d = threadIdx.x;
-            const int t = __ldg(p.path_idx + b * p.max_depth + d);
-            const int prev = d > 0 ? __ldg(p.path_idx + b * p.max_depth + d - 1) : -1;
+            const int t = p.path_idx[b * p.max_depth + d];
+            const int prev = d > 0 ? p.path_idx[b * p.max_depth + d - 1] : -1;
             if (t < 0 || t >= n) fault = SPECA_STATUS_BAD_PATH;
-            else if (p.parent != nullptr && __ldg(p.parent + base + t) != prev) fault = SPECA_STATUS_BAD_PATH;
+            else if (p.parent != nullptr && p.parent[base + t] != prev) fault = SPECA_STATUS_BAD_PATH;
             s_path[d] = t;
             if (!fault) {
                 const long rec = (long(l) * p.T + base + t) * p.H + h;
-                s_alpha[d] = __ldg(p.alpha + rec);
-                s_beta[d] = __ldg(p.beta + rec);
+                s_alpha[d] = p.alpha[rec];
+                s_beta[d] = p.beta[rec];
             }
         }
         constexpr int PIECES = DK / 8;                       // 16-byte pieces per k row
         for (int idx = threadIdx.x; idx < len * PIECES; idx += WARPS * 32) {
             const int d = idx / PIECES, piece = idx % PIECES;
-            const int t = __ldg(p.path_idx + b * p.max_depth + d);
+            const int t = p.path_idx[b * p.max_depth + d];
             if (t >= 0 && t < n) {
                 const long rec = (long(l) * p.T + base + t) * p.H + h;
                 const uint32_t dst = uint32_t(__cvta_generic_to_shared(&s_k[d][piece * 8]));
@@ -283,7 +283,7 @@ commit_kernel(Params p)
         }
         for (int idx = threadIdx.x; idx < len * part_rows; idx += WARPS * 32) {
             const int d = idx / part_rows, r = idx % part_rows;
-            const int t = __ldg(p.path_idx + b * p.max_depth + d);
+            const int t = p.path_idx[b * p.max_depth + d];
             if (t >= 0 && t < n) {
                 const long rec = (long(l) * p.T + base + t) * p.H + h;
                 s_v[d][r] = p.v[rec * p.DV + part * part_rows + r];

@@ -159,8 +159,10 @@ inline int sm_count_of_current_device()
 // Overlapped launches (programmatic dependent launch).  A round is a handful of kernels on one stream, and between two of
 // them the device used to sit idle while one drained and the next was set up.  Every kernel here first waits until the
 // kernel in front of it has completed and its writes are visible, and only then lets the one behind it be set up, beside
-// its own last wave of blocks.  The order matters: the next kernel's blocks start with clean L1 lines only after
-// everything before this kernel has been written, so that its read-only loads are as safe as after a plain launch.
+// its own last wave of blocks.  A kernel is thus already there while the one before it still writes what it is going to
+// read.  Loads through the read-only path (__ldg, const __restrict__ parameters, ld.global.nc) ask for data that nobody
+// writes while the kernel is there, and the compiler may move them above the wait: no kernel launched this way has any, it
+// reads with plain loads.
 // Kernels that are not launched this way, the caller's own among them, are waited for and wait as ever.  The persistent
 // kernels of large calls are launched plainly and carry none of this: the wait alone changed what the compiler made of
 // them (one fused single-pass call of 32 ragged sequences 888 us, with the wait 902, overlapped 915-935).
