@@ -16,6 +16,7 @@ import ctypes
 import importlib.machinery
 import importlib.util
 import os
+import sysconfig
 from dataclasses import dataclass
 from typing import Optional
 
@@ -23,7 +24,9 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libspeca.so")
-MARSHAL_PATH = os.path.join(_HERE, "speca_marshal.so")
+# The marshalling is compiled against the headers of one Python and one torch and reads their objects directly, so its
+# file is named after both: another environment does not find a binary of this one.
+MARSHAL_PATH = os.path.join(_HERE, f"speca_marshal.{sysconfig.get_config_var('SOABI')}.torch-{torch.__version__}.so")
 
 OK = 0
 STATUS_BAD_PARENT, STATUS_BAD_OFFSETS, STATUS_BAD_PATH, STATUS_TOO_DEEP = 1, 2, 4, 8
@@ -118,7 +121,8 @@ def _load_native():
     global _native
     L = lib()
     if not os.path.exists(MARSHAL_PATH):
-        raise SpecaError(f"{MARSHAL_PATH} is missing: build it with `python -m paper_2607_16673_b200.build`")
+        raise SpecaError(f"{MARSHAL_PATH} is missing (it belongs to one Python and one torch): build it with "
+                         "`python -m paper_2607_16673_b200.build`")
     loader = importlib.machinery.ExtensionFileLoader("speca_marshal", MARSHAL_PATH)
     mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("speca_marshal", loader))
     loader.exec_module(mod)

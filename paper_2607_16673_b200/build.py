@@ -1,5 +1,5 @@
-"""Compile libspeca.so (the CUDA library behind the C ABI) for sm_100a with nvcc, and speca_marshal.so (the binding's
-argument marshalling, against torch's headers) with the host compiler.
+"""Compile libspeca.so (the CUDA library behind the C ABI) for sm_100a with nvcc, and the binding's argument
+marshalling (against torch's headers, speca_marshal.*.so) with the host compiler.
 
 Run as ``python -m paper_2607_16673_b200.build``.  The shared objects are written
 next to this file, so they travel with the source tree.  nvcc cross-compiles without a GPU.
@@ -14,7 +14,6 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libspeca.so")
-MARSHAL = os.path.join(HERE, "speca_marshal.so")
 SOURCES = ["api.cu", "plan.cu", "serial.cu", "commit_mma.cu", "direct.cu", "factorized.cu", "effective.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 
@@ -45,6 +44,7 @@ def _start_marshal(tmp: str) -> subprocess.Popen:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    from .binding import MARSHAL_PATH as MARSHAL               # named after this Python and this torch
     newest = _newest_source_mtime()
     if not force and all(os.path.exists(f) and os.path.getmtime(f) >= newest for f in (LIB, MARSHAL)):
         return LIB

@@ -58,3 +58,14 @@ def test_numpy_integers_and_whole_thresholds_are_taken_natively():
     # a number that int() has to convert first is the binding's
     assert native.prune_tree(2.0, 5.0, 2, offs, parent, logp, *out, status) is None
     speca.prune_tree(2.0, 5.0, 2, offs, parent, logp, *out, status)
+
+
+def test_another_torch_does_not_load_this_binary(tmp_path):
+    """The marshalling reads torch's and Python's objects directly: its file carries both versions in its name, and under
+    another version it is missing, not misread."""
+    speca_build.build()
+    assert torch.__version__ in speca.MARSHAL_PATH
+    code = ("import torch\ntorch.__version__ = '0.0.1'\nfrom paper_2607_16673_b200 import binding as speca\ntry:\n"
+            "    speca._load_native()\nexcept speca.SpecaError as e:\n    print('refused', e)\n")
+    run = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0 and run.stdout.startswith("refused") and "build" in run.stdout, run.stderr[-2000:]
