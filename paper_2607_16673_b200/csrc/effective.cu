@@ -15,6 +15,14 @@
 // Accuracy.  Everything is split into bf16 pieces of 8 bits: the fp32 state and x into three each by truncation
 // (exact: 3 x 8 = 24 bits), M likewise; q, k, v are bf16 already.  S0 [K;Q]^T is three products of pieces, exact up
 // to the fp32 accumulation; x M^T keeps the six products down to 2^-16, the dropped ones are 2^-24 of the result.
+// What is left is the accumulation: the tensor core truncates where it adds, so each further product in one accumulator
+// costs half an ulp toward zero.  So the six products go in by size, over all nodes the small ones first, and the Gram blocks
+// in as many chains from zero as their 64 columns of TMEM hold, added up by the solver.  Error against 64 bits, 2-norm of the
+// difference over that of the outputs, x 10^-8, before both / now / the substitution kernel: d_k = 256, 30 nodes 33 / 22 /
+// 26; d_k = 128, 20 nodes 22 / 16 / 15, 60 nodes at 8 levels 24 / 20 / 14 (no columns left for a second chain), at 16 levels
+// 24 / 20 / (a former kernel) 66.  Both cost 2 to 3 % of a unit.  Gram blocks of warp-level MMAs added up in fp32 bring 60
+// nodes to 14 too, and cost 17 % of a unit of 64 nodes, 28 % of one of 40: the solver has no time for them, and the split
+// warps keep the state product waiting.
 //
 // Why this form.  The staged bf16 rows of [K;Q], as TMA lands them, are the B operand: no fp32 operand is built, so
 // the state stream waits for no preparation, only the second product does, a tile later.  The pieces of the state go
@@ -186,6 +194,8 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
 {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
+// chains into which a Gram block of `npad` columns is split
+__device__ __forceinline__ int gram_parts(int npad) { return npad == 16 ? 4 : npad == 32 ? 2 : 1; }
 // one arrival for the whole warp: every lane's earlier writes are ordered before it
 __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane)
 {
@@ -428,12 +438,16 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 if (!(ok = WAIT(1, bar(kGramFree), (gseq & 1) ^ 1))) break;
                 tc_fence_after();
                 const uint32_t idg = make_idesc_bf16(gx.npad);
+                // in as many chains as the 64 columns hold, each from zero: the solver adds them up
+                const int run = 4 * SC / gram_parts(gx.npad);
 #pragma unroll 1
-                for (int c = 0; c < SC; ++c) {
-                    const uint64_t d = make_desc(sbase + LY::OffStage + par * LY::STAGE + c * SCB);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) mma_bf16(tmem_base + kGramOff, d + 2 * k, d + 2 * k, idg, (c | k) != 0, lead);
-                }
+                for (int i = 0, col = kGramOff; i < 4 * SC; i += run, col += gx.npad)
+#pragma unroll 1
+                    for (int k = i; k < i + run; k += 2) {
+                        const uint64_t d = make_desc(sbase + LY::OffStage + par * LY::STAGE + (k >> 2) * SCB + (k & 2) * 32);
+                        mma_bf16(tmem_base + col, d, d, idg, k != i, lead);
+                        mma_bf16(tmem_base + col, d + 2, d + 2, idg, 1, lead);
+                    }
                 mma_commit(bar(kGramFull), lead);
                 mma_commit(bar(kKQFree + par), lead);
                 ++gseq;
@@ -450,14 +464,14 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 tc_fence_after();
                 const uint32_t acc = tmem_base + (q & 1) * kTileCols, xa = tmem_base + kXOff;
                 const uint64_t md = make_desc(sbase + LY::OffM + (small && mbuf ? LY::MBUF2 : 0));
+#pragma unroll
+                for (int order = 2; order >= 0; --order)          // small products first: 2^-16, 2^-8, the large ones
 #pragma unroll 1
-                for (int ks = 0; ks < ksteps; ++ks)
+                    for (int ks = 0; ks < ksteps; ++ks)
 #pragma unroll
-                    for (int xp = 2; xp >= 0; --xp)               // small products first
-#pragma unroll
-                        for (int mp = 2 - xp; mp >= 0; --mp)
-                            mma_bf16_ts(acc, xa + 32 * xp + 8 * ks, md + uint64_t(mp * (LY::MPIECE >> 4) + 2 * ks), idx,
-                                        (ks | (2 - xp)) != 0, lead);
+                        for (int xp = order; xp >= 0; --xp)
+                            mma_bf16_ts(acc, xa + 32 * xp + 8 * ks, md + uint64_t((order - xp) * (LY::MPIECE >> 4) + 2 * ks), idx,
+                                        !(order == 2 && ks == 0 && xp == 2), lead);
                 mma_commit(bar(kOutFull + (q & 1)), lead);
                 if (t == TP - 1) mma_commit(bar(kMFree + mbuf), lead);
             }
@@ -736,17 +750,25 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             {
                 PROF_T0()
                 float *G = (is_k ? Gk - 1 : Gq) + node * GSTR + d;
+                const int end = gram_parts(R) * R;
 #pragma unroll 1
-                for (int c0 = 0; c0 < R; c0 += 16) {
-                    float g[16];
-                    tmem_ld16(gaddr + c0, g);
-                    const uint4 dep = *reinterpret_cast<const uint4 *>(depth_s + c0);
-                    const uint32_t bits = (c0 & 32 ? set_hi : set_lo) >> (c0 & 16);
+                for (int c0 = 0; c0 < R; c0 += 8) {
+                    float g[8];
+                    tmem_ld8(gaddr + c0, g);
+                    const uint2 dep = *reinterpret_cast<const uint2 *>(depth_s + c0);
+                    const uint32_t bits = (c0 & 32 ? set_hi : set_lo) >> (c0 & 24);
                     tmem_ld_wait();
-                    const uint32_t dw[4] = {dep.x, dep.y, dep.z, dep.w};
+#pragma unroll 1
+                    for (int c1 = c0 + R; c1 < end; c1 += R) {
+                        float more[8];
+                        tmem_ld8(gaddr + c1, more);
+                        tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (bits & (1u << i)) G[-int((dw[i >> 2] >> (8 * (i & 3))) & 0xffu)] = g[i];
+                        for (int i = 0; i < 8; ++i) g[i] += more[i];
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (bits & (1u << i)) G[-int(((i < 4 ? dep.x : dep.y) >> (8 * (i & 3))) & 0xffu)] = g[i];
                 }
                 tc_fence_before();
                 warp_arrive(bar(kGramFree), lane);
