@@ -84,7 +84,7 @@ int verify_common(const speca_dims *dims, const float *S0, const uint16_t *q, co
     if (dims->route == SPECA_ROUTE_AUTO && u == nullptr && (reinterpret_cast<uintptr_t>(S0) & 31u) == 0) {
         int most = dims->max_nodes < total_nodes ? dims->max_nodes : total_nodes;
         if (chain && most > dims->max_depth) most = dims->max_depth;
-        const int limit = direct_limit(p, dims->d_k, most, fact || eff);
+        const int limit = direct_limit(p, dims->d_k, most, fact || eff, chain);
         if (limit > 0) {
             rc = cuda_rc(launch_verify_direct(p, dims->d_k, most, limit, st));
             if (rc != SPECA_OK || most <= limit) return rc;

@@ -45,6 +45,7 @@
 // 6.0 TB/s (417); d_k = d_v = 64, 24576 units of 8 / 16 / 32 nodes: 154 / 212 / 342 us (serial walk 343 / 645 / 1364).
 // What bounds it: the state stream up to 16 nodes (93 % of the copy rate), above that the set-up (a chain of about ten
 // latencies, 6-9 us of a CTA's life) and at 32 nodes the MMAs.  For a few users, 384 chains of 8: 10.4 us.
+#include <algorithm>
 #include <atomic>
 
 #include "speca_common.cuh"
@@ -620,10 +621,27 @@ int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_
 
 // Largest sequence this kernel should verify (0: none).  `most` bounds the nodes of any sequence of the call, `piped`
 // says that one of the pipelined tensor-core kernels takes the shape.
-int direct_limit(const Params &p, int d_k, int most, bool piped)
+int direct_limit(const Params &p, int d_k, int most, bool piped, bool chain)
 {
-    if (d_k == 64) return 64;                                // the alternative is the serial walk
-    if (!piped) return 32;
+    if (!piped) {
+        // The alternative is the serial walk, whose time grows with the nodes where this kernel's hardly does.  A chain needs
+        // no plan there, so short ones stay with it; how short, by the elements of a unit and of the call.  us, serial / this
+        // one: 64 x 64, 16 units of 4 / 5 / 8 nodes 3.6 / 4.1, 4.1 / 4.1, 5.5 / 4.1, 12288 units of 2 / 3 / 4 nodes 55 / 74,
+        // 72 / 74, 88 / 74; 64 x 32, 12288 units of 4 / 6 nodes 47 / 64, 65 / 65; 128 x 64, 12288 units of 1 / 2 nodes 70 / 92,
+        // 102 / 93, 192 units of 3 / 4 nodes 5.0 / 5.2, 5.9 / 5.3; 64 x 512, 1536 units of 1 / 2 nodes 37 / 49, 54 / 50.  Trees
+        // (with their plan): 64 x 32, 1536 units of 3 / 4 nodes 9.9 / 10.3, 11.7 / 10.3; 128 x 512, 1536 units of 1 / 2 nodes
+        // 71 / 76, 106 / 77, 16 units of 1 node 5.0 / 4.7.
+        const long unit = long(p.DV) * d_k, call = unit * p.L * p.B * p.H;
+        const bool large = call >= 8L << 20;
+        int few = int(8191 / unit);
+        if (chain) few = std::min(few + 1 + !large + (call <= 1L << 20), 5);
+        else few = call >= 2L << 20 ? std::max(few, 1) : 0;
+        if ((chain && large ? (p.T + p.B - 1) / p.B : most) <= few) return 0;
+        // In a small call the walk of the largest tree is the whole time: where the mean says that there is one left for it, the
+        // others may as well go along (18 units at 64 x 512, trees of up to 68 nodes 47 us, after a launch of this kernel 57).
+        const int limit = d_k == 64 ? 64 : 32;
+        return p.T > long(limit) * p.B && small_batch(p, sm_count_of_current_device()) ? 0 : limit;
+    }
     // us per unit and SM in a large batch, this kernel / the pipelined one: d_k = 128, d_v = 256: 3.6 / 4.0 at 8 nodes,
     // 4.05 / 4.1 at 16, 6.1 / 5.0 at 20..24; d_k = 256: 8.2 / 6.6 at 8.  A few users, us per call with the plan of the
     // pipelined kernel: d_k = 128, d_v = 128, 384 units of 8 / 16 / 32 nodes 10.7 / 16.0 / 19.5, 22.7 / 21.5 / 22.7;

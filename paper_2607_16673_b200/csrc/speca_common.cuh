@@ -116,7 +116,7 @@ bool factorized_fused_supported(const speca_dims *d);
 int launch_verify_factorized(const Params &p, int d_k, bool fused, bool comp, cudaStream_t st);
 void factorized_set_withhold(int on);
 // small draft trees, state streamed straight into registers: largest sequence it should take, and the launch
-int direct_limit(const Params &p, int d_k, int most, bool piped);
+int direct_limit(const Params &p, int d_k, int most, bool piped, bool chain);
 int launch_verify_direct(const Params &p, int d_k, int most, int limit, cudaStream_t st);
 bool effective_supported(const speca_dims *d);
 int launch_verify_effective(const Params &p, int d_k, cudaStream_t st);

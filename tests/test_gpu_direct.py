@@ -97,3 +97,35 @@ def test_state_base_of_sixteen_byte_alignment():
     dp.S = view
     dp.verify_tree()
     assert dp.status_value() == 0 and rel_err(dp.o.cpu().numpy(), oracle_verify(prob)) <= TOL_FP32
+
+
+@pytest.mark.parametrize("L,B,H,d_k,d_v,n,chain,serial", [
+    (1, 4, 4, 64, 64, 3, True, True),            # a few short chains: the serial walk's work is less than the set-up here
+    (1, 4, 4, 64, 64, 6, True, False),
+    (6, 16, 16, 64, 64, 2, True, True),
+    (6, 16, 16, 64, 64, 8, True, False),
+    (6, 16, 16, 64, 32, 3, False, True),         # trees: only units this small, and the plan must not be the whole time
+    (6, 16, 16, 64, 32, 5, False, False),
+    (1, 2, 4, 64, 32, 1, False, False),
+    (4, 64, 16, 256, 64, 1, False, True)])
+def test_short_drafts_stay_with_the_serial_walk(L, B, H, d_k, d_v, n, chain, serial):
+    parents = [synth.chain_parent(n)] * B
+    prob = synth.make_problem(740 + n, L, H, d_k, d_v, parents, max_depth=8)
+    out = {}
+    for route in (speca.ROUTE_AUTO, speca.ROUTE_SERIAL):
+        dp = DevProblem(prob, route=route, max_nodes=n)
+        dp.verify_chain() if chain else dp.verify_tree()
+        assert dp.status_value() == 0
+        out[route] = dp.o
+    assert torch.equal(out[speca.ROUTE_AUTO], out[speca.ROUTE_SERIAL]) == serial        # bit for bit: the same kernel
+    assert float((out[speca.ROUTE_AUTO] - out[speca.ROUTE_SERIAL]).abs().max()) < 1e-5
+    if L * B * H <= 64:
+        assert rel_err(out[speca.ROUTE_AUTO].cpu().numpy(), oracle_verify(prob)) <= TOL_FP32
+
+
+def test_one_large_tree_among_few_takes_the_others_along():
+    """More nodes than a launch of this kernel could take: every sequence is walked serially, none twice or never."""
+    rng = np.random.default_rng(750)
+    prob = synth.make_problem(751, 1, 2, 64, 64, [tree(n, 8, rng) for n in (150, 9, 64)], max_depth=8)
+    check(prob, 160)
+    check(synth.make_problem(752, 1, 2, 64, 64, [tree(n, 8, rng) for n in (66, 9, 64)], max_depth=8), 160)
