@@ -13,8 +13,8 @@ from gpu_util import DevProblem, TOL, TOL_FP32, oracle_commit, oracle_verify, re
 
 pytestmark = pytest.mark.gpu
 
-# the serial walk, the tensor-core routes with split operands (factorised, effective-query) and the single-pass
-# TF32 route; each is held to its own bar (gpu_util.tol_for)
+# the serial walk, the fp32-grade tensor-core routes (factorised, effective-query: one kernel unless u is asked for, see
+# test_gpu_substitution.py) and the single-pass TF32 route; each is held to its own bar (gpu_util.tol_for)
 ROUTES = [speca.ROUTE_SERIAL, speca.ROUTE_FACTORIZED, speca.ROUTE_EFFECTIVE, speca.ROUTE_TF32]
 
 
@@ -39,7 +39,7 @@ def check_verify(prob, route, chain=False, tol=None, want_u=False, max_nodes=Non
 # configuration 1: tiny chain, also against decode steps
 # ---------------------------------------------------------------------------
 def test_unsupported_shapes_fall_back_or_are_refused():
-    """d_k = 64 is outside the factorised route: AUTO takes the serial route, an explicit request is refused."""
+    """d_k = 64 is outside the factorised route: AUTO takes another kernel, an explicit request is refused."""
     prob = synth.config(1)
     dp, _ = check_verify(prob, speca.ROUTE_AUTO, chain=True, tol=TOL_FP32)
     dp = DevProblem(prob, route=speca.ROUTE_FACTORIZED)
