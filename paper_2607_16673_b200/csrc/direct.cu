@@ -60,13 +60,13 @@ __device__ __forceinline__ uint32_t tf32_head(float x) { return (__float_as_uint
 __device__ __forceinline__ uint32_t tf32_tail(float x) { return __float_as_uint(x - __uint_as_float(tf32_head(x))); }
 
 // (not volatile: the compiler may interleave independent products)
-__device__ __forceinline__ void mma_tf32_sync(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+__device__ __forceinline__ void warp_mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ void mma_bf16_sync(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+__device__ __forceinline__ void warp_mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
                  "{%0, %1, %2, %3};"
@@ -74,7 +74,7 @@ __device__ __forceinline__ void mma_bf16_sync(float (&d)[4], const uint32_t (&a)
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 // the product alone (C = 0)
-__device__ __forceinline__ void mma_bf16_first(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+__device__ __forceinline__ void warp_mma_bf16_first(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
                  "{%10, %10, %10, %10};"
@@ -102,10 +102,6 @@ __device__ __forceinline__ bool finite(float x) { return (__float_as_uint(x) & 0
 __device__ __forceinline__ uint32_t finite_pair(uint32_t w)
 {
     return ((w & 0x7f80u) == 0x7f80u ? 0u : w & 0xffffu) | ((w & 0x7f800000u) == 0x7f800000u ? 0u : w & 0xffff0000u);
-}
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 // 16 bytes global -> shared; live == false fills with zeros (the address is not read)
 __device__ __forceinline__ void cp16(void *dst, const void *src, bool live)
@@ -323,8 +319,8 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
             ldsm_x4(a0, pa + 32 * k);
             ldsm_x4(a1, pa + 32 * k + 16);
             float part0[4], part1[4];
-            mma_bf16_first(part0, a0, bq[0], bq[1]);
-            mma_bf16_first(part1, a1, bq[2], bq[3]);
+            warp_mma_bf16_first(part0, a0, bq[0], bq[1]);
+            warp_mma_bf16_first(part1, a1, bq[2], bq[3]);
 #pragma unroll
             for (int e = 0; e < 4; ++e) { acc[e] += part0[e]; acc1[e] += part1[e]; }
         }
@@ -425,9 +421,9 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                         ldsm_x4(a, sW + pc * LY::WP + LY::w_row(16 * mi + (lane & 15)) + 16 * kk + ((lane >> 4) << 3));
 #pragma unroll
                         for (int c = 0; c < 2; ++c) {
-                            if (pc == 2) mma_bf16_first(lo[c], a, kb[2 * c], kb[2 * c + 1]);
-                            else if (pc == 1) mma_bf16_sync(lo[c], a, kb[2 * c], kb[2 * c + 1]);
-                            else mma_bf16_first(hi[c], a, kb[2 * c], kb[2 * c + 1]);
+                            if (pc == 2) warp_mma_bf16_first(lo[c], a, kb[2 * c], kb[2 * c + 1]);
+                            else if (pc == 1) warp_mma_bf16(lo[c], a, kb[2 * c], kb[2 * c + 1]);
+                            else warp_mma_bf16_first(hi[c], a, kb[2 * c], kb[2 * c + 1]);
                         }
                     }
 #pragma unroll
@@ -494,12 +490,12 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                     for (int e2 = 0; e2 < 2; ++e2) {
                         const float4 bh = *reinterpret_cast<const float4 *>(hi_p + 8 * i * LY::BS + 32 * q + 4 * e2);
                         const float4 bl = *reinterpret_cast<const float4 *>(lo_p + 8 * i * LY::BS + 32 * q + 4 * e2);
-                        mma_tf32_sync(part, ah[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
-                        mma_tf32_sync(xx[i], ah[2 * e2], __float_as_uint(bl.x), __float_as_uint(bl.y));
-                        mma_tf32_sync(part, ah[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
-                        mma_tf32_sync(xx[i], al[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
-                        mma_tf32_sync(xx[i], ah[2 * e2 + 1], __float_as_uint(bl.z), __float_as_uint(bl.w));
-                        mma_tf32_sync(xx[i], al[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
+                        warp_mma_tf32(part, ah[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
+                        warp_mma_tf32(xx[i], ah[2 * e2], __float_as_uint(bl.x), __float_as_uint(bl.y));
+                        warp_mma_tf32(part, ah[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
+                        warp_mma_tf32(xx[i], al[2 * e2], __float_as_uint(bh.x), __float_as_uint(bh.y));
+                        warp_mma_tf32(xx[i], ah[2 * e2 + 1], __float_as_uint(bl.z), __float_as_uint(bl.w));
+                        warp_mma_tf32(xx[i], al[2 * e2 + 1], __float_as_uint(bh.z), __float_as_uint(bh.w));
                     }
 #pragma unroll
                     for (int e = 0; e < 4; ++e) hh[i][e] += part[e];
@@ -522,9 +518,9 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                         for (int pc = 2; pc >= 0; --pc) {
                             const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
                             const uint32_t b0 = *reinterpret_cast<const uint32_t *>(mb), b1 = *reinterpret_cast<const uint32_t *>(mb + 8);
-                            if (pc == 2) mma_bf16_first(lo, a, b0, b1);
-                            else if (pc == 1) mma_bf16_sync(lo, a, b0, b1);
-                            else mma_bf16_first(hi, a, b0, b1);
+                            if (pc == 2) warp_mma_bf16_first(lo, a, b0, b1);
+                            else if (pc == 1) warp_mma_bf16(lo, a, b0, b1);
+                            else warp_mma_bf16_first(hi, a, b0, b1);
                         }
 #pragma unroll
                         for (int e = 0; e < 4; ++e) { hh[i][e] += hi[e]; xx[i][e] += lo[e]; }

@@ -56,6 +56,7 @@
 // Every wait is bounded; on expiry the CTA raises SPECA_STATUS_TIMEOUT, drains and exits.
 #include <cuda.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "speca_common.cuh"
@@ -190,10 +191,6 @@ __device__ __forceinline__ bool next_unit(const Walk &w, VUnit &x)
     return false;
 }
 
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
 // chains into which a Gram block of `npad` columns is split
 __device__ __forceinline__ int gram_parts(int npad) { return npad == 16 ? 4 : npad == 32 ? 2 : 1; }
 // one arrival for the whole warp: every lane's earlier writes are ordered before it
@@ -203,17 +200,6 @@ __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane)
     if (lane == 0) mbar_arrive(bar);
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16])
-{
-    uint32_t x[16];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]),
-                   "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]), "=r"(x[13]), "=r"(x[14]), "=r"(x[15])
-                 : "r"(taddr)
-                 : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) r[i] = __uint_as_float(x[i]);
-}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&x)[16])
 {
     asm volatile(
@@ -875,8 +861,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
 
 template <int N> using Int = std::integral_constant<int, N>;
 
-struct DeviceInfo { int sm_count; bool attr_set; };
-DeviceInfo g_dev[64] = {};
+std::atomic<bool> g_opted_in[64];                        // per device: shared memory of every instantiation
 
 }  // namespace
 
@@ -898,12 +883,8 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     if (encode == nullptr) return int(cudaErrorNotSupported);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return int(cudaErrorInvalidDevice);
-    DeviceInfo &di = g_dev[dev];
-    if (di.sm_count == 0) {
-        int n = 0;
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        di.sm_count = n > 0 ? n : 148;
-    }
+    const long sms = sm_count_of_current_device();
+    if (sms <= 0) return int(cudaErrorInvalidDevice);
     // Few units leave SMs idle, or with one unit while others work on two.  A head of two value tiles then counts as two
     // heads of one tile that share keys, queries and gates: states, value rows and outputs already lie that way.  The
     // coefficients are made twice, and a unit's solve takes as long whatever its value rows, so this pays while every half has an SM
@@ -911,7 +892,7 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     // the busiest SM walks fewer tiles of few (192 units: 27.7, whole 29.7; at 16 levels 35.8 / 33.8).
     Params p = call;
     const int heads = p.H;
-    const long sms = di.sm_count, whole = (long(p.L) * p.B * p.H + sms - 1) / sms, halves = (2L * p.L * p.B * p.H + sms - 1) / sms;
+    const long whole = (long(p.L) * p.B * p.H + sms - 1) / sms, halves = (2L * p.L * p.B * p.H + sms - 1) / sms;
     const int share = p.DV == 2 * kRows && (halves == 1 || (p.max_depth <= 8 && halves < 2 * whole && whole <= 4)) ? 1 : 0;
     p.H <<= share;
     p.DV >>= share;
@@ -949,7 +930,7 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
         }
     }
 
-    if (!di.attr_set) {
+    if (!g_opted_in[dev].load(std::memory_order_acquire)) {
         cudaError_t e = cudaSuccess;
         auto opt_in = [&](const void *k, int bytes) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -969,7 +950,7 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
         all(Int<128>{}, Int<64>{});
         all(Int<256>{}, Int<32>{});
         if (e != cudaSuccess) return int(e);
-        di.attr_set = true;
+        g_opted_in[dev].store(true, std::memory_order_release);
     }
     EParams ep;
     ep.p = p;
@@ -982,7 +963,7 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     // 332 units per CTA 1753 / 1807; 32 ragged ones, 83 units 455 / 439; 16 of 40..64 nodes, 41 units 341 / 323.
     ep.heads_per_group = p.H % 4 == 0 && n_units / 4 >= 32 * sms ? 4 : 1;
     const long n_groups = n_units / ep.heads_per_group;
-    const int grid = int(n_groups < di.sm_count ? n_groups : di.sm_count);
+    const int grid = int(n_groups < sms ? n_groups : sms);
     ep.gpl = p.H / ep.heads_per_group;
     ep.dg = grid % ep.gpl;
     ep.db = grid / ep.gpl % p.B;

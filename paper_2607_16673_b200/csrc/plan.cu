@@ -412,7 +412,7 @@ mask_to_parent_kernel(int32_t N, const uint8_t *mask, const int32_t *node_offset
                       int32_t *__restrict__ parent, int32_t *status)
 {
     after_previous_kernel();
-    extern __shared__ int32_t sm[];                     // [N] ancestors-or-self per node, [N] parent
+    extern __shared__ uint4 mask_smem[];                // the staged mask, then int32: [N] ancestors-or-self per node, [N] parent
     const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int base = node_offsets[b], n = node_offsets[b + 1] - base;
     if (n < 0 || n > N) {
@@ -420,8 +420,9 @@ mask_to_parent_kernel(int32_t N, const uint8_t *mask, const int32_t *node_offset
         return;
     }
     const uint8_t *m = mask + size_t(b) * N * N;
+    int32_t *sm = reinterpret_cast<int32_t *>(mask_smem) + (min(N * N, kMaskStage) + 15) / 16 * 4;
     if (n * N <= kMaskStage) {
-        uint8_t *staged = reinterpret_cast<uint8_t *>(sm + 2 * N + ((2 * N) & 3 ? 4 - ((2 * N) & 3) : 0));
+        uint8_t *staged = reinterpret_cast<uint8_t *>(mask_smem);
         if ((N & 3) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15u) == 0)          // every mask starts on 16 bytes
 #pragma unroll 4
             for (int i = threadIdx.x; i < n * N / 16 + (n * N % 16 != 0); i += 256)
@@ -703,8 +704,8 @@ prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *node_offsets,
 int launch_mask_to_parent(int32_t B, int32_t N, const uint8_t *mask, const int32_t *node_offsets, int32_t *parent,
                           int32_t *status, cudaStream_t st)
 {
-    const size_t stage = size_t(N) * N <= kMaskStage ? size_t(N) * N : kMaskStage;
-    launch(mask_to_parent_kernel, B, 256, size_t(2 * N) * sizeof(int32_t) + 32 + stage, st, N, mask, node_offsets,
+    const size_t stage = (size_t(N) * N <= kMaskStage ? size_t(N) * N + 15 : kMaskStage) / 16 * 16;
+    launch(mask_to_parent_kernel, B, 256, size_t(2 * N) * sizeof(int32_t) + stage, st, N, mask, node_offsets,
            parent, status);
     return int(cudaGetLastError());
 }

@@ -210,11 +210,6 @@ verify_serial_kernel(Params p)
 // once; the second tile is asked into L2 when the first is loaded, so that HBM stays busy while the path is staged and
 // walked.  Paths of three nodes, 12288 units of d_k = 128, d_v = 256: a tile a CTA 562 us = 5.8 TB/s, two 490 us = 6.6
 // TB/s, which is the copy rate; four 568 (fewer CTAs start than end).
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 template <int DK, int RS, int WARPS, int TILES>
 __global__ void __launch_bounds__(WARPS * 32, 2048 / (WARPS * 32) / 2)
 commit_kernel(Params p)

@@ -191,6 +191,12 @@ inline cudaError_t launch(void (*kernel)(P...), unsigned grid, unsigned block, s
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// asks for 16-byte aligned memory into L2; reads nothing into the SM
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // Number of on-chip state slots the light-children-first walk can need for a tree of
 // at most n nodes: a node saves its state only if it has two children with
 // children of their own (subtree >= 5 nodes) and every live slot at least halves
