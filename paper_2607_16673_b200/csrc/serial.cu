@@ -139,7 +139,8 @@ verify_serial_kernel(Params p)
     if (CHAIN) {
         n = p.node_offsets[b + 1] - base;
         int fault = 0;
-        if (base < 0 || n < 0 || base + n > p.T) fault = SPECA_STATUS_BAD_OFFSETS;
+        if (base < 0 || n < 0 || base + n > p.T || (b == p.B - 1 && base + n != p.T) || (b == 0 && base != 0))
+            fault = SPECA_STATUS_BAD_OFFSETS;                 // as the plan kernel and direct.cu see it
         else if (n > p.max_nodes) fault = SPECA_STATUS_TOO_MANY;
         else if (n > p.max_depth) fault = SPECA_STATUS_TOO_DEEP;      // a chain of n nodes is n levels deep, on every route
         if (fault) {

@@ -129,3 +129,20 @@ def test_one_large_tree_among_few_takes_the_others_along():
     prob = synth.make_problem(751, 1, 2, 64, 64, [tree(n, 8, rng) for n in (150, 9, 64)], max_depth=8)
     check(prob, 160)
     check(synth.make_problem(752, 1, 2, 64, 64, [tree(n, 8, rng) for n in (66, 9, 64)], max_depth=8), 160)
+
+
+@pytest.mark.parametrize("route", [speca.ROUTE_SERIAL, speca.ROUTE_AUTO])
+@pytest.mark.parametrize("n,bad", [(2, 0), (2, 3), (8, 0), (8, 3)])
+def test_offsets_that_miss_the_ends_are_a_fault_on_every_route(n, bad, route):
+    """Offsets that do not start at 0 or do not end at the number of nodes: the first or last chain is skipped, whichever
+    kernel verifies the call (two nodes: the serial walk, eight: this one)."""
+    prob = synth.make_problem(760 + n, 1, 4, 64, 64, [synth.chain_parent(n)] * 3)
+    good = oracle_verify(prob)
+    dp = DevProblem(prob, route=route, max_nodes=n)
+    dp.node_offsets[bad] += 1 if bad == 0 else -1
+    dp.verify_chain()
+    assert dp.status_value() == speca.STATUS_BAD_OFFSETS
+    skipped = slice(0, n) if bad == 0 else slice(2 * n, 3 * n)
+    o = dp.o.cpu().numpy()
+    assert np.isnan(o[:, skipped]).all()
+    assert rel_err(np.delete(o, np.r_[skipped], 1), np.delete(good, np.r_[skipped], 1)) <= TOL_FP32
