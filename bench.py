@@ -449,7 +449,7 @@ def run_speca(args):
                    "d_k": dk, "d_v": dv, "nodes_per_step_per_gpu": [p["T"] for p in pool],
                    "mean_accepted_len": float(np.mean([p["path_len"].mean() for p in pool])),
                    "input_pool": POOL, "l2": f"inputs larger than L2 (state {L * B * H * dk * dv * 4 / 1e9:.1f} GB)",
-                   "route": {0: "auto: tensor-core route with split operands (fp32-grade)", 1: "serial", 2: "factorised, split operands",
+                   "route": {0: "auto: tensor-core route, state in exact bf16 or TF32 pieces (fp32-grade)", 1: "serial", 2: "factorised, split operands",
                              3: "single-pass TF32", 4: "effective-query"}.get(args.route, str(args.route)),
                    "parallelism": f"dp{world} (sequences partitioned, no collective)"},
         "roofline": {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
@@ -986,7 +986,7 @@ def run_small(args):
 
 
 # ---------------------------------------------------------------------------
-# sweeps behind the figures in the design doc
+# sweeps: commit by path length, verification by unit type, waits of the kernel roles
 # ---------------------------------------------------------------------------
 def run_sweep(args):
     import torch

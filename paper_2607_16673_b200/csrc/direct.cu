@@ -41,10 +41,10 @@
 // over 16-row tiles needs two 32-column steps of registers in flight, not whole tiles: 24 warps fit an SM.  Holding
 // whole tiles in registers through the set-up (16 warps) took 5.1 us per 8-node unit and SM instead of 3.9, at 16
 // nodes 8.0 instead of 4.4.
-// Measured (d_k = 128, d_v = 256, 12288 units): 8 nodes 301 us = 6.0 TB/s (pipelined kernel 411 us), 16 nodes 337 us =
-// 6.0 TB/s (417); d_k = d_v = 64, 24576 units of 8 / 16 / 32 nodes: 154 / 212 / 342 us (serial walk 343 / 645 / 1364).
-// What bounds it: the state stream up to 16 nodes (93 % of the copy rate), above that the set-up (a chain of about ten
-// latencies, 6-9 us of a CTA's life) and at 32 nodes the MMAs.  For a few users, 384 chains of 8: 10.4 us.
+// Measured (d_k = 128, d_v = 256, 12288 units, the pipelined kernel with its plan in brackets): 8 nodes 298 us = 6.1 TB/s
+// (344 us), 16 nodes 369 us = 5.5 TB/s (377); d_k = d_v = 64, 24576 units of 8 / 30 nodes: 148 / 335 us (serial walk 316 /
+// 1244).  What bounds it: the state stream at 8 nodes (93 % of the copy rate; 83 % at 16), above that the set-up (a chain of
+// about ten latencies, 6-9 us of a CTA's life) and at 32 nodes the MMAs.  For a few users, 384 chains of 8: 8.8 us.
 #include <algorithm>
 #include <atomic>
 
@@ -638,10 +638,11 @@ int direct_limit(const Params &p, int d_k, int most, bool piped, bool chain)
         const int limit = d_k == 64 ? 64 : 32;
         return p.T > long(limit) * p.B && small_batch(p, sm_count_of_current_device()) ? 0 : limit;
     }
-    // us per unit and SM in a large batch, this kernel / the pipelined one: d_k = 128, d_v = 256: 3.6 / 4.0 at 8 nodes,
-    // 4.05 / 4.1 at 16, 6.1 / 5.0 at 20..24; d_k = 256: 8.2 / 6.6 at 8.  A few users, us per call with the plan of the
-    // pipelined kernel: d_k = 128, d_v = 128, 384 units of 8 / 16 / 32 nodes 10.7 / 16.0 / 19.5, 22.7 / 21.5 / 22.7;
-    // d_k = 256, 384 units of 8 nodes 30 / 37, 192 units of 16 nodes 25.4 / 24.7.
+    // us per unit and SM in a large batch, this kernel / the pipelined one with its plan: d_k = 128, d_v = 256: 3.6 / 4.1 at 8
+    // nodes, 4.2 / 4.5 at 12, 4.4 / 4.5 at 16, d_v = 128: 2.1 / 3.6 at 8, 2.5 / 3.5 at 16.  Above that its set-up is the longer
+    // one (6.1 / 5.0 at 20..24 nodes; 8.2 / 6.6 at d_k = 256, 8 nodes; both kernels before their large sums were taken apart,
+    // which costs either 2 to 6 %).  A few users, us per call: d_k = 128, d_v = 128, 384 units of 8 / 16 / 32 nodes 8.8 / 15.8,
+    // 14.8 / 15.4, 16.5 / 16.6; d_k = 256, 8 nodes, 192 units 14.2 / 16.8, 384 units 26.4 / 26.4.
     const bool few = small_batch(p, sm_count_of_current_device());
     const int cap = d_k == 128 ? (few ? 32 : 16) : (few ? 8 : 0);
     return most <= cap ? cap : 0;

@@ -42,11 +42,12 @@
 //   warps 20-23   solver, one unit ahead: Gram entries of every row against its own path, back substitution (a thread
 //                 per node, registers), the pieces of M
 // TMEM: two tiles of accumulators (R | G, 128 columns; x M^T overwrites R), two A buffers of 48, x of 96, Gram of 64.
-// Measured in large batches, us per unit and SM (share of the copy rate): d_k = 128, d_v = 256: 8 nodes 4.0 (85 %), 16
-// nodes 4.1 (92 %), 32 nodes 5.3 (85 %), 64 nodes 7.2 (83 %), 64 nodes at 16 levels 8.2; d_k = d_v = 256: 8 nodes 6.6
-// (97 %), 32 nodes 8.1 (97 %).  One split group instead of two: 4.75, 4.8, 5.1, 7.4, 7.9; 8.9, 9.4: a group needs
-// about 750 cycles a slice, the tensor core 280.  What bounds it: HBM at d_k = 256; at d_k = 128 the solver and the epilogue of
-// a unit, which come round twice as often.
+// Measured in large batches, us per unit and SM (share of the copy rate): d_k = 128, d_v = 256: 8 nodes 4.1 (81 %), 16
+// nodes 4.5 (82 %), 32 nodes 5.3 (84 %), 64 nodes 7.8 (76 %), 64 nodes at 16 levels 9.2; d_k = d_v = 256: 8 nodes 7.0
+// (91 %), 32 nodes 8.55 (91 %).  One split group instead of two, before the chains of the Gram blocks: 4.75, 4.8, 5.1, 7.4, 7.9
+// against 4.0, 4.1, 5.3, 7.2, 8.2: a group needs about 750 cycles a slice, the tensor core 280.  What bounds it: HBM at d_k =
+// 256; at d_k = 128 the solver, which never waits for anybody but its own four warps (30 to 40 % of its time reads Gram
+// entries out of TMEM), and next to it the epilogue.
 // Ten roles take turns on four issue slots, so the kernel's size matters as much as its instruction count: loops stay
 // rolled where a role has slack.
 // x M^T runs over all nodes with zeros in M off the path, and zero times a value that is not finite is no zero: where an
@@ -959,8 +960,10 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     ep.share = share;
     // Consecutive heads of one (layer, sequence) that a CTA takes together.  The next head of a group costs a role two
     // additions, the next group some hundred cycles of a chain that short units wait for; but whole groups leave some CTAs
-    // longer lists than others.  Verification in us with groups of 4 / single heads: 128 sequences, half 64-node trees,
-    // 332 units per CTA 1753 / 1807; 32 ragged ones, 83 units 455 / 439; 16 of 40..64 nodes, 41 units 341 / 323.
+    // longer lists than others.  Groups of 4 against single heads, by units per SM: ragged trees of 8..64 nodes +2.6 % at 83,
+    // +1.3 % at 125, +1.7 % at 145, +3.4 % at 166, +1.5 % at 332; trees of 64 nodes 0 at 166, of 32 at d_v = 128 -6.6 % at 166,
+    // ragged at d_v = 128 -2.7 % at 249, chains of 8 -3.5 % at 332, half chains and half 64-node trees -3 % at 332.  The line at
+    // 128 lies where what is lost on ragged trees is less than what short units gain.
     ep.heads_per_group = p.H % 4 == 0 && n_units / 4 >= 32 * sms ? 4 : 1;
     const long n_groups = n_units / ep.heads_per_group;
     const int grid = int(n_groups < sms ? n_groups : sms);
