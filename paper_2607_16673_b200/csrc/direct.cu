@@ -596,7 +596,7 @@ int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
 template <int DK, int MAXD>
 int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_t st)
 {
-    constexpr int C1 = DK == 64 && MAXD == 8 ? 6 : MAXD == 8 && DK == 128 ? 6 : 5, C2 = DK == 64 || MAXD == 8 ? 5 : 4;
+    constexpr int C1 = DK == 128 && MAXD == 8 ? 6 : 5, C2 = DK == 64 || MAXD == 8 ? 5 : 4;
     if (hi <= 8) return launch_one<DK, 1, MAXD, 4, C1>(p, lo, all, sms, st);
     if (hi <= 16) return launch_one<DK, 2, MAXD, 4, C2>(p, lo, all, sms, st);
     if constexpr (DK == 64) {
@@ -628,11 +628,11 @@ int direct_limit(const Params &p, int d_k, int most, bool piped, bool chain)
         // (with their plan): 64 x 32, 1536 units of 3 / 4 nodes 9.9 / 10.3, 11.7 / 10.3; 128 x 512, 1536 units of 1 / 2 nodes
         // 71 / 76, 106 / 77, 16 units of 1 node 5.0 / 4.7.
         const long unit = long(p.DV) * d_k, call = unit * p.L * p.B * p.H;
-        const bool large = call >= 8L << 20;
-        int few = int(8191 / unit);
-        if (chain) few = std::min(few + 1 + !large + (call <= 1L << 20), 5);
-        else few = call >= 2L << 20 ? std::max(few, 1) : 0;
-        if ((chain && large ? (p.T + p.B - 1) / p.B : most) <= few) return 0;
+        const int small_unit = int((d_k == 128 || !chain ? 8191 : 8192) / unit);
+        const int few = chain ? std::min(1 + small_unit + (call < 8L << 20) + (call <= 1L << 20), 5)
+                              : call >= 2L << 20 ? std::max(small_unit, 1) : 0;
+        // many chains take the time of the mean one, a few that of the longest
+        if (chain && call >= 2L << 20 ? p.T <= long(few) * p.B : most <= few) return 0;
         // In a small call the walk of the largest tree is the whole time: where the mean says that there is one left for it, the
         // others may as well go along (18 units at 64 x 512, trees of up to 68 nodes 47 us, after a launch of this kernel 57).
         const int limit = d_k == 64 ? 64 : 32;
