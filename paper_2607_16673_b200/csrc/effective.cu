@@ -35,7 +35,8 @@
 //   warp 0        TMA producer of the state slices (128 rows x 32 columns, 128-byte swizzle)
 //   warp 1        issues S0 [K;Q]^T; owns TMEM
 //   warp 2        issues the Gram blocks [K;Q] K^T (one unit ahead) and x M^T
-//   warp 3        TMA producer of the staged [K;Q] rows (two units) and the value rows (two tiles)
+//   warp 3        walks the list of units and hands records of them to the others; TMA producer of the staged [K;Q] rows
+//                 (two units) and the value rows (two tiles)
 //   warps 4-11    split: slice row per thread -> three bf16 pieces in TMEM; two groups alternate slices, a buffer each
 //   warps 12-19   epilogue, two warps per TMEM lane quarter that share a tile's columns: R out of TMEM, x back into TMEM
 //                 as three pieces; then, while the next tile's product runs, o = scale gamma G + (x M^T), coalesced
@@ -73,6 +74,9 @@ constexpr int kRows = 128;                      // value rows per tile (= TMEM l
 constexpr int kSliceBytes = kRows * 128;        // one ring slot: a K-slice of a tile (128 rows x 32 fp32)
 constexpr int kThreads = 24 * 32;
 constexpr int kWalkSeqs = 128;
+// Records of units.  The walk is one unit ahead of the staged rows, which are two ahead of the state product, and the value
+// rows keep it within two tiles of the epilogue: no role is five units behind it.
+constexpr int kUnitRing = 8;
 // TMEM columns
 constexpr int kTileCols = 128;                  // accumulators of a tile: R, then G
 constexpr int kAOff = 2 * kTileCols, kACols = 48;    // two buffers of three 16-column pieces (32 bf16 columns each)
@@ -97,7 +101,8 @@ template <int DK, int MAXN_, int MAXD> struct Lay {
     static constexpr int OffM = OffStage + 2 * STAGE;
     static constexpr int OffV = OffM + (MAXN > 32 ? 3 : 6) * MPIECE;     // two tiles
     static constexpr int OffRing = OffV + 2 * VBUF;
-    static constexpr int kSmall = 2 * MAXN * GSTR * 4 + 2 * 2 * MAXN * 4 + 2 * MAXN + 4 * 2 * MAXN * 4 + 5 * kWalkSeqs + 16 + 8 * 64;
+    static constexpr int kSmall = 2 * MAXN * GSTR * 4 + 2 * 2 * MAXN * 4 + 2 * MAXN + 4 * 2 * MAXN * 4 + 5 * kWalkSeqs + 32 * kUnitRing +
+                                  16 + 8 * 64;
     static constexpr int kRoom = (227 * 1024 - OffRing - kSmall) / kSliceBytes;
     static constexpr int NS = kRoom > 8 ? 8 : kRoom & ~1;       // ring depth: even, so that a slot is always the same split group's
     static constexpr int OffGk = OffRing + NS * kSliceBytes;    // [MAXN][GSTR] k_node . k_(ancestor at distance i + 1)
@@ -106,7 +111,8 @@ template <int DK, int MAXN_, int MAXD> struct Lay {
     static constexpr int OffGam = OffAB + 2 * 2 * MAXN * 4;     // four units of float gamma in x, factor of G [MAXN]
     static constexpr int OffDepth = OffGam + 4 * 2 * MAXN * 4;  // two units of uint8 [MAXN]
     static constexpr int OffWalk = OffDepth + 2 * MAXN;
-    static constexpr int OffMisc = OffWalk + 5 * kWalkSeqs;     // abort flag, TMEM base
+    static constexpr int OffUnit = OffWalk + 5 * kWalkSeqs;     // records of units, 32 bytes each
+    static constexpr int OffMisc = OffUnit + 32 * kUnitRing;    // abort flag, TMEM base
     static constexpr int OffBars = OffMisc + 16;
     static constexpr int Bytes = OffBars + 8 * 64;
     static_assert(Bytes - OffGk == kSmall, "small regions");
@@ -134,7 +140,8 @@ enum Bar {
     kMReady = kGamReady + 2,           // [2] solver -> MMA: M of a unit
     kMFree = kMReady + 2,              // [2] MMA -> solver
     kSync = kMFree + 2,                // solver, role-internal
-    kDrain,
+    kUnit,                             // [8] walk -> all: record of a unit
+    kDrain = kUnit + 8,
     kBarCount
 };
 static_assert(kBarCount <= 64, "barrier region too small");
@@ -152,44 +159,39 @@ struct EParams {
 
 // A unit is one (layer, sequence, head); with u requested it is walked twice (kind 0: o rows, kind 1: u rows).
 // Units are taken in groups of HG consecutive heads of one (layer, sequence): group blockIdx.x, += gridDim.x, kept as
-// (layer, sequence, group of heads) and advanced by carries, not divisions: every role walks the list by itself, so
-// this code is there ten times.
-struct VUnit {
-    int l, b, h, u, n, npad, base, kind, hi;
-    int nl, nb, ng;                                              // the group after this one
-};
+// (layer, sequence, group of heads) and advanced by carries, not divisions.  One warp walks the list and hands a record of
+// every unit to the others through a ring in shared memory.  With the walk in every role, 24 warps spent some fifty
+// instructions a unit on it, and the registers of its state (us per unit and SM, walk in every role / records: d_k = 128, d_v =
+// 256, 20 nodes 4.66 / 4.51, 32 nodes 5.00 / 4.76, 64 nodes 7.52 / 7.41, 64 and 24 nodes at 16 levels 8.24 / 7.80 and 6.29 /
+// 5.35; d_v = 128, 32 nodes 3.96 / 3.27; d_k = 256, 24 nodes 8.07 / 7.74).
+struct Unit { int u, n, z, h, base, kind; };                     // z: layer's first record + base; n = 0: the list has ended
 struct Walk {
-    int HG, gpl, L, B, H, dl, db, dg, two;                       // d*: a step of gridDim.x groups
+    int HG, gpl, L, B, H, T, dl, db, dg, two;                    // d*: a step of gridDim.x groups
     const int32_t *seq_n; const int32_t *offs;
     const uint8_t *tab;
+    int hi, nl, nb, ng;                                          // head of the group; the group after this one
 };
 
-__device__ __forceinline__ bool next_unit(const Walk &w, VUnit &x)
+__device__ __forceinline__ void next_unit(Walk &w, Unit &x)
 {
-    if (w.two && x.kind == 0) { x.kind = 1; return true; }
+    if (w.two && x.kind == 0) { x.kind = 1; return; }
     x.kind = 0;
-    if (++x.hi < w.HG) { ++x.h; ++x.u; return true; }
-    while (x.nl < w.L) {
-        x.l = x.nl; x.b = x.nb;
-        const int g = x.ng;
-        x.ng += w.dg; x.nb += w.db; x.nl += w.dl;
-        if (x.ng >= w.gpl) { x.ng -= w.gpl; ++x.nb; }
-        if (x.nb >= w.B) { x.nb -= w.B; ++x.nl; }
-        const bool in_tab = x.b < kWalkSeqs;
-        x.n = in_tab ? int(reinterpret_cast<const int8_t *>(w.tab + 4 * kWalkSeqs)[x.b]) : w.seq_n[x.b];
-        if (x.n > 0) {
-            x.hi = 0;
-            x.h = g * w.HG;
-            x.u = (x.l * w.B + x.b) * w.H + x.h;
-            x.npad = (x.n + 15) & ~15;
-            x.base = in_tab ? reinterpret_cast<const int32_t *>(w.tab)[x.b] : w.offs[x.b];
-            return true;
-        }
-    }
+    if (++w.hi < w.HG) { ++x.h; ++x.u; return; }
     x.n = 0;
-    x.hi = w.HG;
-    x.kind = 1;
-    return false;
+    while (w.nl < w.L && x.n <= 0) {
+        const int l = w.nl, b = w.nb, g = w.ng;
+        w.ng += w.dg; w.nb += w.db; w.nl += w.dl;
+        if (w.ng >= w.gpl) { w.ng -= w.gpl; ++w.nb; }
+        if (w.nb >= w.B) { w.nb -= w.B; ++w.nl; }
+        const bool in_tab = b < kWalkSeqs;
+        x.n = in_tab ? int(reinterpret_cast<const int8_t *>(w.tab + 4 * kWalkSeqs)[b]) : w.seq_n[b];
+        w.hi = 0;
+        x.h = g * w.HG;
+        x.u = (l * w.B + b) * w.H + x.h;
+        x.base = in_tab ? reinterpret_cast<const int32_t *>(w.tab)[b] : w.offs[b];
+        x.z = l * w.T + x.base;
+    }
+    if (x.n < 0) x.n = 0;
 }
 
 // chains into which a Gram block of `npad` columns is split
@@ -325,6 +327,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         mbar_init(bar(kGramFree), 4);
         mbar_init(bar(kSync), 4);
         mbar_init(bar(kDrain), 2);
+#pragma unroll 1
+        for (int i = 0; i < kUnitRing; ++i) mbar_init(bar(kUnit + i), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if constexpr (FEW) {
@@ -345,18 +349,19 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    Walk walk;
-    walk.HG = ep.heads_per_group; walk.gpl = ep.gpl;
-    walk.L = p.L; walk.B = p.B; walk.H = p.H;
-    walk.dl = ep.dl; walk.db = ep.db; walk.dg = ep.dg;
-    walk.two = ep.want_u;
-    walk.seq_n = p.ws.seq_n; walk.offs = p.node_offsets;
-    walk.tab = smem + LY::OffWalk;
-    VUnit x;                                                     // before the first unit
-    x.kind = 1; x.hi = walk.HG; x.n = 0;
-    x.ng = int(blockIdx.x) % ep.gpl; x.nb = int(blockIdx.x) / ep.gpl % p.B; x.nl = int(blockIdx.x) / ep.gpl / p.B;
+    // record of unit `s` of this CTA's list; false: the list has ended, or (ok == false) the CTA is aborting
     bool ok = true;
-    auto head_of = [&](const VUnit &y) { return FEW ? y.h >> ep.share : y.h; };
+    Unit x;
+    auto unit = [&](uint32_t s, Unit &y) -> bool {
+        if (!(ok = wait_fast(bar(kUnit + (s % kUnitRing)), (s / kUnitRing) & 1, abort_flag))) return false;
+        const int4 *rec = reinterpret_cast<const int4 *>(smem + LY::OffUnit) + 2 * (s % kUnitRing);
+        const int4 r = rec[0];
+        const int2 e = *reinterpret_cast<const int2 *>(rec + 1);
+        y = Unit{r.x, r.y, r.z, r.w, e.x, e.y};
+        return r.y > 0;
+    };
+    auto padded = [](const Unit &y) { return (y.n + 15) & ~15; };
+    auto head_of = [&](const Unit &y) { return FEW ? y.h >> ep.share : y.h; };
 
     const uint32_t lead = elect_one();                           // the thread that issues this warp's tcgen05 instructions
 
@@ -364,7 +369,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         // ------------------------------------------------------------- TMA producer: state slices
         uint32_t it = 0;
         PROF_DECL
-        while (ok && next_unit(walk, x)) {
+        for (uint32_t useq = 0; ok && unit(useq, x); ++useq) {
 #pragma unroll 1
             for (int e = 0; e < TP * NC; ++e, ++it) {
                 const int s = it % NS;
@@ -381,9 +386,9 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         // ------------------------------------------------------------- MMA issuer: S0 [K;Q]^T
         uint32_t it = 0, q = 0, useq = 0;                        // slices, tiles, units
         PROF_DECL
-        for (; ok && next_unit(walk, x); ++useq) {
+        for (; ok && unit(useq, x); ++useq) {
             const int par = useq & 1;
-            const uint32_t idm = make_idesc_bf16(2 * x.npad);
+            const uint32_t idm = make_idesc_bf16(2 * padded(x));
             const uint32_t stage = sbase + LY::OffStage + par * LY::STAGE;
             if (!(ok = WAIT(0, bar(kKQFull + par), (useq >> 1) & 1))) break;
 #pragma unroll 1
@@ -414,21 +419,20 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
     } else if (warp == 2) {
         // ------------------------------------------------------------- MMA issuer: Gram blocks one unit ahead, x M^T
         uint32_t q = 0, useq = 0, gseq = 0;
-        VUnit gx = x;
         PROF_DECL
         // pass s issues the Gram block of unit s, [K;Q] (128 rows) x K^T (R columns) from the staged rows, and the
         // products of unit s - 1
         for (bool first = true; ok; first = false) {
-            if (next_unit(walk, gx)) {
-                const int par = gseq & 1;
+            if (unit(gseq, x)) {
+                const int par = gseq & 1, npad = padded(x);
                 if (!(ok = WAIT(0, bar(kKQFull + par), (gseq >> 1) & 1))) break;
                 if (!(ok = WAIT(1, bar(kGramFree), (gseq & 1) ^ 1))) break;
                 tc_fence_after();
-                const uint32_t idg = make_idesc_bf16(gx.npad);
+                const uint32_t idg = make_idesc_bf16(npad);
                 // in as many chains as the 64 columns hold, each from zero: the solver adds them up
-                const int run = 4 * SC / gram_parts(gx.npad);
+                const int run = 4 * SC / gram_parts(npad);
 #pragma unroll 1
-                for (int i = 0, col = kGramOff; i < 4 * SC; i += run, col += gx.npad)
+                for (int i = 0, col = kGramOff; i < 4 * SC; i += run, col += npad)
 #pragma unroll 1
                     for (int k = i; k < i + run; k += 2) {
                         const uint64_t d = make_desc(sbase + LY::OffStage + par * LY::STAGE + (k >> 2) * SCB + (k & 2) * 32);
@@ -440,10 +444,11 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 ++gseq;
             }
             if (first) continue;
-            if (!next_unit(walk, x)) break;
-            const bool small = x.npad <= 32;
-            const int ksteps = x.npad >> 4, mbuf = useq & 1;
-            const uint32_t idx = make_idesc_bf16(x.npad);
+            if (!ok || !unit(useq, x)) break;
+            const int npad = padded(x);
+            const bool small = npad <= 32;
+            const int ksteps = npad >> 4, mbuf = useq & 1;
+            const uint32_t idx = make_idesc_bf16(npad);
             if (!(ok = WAIT(2, bar(kMReady + mbuf), (useq >> 1) & 1))) break;
 #pragma unroll 1
             for (int t = 0; t < TP; ++t, ++q) {
@@ -467,35 +472,61 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         PROF_STORE()
     } else if (warp == 3) {
         // ------------------------------------------------------------- TMA producer: staged [K;Q] rows, value rows
-        uint32_t kseq = 0, q = 0;
-        VUnit kx = x;
+        // (and the walk: unit s + 1 is handed out before the rows of unit s are asked for)
+        Walk walk;
+        walk.HG = ep.heads_per_group; walk.gpl = ep.gpl;
+        walk.L = p.L; walk.B = p.B; walk.H = p.H; walk.T = p.T;
+        walk.dl = ep.dl; walk.db = ep.db; walk.dg = ep.dg;
+        walk.two = ep.want_u;
+        walk.seq_n = p.ws.seq_n; walk.offs = p.node_offsets;
+        walk.tab = smem + LY::OffWalk;
+        walk.hi = walk.HG;                                       // before the first unit
+        walk.ng = int(blockIdx.x) % ep.gpl; walk.nb = int(blockIdx.x) / ep.gpl % p.B; walk.nl = int(blockIdx.x) / ep.gpl / p.B;
+        Unit kx, ux;
+        ux.kind = 1;
+        uint32_t kseq = 0, q = 0, pub = 0, useq = 0;
+        auto publish = [&]() {
+            next_unit(walk, ux);
+            if (lane == 0) {
+                int4 *rec = reinterpret_cast<int4 *>(smem + LY::OffUnit) + 2 * (pub % kUnitRing);
+                rec[0] = make_int4(ux.u, ux.n, ux.z, ux.h);
+                rec[1] = make_int4(ux.base, ux.kind, 0, 0);
+                mbar_arrive(bar(kUnit + (pub % kUnitRing)));
+            }
+            __syncwarp();
+            ++pub;
+        };
         PROF_DECL
+        publish();
+        kx = ux;
         for (bool first = true; ok; first = false) {             // staged rows one unit ahead of the value rows
-            if (next_unit(walk, kx)) {
-                const int par = kseq & 1;
+            if (kx.n > 0) {
+                publish();
+                const int par = kseq & 1, npad = padded(kx);
                 if (!(ok = WAIT(0, bar(kKQFree + par), ((kseq >> 1) & 1) ^ 1))) break;
                 if (lane == 0) {
-                    const int m = (kx.npad >> 4) - 1, z = kx.l * p.T + kx.base;
+                    const int m = (npad >> 4) - 1, z = kx.z;
                     const uint32_t stage = sbase + LY::OffStage + par * LY::STAGE;
-                    mbar_arrive_expect_tx(bar(kKQFull + par), uint32_t(4 * kx.npad * DK));
+                    mbar_arrive_expect_tx(bar(kKQFull + par), uint32_t(4 * npad * DK));
 #pragma unroll 1
                     for (int c = 0; c < SC; ++c) {
                         tma_load_3d(stage + c * SCB, &maps.k[m], c * 64, head_of(kx), z, bar(kKQFull + par));
-                        tma_load_3d(stage + c * SCB + kx.npad * 128, &maps.q[m], c * 64, head_of(kx), z, bar(kKQFull + par));
+                        tma_load_3d(stage + c * SCB + npad * 128, &maps.q[m], c * 64, head_of(kx), z, bar(kKQFull + par));
                     }
                 }
                 __syncwarp();
                 ++kseq;
+                kx = ux;
             }
             if (first) continue;
-            if (!next_unit(walk, x)) break;
+            if (!unit(useq++, x)) break;
 #pragma unroll 1
             for (int t = 0; t < TP; ++t, ++q) {
                 const int vb = q & 1;
                 if (!(ok = WAIT(1, bar(kVFree + vb), ((q >> 1) & 1) ^ 1))) break;
                 if (lane == 0) {
-                    mbar_arrive_expect_tx(bar(kVFull + vb), uint32_t(x.npad * kRows * 2));
-                    tma_load_3d(sbase + LY::OffV + vb * LY::VBUF, &maps.v[(x.npad >> 4) - 1], t * kRows, x.h, x.l * p.T + x.base,
+                    mbar_arrive_expect_tx(bar(kVFull + vb), uint32_t(padded(x) * kRows * 2));
+                    tma_load_3d(sbase + LY::OffV + vb * LY::VBUF, &maps.v[(padded(x) >> 4) - 1], t * kRows, x.h, x.z,
                                 bar(kVFull + vb));
                 }
                 __syncwarp();
@@ -509,7 +540,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         const uint32_t abase = tmem_base + kAOff + (uint32_t(32 * (warp & 3)) << 16);
         uint32_t it = 0;
         PROF_DECL
-        while (ok && next_unit(walk, x)) {
+        for (uint32_t useq = 0; ok && unit(useq, x); ++useq) {
 #pragma unroll 1
             for (int e = 0; e < TP * NC; ++e, ++it) {
                 const int s = it % NS, ab = it & 1;
@@ -550,7 +581,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         const uint32_t xb = tmem_base + kXOff + lane_addr;
         const size_t stride = size_t(p.H) * p.DV;
         uint32_t q = 0, useq = 0xffffffffu;
-        int t = TP - 1, pn = 0, pR = 0;                          // tile of the unit; nodes and rows of the last tile's unit (0: none)
+        int t = TP - 1, npad = 0, pn = 0, pR = 0;                // tile of the unit; nodes and rows of the last tile's unit (0: none)
         const float *pgf = nullptr;
         float *pdst = nullptr;
         bool more = true;
@@ -559,9 +590,10 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             if (more && ++t == TP) {
                 t = 0;
                 ++useq;
-                more = next_unit(walk, x);
+                more = unit(useq, x);
+                npad = padded(x);
             }
-            if (pn == 0 && !more) break;
+            if (!ok || (pn == 0 && !more)) break;
             const uint32_t slot = q & 1, ps = slot ^ 1;
             if (pn > 0 && !(ok = WAIT(4, bar(kOutFull + ps), ((q - 1) >> 1) & 1))) break;
             const float *gx = reinterpret_cast<const float *>(smem + LY::OffGam) + (useq & 3) * 2 * MAXN;
@@ -628,13 +660,13 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 float2 zero = make_float2(0.f, 0.f);
                 uint32_t none = 0u;
 #pragma unroll 1
-                for (int c0 = 8 * grp; c0 < x.npad; c0 += 16) make_x(c0, false, zero, none);
+                for (int c0 = 8 * grp; c0 < npad; c0 += 16) make_x(c0, false, zero, none);
                 if (__any_sync(0xffffffffu, !(zero.x + zero.y == 0.f))) {
                     // Both warps of the lane quarter may come here: each looks at all nodes, so that both write the same G.
                     // (R stays until all epilogue warps have arrived below.)
                     uint32_t odd_lo = 0u, odd_hi = 0u;
 #pragma unroll 1
-                    for (int c0 = 0; c0 < x.npad; c0 += 8) {
+                    for (int c0 = 0; c0 < npad; c0 += 8) {
                         uint32_t odd = 0u;
                         make_x(c0, true, zero, odd);
                         if (c0 < 32) odd_lo |= odd << c0;
@@ -643,8 +675,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
 #pragma unroll 1
                     for (int i = 0; i < x.n; ++i) {
                         const int2 set = reinterpret_cast<const int2 *>(p.ws.set)[x.base + i];
-                        const float g = tmem_ld1(acc + x.npad + i);
-                        tmem_st1(acc + x.npad + i, ((uint32_t(set.x) & odd_lo) | (uint32_t(set.y) & odd_hi)) != 0u ? NAN : g);
+                        const float g = tmem_ld1(acc + npad + i);
+                        tmem_st1(acc + npad + i, ((uint32_t(set.x) & odd_lo) | (uint32_t(set.y) & odd_hi)) != 0u ? NAN : g);
                     }
                 }
                 tmem_st_wait();
@@ -655,9 +687,9 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             }
             pn = 0;
             if (more) {
-                pn = x.n; pR = x.npad;
+                pn = x.n; pR = npad;
                 pgf = gx + MAXN;
-                pdst = (x.kind == 0 ? p.o : p.u) + size_t((x.l * p.T + x.base) * p.H + x.h) * p.DV + t * kRows + row;
+                pdst = (x.kind == 0 ? p.o : p.u) + size_t(x.z * p.H + x.h) * p.DV + t * kRows + row;
             }
             ++q;
         }
@@ -682,8 +714,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         uint32_t up_n[4] = {0u, 0u, 0u, 0u}, lo_n = 0u, hi_n = 0u;
         int d_n = 0;
         float alpha_n = 1.f, beta_n = 0.f;
-        auto fetch_topo = [&](const VUnit &y) {
-            const int node = grow < y.npad ? grow : grow - y.npad;
+        auto fetch_topo = [&](const Unit &y) {
+            const int node = grow < padded(y) ? grow : grow - padded(y);
             d_n = 0;
             if (node < y.n) {
                 const int i = y.base + node;
@@ -697,17 +729,17 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 const int2 s = reinterpret_cast<const int2 *>(p.ws.set)[i];
                 lo_n = uint32_t(s.x); hi_n = uint32_t(s.y);
                 d_n = p.ws.depth[i];
-                const int r = FEW ? ((y.l * p.T + i) * p.H + y.h) >> ep.share : (y.l * p.T + i) * p.H + y.h;
+                const int r = FEW ? ((y.z + node) * p.H + y.h) >> ep.share : (y.z + node) * p.H + y.h;
                 alpha_n = p.alpha[r];
                 beta_n = p.beta[r];
             }
         };
-        VUnit nx = x;
-        bool have = next_unit(walk, nx);
+        Unit nx;
+        bool have = unit(0, nx);
         if (have) fetch_topo(nx);
         for (; have && ok; ++useq) {
             x = nx;
-            const int R = x.npad;
+            const int R = padded(x);
             const bool is_k = grow < R, small = R <= 32;
             const int node = is_k ? grow : grow - R;
             const int d = grow < 2 * R ? d_n : 0;                // zero: a row without a node
@@ -726,7 +758,8 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                 else set_hi &= ~(1u << (node & 31));
             }
             auto path = [&](int r) -> int { return int((up[r >> 2] >> (8 * (r & 3))) & 0xffu); };
-            have = next_unit(walk, nx);
+            have = unit(useq + 1, nx);
+            if (!ok) break;
             if (have) fetch_topo(nx);
             if (!(ok = role_sync())) break;                      // depths and gates visible; the last unit's entries are dead
 
