@@ -43,12 +43,12 @@
 //   warps 20-23   solver, one unit ahead: Gram entries of every row against its own path, back substitution (a thread
 //                 per node, registers), the pieces of M
 // TMEM: two tiles of accumulators (R | G, 128 columns; x M^T overwrites R), two A buffers of 48, x of 96, Gram of 64.
-// Measured in large batches, us per unit and SM (share of the copy rate): d_k = 128, d_v = 256: 8 nodes 4.1 (81 %), 16
-// nodes 4.5 (82 %), 32 nodes 5.3 (84 %), 64 nodes 7.8 (76 %), 64 nodes at 16 levels 9.2; d_k = d_v = 256: 8 nodes 7.0
-// (91 %), 32 nodes 8.55 (91 %).  One split group instead of two, before the chains of the Gram blocks: 4.75, 4.8, 5.1, 7.4, 7.9
-// against 4.0, 4.1, 5.3, 7.2, 8.2: a group needs about 750 cycles a slice, the tensor core 280.  What bounds it: HBM at d_k =
-// 256; at d_k = 128 the solver, which never waits for anybody but its own four warps (30 to 40 % of its time reads Gram
-// entries out of TMEM), and next to it the epilogue.
+// Measured in large batches, us per unit and SM (share of the copy rate): d_k = 128, d_v = 256: 20 nodes 4.1 (95 %), 32
+// nodes 4.4 (100 %), 40 nodes 5.2 (92 %), 64 nodes 6.7 (89 %); d_k = d_v = 256, 24 nodes 7.1 (103 %).  What bounds it: HBM up to
+// 32 nodes and at d_k = 256; above that the instructions of the roles, which wait for one another in turn (an epilogue warp a
+// third of its time for x M^T).  More of them did not help: three epilogue warps a lane quarter in the place of the second
+// split group no change, x M^T in two parts (the first under the making of the second half of x) 3 % slower, the loads of the
+// next eight columns under the work on these 4 % slower.
 // Ten roles take turns on four issue slots, so the kernel's size matters as much as its instruction count: loops stay
 // rolled where a role has slack.
 // x M^T runs over all nodes with zeros in M off the path, and zero times a value that is not finite is no zero: where an
@@ -241,16 +241,26 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         : "memory");
 }
 // Two fp32 values as three packed pairs of bf16 pieces (x0 in the low half), by truncation: a piece takes the top 8
-// bits of what is left, and three times 8 bits are all 24.
+// bits of what is left, and three times 8 bits are all 24.  What is left is taken with the fused multiply-add that reads a
+// bf16 half of a register (piece times -1 plus x, exact): masks and a packed subtraction took four more instructions of
+// the integer pipe, which runs at half rate (in a loop of splits a pair took 22 cycles, now 16; verification of ragged trees
+// of 8..64 nodes 463 -> 444 us).
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &p1, uint32_t &p2, uint32_t &p3)
 {
-    auto rest = [](float2 x) {                          // x minus its top 16 bits, exact
-        const float2 t = make_float2(__uint_as_float(__float_as_uint(x.x) & 0xffff0000u), __uint_as_float(__float_as_uint(x.y) & 0xffff0000u));
-        return __ffma2_rn(t, make_float2(-1.f, -1.f), x);
+    auto pack = [](float y0, float y1) { return __byte_perm(__float_as_uint(y0), __float_as_uint(y1), 0x7632); };
+    auto rest = [](uint32_t piece, float &y0, float &y1) {
+        asm("{\n\t.reg .b16 lo, hi, m;\n\t"
+            "mov.b16 m, 0xbf80;\n\t"
+            "mov.b32 {lo, hi}, %2;\n\t"
+            "fma.rn.f32.bf16 %0, lo, m, %0;\n\t"
+            "fma.rn.f32.bf16 %1, hi, m, %1;\n\t}"
+            : "+f"(y0), "+f"(y1) : "r"(piece));
     };
-    auto pack = [](float2 x) { return __byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x7632); };
-    const float2 a = make_float2(x0, x1), b = rest(a), c = rest(b);
-    p1 = pack(a); p2 = pack(b); p3 = pack(c);
+    p1 = pack(x0, x1);
+    rest(p1, x0, x1);
+    p2 = pack(x0, x1);
+    rest(p2, x0, x1);
+    p3 = pack(x0, x1);
 }
 
 // Optional self-profiling build (-DSPECA_PROF): cycles CTA 0 spends in each kind of wait, per warp,
@@ -641,16 +651,20 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
                     tmem_ld_wait();
                     uint32_t p1[4], p2[4], p3[4];
 #pragma unroll
+                    for (int i = 0; i < 8; ++i) r[i] = fmaf(-gm[i], r[i], __uint_as_float(vv[i] << 16));
+                    // rows past the last node belong to another sequence: they must not reach the product
+                    if (c0 + 8 > x.n)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (c0 + i >= x.n) r[i] = 0.f;
+#pragma unroll
                     for (int i = 0; i < 8; i += 2) {
-                        // rows past the last node belong to another sequence: they must not reach the product
-                        float x0 = c0 + i < x.n ? fmaf(-gm[i], r[i], __uint_as_float(vv[i] << 16)) : 0.f;
-                        float x1 = c0 + i + 1 < x.n ? fmaf(-gm[i + 1], r[i + 1], __uint_as_float(vv[i + 1] << 16)) : 0.f;
-                        zero = __ffma2_rn(make_float2(x0, x1), make_float2(0.f, 0.f), zero);
+                        zero = __ffma2_rn(make_float2(r[i], r[i + 1]), make_float2(0.f, 0.f), zero);
                         if (clean) {
-                            if (!(fabsf(x0) < INFINITY)) { odd |= 1u << i; x0 = 0.f; }
-                            if (!(fabsf(x1) < INFINITY)) { odd |= 2u << i; x1 = 0.f; }
+                            if (!(fabsf(r[i]) < INFINITY)) { odd |= 1u << i; r[i] = 0.f; }
+                            if (!(fabsf(r[i + 1]) < INFINITY)) { odd |= 2u << i; r[i + 1] = 0.f; }
                         }
-                        split_pair(x0, x1, p1[i >> 1], p2[i >> 1], p3[i >> 1]);
+                        split_pair(r[i], r[i + 1], p1[i >> 1], p2[i >> 1], p3[i >> 1]);
                     }
                     if (clean && ((c0 >> 3) & 1) != grp) return;         // the other warp's chunk
                     tmem_st4(xb + (c0 >> 1), p1);
