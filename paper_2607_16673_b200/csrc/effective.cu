@@ -37,14 +37,16 @@
 //   warp 2        issues the Gram blocks [K;Q] K^T (one unit ahead) and x M^T
 //   warp 3        walks the list of units and hands records of them to the others; TMA producer of the staged [K;Q] rows
 //                 (two units) and the value rows (two tiles)
-//   warps 4-11    split: slice row per thread -> three bf16 pieces in TMEM; two groups alternate slices, a buffer each
+//   warps 4-11    split: slice row per thread -> three bf16 pieces in TMEM; two groups alternate slices, a buffer each (trees
+//                 of more than 8 levels: one group, and the roles below four warps earlier)
 //   warps 12-19   epilogue, two warps per TMEM lane quarter that share a tile's columns: R out of TMEM, x back into TMEM
 //                 as three pieces; then, while the next tile's product runs, o = scale gamma G + (x M^T), coalesced
 //   warps 20-23   solver, one unit ahead: Gram entries of every row against its own path, back substitution (a thread
 //                 per node, registers), the pieces of M
 // TMEM: two tiles of accumulators (R | G, 128 columns; x M^T overwrites R), two A buffers of 48, x of 96, Gram of 64.
 // Measured in large batches, us per unit and SM (share of the copy rate): d_k = 128, d_v = 256: 20 nodes 4.1 (95 %), 32
-// nodes 4.4 (100 %), 40 nodes 5.2 (92 %), 64 nodes 6.7 (89 %); d_k = d_v = 256, 24 nodes 7.1 (103 %).  What bounds it: HBM up to
+// nodes 4.4 (100 %), 40 nodes 5.2 (92 %), 64 nodes 6.7 (89 %); d_k = d_v = 256, 24 nodes 7.1 (103 %); 16 levels: 24 nodes 4.6
+// (88 %), 64 nodes 7.0 (85 %).  What bounds it: HBM up to
 // 32 nodes and at d_k = 256; above that the instructions of the roles, which wait for one another in turn (an epilogue warp a
 // third of its time for x M^T).  More of them did not help: three epilogue warps a lane quarter in the place of the second
 // split group no change, x M^T in two parts (the first under the making of the second half of x) 3 % slower, the loads of the
@@ -72,7 +74,6 @@ using namespace tc;
 
 constexpr int kRows = 128;                      // value rows per tile (= TMEM lanes = MMA M)
 constexpr int kSliceBytes = kRows * 128;        // one ring slot: a K-slice of a tile (128 rows x 32 fp32)
-constexpr int kThreads = 24 * 32;
 constexpr int kWalkSeqs = 128;
 // Records of units.  The walk is one unit ahead of the staged rows, which are two ahead of the state product, and the value
 // rows keep it within two tiles of the epilogue: no role is five units behind it.
@@ -84,6 +85,15 @@ constexpr int kXOff = kAOff + 2 * kACols;       // x: three 32-column pieces (64
 constexpr int kGramOff = kXOff + 96;
 constexpr int kTmemCols = 512;
 static_assert(kGramOff + 64 == kTmemCols, "TMEM columns");
+
+// Split groups, four warps each, and with them the first warps of the epilogue and of the solver.  Up to 8 levels two: one takes
+// as long at 64 nodes, 4 % longer at 20.  Beyond that the solver's coefficients want the registers of four warps (96 a thread
+// instead of 80), and one group keeps up with it.  us per unit and SM, two groups / one: d_k = 128, d_v = 256, 16 levels, 24
+// nodes 5.34 / 4.64, 40 nodes 6.16 / 5.37, 64 nodes 7.25 / 7.00; 192 units of d_k = d_v = 256, 32 nodes 25.5 / 23.9 us.
+template <int DK, int MAXD> struct Roles {
+    static constexpr int kSplits = MAXD > 8 ? 1 : 2;
+    static constexpr int kEpilogue = 4 + 4 * kSplits, kSolver = kEpilogue + 8, kThreads = 32 * (kSolver + 4);
+};
 
 // shared-memory carve-up per instantiation
 template <int DK, int MAXN_, int MAXD> struct Lay {
@@ -296,10 +306,11 @@ __device__ __forceinline__ bool prof_wait(long long &acc, uint32_t bar, uint32_t
 // FEW = a call of a few units per SM: launched beside the plan kernel, value tiles of a head on two SMs.  (In a long call
 // every instruction of the ten roles counts, and the plain form is 1 to 2 % faster.)
 template <int TP, int DK, int MAXN, int MAXD, bool FEW>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Roles<DK, MAXD>::kThreads, 1)
 verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid_constant__ EMaps maps, EParams ep)
 {
     using LY = Lay<DK, MAXN, MAXD>;
+    using RO = Roles<DK, MAXD>;
     constexpr int NS = LY::NS, NC = LY::NC, SC = LY::SC, SCB = LY::SCB;
     extern __shared__ __align__(1024) uint8_t smem[];
     const Params &p = ep.p;
@@ -543,7 +554,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             }
         }
         PROF_STORE()
-    } else if (warp < 12) {
+    } else if (warp < RO::kEpilogue) {
         // ------------------------------------------------------------- split: slice -> three bf16 pieces in TMEM
         const int row = 32 * (warp & 3) + lane;                  // slice row = TMEM lane of this thread
         const int sgrp = (warp - 4) >> 2;                   // two groups, alternating slices
@@ -554,7 +565,7 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
 #pragma unroll 1
             for (int e = 0; e < TP * NC; ++e, ++it) {
                 const int s = it % NS, ab = it & 1;
-                if (ab != sgrp) continue;
+                if (RO::kSplits == 2 && ab != sgrp) continue;
                 if (!(ok = WAIT(0, bar(kFull + s), (it / NS) & 1))) break;
                 const uint8_t *src = smem + LY::OffRing + s * kSliceBytes + row * 128;
                 uint32_t p1[16], p2[16], p3[16];
@@ -579,13 +590,13 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
             }
         }
         PROF_STORE()
-    } else if (warp < 20) {
+    } else if (warp < RO::kSolver) {
         // ------------------------------------------------------------- epilogue
         // Step s takes tile s - 1 from x M^T to o, which frees its accumulators, and then tile s from R to x: the state product
         // of a tile runs under the second product of the one before it and under both of these.  (The other way round the
         // accumulators came free a whole state product later: 8-node units 4.9 us instead of 4.6.)  Columns go in chunks of
         // 8 nodes, alternately to the two warps of a lane quarter.
-        const int grp = (warp - 12) >> 2;
+        const int grp = (warp - RO::kEpilogue) >> 2;
         const int row = 32 * (warp & 3) + lane;
         const uint32_t lane_addr = uint32_t(32 * (warp & 3)) << 16;
         const uint32_t xb = tmem_base + kXOff + lane_addr;
@@ -1025,9 +1036,9 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     const bool few = share != 0 || n_units < 8 * sms;
     auto go = [&](auto tp, auto dk, auto mn, auto md) {
         constexpr int TP = decltype(tp)::value, DK = decltype(dk)::value, MN = decltype(mn)::value, MD = decltype(md)::value;
-        constexpr int bytes = Lay<DK, MN, MD>::Bytes;
-        if (few) launch(verify_effective_kernel<TP, DK, MN, MD, true>, grid, kThreads, bytes, st, map, em, ep);
-        else verify_effective_kernel<TP, DK, MN, MD, false><<<grid, kThreads, bytes, st>>>(map, em, ep);
+        constexpr int bytes = Lay<DK, MN, MD>::Bytes, threads = Roles<DK, MD>::kThreads;
+        if (few) launch(verify_effective_kernel<TP, DK, MN, MD, true>, grid, threads, bytes, st, map, em, ep);
+        else verify_effective_kernel<TP, DK, MN, MD, false><<<grid, threads, bytes, st>>>(map, em, ep);
     };
     auto pick = [&](auto dk, auto mn) {
         if (one_tile) deep ? go(Int<1>{}, dk, mn, Int<16>{}) : go(Int<1>{}, dk, mn, Int<8>{});
