@@ -174,6 +174,11 @@ plan_kernel(const int32_t *node_offsets, const int32_t *parent,
 
 // One warp per sequence.  Each lane takes nodes t = lane, lane+32, ... and walks t's
 // root path checking every token against the prediction made at its parent.
+// Parents, and whether a node's token is the one predicted at its parent, are staged in shared memory for up to kAcceptNodes
+// nodes: the loads of a node's three words are then in flight together, and a step up the path is one read of shared memory
+// instead of three dependent ones of global memory (128 sequences of 8..64 nodes 4.8 -> 3.6 us, one of 8 nodes 2.2 -> 1.8).
+// Larger sequences are walked in place.
+constexpr int kAcceptNodes = 128;
 __global__ void __launch_bounds__(128)
 accept_kernel(int32_t B, int32_t max_depth, const int32_t *node_offsets,
               const int32_t *parent, const int32_t *draft_tok,
@@ -190,9 +195,48 @@ accept_kernel(int32_t B, int32_t max_depth, const int32_t *node_offsets,
     const int root_pred = root_target_tok[b];
     int fault = 0;
     if (base < 0 || n < 0) fault = SPECA_STATUS_BAD_OFFSETS;
+    __shared__ int32_t s_target[4][kAcceptNodes];
+    __shared__ int16_t s_step[4][kAcceptNodes];        // parent, or kStop - parent where the walk ends at this node's token
+    constexpr int kStop = -16, kBad = -4;              // (kBad: no parent of this node)
+    int32_t *target = s_target[threadIdx.x >> 5];
+    int16_t *step = s_step[threadIdx.x >> 5];
+    const bool staged = !fault && n <= kAcceptNodes;
     // best = (depth << 16) | (0xffff - index): max picks the deepest, then the lowest index
     int best = -1;
-    if (!fault) {
+    if (staged) {
+        int pa[kAcceptNodes / 32], draft[kAcceptNodes / 32];
+#pragma unroll
+        for (int k = 0; k < kAcceptNodes / 32; ++k) {
+            const int t = 32 * k + lane;
+            if (t < n) {
+                pa[k] = parent[base + t];
+                draft[k] = draft_tok[base + t];
+                target[t] = target_tok[base + t];
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < kAcceptNodes / 32; ++k) {
+            const int t = 32 * k + lane;
+            if (t < n) {
+                const int p = pa[k];
+                const bool bad = p < -1 || p >= t;
+                const int pred = bad ? 0 : p < 0 ? root_pred : target[p];
+                step[t] = int16_t(bad ? kBad : draft[k] == pred ? p : kStop - p);
+            }
+        }
+        __syncwarp();
+        for (int t = lane; t < n; t += 32) {
+            int d = 0, a = t;
+            while (a >= 0) {
+                a = step[a];
+                if (a < -1) break;
+                if (++d > max_depth) { fault |= SPECA_STATUS_TOO_DEEP; a = kStop; break; }
+            }
+            if (a == kBad) fault |= SPECA_STATUS_BAD_PARENT;
+            if (a == -1) best = max(best, (d << 16) | (0xffff - t));
+        }
+    } else if (!fault) {
         for (int t = lane; t < n; t += 32) {
             int d = 0, ok = 1;
             for (int a = t; a >= 0;) {
@@ -207,23 +251,25 @@ accept_kernel(int32_t B, int32_t max_depth, const int32_t *node_offsets,
         }
     }
     if (n > 0x10000) fault |= SPECA_STATUS_TOO_MANY;
-    for (int off = 16; off; off >>= 1) {
-        best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
-        fault |= __shfl_xor_sync(0xffffffffu, fault, off);
-    }
-    if (lane != 0) return;
+    best = __reduce_max_sync(0xffffffffu, best);
+    fault = __reduce_or_sync(0xffffffffu, fault);
     if (fault) {                       // skip the sequence: nothing accepted
-        atomicOr(status, fault);
+        if (lane == 0) atomicOr(status, fault);
         best = -1;
     }
     const int len = best < 0 ? 0 : (best >> 16);
     int node = best < 0 ? -1 : 0xffff - (best & 0xffff);
-    path_len[b] = len;
-    next_tok[b] = (node < 0) ? root_pred : target_tok[base + node];
-    for (int d = max_depth - 1; d >= 0; --d) {
-        if (d < len) { path_idx[b * max_depth + d] = node; node = parent[base + node]; }
-        else path_idx[b * max_depth + d] = -1;
+    if (lane == 0) {
+        path_len[b] = len;
+        next_tok[b] = (node < 0) ? root_pred : staged ? target[node] : target_tok[base + node];
     }
+    // lane d writes entry d of the path; every lane walks
+    int mine = -1;
+    for (int d = len - 1; d >= 0; --d) {
+        if (d == lane) mine = node;
+        node = staged ? step[node] : parent[base + node];
+    }
+    if (lane < max_depth) path_idx[b * max_depth + lane] = mine;
 }
 
 // Stochastic posterior selection given per-node probabilities: one warp per sequence.
@@ -248,29 +294,27 @@ stochastic_accept_kernel(int32_t B, int32_t max_depth, const int32_t *node_offse
     if (base < 0 || n < 0) fault = SPECA_STATUS_BAD_OFFSETS;
     if (n > 0x10000) fault |= SPECA_STATUS_TOO_MANY;
     auto passes = [&](int t) { return __fmul_rn(uniform[base + t], p_draft[base + t]) < p_target[base + t]; };
-    // Parents and verdicts of up to kStochNodes nodes are staged in shared memory: a walk that chases parents and lower
-    // siblings through global memory is a chain of loads of half a microsecond each (128 trees of 24..64 nodes: 15.0 us,
-    // staged 7.7 us).  Larger sequences are walked in place.
+    // Parents and, of every node (and the committed state, entry 0), the first child that passes are staged in shared memory
+    // for up to kStochNodes nodes: a walk that chases parents and lower siblings through global memory is a chain of loads of
+    // half a microsecond each, and a search through the lower siblings one of as many reads of shared memory (128 trees of
+    // 24..64 nodes: 15.0 us in place, 7.6 searching, 3.7 so).  Larger sequences are walked in place.
     constexpr int kStochNodes = 256;
     __shared__ int16_t s_par[4][kStochNodes];
-    __shared__ uint8_t s_pass[4][kStochNodes], s_chosen[4][kStochNodes];
+    __shared__ int32_t s_first[4][kStochNodes + 1];
     int16_t *par = s_par[threadIdx.x >> 5];
-    uint8_t *ps = s_pass[threadIdx.x >> 5], *chosen = s_chosen[threadIdx.x >> 5];
+    int32_t *first = s_first[threadIdx.x >> 5];
+    const bool staged = !fault && n <= kStochNodes;
     int best = -1;                     // (depth << 16) | (0xffff - index) of the deepest node whose root path is all chosen
-    if (!fault && n <= kStochNodes) {
+    if (staged) {
+        for (int t = lane; t <= n; t += 32) first[t] = kStochNodes;
+        __syncwarp();
+#pragma unroll 2
         for (int t = lane; t < n; t += 32) {
             const int pa = parent[base + t];
+            const bool pass = passes(t);
             const bool bad = pa < -1 || pa >= t;
             par[t] = int16_t(bad ? -2 : pa);
-            ps[t] = passes(t);
-        }
-        __syncwarp();
-        // chosen: passing, with no passing sibling of lower index
-        for (int t = lane; t < n; t += 32) {
-            int ok = ps[t];
-            const int pa = par[t];
-            for (int s2 = pa + 1; s2 < t && ok && pa >= -1; ++s2) ok = !(par[s2] == pa && ps[s2]);
-            chosen[t] = uint8_t(ok);
+            if (pass && !bad) atomicMin(&first[pa + 1], t);
         }
         __syncwarp();
         for (int t = lane; t < n; t += 32) {
@@ -278,7 +322,7 @@ stochastic_accept_kernel(int32_t B, int32_t max_depth, const int32_t *node_offse
             for (int a = t; a >= 0;) {
                 const int pa = par[a];
                 if (pa < -1) { fault |= SPECA_STATUS_BAD_PARENT; ok = 0; break; }
-                if (!chosen[a]) { ok = 0; break; }
+                if (first[pa + 1] != a) { ok = 0; break; }         // fails, or a sibling of lower index passes
                 if (++d > max_depth) { fault |= SPECA_STATUS_TOO_DEEP; ok = 0; break; }
                 a = pa;
             }
@@ -301,22 +345,21 @@ stochastic_accept_kernel(int32_t B, int32_t max_depth, const int32_t *node_offse
             if (ok) best = max(best, (d << 16) | (0xffff - t));
         }
     }
-    for (int off = 16; off; off >>= 1) {
-        best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
-        fault |= __shfl_xor_sync(0xffffffffu, fault, off);
-    }
-    if (lane != 0) return;
+    best = __reduce_max_sync(0xffffffffu, best);
+    fault = __reduce_or_sync(0xffffffffu, fault);
     if (fault) {                       // skip the sequence: nothing accepted
-        atomicOr(status, fault);
+        if (lane == 0) atomicOr(status, fault);
         best = -1;
     }
     const int len = best < 0 ? 0 : (best >> 16);
     int node = best < 0 ? -1 : 0xffff - (best & 0xffff);
-    path_len[b] = len;
-    for (int d = max_depth - 1; d >= 0; --d) {
-        if (d < len) { path_idx[b * max_depth + d] = node; node = parent[base + node]; }
-        else path_idx[b * max_depth + d] = -1;
+    if (lane == 0) path_len[b] = len;
+    int mine = -1;                     // lane d writes entry d of the path; every lane walks
+    for (int d = len - 1; d >= 0; --d) {
+        if (d == lane) mine = node;
+        node = staged ? par[node] : parent[base + node];
     }
+    if (lane < max_depth) path_idx[b * max_depth + lane] = mine;
 }
 
 // Pending accepted paths of the fused commit-and-verify call, one thread per sequence:
@@ -473,7 +516,8 @@ chain_decompose_kernel(int32_t N, const int32_t *node_offsets, const int32_t *pa
                        int32_t *__restrict__ chain_head, int32_t *__restrict__ n_chains, int32_t *status)
 {
     after_previous_kernel();
-    extern __shared__ int32_t sm[];                     // [N] subtree size, [N] key of the heavy child
+    extern __shared__ int32_t sm[];                     // [N] subtree size, [N] key of the heavy child, [N] parent
+    int32_t *par = sm + 2 * N;
     __shared__ int32_t s_flag, s_count;
     const int b = blockIdx.x;
     const int base = node_offsets[b], n = node_offsets[b + 1] - base;
@@ -490,6 +534,7 @@ chain_decompose_kernel(int32_t N, const int32_t *node_offsets, const int32_t *pa
         sm[i] = 1;
         sm[N + i] = -1;
         const int pa = parent[base + i];
+        par[i] = pa;
         if (pa < -1 || pa >= i) atomicOr(&s_flag, 1);
     }
     __syncthreads();
@@ -498,17 +543,17 @@ chain_decompose_kernel(int32_t N, const int32_t *node_offsets, const int32_t *pa
         return;
     }
     for (int i = threadIdx.x; i < n; i += blockDim.x)
-        for (int a = parent[base + i]; a >= 0; a = parent[base + a]) atomicAdd(&sm[a], 1);
+        for (int a = par[i]; a >= 0; a = par[a]) atomicAdd(&sm[a], 1);
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int pa = parent[base + i];
+        const int pa = par[i];
         if (pa >= 0) atomicMax(&sm[N + pa], (sm[i] << 16) | (0xffff - i));       // largest subtree, then lowest index
     }
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         int h = i;
         for (;;) {
-            const int pa = parent[base + h];
+            const int pa = par[h];
             if (pa < 0 || 0xffff - (sm[N + pa] & 0xffff) != h) break;            // h heads its chain
             h = pa;
         }
@@ -713,7 +758,7 @@ int launch_mask_to_parent(int32_t B, int32_t N, const uint8_t *mask, const int32
 int launch_chain_decompose(int32_t B, int32_t N, const int32_t *node_offsets, const int32_t *parent,
                            int32_t *chain_head, int32_t *n_chains, int32_t *status, cudaStream_t st)
 {
-    launch(chain_decompose_kernel, B, 256, size_t(2 * N) * sizeof(int32_t), st, N, node_offsets, parent, chain_head,
+    launch(chain_decompose_kernel, B, 256, size_t(3 * N) * sizeof(int32_t), st, N, node_offsets, parent, chain_head,
            n_chains, status);
     return int(cudaGetLastError());
 }
