@@ -398,48 +398,54 @@ pending_check_kernel(int32_t B, int32_t Tp, int32_t max_depth, int32_t max_len, 
     rec[9] = base;
 }
 
-// Convolution-state commit: one CTA per (layer, sequence), a thread per 8 channels.  A thread reads the
+// Convolution-state commit, a thread per kConvPieces pieces of 8 channels of one (layer, sequence).  A thread reads the
 // W rows that make up the new register (old rows and accepted inputs) into registers, then writes them,
-// so the in-place update never reads a row it has already overwritten.
-constexpr int kConvMaxWidth = 8;
+// so the in-place update never reads a row it has already overwritten.  The path is asked for together with its length, an
+// entry a lane, and checked by the warp.  All rows of a thread's pieces are in flight together, and a row of many channels is
+// spread over several CTAs (3072 x 3 rows of 8192 channels: 42.5 us with a CTA per (layer, sequence) and a piece at a time,
+// 37.2 = 6.1 TB/s now).
+constexpr int kConvMaxWidth = 8, kConvPieces = 2;
+template <int MAXW>
 __global__ void __launch_bounds__(256)
-conv_commit_kernel(int32_t B, int32_t channels, int32_t W, int32_t T, int32_t max_depth, uint4 *__restrict__ C,
+conv_commit_kernel(int32_t B, int32_t vec, int32_t parts, int32_t W, int32_t T, int32_t max_depth, uint4 *__restrict__ C,
                    const uint4 *x, const int32_t *node_offsets,
                    const int32_t *path_idx, const int32_t *path_len, int32_t *status)
 {
     after_previous_kernel();
-    const int l = blockIdx.x / B, b = blockIdx.x % B;
+    const int part = blockIdx.x % parts, l = blockIdx.x / parts / B, b = blockIdx.x / parts % B, lane = threadIdx.x & 31;
     const int A = path_len[b];
-    if (A == 0) return;
+    const int entry = lane < max_depth ? path_idx[b * max_depth + lane] : 0;
     const int base = node_offsets[b], n = node_offsets[b + 1] - base;
+    if (A == 0) return;
     int fault = 0;
     if (A < 0 || A > max_depth) fault = SPECA_STATUS_TOO_DEEP;
     else if (base < 0 || n < 0 || base + n > T) fault = SPECA_STATUS_BAD_OFFSETS;
-    else
-        for (int d = 0; d < A; ++d) {
-            const int t = path_idx[b * max_depth + d];
-            if (t < 0 || t >= n) fault = SPECA_STATUS_BAD_PATH;
-        }
+    else if (__any_sync(0xffffffffu, lane < A && (entry < 0 || entry >= n))) fault = SPECA_STATUS_BAD_PATH;
     if (fault) {
-        if (threadIdx.x == 0 && l == 0) atomicOr(status, fault);
+        if (threadIdx.x == 0 && l == 0 && part == 0) atomicOr(status, fault);
         return;
     }
-    const int vec = channels / 8;                       // 16-byte pieces per row
     uint4 *Cb = C + (size_t(l) * B + b) * W * vec;
-    for (int c = threadIdx.x; c < vec; c += blockDim.x) {
-        uint4 row[kConvMaxWidth];
+    const uint4 *xb = x + (size_t(l) * T + base) * vec;
+    const int c0 = part * (256 * kConvPieces) + threadIdx.x;    // this thread's pieces: c0, c0 + 256
+    uint4 row[kConvPieces][MAXW];
 #pragma unroll
-        for (int w = 0; w < kConvMaxWidth; ++w) {
-            if (w < W) {
-                const int s = A + w;                    // index in (old rows, accepted rows); the last W are kept
-                if (s < W) row[w] = Cb[s * vec + c];
-                else row[w] = x[(size_t(l) * T + base + path_idx[b * max_depth + (s - W)]) * vec + c];
-            }
+    for (int w = 0; w < MAXW; ++w) {
+        const int s = A + w;                                    // index in (old rows, accepted rows); the last W are kept
+        const int node = __shfl_sync(0xffffffffu, entry, s >= W ? (s - W) & 31 : 0);
+        if (w < W) {
+            const uint4 *src = s < W ? Cb + s * vec : xb + size_t(node) * vec;
+#pragma unroll
+            for (int i = 0; i < kConvPieces; ++i)
+                if (c0 + 256 * i < vec) row[i][w] = src[c0 + 256 * i];
         }
-#pragma unroll
-        for (int w = 0; w < kConvMaxWidth; ++w)
-            if (w < W) Cb[w * vec + c] = row[w];
     }
+#pragma unroll
+    for (int w = 0; w < MAXW; ++w)
+        if (w < W)
+#pragma unroll
+            for (int i = 0; i < kConvPieces; ++i)
+                if (c0 + 256 * i < vec) Cb[w * vec + c0 + 256 * i] = row[i][w];
 }
 
 // Proposal converter: tree attention mask -> parent array.  One CTA per sequence, a warp per row of the mask: the
@@ -781,7 +787,9 @@ int launch_conv_commit(int32_t L, int32_t B, int32_t channels, int32_t W, int32_
                        const void *x, const int32_t *node_offsets, const int32_t *path_idx, const int32_t *path_len,
                        int32_t *status, cudaStream_t st)
 {
-    launch(conv_commit_kernel, L * B, 256, 0, st, B, channels, W, T, max_depth, static_cast<uint4 *>(C),
+    const int vec = channels / 8, parts = (vec + 256 * kConvPieces - 1) / (256 * kConvPieces);     // 16-byte pieces of a row
+    auto kern = W <= 4 ? conv_commit_kernel<4> : conv_commit_kernel<kConvMaxWidth>;
+    launch(kern, unsigned(L) * B * parts, 256, 0, st, B, vec, parts, W, T, max_depth, static_cast<uint4 *>(C),
            static_cast<const uint4 *>(x), node_offsets, path_idx, path_len, status);
     return int(cudaGetLastError());
 }
