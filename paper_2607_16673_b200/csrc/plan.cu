@@ -469,6 +469,43 @@ mask_to_parent_kernel(int32_t N, const uint8_t *mask, const int32_t *node_offset
         return;
     }
     const uint8_t *m = mask + size_t(b) * N * N;
+    if (n <= 64) {
+        // Rows as 64-bit sets, straight out of global memory (the bytes of all rows of a warp are in flight together); then a
+        // thread per node goes through its own ancestors, which are few, instead of a warp through all nodes (128 masks of 64 x
+        // 64: 5.8 us staged as below, 3.2 so).
+        __shared__ uint2 s_row[64];
+        uint8_t lo[8], hi[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int i = warp + 8 * k;
+            lo[k] = i < n && lane < n ? m[i * N + lane] : 0;
+            hi[k] = i < n && lane + 32 < n ? m[i * N + lane + 32] : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint2 row = make_uint2(__ballot_sync(0xffffffffu, lo[k] != 0), __ballot_sync(0xffffffffu, hi[k] != 0));
+            if (lane == 0) s_row[warp + 8 * k] = row;
+        }
+        __syncthreads();
+        int bad = 0, best = -1;                         // best: (ancestors << 16) | (0xffff - index): the most, then the lowest index
+        const int i = threadIdx.x;
+        if (i < n) {
+            const uint2 row = s_row[i];
+            const unsigned long long set = row.x | (unsigned long long)(row.y) << 32, self = 1ull << i;
+            bad = !(set & self) || (set & ~(2 * self - 1)) != 0;
+            for (unsigned long long rest = set & ~self; rest != 0; rest &= rest - 1) {
+                const int j = __ffsll(rest) - 1;
+                best = max(best, ((__popc(s_row[j].x) + __popc(s_row[j].y)) << 16) | (0xffff - j));
+            }
+            bad |= (best < 0 ? 0 : best >> 16) != __popcll(set) - 1;
+        }
+        if (__syncthreads_or(bad)) {
+            if (threadIdx.x == 0) atomicOr(status, SPECA_STATUS_BAD_PARENT);
+            return;
+        }
+        if (i < n) parent[base + i] = best < 0 ? -1 : 0xffff - (best & 0xffff);
+        return;
+    }
     int32_t *sm = reinterpret_cast<int32_t *>(mask_smem) + (min(N * N, kMaskStage) + 15) / 16 * 4;
     if (n * N <= kMaskStage) {
         uint8_t *staged = reinterpret_cast<uint8_t *>(mask_smem);
