@@ -616,8 +616,8 @@ chain_decompose_kernel(int32_t N, const int32_t *node_offsets, const int32_t *pa
 // 1 .. b -- ~count, or the final offset if that sequence was quicker -- and replaces its own entry by the offset.
 // Every entry is either of the two whenever it is read, so the sum does not depend on who comes first.  (One CTA that
 // packed the sequences in turn took 86 us for 128 of them, its serial selection 15; both runs together 21 us.)
-// What bounds it: a chain of shared-memory and L2 latencies per sequence.  The five drafting utilities of 128 trees of 24..64 nodes
-// take 102.7 us with two barriers per tree level, 96.9 with every node's path in registers and the scan's loads together.
+// What bounds it: a chain of shared-memory and L2 latencies per sequence; every node's path stays in registers instead of two
+// barriers per tree level.
 constexpr int kPruneLevels = 16;
 
 // Calls step(i, parent of i) for every node with a parent, parents first: level by level, all threads of the CTA, for
@@ -787,6 +787,133 @@ prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *node_offsets,
         }
 }
 
+// The same for up to kPruneSeqs sequences of at most 64 nodes, in one launch: a warp per sequence, spread over a cluster of
+// CTAs that tell one another their counts through shared memory, so that nothing has to be done twice.  Sets of nodes are 64-bit
+// words, and a warp needs no barrier.  What is left is a chain of two loads, the levels of the tree, the 64 comparisons of
+// a node and one barrier of the cluster.  128 trees of 24..64 nodes: 11.9 us for the two runs of prune_kernel, 5.0 so.  More
+// sequences than warps, or more nodes than bits, go the other way.
+constexpr int kPruneCtas = 8, kPruneSeqs = 128;
+__global__ void __cluster_dims__(kPruneCtas, 1, 1) __launch_bounds__(kPruneSeqs / kPruneCtas * 32)
+prune_small_kernel(int32_t B, int32_t N, float tau, int32_t budget, const int32_t *node_offsets, const int32_t *parent,
+                   const float *logp, int32_t *__restrict__ out_offsets, int32_t *__restrict__ out_parent,
+                   int32_t *__restrict__ out_index, int32_t *status)
+{
+    after_previous_kernel();
+    __shared__ int32_t s_count[kPruneSeqs];
+    __shared__ __align__(16) float s_q[kPruneSeqs / kPruneCtas][64];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = warp * kPruneCtas + blockIdx.x;
+    float *q = s_q[warp];
+    typedef unsigned long long Set;
+    auto set_of = [](bool lo, bool hi) -> Set {
+        return __ballot_sync(0xffffffffu, lo) | Set(__ballot_sync(0xffffffffu, hi)) << 32;
+    };
+    auto in = [](Set s, int i) -> bool { return (s >> i) & 1; };
+
+    int base = 0, n = 0, fault = 0;
+    if (b < B) {
+        base = node_offsets[b];
+        n = node_offsets[b + 1] - base;
+        if (n < 0 || base < 0) fault = SPECA_STATUS_BAD_OFFSETS;
+        else if (n > N) fault = SPECA_STATUS_TOO_MANY;
+    }
+    if (fault) n = 0;
+    int par[2] = {-1, -1};
+    float lp[2] = {0.f, 0.f};
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int i = lane + 32 * k;
+        if (i < n) {
+            par[k] = parent[base + i];
+            lp[k] = logp[base + i];
+            bad |= par[k] < -1 || par[k] >= i;
+        }
+    }
+    if (__any_sync(0xffffffffu, bad)) {
+        fault = SPECA_STATUS_BAD_PARENT;
+        n = 0;
+    }
+    if (fault && lane == 0) atomicOr(status, fault);
+
+    // scores: a level a turn, a node adds its own to its parent's (entries past the last node compare as false)
+    const bool live[2] = {lane < n, lane + 32 < n};
+    float mine[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        mine[k] = live[k] ? lp[k] : NAN;
+        q[lane + 32 * k] = mine[k];
+    }
+    __syncwarp();
+    Set done = set_of(!live[0] || par[0] < 0, !live[1] || par[1] < 0);
+    while (done != ~Set(0)) {
+        bool now[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            now[k] = !in(done, lane + 32 * k) && in(done, par[k] & 63);
+            if (now[k]) mine[k] = q[par[k]] + lp[k];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (now[k]) q[lane + 32 * k] = mine[k];
+        done |= set_of(now[0], now[1]);
+    }
+    __syncwarp();
+    float best = fmaxf(mine[0], mine[1]);
+    for (int off = 16; off; off >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, off));
+    best = fmaxf(best, -INFINITY);
+    if (n > 0 && q[0] != q[0]) best = q[0];             // a score that is no number in front keeps nothing
+    const float thr = best - tau;
+    // nodes that go before this one: better, or as good and of lower index (where this one is in the window, so are they)
+    int rank[2] = {0, 0};
+#pragma unroll 2
+    for (int j0 = 0; j0 < n; j0 += 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(q + j0);
+        const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                rank[k] += f[e] > mine[k] || (f[e] == mine[k] && j0 + e < lane + 32 * k);
+    }
+    const Set keep = set_of(live[0] && mine[0] >= thr && rank[0] < budget, live[1] && mine[1] >= thr && rank[1] < budget);
+    // a node goes with its parent
+    Set kept = 0;
+    for (Set more = keep; more != kept;) {
+        kept = more;
+        more = set_of(in(kept, lane) && (par[0] < 0 || in(kept, par[0] & 63)),
+                      in(kept, lane + 32) && (par[1] < 0 || in(kept, par[1] & 63)));
+    }
+    const int count = __popcll(kept);
+
+    // every CTA learns every count
+    const uint32_t slot = uint32_t(__cvta_generic_to_shared(&s_count[b]));
+    if (lane < kPruneCtas) {
+        uint32_t remote;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(slot), "r"(lane));
+        asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote), "r"(count) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (b >= B) return;
+    int dst = 0;
+#pragma unroll
+    for (int k = 0; k < kPruneSeqs / 32; ++k) dst += lane + 32 * k < b ? s_count[lane + 32 * k] : 0;
+    dst = __reduce_add_sync(0xffffffffu, dst);
+    if (lane == 0) {
+        out_offsets[b + 1] = dst + count;
+        if (b == 0) out_offsets[0] = 0;
+    }
+    auto before = [&](int i) { return __popcll(kept & ((Set(1) << i) - 1)); };
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int i = lane + 32 * k;
+        if (in(kept, i)) {
+            out_parent[dst + before(i)] = par[k] < 0 ? -1 : before(par[k]);
+            out_index[dst + before(i)] = i;
+        }
+    }
+}
+
 }  // namespace
 
 int launch_mask_to_parent(int32_t B, int32_t N, const uint8_t *mask, const int32_t *node_offsets, int32_t *parent,
@@ -810,6 +937,11 @@ int launch_prune(int32_t B, int32_t N, float tau, int32_t budget, const int32_t 
                  const float *logp, int32_t *out_offsets, int32_t *out_parent, int32_t *out_index, int32_t *status,
                  cudaStream_t st)
 {
+    if (N <= 64 && B <= kPruneSeqs) {
+        launch(prune_small_kernel, kPruneCtas, kPruneSeqs / kPruneCtas * 32, 0, st, B, N, tau, budget, node_offsets, parent,
+               logp, out_offsets, out_parent, out_index, status);
+        return int(cudaGetLastError());
+    }
     const size_t smem = size_t(5 * N) * sizeof(int32_t);
     launch(prune_kernel<false>, B, 128, smem, st, N, tau, budget, node_offsets, parent, logp, out_offsets, out_parent,
            out_index, status);
