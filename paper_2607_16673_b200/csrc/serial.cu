@@ -218,8 +218,11 @@ commit_kernel(Params p)
     after_previous_kernel();
     constexpr int G = Map<DK>::G, RPS = Map<DK>::RPS, ROWS = WARPS * RS * RPS, part_rows = ROWS * TILES;
     const int parts = p.DV / part_rows;
-    const long unit = blockIdx.x / parts;
-    const int part = blockIdx.x % parts;
+    // Large calls go through the units backwards: the verification before this one went forwards, and what it read last is
+    // still in L2 (16 sequences, 805 MB of state: round 495 -> 488 us; where everything fits in L2 it only costs 0.2 us).
+    const unsigned block = TILES > 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const long unit = block / parts;
+    const int part = block % parts;
     const int h = int(unit % p.H), b = int((unit / p.H) % p.B), l = int(unit / (long(p.H) * p.B));
     const int lane = threadIdx.x & 31, g = lane % G, sub = lane / G;
 
@@ -227,6 +230,12 @@ commit_kernel(Params p)
     const int len = p.path_len[b];
     const int base = p.node_offsets[b];
     const int n = p.node_offsets[b + 1] - base;
+    // (the path is asked for together with its length: the reads below then find it in L1.  4608 units of d_k = d_v = 64 27.6
+    // -> 26.4 us, 6144 units of 128 x 256 190.0 -> 185.3)
+    int entry = 0;
+    if (lane < p.max_depth)
+        asm volatile("ld.global.s32 %0, [%1];" : "=r"(entry) : "l"(p.path_idx + b * p.max_depth + lane) : "memory");
+    const int before = __shfl_up_sync(0xffffffffu, entry, 1);
     if (len == 0) return;
     // paths the tensor-core commit takes (it validates them itself)
     if (p.long_min > 0 && len >= p.long_min && len <= 8 && len <= p.max_depth) return;
@@ -255,8 +264,8 @@ commit_kernel(Params p)
     else {
         if (int(threadIdx.x) < len) {
             const int d = threadIdx.x;
-            const int t = p.path_idx[b * p.max_depth + d];
-            const int prev = d > 0 ? p.path_idx[b * p.max_depth + d - 1] : -1;
+            const int t = entry;
+            const int prev = d > 0 ? before : -1;
             if (t < 0 || t >= n) fault = SPECA_STATUS_BAD_PATH;
             else if (p.parent != nullptr && p.parent[base + t] != prev) fault = SPECA_STATUS_BAD_PATH;
             s_path[d] = t;
