@@ -43,8 +43,9 @@
 // nodes 8.0 instead of 4.4.
 // Measured (d_k = 128, d_v = 256, 12288 units, the pipelined kernel with its plan in brackets): 8 nodes 298 us = 6.1 TB/s
 // (344 us), 16 nodes 369 us = 5.5 TB/s (377); d_k = d_v = 64, 24576 units of 8 / 30 nodes: 148 / 335 us (serial walk 316 /
-// 1244).  What bounds it: the state stream at 8 nodes (93 % of the copy rate; 83 % at 16), above that the set-up (a chain of
-// about ten latencies, 6-9 us of a CTA's life) and at 32 nodes the MMAs.  For a few users, 384 chains of 8: 8.8 us.
+// 1244).  At d_k = 64 a unit of 17 nodes is 6400 warp instructions around 16 KB of state (half of the issue slots, 22 % of HBM);
+// several heads a CTA with their records loaded ahead, or five CTAs an SM instead of four, gained nothing there.  What bounds it: the state stream at 8 nodes (93 % of the copy rate; 83 % at 16), above that the set-up (some
+// thousand instructions a warp between ten barriers, issued every seventh cycle) and at 32 nodes the MMAs.  For a few users, 384 chains of 8: 8.8 us.
 #include <algorithm>
 #include <atomic>
 
@@ -140,11 +141,41 @@ template <int DK, int NT, int MAXD> struct Lay {
     static constexpr int bytes(int rows) { return OffV + NK * (rows + 8) * 2; }
 };
 
+// Division by a number that is the same for the whole call, for dividends below 2^31: a product and a shift instead of some
+// twenty instructions, of which every thread of a small unit had six.  (With the enumeration of the Gram blocks, us: 4608 units
+// of 5..40 nodes at d_k = d_v = 64 90.7 -> 83.1, 9216 units of 9..16 nodes 78.7 -> 73.3, of 48..64 nodes 335 -> 309; one user
+// of 64-wide heads, 20..40 nodes, 8.3 -> 7.6; chains of 8 at d_k = 128 9.0 -> 8.8.)
+struct Divisor {
+    uint32_t d, mul, shift;
+    Divisor() = default;
+    explicit Divisor(uint32_t by) : d(by), shift(31)
+    {
+        for (uint32_t x = by - 1; x != 0; x >>= 1) ++shift;     // 31 + ceil(log2 by)
+        mul = uint32_t(((uint64_t(1) << shift) + by - 1) / by);
+    }
+    __device__ __forceinline__ int quotient(int n) const { return int(uint64_t(uint32_t(n)) * mul >> shift); }
+};
+
 struct DirectArgs {
     Params p;
-    int32_t parts, rows;        // value-row slices per unit, rows per slice
+    Divisor parts, H, B, vp;    // value-row slices per unit; heads, sequences; 16-byte pieces of a slice of a value row
+    int32_t rows;               // value rows per slice
     int32_t lo;                 // sequences of at most this many nodes belong to another launch
     int32_t early;              // ask for the state before the records: see launch_one
+};
+
+// what a CTA works on
+struct Unit {
+    int part, unit, h, b, l;
+    __device__ __forceinline__ explicit Unit(const DirectArgs &da)
+    {
+        unit = da.parts.quotient(int(blockIdx.x));
+        part = int(blockIdx.x) - unit * int(da.parts.d);
+        const int lb = da.H.quotient(unit);
+        h = unit - lb * int(da.H.d);
+        l = da.B.quotient(lb);
+        b = lb - l * int(da.B.d);
+    }
 };
 
 // After a pass with an output that is not finite.  First pass: keys and value elements that are not finite are replaced by
@@ -156,8 +187,8 @@ __device__ __forceinline__ bool repair(const DirectArgs &da, uint8_t *smem, int 
     using LY = Lay<DK, NT, MAXD>;
     constexpr int N = LY::N;
     const Params &p = da.p;
-    const int part = int(blockIdx.x % unsigned(da.parts)), unit = int(blockIdx.x / unsigned(da.parts)), rows = da.rows;
-    const int h = unit % p.H, lb = unit / p.H, b = lb % p.B, l = lb / p.B;
+    const Unit un(da);
+    const int part = un.part, h = un.h, b = un.b, l = un.l, rows = da.rows;
     const int base = p.node_offsets[b], n = p.node_offsets[b + 1] - base;
     const long rec0 = (long(l) * p.T + base) * p.H + h;
     if (pass == 0) {
@@ -200,9 +231,8 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
     const Params &p = da.p;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
 
-    const int part = int(blockIdx.x % unsigned(da.parts));
-    const int unit = int(blockIdx.x / unsigned(da.parts));
-    const int h = unit % p.H, lb = unit / p.H, b = lb % p.B, l = lb / p.B;
+    const Unit un(da);
+    const int part = un.part, unit = un.unit, h = un.h, b = un.b, l = un.l;
     const int row0 = part * da.rows;
 
     // the first tiles are asked into L2 before anything else is known when the sequence is certainly ours
@@ -266,7 +296,7 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
         asm volatile("cp.async.commit_group;" ::: "memory");
         const int vp = da.rows >> 3, vrows = (n + 15) & ~15;
         for (int i = tid; i < vrows * vp; i += THREADS) {
-            const int node = i / vp, c = i % vp;
+            const int node = da.vp.quotient(i), c = i - node * vp;
             const bool live = node < n;
             cp16(sV + node * vstride + 8 * c, p.v + (rec0 + long(live ? node : 0) * H) * p.DV + row0 + 8 * c, live);
         }
@@ -305,10 +335,13 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
     }
 
     // ---- Gram rows of keys and queries against the keys
-    for (int job = WARPS - 1 - warp; job < nt * nt; job += WARPS) {      // (warp 0 walks the paths meanwhile)
-        // one MMA row block: keys 8 mi .. in rows 0-7, queries 8 mi .. in rows 8-15; a node's path holds no later node
-        const int mi = job / nt, ni = job % nt;
-        if (ni > mi) continue;
+    for (int job = WARPS - 1 - warp; job < nt * (nt + 1) / 2; job += WARPS) {      // (warp 0 walks the paths meanwhile)
+        // one MMA row block: keys 8 mi .. in rows 0-7, queries 8 mi .. in rows 8-15; a node's path holds no later node, so
+        // ni <= mi: the triangle row by row
+        int mi = 0;
+#pragma unroll
+        for (int m = 1; m < NT; ++m) mi += job >= m * (m + 1) / 2;
+        const int ni = job - mi * (mi + 1) / 2;
         float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
         const __nv_bfloat16 *pa = sKQ + ((lane & 8 ? N : 0) + 8 * mi + (lane & 7)) * LY::KQS + ((lane >> 4) << 3);
         const __nv_bfloat16 *pb = sKQ + (8 * ni + (lane & 7)) * LY::KQS + ((lane >> 3) << 3);
@@ -575,7 +608,11 @@ int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
         rows /= 2;
     }
     da.rows = rows;
-    da.parts = p.DV / rows;
+    const int parts = p.DV / rows;
+    da.parts = Divisor(parts);
+    da.H = Divisor(p.H);
+    da.B = Divisor(p.B);
+    da.vp = Divisor(rows >> 3);
     const int smem = LY::bytes(rows);
     static std::atomic<int> opted[64];
     int dev = 0;
@@ -586,7 +623,7 @@ int launch_one(const Params &p, int lo, bool all, int sms, cudaStream_t st)
         if (e != cudaSuccess) return int(e);
         opted[dev].store(1, std::memory_order_release);
     }
-    launch(kern, unsigned(units * da.parts), WARPS * 32, smem, st, da);
+    launch(kern, unsigned(units * parts), WARPS * 32, smem, st, da);
     return int(cudaGetLastError());
 }
 
