@@ -91,14 +91,13 @@ int verify_common(const speca_dims *dims, const float *S0, const uint16_t *q, co
             p.skip_nodes = limit;
         }
     }
-    if (!chain || fact || eff || tf32) {
-        p.plan_paths_only = eff;
+    if (eff) return cuda_rc(launch_verify_effective(p, dims->d_k, st));       // (and the plan, where it wants one)
+    if (!chain || fact || tf32) {
         // with parent == NULL (chain entry point) the plan kernel assumes parent[i] = i - 1
         rc = cuda_rc(launch_plan(p, st));
         if (rc != SPECA_OK) return rc;
     }
     if (fact) return cuda_rc(launch_verify_factorized(p, dims->d_k, false, true, st));
-    if (eff) return cuda_rc(launch_verify_effective(p, dims->d_k, st));
     if (tf32) return cuda_rc(launch_verify_factorized(p, dims->d_k, false, false, st));
     return cuda_rc(launch_verify_serial(p, dims->d_k, chain, st));
 }

@@ -163,6 +163,7 @@ struct EParams {
     int32_t share;                   // log2 of the units that share a head's keys and queries: see launch_verify_effective
     int32_t withhold_first_load;     // failure-detection test: CTA 0 never requests its first state slice
     int32_t want_u;
+    int32_t own_plan;                // FEW: the sequences are checked and their paths written here, no plan kernel ran
     int32_t heads_per_group;
     int32_t gpl, dl, db, dg;         // groups of heads per (layer, sequence); a step of gridDim.x groups as (layers, sequences, groups)
 };
@@ -302,6 +303,55 @@ __device__ __forceinline__ bool prof_wait(long long &acc, uint32_t bar, uint32_t
 #endif
 
 
+// What the plan kernel does for this one, done by every CTA for itself: a warp per sequence checks the topology and writes the
+// paths of its nodes to the workspace (all CTAs the same values; a CTA reads what it has written).  A launch and its latencies
+// less in front of a call of a few units.  scratch: 64 bytes a warp.
+__device__ __forceinline__ void plan_paths(const Params &p, int warp, int n_warps, int lane, int8_t *scratch, int32_t *tab_base, int8_t *tab_n)
+{
+    int8_t *par = scratch + 64 * warp;
+    for (int b = warp; b < p.B; b += n_warps) {
+        const int base = p.node_offsets[b], n = p.node_offsets[b + 1] - base;
+        int fault = 0;
+        if (base < 0 || n < 0 || base + n > p.T || (b == p.B - 1 && base + n != p.T) || (b == 0 && base != 0))
+            fault = SPECA_STATUS_BAD_OFFSETS;
+        else if (n > p.max_nodes)
+            fault = SPECA_STATUS_TOO_MANY;
+        if (!fault) {
+            for (int i = lane; i < n; i += 32) {
+                const int pa = p.parent != nullptr ? p.parent[base + i] : i - 1;       // no parent array: chain
+                if (pa < -1 || pa >= i) fault = SPECA_STATUS_BAD_PARENT;
+                par[i] = int8_t(pa);
+            }
+            fault = __reduce_or_sync(0xffffffffu, fault);
+        }
+        if (!fault)
+            for (int i = lane; i < n; i += 32) {
+                uint32_t up[4] = {0u, 0u, 0u, 0u}, lo = 0u, hi = 0u;
+                int d = 0;
+                for (int a = i; a >= 0; a = par[a], ++d) {
+                    const uint32_t byte = uint32_t(a) << (8 * (d & 3));
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) up[w] |= (d >> 2) == w ? byte : 0u;
+                    if (a < 32) lo |= 1u << a;
+                    else hi |= 1u << (a - 32);
+                }
+                p.ws.depth[base + i] = d;
+                reinterpret_cast<int4 *>(p.ws.up)[base + i] = make_int4(int(up[0]), int(up[1]), int(up[2]), int(up[3]));
+                reinterpret_cast<int2 *>(p.ws.set)[base + i] = make_int2(int(lo), int(hi));
+                if (d > p.max_depth) fault |= SPECA_STATUS_TOO_DEEP;
+                if (p.depth_in != nullptr && p.depth_in[base + i] != d) fault |= SPECA_STATUS_BAD_DEPTH;
+            }
+        fault = __reduce_or_sync(0xffffffffu, fault);
+        if (lane == 0) {
+            if (fault && blockIdx.x == 0) atomicOr(p.status, fault);
+            tab_base[b] = base;
+            tab_n[b] = int8_t(fault ? -1 : n);
+        }
+        __syncwarp();
+    }
+    fence_proxy_async();                                         // the scratch becomes a slot of the TMA ring
+}
+
 // TP = value tiles per unit (d_v / 128), DK = key width, MAXN = nodes per sequence, MAXD = tree depth.
 // FEW = a call of a few units per SM: launched beside the plan kernel, value tiles of a head on two SMs.  (In a long call
 // every instruction of the ten roles counts, and the plain form is 1 to 2 % faster.)
@@ -353,13 +403,16 @@ verify_effective_kernel(const __grid_constant__ CUtensorMap s0_map, const __grid
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if constexpr (FEW) {
-        // The plan kernel runs just before this one and writes none of the state: the first tile of the first unit is on
-        // its way into L2 while the plan is made.
+        // While the kernel in front drains (it may still write the state: this only brings it into L2), the first tile of the
+        // first unit is on its way.
         if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), kTmemCols);
         if (threadIdx.x == 0) prefetch_l2(p.S0 + size_t(blockIdx.x) * p.DV * DK, uint32_t(kRows * DK * 4));
         wait_for_previous_kernel();
+        if (ep.own_plan)
+            plan_paths(p, warp, RO::kThreads / 32, lane, reinterpret_cast<int8_t *>(smem + LY::OffRing),
+                       reinterpret_cast<int32_t *>(smem + LY::OffWalk), reinterpret_cast<int8_t *>(smem + LY::OffWalk + 4 * kWalkSeqs));
     }
-    for (int b = threadIdx.x; b < p.B && b < kWalkSeqs; b += blockDim.x) {
+    for (int b = threadIdx.x; b < p.B && b < kWalkSeqs && !(FEW && ep.own_plan); b += blockDim.x) {
         const int n = p.ws.seq_n[b];
         reinterpret_cast<int32_t *>(smem + LY::OffWalk)[b] = p.node_offsets[b];
         reinterpret_cast<int8_t *>(smem + LY::OffWalk + 4 * kWalkSeqs)[b] = int8_t(n < 0 ? -1 : n);
@@ -956,6 +1009,16 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     p.H <<= share;
     p.DV >>= share;
     const long n_units = long(p.L) * p.B * p.H;
+    // Launched beside the plan kernel where that is a part of the whole that counts (384 units of 64 nodes 37.9 -> 35.8 us,
+    // 12288 units not measurable), or without one while every warp of a CTA has a sequence at most (us with / without: 192 units
+    // of one sequence at d_k = 256 24.2 / 21.2, 16 units 10.1 / 9.5, 768 units of 2 sequences 42.5 / 41.5, 384 of 24 27.3 / 26.9;
+    // of 32 34.5 / 36.3, of 40 35.9 / 37.2).
+    const bool few = share != 0 || n_units < 8 * sms, own_plan = few && p.B <= 20 && p.skip_nodes == 0;
+    if (!own_plan) {
+        p.plan_paths_only = 1;
+        const int rc = launch_plan(p, st);
+        if (rc != 0) return rc;
+    }
     const cuuint32_t es[3] = {1, 1, 1};
     CUtensorMap map;
     {
@@ -1016,6 +1079,7 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     ep.want_u = p.u != nullptr ? 1 : 0;
     ep.withhold_first_load = g_withhold_first_load;
     ep.share = share;
+    ep.own_plan = own_plan;
     // Consecutive heads of one (layer, sequence) that a CTA takes together.  The next head of a group costs a role two
     // additions, the next group some hundred cycles of a chain that short units wait for; but whole groups leave some CTAs
     // longer lists than others.  Groups of 4 against single heads, by units per SM: ragged trees of 8..64 nodes +2.6 % at 83,
@@ -1031,9 +1095,6 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     ep.dl = grid / ep.gpl / p.B;
     const bool one_tile = p.DV == kRows;
     const bool deep = p.max_depth > 8;
-    // Launched beside the plan kernel where that is a part of the whole that counts (384 units of 64 nodes 37.9 -> 35.8 us,
-    // 12288 units not measurable).
-    const bool few = share != 0 || n_units < 8 * sms;
     auto go = [&](auto tp, auto dk, auto mn, auto md) {
         constexpr int TP = decltype(tp)::value, DK = decltype(dk)::value, MN = decltype(mn)::value, MD = decltype(md)::value;
         constexpr int bytes = Lay<DK, MN, MD>::Bytes, threads = Roles<DK, MD>::kThreads;
