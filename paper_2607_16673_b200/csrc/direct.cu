@@ -17,8 +17,8 @@
 // state; while one CTA builds its coefficients the other resident CTAs stream.  The pipelined tcgen05 kernel
 // spends most of a small unit on hand-overs between its roles instead.
 //
-// fp32 accuracy: both operands are split into a TF32 head and the remainder (three products; the dropped one is 2^-22 of
-// the result); M and the weights of the keys are split into three bf16 pieces and multiply bf16 rows exactly.  The tensor
+// fp32 accuracy: both operands are split into a TF32 head and the remainder, from 17 nodes on into two fp16 of 11 bits each under a
+// common scale (three products; the dropped one is 2^-22 of the result); M and the weights of the keys are split into three bf16 pieces and multiply bf16 rows exactly.  The tensor
 // core truncates where it adds, relative to the largest term, accumulator included; a long chain of products in one
 // accumulator loses a bit or two toward zero.  So the large sums (Gram entries, leading pieces, 32-column steps of the
 // state product) start from zero and are added up in fp32 proper.  Error against 64 bits, 2-norm of the difference over
@@ -48,6 +48,8 @@
 // thousand instructions a warp between ten barriers, issued every seventh cycle) and at 32 nodes the MMAs.  For a few users, 384 chains of 8: 8.8 us.
 #include <algorithm>
 #include <atomic>
+
+#include <cuda_fp16.h>
 
 #include "speca_common.cuh"
 #include "tc_ptx.cuh"
@@ -81,6 +83,46 @@ __device__ __forceinline__ void warp_mma_bf16_first(float (&d)[4], const uint32_
                  "{%10, %10, %10, %10};"
                  : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+template <bool FIRST> __device__ __forceinline__ void warp_mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    if (FIRST)
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+    else
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+            : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Power of two that brings values of up to m into [2^14, 2^15), and its inverse (m below 2^-112 counts as that; one that is not
+// finite keeps what it multiplies from being finite)
+__device__ __forceinline__ void half_scale(float m, float &up, float &down)
+{
+    const uint32_t e = max(__float_as_uint(m) & 0x7f800000u, 15u << 23);
+    up = __uint_as_float((268u << 23) - e);
+    down = __uint_as_float(e - (14u << 23));
+}
+// Two scaled values as a pair of fp16 and what is left of them as another, both rounded: 2^-23 of the value is lost at most, as
+// with TF32.
+__device__ __forceinline__ void half_split(float x0, float x1, uint32_t &hi, uint32_t &lo)
+{
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(x1), "f"(x0));
+    asm("{\n\t.reg .b16 h0, h1, m;\n\t"
+        "mov.b16 m, 0xbc00;\n\t"                                // -1
+        "mov.b32 {h0, h1}, %2;\n\t"
+        "fma.rn.f32.f16 %0, h0, m, %0;\n\t"
+        "fma.rn.f32.f16 %1, h1, m, %1;\n\t}"
+        : "+f"(x0), "+f"(x1) : "r"(hi));
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(x1), "f"(x0));
+}
+// largest magnitude of 8 values, and of what the four lanes of a row hold
+__device__ __forceinline__ float row_max(const float (&x)[8])
+{
+    float m = fmaxf(fmaxf(fmaxf(fabsf(x[0]), fabsf(x[1])), fmaxf(fabsf(x[2]), fabsf(x[3]))),
+                    fmaxf(fmaxf(fabsf(x[4]), fabsf(x[5])), fmaxf(fabsf(x[6]), fabsf(x[7]))));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    return fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
 }
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void *p)
 {
@@ -116,7 +158,14 @@ template <int DK, int NT, int MAXD> struct Lay {
     static constexpr int N = 8 * NT;
     static constexpr int NK = (N + 15) & ~15;                   // contraction width of the value term
     static constexpr int KQS = DK + 8;                          // bf16 per staged key / query row (16 bytes of padding)
+    // From 17 nodes on the tensor pipe bounds the state product (77 % of it, 384 units of 32 nodes), and its operands are pairs of
+    // fp16, scaled by row and 32-column step: six products of 16 columns in the place of twelve of 8 in TF32.  us, TF32 / fp16:
+    // 384 units of 32 nodes at d_k = d_v = 128 16.9 / 14.9, 192 at d_v = 256 18.0 / 15.5; d_k = d_v = 64, 9216 units of 16..32 nodes
+    // 117 / 110, of 48..64 309 / 295.  Below that the conversions cost more than the products.
+    static constexpr bool kHalf = NT >= 4;
+    static constexpr int NS = DK / 32;                          // 32-column steps
     static constexpr int BS = DK + 4;                           // floats per effective-query row (16 bytes of padding)
+    static constexpr int BSH = DK + 32;                         // fp16 per effective-query row (64 bytes: eight lanes, two rows, no conflict)
     static constexpr int MS = NK + 8;                           // bf16 per row of a piece of M
     static constexpr int GS = N + 1;
     static constexpr int NR = NK;                               // rows of the weight pieces: whole MMA row blocks
@@ -125,18 +174,20 @@ template <int DK, int NT, int MAXD> struct Lay {
     static constexpr int WP = w_row(NR);                        // bf16 per piece
     static constexpr int OffKQ = 0;                             // bf16 [2N][KQS]: key rows, query rows
     static constexpr int OffHi = OffKQ + 2 * N * KQS * 2;       // float [N][BS]
-    static constexpr int OffLo = OffHi + N * BS * 4;
-    static constexpr int OffM = OffLo + N * BS * 4;             // bf16 [3][N][MS]
+    static constexpr int OffLo = OffHi + (kHalf ? N * BSH * 2 : N * BS * 4);
+    static constexpr int OffS = OffLo + N * BSH * 2;            // kHalf: float [NS][N], what undoes the scale of a node's 32 columns
     static constexpr int OffG = OffHi;                          // float [2N][GS]: Gram rows of keys, queries (dead before Hi is written)
+    static constexpr int kQEnd = kHalf ? OffS + NS * N * 4 : OffLo + N * BS * 4;
+    static constexpr int kREnd = kQEnd > OffG + 2 * N * GS * 4 ? kQEnd : (OffG + 2 * N * GS * 4 + 15) & ~15;
+    static constexpr int OffM = kREnd;                          // bf16 [3][N][MS]
     static constexpr int OffW = OffM + 3 * N * MS * 2;          // bf16 [3][WP]: weights of the keys in qeff
     static constexpr int OffP = OffW + 3 * WP * 2;         // int32 parent[N], float alpha[N], beta[N], scale gamma[NR]
     // rows of the back substitution: float c beta [N][MAXD], float rho [N][MAXD], uint8 path [N][MAXD]; behind the Gram
     // rows where those leave room, else over them (one barrier more), and as dead as they are afterwards
     static constexpr int GEnd = (OffG + 2 * N * GS * 4 + 15) & ~15, CBytes = 9 * N * MAXD;
-    static constexpr bool kOver = GEnd + CBytes > OffHi + 2 * N * BS * 4;
+    static constexpr bool kOver = GEnd + CBytes > kREnd;
     static constexpr int OffC = kOver ? OffG : GEnd;
     static constexpr int OffV = OffP + (3 * N + NR) * 4;        // bf16 [NK][rows + 8]
-    static_assert(2 * N * GS <= 2 * N * BS, "Gram rows do not fit the space of the effective queries");
     static_assert(OffG + CBytes <= GEnd || !kOver, "rows of the back substitution do not fit the space of the Gram rows");
     static constexpr int bytes(int rows) { return OffV + NK * (rows + 8) * 2; }
 };
@@ -262,6 +313,8 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
     if (n <= da.lo || n > N) return;                         // nothing to do, or another launch's
     __nv_bfloat16 *sKQ = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffKQ);
     float *sHi = reinterpret_cast<float *>(smem + LY::OffHi), *sLo = reinterpret_cast<float *>(smem + LY::OffLo);
+    uint16_t *hHi = reinterpret_cast<uint16_t *>(smem + LY::OffHi), *hLo = reinterpret_cast<uint16_t *>(smem + LY::OffLo);
+    float *sSc = reinterpret_cast<float *>(smem + LY::OffS);
     __nv_bfloat16 *sM = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffM);
     float *sG = reinterpret_cast<float *>(smem + LY::OffG);
     __nv_bfloat16 *sW = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffW);
@@ -428,14 +481,15 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
 
         // ---- effective queries (scale gamma q + W K, the weights in three bf16 pieces), split into head and remainder
         {
+            constexpr int CW = LY::kHalf ? 32 : 16, CB = CW / 8;     // columns of a job, in blocks of 8
             const int nm = (n + 15) >> 4;
-            for (int job = warp; job < nm * (DK / 16); job += WARPS) {
-                const int mi = job / (DK / 16), c0 = (job % (DK / 16)) * 16;
+            for (int job = warp; job < nm * (DK / CW); job += WARPS) {
+                const int mi = job / (DK / CW), c0 = (job % (DK / CW)) * CW;
                 const int r0 = 16 * mi + g, r1 = r0 + 8;
                 const float g0 = sGam[r0], g1 = sGam[r1];
-                float acc[2][4];
+                float acc[CB][4];
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
+                for (int c = 0; c < CB; ++c) {
                     // rows past the staged ones weigh nothing; clamp keeps the read inside the buffer
                     const uint32_t q0 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r0, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
                     const uint32_t q1 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r1, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
@@ -444,29 +498,46 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                     acc[c][3] = r1 < 8 * nt ? g1 * __uint_as_float(q1 & 0xffff0000u) : 0.f;
                 }
                 for (int kk = 0; kk <= mi; ++kk) {               // a node's path holds no later node
-                    uint32_t kb[4];                              // key rows 16 kk .. + 15, columns c0 .. + 15
+                    uint32_t kb[CB / 2][4];                      // key rows 16 kk .. + 15, columns c0 .. + CW - 1
                     const int kr = 16 * kk + (lane & 15);
-                    ldsm_x4_t(kb, sKQ + min(kr, 8 * nt - 1) * LY::KQS + c0 + ((lane >> 4) << 3));
-                    float lo[2][4], hi[2][4];
+#pragma unroll
+                    for (int c = 0; c < CB / 2; ++c)
+                        ldsm_x4_t(kb[c], sKQ + min(kr, 8 * nt - 1) * LY::KQS + c0 + 16 * c + ((lane >> 4) << 3));
+                    float lo[CB][4], hi[CB][4];
 #pragma unroll
                     for (int pc = 2; pc >= 0; --pc) {
                         uint32_t a[4];
                         ldsm_x4(a, sW + pc * LY::WP + LY::w_row(16 * mi + (lane & 15)) + 16 * kk + ((lane >> 4) << 3));
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
-                            if (pc == 2) warp_mma_bf16_first(lo[c], a, kb[2 * c], kb[2 * c + 1]);
-                            else if (pc == 1) warp_mma_bf16(lo[c], a, kb[2 * c], kb[2 * c + 1]);
-                            else warp_mma_bf16_first(hi[c], a, kb[2 * c], kb[2 * c + 1]);
+                        for (int c = 0; c < CB; ++c) {
+                            const uint32_t b0 = kb[c >> 1][2 * (c & 1)], b1 = kb[c >> 1][2 * (c & 1) + 1];
+                            if (pc == 2) warp_mma_bf16_first(lo[c], a, b0, b1);
+                            else if (pc == 1) warp_mma_bf16(lo[c], a, b0, b1);
+                            else warp_mma_bf16_first(hi[c], a, b0, b1);
                         }
                     }
 #pragma unroll
-                    for (int c = 0; c < 2; ++c)
+                    for (int c = 0; c < CB; ++c)
 #pragma unroll
                         for (int e = 0; e < 4; ++e) acc[c][e] += hi[c][e] + lo[c][e];
                 }
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
                     const int r = half ? r1 : r0;
+                    if constexpr (LY::kHalf) {
+                        float x[8], up, down;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) { x[2 * c] = acc[c][2 * half]; x[2 * c + 1] = acc[c][2 * half + 1]; }
+                        half_scale(row_max(x), up, down);
+                        if (r < 8 * nt) {
+                            uint32_t *ph = reinterpret_cast<uint32_t *>(hHi + r * LY::BSH + c0 + 2 * t4);
+                            uint32_t *pl = reinterpret_cast<uint32_t *>(hLo + r * LY::BSH + c0 + 2 * t4);
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) half_split(x[2 * c] * up, x[2 * c + 1] * up, ph[4 * c], pl[4 * c]);
+                            if (t4 == 0) sSc[(c0 >> 5) * N + r] = down;
+                        }
+                        continue;
+                    }
                     if (r >= 8 * nt) break;
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
@@ -486,6 +557,7 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
         // columns 8 t + 2 e and 8 t + 2 e + 1 of the four lanes
         const int half = PARTS == 1 ? 0 : warp % PARTS, i0 = half * NTP;         // this warp's column tiles: i0 ..
         const float *hi_p = sHi + (8 * i0 + g) * LY::BS + 8 * t4, *lo_p = sLo + (8 * i0 + g) * LY::BS + 8 * t4;
+        const uint16_t *hh_p = hHi + (8 * i0 + g) * LY::BSH + 8 * t4, *hl_p = hLo + (8 * i0 + g) * LY::BSH + 8 * t4;
         const int nk = (n + 15) >> 4, ntp = nt - i0;
         const int tile_end = PARTS > 1 && ntp <= 0 ? 0 : tiles;
         float *o0 = p.o + rec0 * p.DV + row0 + g;
@@ -503,6 +575,45 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
             const float *cur = Su + long(tile) * 16 * DK, *nxt = cur + STRIDE * 16 * DK - NS * 32;
 #pragma unroll
             for (int q = 0; q < NS; ++q) {
+                if constexpr (LY::kHalf) {
+                    // k-steps j = 0, 1 of 16 contract columns 8 t + 4 j .. + 3 of the four lanes
+                    uint32_t ah[2][4], al[2][4];
+                    float up_a, down_a, up_b, down_b;
+                    half_scale(row_max(sa[q & 1]), up_a, down_a);
+                    half_scale(row_max(sb[q & 1]), up_b, down_b);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            const int e = 4 * j + 2 * c;
+                            half_split(sa[q & 1][e] * up_a, sa[q & 1][e + 1] * up_a, ah[j][2 * c], al[j][2 * c]);
+                            half_split(sb[q & 1][e] * up_b, sb[q & 1][e + 1] * up_b, ah[j][2 * c + 1], al[j][2 * c + 1]);
+                        }
+                    if (q + 2 < NS || next) {
+                        const float *src = (q + 2 < NS ? cur : nxt) + 32 * (q + 2);
+                        ld_state(sa[q & 1], src);
+                        ld_state(sb[q & 1], src + 8 * DK);
+                    }
+#pragma unroll
+                    for (int i = 0; i < NTP; ++i) {
+                        if (NTP > 1 && i >= ntp) break;
+                        const uint4 bh = *reinterpret_cast<const uint4 *>(hh_p + 8 * i * LY::BSH + 32 * q);
+                        const uint4 bl = *reinterpret_cast<const uint4 *>(hl_p + 8 * i * LY::BSH + 32 * q);
+                        const float2 sc = *reinterpret_cast<const float2 *>(sSc + q * N + 8 * (i0 + i) + 2 * t4);
+                        float part[4];                           // small products first
+                        warp_mma_f16<true>(part, al[0], bh.x, bh.y);
+                        warp_mma_f16<false>(part, al[1], bh.z, bh.w);
+                        warp_mma_f16<false>(part, ah[0], bl.x, bl.y);
+                        warp_mma_f16<false>(part, ah[1], bl.z, bl.w);
+                        warp_mma_f16<false>(part, ah[0], bh.x, bh.y);
+                        warp_mma_f16<false>(part, ah[1], bh.z, bh.w);
+                        hh[i][0] = fmaf(part[0] * down_a, sc.x, hh[i][0]);
+                        hh[i][1] = fmaf(part[1] * down_a, sc.y, hh[i][1]);
+                        hh[i][2] = fmaf(part[2] * down_b, sc.x, hh[i][2]);
+                        hh[i][3] = fmaf(part[3] * down_b, sc.y, hh[i][3]);
+                    }
+                    continue;
+                }
                 uint32_t ah[4][4], al[4][4];                     // [k-step][fragment register]
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -641,11 +752,11 @@ int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_
         return launch_one<DK, 8, MAXD, 8, 2>(p, lo, all, sms, st);
     } else {
         // between two and three units per SM one wave of smaller CTAs beats two of the others (d_k = d_v = 128, 32 nodes: 384
-        // units 24.6 us, with eight warps 26.6; 432 units the same; 576 units take two waves either way); at d_v > 128 three
-        // do not fit in shared memory
+        // units 24.6 us, with eight warps 26.6; 432 units the same; 576 units take two waves either way; d_v = 256, 384 units of 24 /
+        // 32 nodes 22.1 / 25.6, with eight warps 25.1 / 29.0)
         const long units = long(p.L) * p.B * p.H;
         if constexpr (DK == 128)
-            if (p.DV <= 128 && units > 2 * sms && units <= 3 * sms) return launch_one<DK, 4, MAXD, 4, 3>(p, lo, all, sms, st);
+            if (p.DV <= 256 && units > 2 * sms && units <= 3 * sms) return launch_one<DK, 4, MAXD, 4, 3>(p, lo, all, sms, st);
         return launch_one<DK, 4, MAXD, 8, 2>(p, lo, all, sms, st);
     }
 }
