@@ -211,17 +211,19 @@ verify_serial_kernel(Params p)
 // once; the second tile is asked into L2 when the first is loaded, so that HBM stays busy while the path is staged and
 // walked.  Paths of three nodes, 12288 units of d_k = 128, d_v = 256: a tile a CTA 562 us = 5.8 TB/s, two 490 us = 6.6
 // TB/s, which is the copy rate; four 568 (fewer CTAs start than end).
-template <int DK, int RS, int WARPS, int TILES>
+// HEADS = 2: the tiles are whole units of two neighbouring heads, whose states and records lie one behind the other.
+template <int DK, int RS, int WARPS, int TILES, int HEADS>
 __global__ void __launch_bounds__(WARPS * 32, 2048 / (WARPS * 32) / 2)
 commit_kernel(Params p)
 {
     after_previous_kernel();
     constexpr int G = Map<DK>::G, RPS = Map<DK>::RPS, ROWS = WARPS * RS * RPS, part_rows = ROWS * TILES;
-    const int parts = p.DV / part_rows;
+    static_assert(HEADS == 1 || HEADS == TILES, "a tile per head");
+    const int parts = HEADS > 1 ? 1 : p.DV / part_rows;
     // Large calls go through the units backwards: the verification before this one went forwards, and what it read last is
     // still in L2 (16 sequences, 805 MB of state: round 495 -> 488 us; where everything fits in L2 it only costs 0.2 us).
-    const unsigned block = TILES > 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
-    const long unit = block / parts;
+    const unsigned block = TILES > HEADS ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const long unit = long(block / parts) * HEADS;
     const int part = block % parts;
     const int h = int(unit % p.H), b = int((unit / p.H) % p.B), l = int(unit / (long(p.H) * p.B));
     const int lane = threadIdx.x & 31, g = lane % G, sub = lane / G;
@@ -255,8 +257,8 @@ commit_kernel(Params p)
     // are staged in shared memory while the state tile is in flight, so that the token-by-token
     // recurrence below never waits on global memory.
     __shared__ int s_path[16];
-    __shared__ __align__(16) __nv_bfloat16 s_k[16][DK];
-    __shared__ float s_alpha[16], s_beta[16];
+    __shared__ __align__(16) __nv_bfloat16 s_k[16][DK * HEADS];
+    __shared__ float s_alpha[HEADS][16], s_beta[HEADS][16];
     __shared__ __nv_bfloat16 s_v[16][part_rows];
     int fault = 0;
     if (!len_ok) fault = SPECA_STATUS_TOO_DEEP;
@@ -271,11 +273,14 @@ commit_kernel(Params p)
             s_path[d] = t;
             if (!fault) {
                 const long rec = (long(l) * p.T + base + t) * p.H + h;
-                s_alpha[d] = p.alpha[rec];
-                s_beta[d] = p.beta[rec];
+#pragma unroll
+                for (int i = 0; i < HEADS; ++i) {
+                    s_alpha[i][d] = p.alpha[rec + i];
+                    s_beta[i][d] = p.beta[rec + i];
+                }
             }
         }
-        constexpr int PIECES = DK / 8;                       // 16-byte pieces per k row
+        constexpr int PIECES = DK * HEADS / 8;               // 16-byte pieces per k row
         for (int idx = threadIdx.x; idx < len * PIECES; idx += WARPS * 32) {
             const int d = idx / PIECES, piece = idx % PIECES;
             const int t = p.path_idx[b * p.max_depth + d];
@@ -316,11 +321,11 @@ commit_kernel(Params p)
             float2 kx[8];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const uint2 raw = *(reinterpret_cast<const uint2 *>(&s_k[d][0]) + g + G * c);
+                const uint2 raw = *(reinterpret_cast<const uint2 *>(&s_k[d][HEADS > 1 ? tile * DK : 0]) + g + G * c);
                 kx[2 * c + 0] = make_float2(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u));
                 kx[2 * c + 1] = make_float2(__uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
             }
-            const float alpha = s_alpha[d], beta = s_beta[d];
+            const float alpha = s_alpha[HEADS > 1 ? tile : 0][d], beta = s_beta[HEADS > 1 ? tile : 0][d];
 #pragma unroll
             for (int r = 0; r < RS; ++r) {
                 const float sk = group_sum<G>(dot16(s[r], kx));
@@ -367,12 +372,16 @@ template <int DK, int RS, int WARPS> struct LaunchCommit {
         const long tiles = n_units(p) * (p.DV / ROWS);
         // Two tiles a CTA from four rounds of such CTAs on (d_k = 128, d_v = 256, 1536 units: 74.8 -> 72.0 us); below that
         // twice the CTAs serve the device better, and a 64-wide tile is done before its second is there (24576 units of
-        // d_k = d_v = 64: 162 us, two tiles 166).
+        // d_k = d_v = 64: 162 us, two tiles 166).  Two neighbouring heads of 64 x 64, which share the path, do pay (us, one / two, paths
+        // of three nodes: 4608 units 26.0 / 25.7, 6144 41.7 / 40.6, 9216 61.1 / 57.6, 18432 117.5 / 103.3; of one node 21.4 / 21.7,
+        // 35.1 / 34.7, 51.8 / 52.0, 100.3 / 97.2).
         const long round = long(sm_count_of_current_device()) * (2048 / (WARPS * 32) / 2);
         if (DK > 64 && p.DV % (2 * ROWS) == 0 && tiles >= 8 * round)
-            launch(commit_kernel<DK, RS, WARPS, 2>, unsigned(tiles / 2), WARPS * 32, 0, st, p);
+            launch(commit_kernel<DK, RS, WARPS, 2, 1>, unsigned(tiles / 2), WARPS * 32, 0, st, p);
+        else if (DK == 64 && p.DV == ROWS && p.H % 2 == 0 && tiles >= 5 * round)
+            launch(commit_kernel<DK, RS, WARPS, DK == 64 ? 2 : 1, DK == 64 ? 2 : 1>, unsigned(tiles / 2), WARPS * 32, 0, st, p);
         else
-            launch(commit_kernel<DK, RS, WARPS, 1>, unsigned(tiles), WARPS * 32, 0, st, p);
+            launch(commit_kernel<DK, RS, WARPS, 1, 1>, unsigned(tiles), WARPS * 32, 0, st, p);
         return int(cudaGetLastError());
     }
 };
