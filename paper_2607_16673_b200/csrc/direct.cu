@@ -17,17 +17,20 @@
 // state; while one CTA builds its coefficients the other resident CTAs stream.  The pipelined tcgen05 kernel
 // spends most of a small unit on hand-overs between its roles instead.
 //
-// fp32 accuracy: both operands are split into a TF32 head and the remainder, from 17 nodes on into two fp16 of 11 bits each under a
-// common scale (three products; the dropped one is 2^-22 of the result); M and the weights of the keys are split into three bf16 pieces and multiply bf16 rows exactly.  The tensor
-// core truncates where it adds, relative to the largest term, accumulator included; a long chain of products in one
-// accumulator loses a bit or two toward zero.  So the large sums (Gram entries, leading pieces, 32-column steps of the
-// state product) start from zero and are added up in fp32 proper.  Error against 64 bits, 2-norm of the difference over
-// that of the outputs, x 10^-8, chained / now / the route that takes the shape without this kernel: d_k = d_v = 64 (serial
-// walk): chains of 8 15.0 / 7.2 / 7.2, of 16 15.0 / 7.9 / 7.1, trees of 30 15.0 / 6.9 / 7.2; 128 x 64 (serial walk): chains
-// of 8 17.7 / 7.7 / 7.6, trees of 30 17.6 / 7.4 / 7.7; 128 x 256 (substitution kernel): chains of 8 17.6 / 7.7 / 15.4, trees
-// of 30 17.6 / 7.3 / 14.1; 256 x 256, chains of 8 24.2 / 8.7 / 30.3.  (Of the part that comes from the state alone 14, the
-// serial walk 7.6, the substitution kernel 90.)  It costs 2 to 6 % of a unit: 24576 units of 8 / 30 nodes at 64 x 64 142 /
-// 326 us chained, 148 / 336 now, 12288 units of 16 nodes at 128 x 256 388 and 394.
+// fp32 accuracy: both operands are split into a TF32 head and the remainder, from 17 nodes on into two fp16 of 11 bits each
+// under a common scale, the low one apart by another 2^11 (three products; the dropped one is 2^-22 of the result).  fp16 has
+// five bits of exponent: values that do not keep their bits under the scale of their 32 columns are looked for among the
+// effective queries, and, only where these are so uneven that it could show, among the rows of the state, and are multiplied in
+// TF32 instead.  M and the weights of the keys are split into three bf16 pieces and multiply bf16 rows exactly.  The tensor core
+// truncates where it adds, relative to the largest term, accumulator included; a long chain of products in one accumulator
+// loses a bit or two toward zero.  So the large sums (Gram entries, leading pieces, 32-column steps of the state product) start
+// from zero and are added up in fp32 proper.  Error against 64 bits, 2-norm of the difference over that of the outputs, x
+// 10^-8, chained / now / the route that takes the shape without this kernel: d_k = d_v = 64 (serial walk): chains of 8 15.0 /
+// 7.2 / 7.2, of 16 15.0 / 7.9 / 7.1, trees of 30 15.0 / 6.9 / 7.2; 128 x 64 (serial walk): chains of 8 17.7 / 7.7 / 7.6, trees
+// of 30 17.6 / 7.4 / 7.7; 128 x 256 (substitution kernel): chains of 8 17.6 / 7.7 / 15.4, trees of 30 17.6 / 7.3 / 14.1; 256 x
+// 256, chains of 8 24.2 / 8.7 / 30.3.  (Of the part that comes from the state alone 14, the serial walk 7.6, the substitution
+// kernel 90.)  It costs 2 to 6 % of a unit: 24576 units of 8 / 30 nodes at 64 x 64 142 / 326 us chained, 148 / 336 now, 12288
+// units of 16 nodes at 128 x 256 388 and 394.
 //
 // The products run over all nodes of a block with zero weights off the path, and zero times a value that is not finite
 // is no zero.  So where an output is not finite the CTA looks for such records (repair), takes them out of the products and
@@ -95,26 +98,48 @@ template <bool FIRST> __device__ __forceinline__ void warp_mma_f16(float (&d)[4]
             : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
             : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// Power of two that brings values of up to m into [2^14, 2^15), and its inverse (m below 2^-112 counts as that; one that is not
-// finite keeps what it multiplies from being finite)
-__device__ __forceinline__ void half_scale(float m, float &up, float &down)
+// Scale of a group of values of which the largest is m: the power of two that brings m into [2^14, 2^15), and its inverse (m
+// below 2^-112 counts as that).
+struct HalfScale {
+    float up, down, top;
+    __device__ __forceinline__ explicit HalfScale(float m) : top(m)
+    {
+        const uint32_t e = max(__float_as_uint(m) & 0x7f800000u, 15u << 23);
+        up = __uint_as_float((268u << 23) - e);
+        down = __uint_as_float(e - (14u << 23));
+    }
+    // some value that is not zero does not keep its bits in a pair (in a group that is not finite all others)
+    __device__ __forceinline__ bool loses(const float (&x)[8]) const
+    {
+        bool any = false;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) any |= x[e] != 0.f && fabsf(x[e] * up) < 1.f / 8192.f;
+        return any;
+    }
+};
+constexpr float kLowPiece = 1.f / 2048.f;                        // what a low piece counts
+__device__ __forceinline__ __half2 as_half2(uint32_t x) { return *reinterpret_cast<const __half2 *>(&x); }
+// Two values, scaled, as a pair of fp16 and 2^11 times what is left of them as another, both rounded.  At most 2^-23 of a value
+// is lost, as with TF32, down to 2^-27 of the largest of its group; below that 2^-51 of the largest.  (Were the low piece not
+// scaled, it would be subnormal from 2^-16 of the largest on and lose a bit per binade.)
+__device__ __forceinline__ void half_split(float x0, float x1, float up, uint32_t &hi, uint32_t &lo)
 {
-    const uint32_t e = max(__float_as_uint(m) & 0x7f800000u, 15u << 23);
-    up = __uint_as_float((268u << 23) - e);
-    down = __uint_as_float(e - (14u << 23));
-}
-// Two scaled values as a pair of fp16 and what is left of them as another, both rounded: 2^-23 of the value is lost at most, as
-// with TF32.
-__device__ __forceinline__ void half_split(float x0, float x1, uint32_t &hi, uint32_t &lo)
-{
-    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(x1), "f"(x0));
+    const float2 y = __fmul2_rn(make_float2(x0, x1), make_float2(up, up));
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(y.y), "f"(y.x));
+    float2 z = __fmul2_rn(y, make_float2(2048.f, 2048.f));
     asm("{\n\t.reg .b16 h0, h1, m;\n\t"
-        "mov.b16 m, 0xbc00;\n\t"                                // -1
+        "mov.b16 m, 0xe800;\n\t"                                // -2^11
         "mov.b32 {h0, h1}, %2;\n\t"
         "fma.rn.f32.f16 %0, h0, m, %0;\n\t"
         "fma.rn.f32.f16 %1, h1, m, %1;\n\t}"
-        : "+f"(x0), "+f"(x1) : "r"(hi));
-    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(x1), "f"(x0));
+        : "+f"(z.x), "+f"(z.y) : "r"(hi));
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(z.y), "f"(z.x));
+}
+// smallest magnitude of 8 values
+__device__ __forceinline__ float least_of(const float (&x)[8])
+{
+    return fminf(fminf(fminf(fabsf(x[0]), fabsf(x[1])), fminf(fabsf(x[2]), fabsf(x[3]))),
+                 fminf(fminf(fabsf(x[4]), fabsf(x[5])), fminf(fabsf(x[6]), fabsf(x[7]))));
 }
 // largest magnitude of 8 values, and of what the four lanes of a row hold
 __device__ __forceinline__ float row_max(const float (&x)[8])
@@ -158,14 +183,16 @@ template <int DK, int NT, int MAXD> struct Lay {
     static constexpr int N = 8 * NT;
     static constexpr int NK = (N + 15) & ~15;                   // contraction width of the value term
     static constexpr int KQS = DK + 8;                          // bf16 per staged key / query row (16 bytes of padding)
-    // From 17 nodes on the tensor pipe bounds the state product (77 % of it, 384 units of 32 nodes), and its operands are pairs of
-    // fp16, scaled by row and 32-column step: six products of 16 columns in the place of twelve of 8 in TF32.  us, TF32 / fp16:
-    // 384 units of 32 nodes at d_k = d_v = 128 16.9 / 14.9, 192 at d_v = 256 18.0 / 15.5; d_k = d_v = 64, 9216 units of 16..32 nodes
-    // 117 / 110, of 48..64 309 / 295.  Below that the conversions cost more than the products.
+    // From 17 nodes on the tensor pipe bounds the state product (77 % of it, 384 units of 32 nodes), and its operands are pairs
+    // of fp16, scaled by row and 32-column step: six products of 16 columns in the place of twelve of 8 in TF32.  us, TF32 /
+    // fp16: 384 units of 32 nodes at d_k = d_v = 128 17.7 / 15.6, 192 at d_v = 256 18.0 / 15.4; d_k = d_v = 64, 9216 units of
+    // 17..32 nodes 117.3 / 110.8, of 48..64 308 / 296; 256 x 64, 768 units of 32 nodes 66.2 / 38.6.  Below that the conversions
+    // cost more than the products.
     static constexpr bool kHalf = NT >= 4;
     static constexpr int NS = DK / 32;                          // 32-column steps
     static constexpr int BS = DK + 4;                           // floats per effective-query row (16 bytes of padding)
-    static constexpr int BSH = DK + 32;                         // fp16 per effective-query row (64 bytes: eight lanes, two rows, no conflict)
+    static constexpr int BSH = DK + 32;                         // fp16 per effective-query row (64 bytes: eight lanes, two rows, no
+                                                                // conflict)
     static constexpr int MS = NK + 8;                           // bf16 per row of a piece of M
     static constexpr int GS = N + 1;
     static constexpr int NR = NK;                               // rows of the weight pieces: whole MMA row blocks
@@ -187,7 +214,8 @@ template <int DK, int NT, int MAXD> struct Lay {
     static constexpr int GEnd = (OffG + 2 * N * GS * 4 + 15) & ~15, CBytes = 9 * N * MAXD;
     static constexpr bool kOver = GEnd + CBytes > kREnd;
     static constexpr int OffC = kOver ? OffG : GEnd;
-    static constexpr int OffV = OffP + (3 * N + NR) * 4;        // bf16 [NK][rows + 8]
+    static constexpr int OffU = OffP + (3 * N + NR) * 4;        // kHalf: int, steps whose effective queries are uneven
+    static constexpr int OffV = OffU + (kHalf ? 16 : 0);        // bf16 [NK][rows + 8]
     static_assert(OffG + CBytes <= GEnd || !kOver, "rows of the back substitution do not fit the space of the Gram rows");
     static constexpr int bytes(int rows) { return OffV + NK * (rows + 8) * 2; }
 };
@@ -320,6 +348,7 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
     __nv_bfloat16 *sW = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffW);
     int *sPar = reinterpret_cast<int *>(smem + LY::OffP);
     float *sAl = reinterpret_cast<float *>(sPar + N), *sBe = sAl + N, *sGam = sBe + N;
+    int *sUneven = reinterpret_cast<int *>(smem + LY::OffU);
     float *sC = reinterpret_cast<float *>(smem + LY::OffC);
     uint8_t *sPath = smem + LY::OffC + 8 * N * MAXD;
     __nv_bfloat16 *sV = reinterpret_cast<__nv_bfloat16 *>(smem + LY::OffV);
@@ -358,6 +387,7 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
         for (int i = tid; i < 3 * N * LY::MS / 8; i += THREADS) reinterpret_cast<uint4 *>(sM)[i] = make_uint4(0u, 0u, 0u, 0u);
         for (int i = tid; i < 3 * LY::WP / 8; i += THREADS) reinterpret_cast<uint4 *>(sW)[i] = make_uint4(0u, 0u, 0u, 0u);
         if (tid < LY::NR) sGam[tid] = 0.f;
+        if (LY::kHalf && tid == 0) *sUneven = 0;
     }
     if (tid < n) {
         if (pa < -1 || pa >= tid) fault = SPECA_STATUS_BAD_PARENT;
@@ -525,16 +555,33 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                 for (int half = 0; half < 2; ++half) {
                     const int r = half ? r1 : r0;
                     if constexpr (LY::kHalf) {
-                        float x[8], up, down;
+                        float x[8];
 #pragma unroll
                         for (int c = 0; c < 4; ++c) { x[2 * c] = acc[c][2 * half]; x[2 * c + 1] = acc[c][2 * half + 1]; }
-                        half_scale(row_max(x), up, down);
+                        const HalfScale scale(row_max(x));
+                        uint32_t *ph = reinterpret_cast<uint32_t *>(hHi + r * LY::BSH + c0 + 2 * t4);
+                        uint32_t *pl = reinterpret_cast<uint32_t *>(hLo + r * LY::BSH + c0 + 2 * t4);
                         if (r < 8 * nt) {
-                            uint32_t *ph = reinterpret_cast<uint32_t *>(hHi + r * LY::BSH + c0 + 2 * t4);
-                            uint32_t *pl = reinterpret_cast<uint32_t *>(hLo + r * LY::BSH + c0 + 2 * t4);
 #pragma unroll
-                            for (int c = 0; c < 4; ++c) half_split(x[2 * c] * up, x[2 * c + 1] * up, ph[4 * c], pl[4 * c]);
-                            if (t4 == 0) sSc[(c0 >> 5) * N + r] = down;
+                            for (int c = 0; c < 4; ++c) half_split(x[2 * c], x[2 * c + 1], scale.up, ph[4 * c], pl[4 * c]);
+                            if (t4 == 0) sSc[(c0 >> 5) * N + r] = scale.down;
+                        }
+                        // Where no value is less than 2^-23 of the largest of its 32, the column in which a row of the state has
+                        // its largest brings at least 2^-23 a_max b_max, and the 2^-51 a_max that its smallest values may lose
+                        // are no more than 2^-23 of what the products come to.  Else the state is looked at below.
+                        if (__any_sync(0xffffffffu, least_of(x) < scale.top * 0x1p-23f)) {
+                            const uint32_t raw = __ballot_sync(0xffffffffu, scale.loses(x));
+                            if (lane == 0) atomicOr(sUneven, (raw ? 257 : 1) << (c0 >> 5));
+                            // what does not fit fp16 pairs stays as it is, in halves, under a scale of zero
+                            if (r < 8 * nt && (raw >> (lane & 28) & 15u) != 0u) {
+#pragma unroll
+                                for (int c = 0; c < 4; ++c) {
+                                    const uint32_t x0 = __float_as_uint(x[2 * c]), x1 = __float_as_uint(x[2 * c + 1]);
+                                    ph[4 * c] = __byte_perm(x0, x1, 0x7632);
+                                    pl[4 * c] = __byte_perm(x0, x1, 0x5410);
+                                }
+                                if (t4 == 0) sSc[(c0 >> 5) * N + r] = 0.f;
+                            }
                         }
                         continue;
                     }
@@ -563,6 +610,50 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
         float *o0 = p.o + rec0 * p.DV + row0 + g;
         const long node_stride = long(H) * p.DV;
         float zero = 0.f;                                        // the sum of the outputs times zero
+        // adds the value term and writes the outputs
+        auto finish_tile = [&](int tile, float (&hh)[NTP][4], float (&xx)[NTP][4]) {
+            // value term: rows of V^T (16 value rows x 16 nodes) x M, piece by piece
+            {
+                const __nv_bfloat16 *va = sV + ((lane & 7) + ((lane >> 4) << 3)) * vstride + tile * 16 + (lane & 8);
+#pragma unroll
+                for (int kk = 0; kk < LY::NK / 16; ++kk) {
+                    if (LY::NK > 16 && kk >= nk) break;
+                    uint32_t a[4];
+                    ldsm_x4_t(a, va + kk * 16 * vstride);
+#pragma unroll
+                    for (int i = 0; i < NTP; ++i) {
+                        if (NTP > 1 && i >= ntp) break;
+                        if (8 * (i0 + i) + 7 < 16 * kk) continue;       // a node's path holds no later node
+                        float lo[4], hi[4];
+#pragma unroll
+                        for (int pc = 2; pc >= 0; --pc) {
+                            const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
+                            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(mb);
+                            const uint32_t b1 = *reinterpret_cast<const uint32_t *>(mb + 8);
+                            if (pc == 2) warp_mma_bf16_first(lo, a, b0, b1);
+                            else if (pc == 1) warp_mma_bf16(lo, a, b0, b1);
+                            else warp_mma_bf16_first(hi, a, b0, b1);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) { hh[i][e] += hi[e]; xx[i][e] += lo[e]; }
+                    }
+                }
+            }
+            float *ot = o0 + tile * 16;
+#pragma unroll
+            for (int i = 0; i < NTP; ++i) {
+                if (NTP > 1 && i >= ntp) break;
+                const int n0 = 8 * (i0 + i) + 2 * t4;
+                float *od = ot + n0 * node_stride;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    hh[i][e] += xx[i][e];
+                    zero = fmaf(hh[i][e], 0.f, zero);
+                }
+                if (n0 < n) { od[0] = hh[i][0]; od[8] = hh[i][2]; }
+                if (n0 + 1 < n) { od[node_stride] = hh[i][1]; od[node_stride + 8] = hh[i][3]; }
+            }
+        };
 #pragma unroll 1
         for (int tile = warp / PARTS; tile < tile_end; tile += STRIDE) {
             if (lane == 0 && half == 0 && tile + AHEAD < tiles) prefetch_l2(S_cta + long(tile + AHEAD) * 16 * DK, 16 * DK * 4);
@@ -578,16 +669,14 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                 if constexpr (LY::kHalf) {
                     // k-steps j = 0, 1 of 16 contract columns 8 t + 4 j .. + 3 of the four lanes
                     uint32_t ah[2][4], al[2][4];
-                    float up_a, down_a, up_b, down_b;
-                    half_scale(row_max(sa[q & 1]), up_a, down_a);
-                    half_scale(row_max(sb[q & 1]), up_b, down_b);
+                    const HalfScale scale_a(row_max(sa[q & 1])), scale_b(row_max(sb[q & 1]));
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
 #pragma unroll
                         for (int c = 0; c < 2; ++c) {
                             const int e = 4 * j + 2 * c;
-                            half_split(sa[q & 1][e] * up_a, sa[q & 1][e + 1] * up_a, ah[j][2 * c], al[j][2 * c]);
-                            half_split(sb[q & 1][e] * up_b, sb[q & 1][e + 1] * up_b, ah[j][2 * c + 1], al[j][2 * c + 1]);
+                            half_split(sa[q & 1][e], sa[q & 1][e + 1], scale_a.up, ah[j][2 * c], al[j][2 * c]);
+                            half_split(sb[q & 1][e], sb[q & 1][e + 1], scale_b.up, ah[j][2 * c + 1], al[j][2 * c + 1]);
                         }
                     if (q + 2 < NS || next) {
                         const float *src = (q + 2 < NS ? cur : nxt) + 32 * (q + 2);
@@ -600,17 +689,22 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                         const uint4 bh = *reinterpret_cast<const uint4 *>(hh_p + 8 * i * LY::BSH + 32 * q);
                         const uint4 bl = *reinterpret_cast<const uint4 *>(hl_p + 8 * i * LY::BSH + 32 * q);
                         const float2 sc = *reinterpret_cast<const float2 *>(sSc + q * N + 8 * (i0 + i) + 2 * t4);
-                        float part[4];                           // small products first
-                        warp_mma_f16<true>(part, al[0], bh.x, bh.y);
-                        warp_mma_f16<false>(part, al[1], bh.z, bh.w);
-                        warp_mma_f16<false>(part, ah[0], bl.x, bl.y);
-                        warp_mma_f16<false>(part, ah[1], bl.z, bl.w);
-                        warp_mma_f16<false>(part, ah[0], bh.x, bh.y);
+                        float low[4], part[4];
+                        warp_mma_f16<true>(low, al[0], bh.x, bh.y);
+                        warp_mma_f16<true>(part, ah[0], bh.x, bh.y);
+                        warp_mma_f16<false>(low, al[1], bh.z, bh.w);
                         warp_mma_f16<false>(part, ah[1], bh.z, bh.w);
-                        hh[i][0] = fmaf(part[0] * down_a, sc.x, hh[i][0]);
-                        hh[i][1] = fmaf(part[1] * down_a, sc.y, hh[i][1]);
-                        hh[i][2] = fmaf(part[2] * down_b, sc.x, hh[i][2]);
-                        hh[i][3] = fmaf(part[3] * down_b, sc.y, hh[i][3]);
+                        warp_mma_f16<false>(low, ah[0], bl.x, bl.y);
+                        warp_mma_f16<false>(low, ah[1], bl.z, bl.w);
+#pragma unroll
+                        for (int e = 0; e < 4; e += 2) {
+                            const float down = e < 2 ? scale_a.down : scale_b.down;
+                            float2 x = __ffma2_rn(make_float2(low[e], low[e + 1]), make_float2(kLowPiece, kLowPiece),
+                                                  make_float2(part[e], part[e + 1]));
+                            x = __ffma2_rn(__fmul2_rn(x, make_float2(down, down)), sc, make_float2(hh[i][e], hh[i][e + 1]));
+                            hh[i][e] = x.x;
+                            hh[i][e + 1] = x.y;
+                        }
                     }
                     continue;
                 }
@@ -645,45 +739,57 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                     for (int e = 0; e < 4; ++e) hh[i][e] += part[e];
                 }
             }
-            // value term: rows of V^T (16 value rows x 16 nodes) x M, piece by piece
-            {
-                const __nv_bfloat16 *va = sV + ((lane & 7) + ((lane >> 4) << 3)) * vstride + tile * 16 + (lane & 8);
+            finish_tile(tile, hh, xx);
+        }
+        // Where the effective queries are uneven, tiles that do not fit fp16 pairs, or all of them if the queries do not: once
+        // more, in TF32 as below 17 nodes.  (Looking for such tiles in the loop above cost 2 to 10 % of a call.)
+        if (LY::kHalf && *sUneven != 0) {
+            const int uneven = *sUneven;                         // (bits 8 ..: steps with queries that do not fit)
+#pragma unroll 1
+            for (int tile = warp / PARTS; tile < tile_end; tile += STRIDE) {
+                const float *cur = Su + long(tile) * 16 * DK;
+                bool loses = uneven >= 256;
+#pragma unroll 1
+                for (int q = 0; q < NS && uneven < 256; ++q) {
+                    if (!(uneven >> q & 1)) continue;
+                    float xa[8], xb[8];
+                    ld_state(xa, cur + 32 * q);
+                    ld_state(xb, cur + 32 * q + 8 * DK);
+                    const HalfScale scale_a(row_max(xa)), scale_b(row_max(xb));
+                    loses |= scale_a.loses(xa) || scale_b.loses(xb);
+                }
+                if (!__any_sync(0xffffffffu, loses)) continue;
+                float hh[NTP][4] = {}, xx[NTP][4] = {};
+#pragma unroll 1
+                for (int q = 0; q < NS; ++q) {
+                    float part[NTP][4] = {};
+#pragma unroll 1
+                    for (int e = 32 * q; e < 32 * q + 8; e += 2) {
+                        const float2 xa = *reinterpret_cast<const float2 *>(cur + e), xb = *reinterpret_cast<const float2 *>(cur + e + 8 * DK);
+                        const uint32_t ah[4] = {tf32_head(xa.x), tf32_head(xb.x), tf32_head(xa.y), tf32_head(xb.y)};
+                        const uint32_t al[4] = {tf32_tail(xa.x), tf32_tail(xb.x), tf32_tail(xa.y), tf32_tail(xb.y)};
 #pragma unroll
-                for (int kk = 0; kk < LY::NK / 16; ++kk) {
-                    if (LY::NK > 16 && kk >= nk) break;
-                    uint32_t a[4];
-                    ldsm_x4_t(a, va + kk * 16 * vstride);
-#pragma unroll
-                    for (int i = 0; i < NTP; ++i) {
-                        if (NTP > 1 && i >= ntp) break;
-                        if (8 * (i0 + i) + 7 < 16 * kk) continue;       // a node's path holds no later node
-                        float lo[4], hi[4];
-#pragma unroll
-                        for (int pc = 2; pc >= 0; --pc) {
-                            const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
-                            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(mb), b1 = *reinterpret_cast<const uint32_t *>(mb + 8);
-                            if (pc == 2) warp_mma_bf16_first(lo, a, b0, b1);
-                            else if (pc == 1) warp_mma_bf16(lo, a, b0, b1);
-                            else warp_mma_bf16_first(hi, a, b0, b1);
+                        for (int i = 0; i < NTP; ++i) {
+                            if (NTP > 1 && i >= ntp) break;
+                            const uint32_t hi = *reinterpret_cast<const uint32_t *>(hh_p + 8 * i * LY::BSH + e);
+                            const uint32_t lo = *reinterpret_cast<const uint32_t *>(hl_p + 8 * i * LY::BSH + e);
+                            const float sc = sSc[q * N + 8 * (i0 + i) + g];
+                            const float2 h = __half22float2(as_half2(hi)), l = __half22float2(as_half2(lo));
+                            float w0 = fmaf(l.x, kLowPiece, h.x) * sc, w1 = fmaf(l.y, kLowPiece, h.y) * sc;
+                            w0 = sc != 0.f ? w0 : __uint_as_float(__byte_perm(lo, hi, 0x5410));
+                            w1 = sc != 0.f ? w1 : __uint_as_float(__byte_perm(lo, hi, 0x7632));
+                            const uint32_t b0 = tf32_head(w0), b1 = tf32_head(w1);
+                            warp_mma_tf32(xx[i], al, b0, b1);
+                            warp_mma_tf32(xx[i], ah, tf32_tail(w0), tf32_tail(w1));
+                            warp_mma_tf32(part[i], ah, b0, b1);
                         }
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) { hh[i][e] += hi[e]; xx[i][e] += lo[e]; }
                     }
-                }
-            }
-            float *ot = o0 + tile * 16;
 #pragma unroll
-            for (int i = 0; i < NTP; ++i) {
-                if (NTP > 1 && i >= ntp) break;
-                const int n0 = 8 * (i0 + i) + 2 * t4;
-                float *od = ot + n0 * node_stride;
+                    for (int i = 0; i < NTP; ++i)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    hh[i][e] += xx[i][e];
-                    zero = fmaf(hh[i][e], 0.f, zero);
+                        for (int e = 0; e < 4; ++e) hh[i][e] += part[i][e];
                 }
-                if (n0 < n) { od[0] = hh[i][0]; od[8] = hh[i][2]; }
-                if (n0 + 1 < n) { od[node_stride] = hh[i][1]; od[node_stride + 8] = hh[i][3]; }
+                finish_tile(tile, hh, xx);
             }
         }
         const bool odd = __syncthreads_or(!(zero == 0.f));
