@@ -98,15 +98,17 @@ template <bool FIRST> __device__ __forceinline__ void warp_mma_f16(float (&d)[4]
             : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
             : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// Scale of a group of values of which the largest is m: the power of two that brings m into [2^14, 2^15), and its inverse (m
-// below 2^-112 counts as that).
+// Scale of a group of values of which the largest is m: the power of two that brings m into [2^14, 2^15), and the one that m
+// has (m below 2^-112 counts as that).  32 products of two scaled values come to less than 2^36.  What undoes the scales is
+// multiplied in so that no step leaves the range unless the result does: 2^-35 size of the state first, then 2^7 size of the
+// effective query (up to kMostHalf, beyond that TF32).
 struct HalfScale {
-    float up, down, top;
-    __device__ __forceinline__ explicit HalfScale(float m) : top(m)
+    float up, size;
+    __device__ __forceinline__ explicit HalfScale(float m)
     {
         const uint32_t e = max(__float_as_uint(m) & 0x7f800000u, 15u << 23);
         up = __uint_as_float((268u << 23) - e);
-        down = __uint_as_float(e - (14u << 23));
+        size = __uint_as_float(e);
     }
     // some value that is not zero does not keep its bits in a pair (in a group that is not finite all others)
     __device__ __forceinline__ bool loses(const float (&x)[8]) const
@@ -118,6 +120,7 @@ struct HalfScale {
     }
 };
 constexpr float kLowPiece = 1.f / 2048.f;                        // what a low piece counts
+constexpr float kUndoState = 0x1p-35f, kUndoQuery = 0x1p7f, kMostHalf = 0x1p120f;
 __device__ __forceinline__ __half2 as_half2(uint32_t x) { return *reinterpret_cast<const __half2 *>(&x); }
 // Two values, scaled, as a pair of fp16 and 2^11 times what is left of them as another, both rounded.  At most 2^-23 of a value
 // is lost, as with TF32, down to 2^-27 of the largest of its group; below that 2^-51 of the largest.  (Were the low piece not
@@ -558,19 +561,20 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                         float x[8];
 #pragma unroll
                         for (int c = 0; c < 4; ++c) { x[2 * c] = acc[c][2 * half]; x[2 * c + 1] = acc[c][2 * half + 1]; }
-                        const HalfScale scale(row_max(x));
+                        const float top = row_max(x);
+                        const HalfScale scale(top);
                         uint32_t *ph = reinterpret_cast<uint32_t *>(hHi + r * LY::BSH + c0 + 2 * t4);
                         uint32_t *pl = reinterpret_cast<uint32_t *>(hLo + r * LY::BSH + c0 + 2 * t4);
                         if (r < 8 * nt) {
 #pragma unroll
                             for (int c = 0; c < 4; ++c) half_split(x[2 * c], x[2 * c + 1], scale.up, ph[4 * c], pl[4 * c]);
-                            if (t4 == 0) sSc[(c0 >> 5) * N + r] = scale.down;
+                            if (t4 == 0) sSc[(c0 >> 5) * N + r] = scale.size * kUndoQuery;
                         }
                         // Where no value is less than 2^-23 of the largest of its 32, the column in which a row of the state has
                         // its largest brings at least 2^-23 a_max b_max, and the 2^-51 a_max that its smallest values may lose
                         // are no more than 2^-23 of what the products come to.  Else the state is looked at below.
-                        if (__any_sync(0xffffffffu, least_of(x) < scale.top * 0x1p-23f)) {
-                            const uint32_t raw = __ballot_sync(0xffffffffu, scale.loses(x));
+                        if (__any_sync(0xffffffffu, least_of(x) < top * 0x1p-23f || top > kMostHalf)) {
+                            const uint32_t raw = __ballot_sync(0xffffffffu, scale.loses(x) || top > kMostHalf);
                             if (lane == 0) atomicOr(sUneven, (raw ? 257 : 1) << (c0 >> 5));
                             // what does not fit fp16 pairs stays as it is, in halves, under a scale of zero
                             if (r < 8 * nt && (raw >> (lane & 28) & 15u) != 0u) {
@@ -698,7 +702,7 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                         warp_mma_f16<false>(low, ah[1], bl.z, bl.w);
 #pragma unroll
                         for (int e = 0; e < 4; e += 2) {
-                            const float down = e < 2 ? scale_a.down : scale_b.down;
+                            const float down = (e < 2 ? scale_a.size : scale_b.size) * kUndoState;
                             float2 x = __ffma2_rn(make_float2(low[e], low[e + 1]), make_float2(kLowPiece, kLowPiece),
                                                   make_float2(part[e], part[e + 1]));
                             x = __ffma2_rn(__fmul2_rn(x, make_float2(down, down)), sc, make_float2(hh[i][e], hh[i][e + 1]));
@@ -775,7 +779,8 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                             const uint32_t lo = *reinterpret_cast<const uint32_t *>(hl_p + 8 * i * LY::BSH + e);
                             const float sc = sSc[q * N + 8 * (i0 + i) + g];
                             const float2 h = __half22float2(as_half2(hi)), l = __half22float2(as_half2(lo));
-                            float w0 = fmaf(l.x, kLowPiece, h.x) * sc, w1 = fmaf(l.y, kLowPiece, h.y) * sc;
+                            constexpr float kOne = 0x1p-14f / kUndoQuery;        // of a scaled value, under what undoes its scale
+                            float w0 = fmaf(l.x, kLowPiece, h.x) * kOne * sc, w1 = fmaf(l.y, kLowPiece, h.y) * kOne * sc;
                             w0 = sc != 0.f ? w0 : __uint_as_float(__byte_perm(lo, hi, 0x5410));
                             w1 = sc != 0.f ? w1 : __uint_as_float(__byte_perm(lo, hi, 0x7632));
                             const uint32_t b0 = tf32_head(w0), b1 = tf32_head(w1);

@@ -89,3 +89,13 @@ def test_columns_of_every_magnitude(d_k, d_v, n, depth):
     prob.q[:] = synth.f32_to_bf16_bits((synth.bf16_bits_to_f32(prob.q) / columns).astype(np.float32))
     prob.S0[rng.random(prob.S0.shape) < 0.01] = 0.0
     assert error_norm(prob, n) <= TOL_PRODUCTS
+
+
+@pytest.mark.parametrize("d_k,d_v,n,depth", SHAPES)
+@pytest.mark.parametrize("state,query", [(112, 0), (118, 0), (118, -30), (-30, 118), (-60, 122), (-100, 0), (-60, -40), (60, 60)])
+def test_results_inside_the_range_stay_inside(d_k, d_v, n, depth, state, query):
+    """State and queries of 2^state and 2^query: the products are of 2^(state + query), and so are the outputs."""
+    prob = state_only(d_k, d_v, n, depth)
+    prob.S0 *= np.float32(2.0 ** state)
+    prob.q[:] = synth.f32_to_bf16_bits((synth.bf16_bits_to_f32(prob.q) * np.float32(2.0 ** query)).astype(np.float32))
+    assert error_norm(prob, n) <= TOL_PRODUCTS
