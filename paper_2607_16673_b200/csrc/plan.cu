@@ -799,6 +799,8 @@ prune_small_kernel(int32_t B, int32_t N, float tau, int32_t budget, const int32_
                    int32_t *__restrict__ out_index, int32_t *status)
 {
     after_previous_kernel();
+    // (every CTA of the cluster has to have started before its shared memory is written; waited for below, behind the loads)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     __shared__ int32_t s_count[kPruneSeqs];
     __shared__ __align__(16) float s_q[kPruneSeqs / kPruneCtas][64];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = warp * kPruneCtas + blockIdx.x;
@@ -887,12 +889,15 @@ prune_small_kernel(int32_t B, int32_t N, float tau, int32_t budget, const int32_
     const int count = __popcll(kept);
 
     // every CTA learns every count
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     const uint32_t slot = uint32_t(__cvta_generic_to_shared(&s_count[b]));
     if (lane < kPruneCtas) {
         uint32_t remote;
         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(slot), "r"(lane));
         asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote), "r"(count) : "memory");
     }
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (b >= B) return;
     int dst = 0;
