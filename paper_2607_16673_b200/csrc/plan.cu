@@ -858,9 +858,9 @@ prune_small_kernel(int32_t B, int32_t N, float tau, int32_t budget, const int32_
 #pragma unroll
         for (int k = 0; k < 2; ++k)
             if (now[k]) q[lane + 32 * k] = mine[k];
+        __syncwarp();
         done |= set_of(now[0], now[1]);
     }
-    __syncwarp();
     float best = fmaxf(mine[0], mine[1]);
     for (int off = 16; off; off >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, off));
     best = fmaxf(best, -INFINITY);

@@ -1,5 +1,6 @@
 """Shared memory that one thread writes and another reads, in the source: stores into another CTA's shared memory come after all
-CTAs of the cluster have started, and are waited for before they are read."""
+CTAs of the cluster have started, and are waited for before they are read; between the lanes of a warp stands a __syncwarp, since
+votes and reductions order no memory."""
 import os
 import re
 
@@ -47,3 +48,26 @@ def test_other_ctas_have_started_before_their_memory_is_written(name, kernel):
     assert not re.search(r"\breturn;", text[:last])                 # nobody leaves before
     assert "release" in text[last:].split("barrier.cluster.arrive")[1][:20]
     assert "acquire" in text[last:].split("barrier.cluster.wait")[1][:20]
+
+
+# file, function, how the loop around both starts (None: they follow one another), the write, the read by other lanes
+HANDED_OVER = [
+    ("plan.cu", "accept_kernel", None, "target[t] = target_tok[base + t];", "target[p];"),
+    ("plan.cu", "accept_kernel", None, "step[t] = ", "a = step[a];"),
+    ("plan.cu", "stochastic_accept_kernel", None, "first[t] = kStochNodes;", "atomicMin(&first"),
+    ("plan.cu", "stochastic_accept_kernel", None, "atomicMin(&first", "first[pa + 1] != a"),
+    ("plan.cu", "prune_small_kernel", None, "q[lane + 32 * k] = mine[k];", "q[par[k]]"),
+    ("plan.cu", "prune_small_kernel", "while (done", "q[lane + 32 * k] = mine[k];", "q[par[k]]"),
+    ("plan.cu", "prune_small_kernel", "while (done", "q[par[k]]", "q[lane + 32 * k] = mine[k];"),
+]
+
+
+@pytest.mark.parametrize("name,func,loop,write,read", HANDED_OVER)
+def test_lanes_synchronise_between_writing_and_reading(name, func, loop, write, read):
+    text = function(name, func)
+    if loop:
+        text = 2 * block(text, text.index(loop))                     # one turn and the next
+        text = text[text.index(write):]
+    between = text[text.index(write):]
+    between = between[:between.index(read)]
+    assert re.search(r"__sync(warp|threads)\(\)", between)
