@@ -323,6 +323,7 @@ __device__ __forceinline__ void plan_paths(const Params &p, int warp, int n_warp
                 par[i] = int8_t(pa);
             }
             fault = __reduce_or_sync(0xffffffffu, fault);
+            __syncwarp();                                        // (the reduction orders no memory)
         }
         if (!fault)
             for (int i = lane; i < n; i += 32) {
