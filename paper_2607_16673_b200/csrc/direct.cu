@@ -260,6 +260,69 @@ struct Unit {
     }
 };
 
+// some value of a tile does not keep its bits in an fp16 pair (cur: this lane's part of row g; only the steps given)
+template <int DK> __device__ __forceinline__ bool loses_bits(const float *cur, int steps)
+{
+    bool loses = false;
+#pragma unroll 1
+    for (int q = 0; q < DK / 32; ++q) {
+        if (!(steps >> q & 1)) continue;
+        float xa[8], xb[8];
+        ld_state(xa, cur + 32 * q);
+        ld_state(xb, cur + 32 * q + 8 * DK);
+        const HalfScale scale_a(row_max(xa)), scale_b(row_max(xb));
+        loses |= scale_a.loses(xa) || scale_b.loses(xb);
+    }
+    return __any_sync(0xffffffffu, loses);
+}
+// The product of a tile with the effective queries in TF32 as below 17 nodes; these are put together again from their pairs, or
+// taken as they are where they did not fit.
+template <class LY, int NTP>
+__device__ __forceinline__ void state_in_tf32(float (&x)[NTP][4], const float *cur, const uint16_t *high,
+                                              const uint16_t *low, const float *scale, int ntp)
+{
+    constexpr float kOne = 0x1p-14f / kUndoQuery;                // of a scaled value, under what undoes its scale
+    float xx[NTP][4] = {};                                       // the cross products
+#pragma unroll
+    for (int i = 0; i < NTP; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[i][e] = 0.f;
+#pragma unroll 1
+    for (int q = 0; q < LY::NS; ++q) {
+        float part[NTP][4] = {};
+#pragma unroll 1
+        for (int e = 32 * q; e < 32 * q + 8; e += 2) {
+            const float2 xa = *reinterpret_cast<const float2 *>(cur + e);
+            const float2 xb = *reinterpret_cast<const float2 *>(cur + e + 8 * 32 * LY::NS);
+            const uint32_t ah[4] = {tf32_head(xa.x), tf32_head(xb.x), tf32_head(xa.y), tf32_head(xb.y)};
+            const uint32_t al[4] = {tf32_tail(xa.x), tf32_tail(xb.x), tf32_tail(xa.y), tf32_tail(xb.y)};
+#pragma unroll
+            for (int i = 0; i < NTP; ++i) {
+                if (NTP > 1 && i >= ntp) break;
+                const uint32_t hi = *reinterpret_cast<const uint32_t *>(high + 8 * i * LY::BSH + e);
+                const uint32_t lo = *reinterpret_cast<const uint32_t *>(low + 8 * i * LY::BSH + e);
+                const float sc = scale[q * LY::N + 8 * i];
+                const float2 h = __half22float2(as_half2(hi)), l = __half22float2(as_half2(lo));
+                float w0 = fmaf(l.x, kLowPiece, h.x) * kOne * sc, w1 = fmaf(l.y, kLowPiece, h.y) * kOne * sc;
+                w0 = sc != 0.f ? w0 : __uint_as_float(__byte_perm(lo, hi, 0x5410));
+                w1 = sc != 0.f ? w1 : __uint_as_float(__byte_perm(lo, hi, 0x7632));
+                const uint32_t b0 = tf32_head(w0), b1 = tf32_head(w1);
+                warp_mma_tf32(xx[i], al, b0, b1);
+                warp_mma_tf32(xx[i], ah, tf32_tail(w0), tf32_tail(w1));
+                warp_mma_tf32(part[i], ah, b0, b1);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NTP; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[i][e] += part[i][e];
+    }
+#pragma unroll
+    for (int i = 0; i < NTP; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[i][e] += xx[i][e];
+}
+
 // After a pass with an output that is not finite.  First pass: keys and value elements that are not finite are replaced by
 // zero in shared memory; true if there were any.  Second pass: the value elements are added for the nodes that have them on
 // their path.
@@ -614,50 +677,6 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
         float *o0 = p.o + rec0 * p.DV + row0 + g;
         const long node_stride = long(H) * p.DV;
         float zero = 0.f;                                        // the sum of the outputs times zero
-        // adds the value term and writes the outputs
-        auto finish_tile = [&](int tile, float (&hh)[NTP][4], float (&xx)[NTP][4]) {
-            // value term: rows of V^T (16 value rows x 16 nodes) x M, piece by piece
-            {
-                const __nv_bfloat16 *va = sV + ((lane & 7) + ((lane >> 4) << 3)) * vstride + tile * 16 + (lane & 8);
-#pragma unroll
-                for (int kk = 0; kk < LY::NK / 16; ++kk) {
-                    if (LY::NK > 16 && kk >= nk) break;
-                    uint32_t a[4];
-                    ldsm_x4_t(a, va + kk * 16 * vstride);
-#pragma unroll
-                    for (int i = 0; i < NTP; ++i) {
-                        if (NTP > 1 && i >= ntp) break;
-                        if (8 * (i0 + i) + 7 < 16 * kk) continue;       // a node's path holds no later node
-                        float lo[4], hi[4];
-#pragma unroll
-                        for (int pc = 2; pc >= 0; --pc) {
-                            const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
-                            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(mb);
-                            const uint32_t b1 = *reinterpret_cast<const uint32_t *>(mb + 8);
-                            if (pc == 2) warp_mma_bf16_first(lo, a, b0, b1);
-                            else if (pc == 1) warp_mma_bf16(lo, a, b0, b1);
-                            else warp_mma_bf16_first(hi, a, b0, b1);
-                        }
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) { hh[i][e] += hi[e]; xx[i][e] += lo[e]; }
-                    }
-                }
-            }
-            float *ot = o0 + tile * 16;
-#pragma unroll
-            for (int i = 0; i < NTP; ++i) {
-                if (NTP > 1 && i >= ntp) break;
-                const int n0 = 8 * (i0 + i) + 2 * t4;
-                float *od = ot + n0 * node_stride;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    hh[i][e] += xx[i][e];
-                    zero = fmaf(hh[i][e], 0.f, zero);
-                }
-                if (n0 < n) { od[0] = hh[i][0]; od[8] = hh[i][2]; }
-                if (n0 + 1 < n) { od[node_stride] = hh[i][1]; od[node_stride + 8] = hh[i][3]; }
-            }
-        };
 #pragma unroll 1
         for (int tile = warp / PARTS; tile < tile_end; tile += STRIDE) {
             if (lane == 0 && half == 0 && tile + AHEAD < tiles) prefetch_l2(S_cta + long(tile + AHEAD) * 16 * DK, 16 * DK * 4);
@@ -743,58 +762,73 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
                     for (int e = 0; e < 4; ++e) hh[i][e] += part[e];
                 }
             }
-            finish_tile(tile, hh, xx);
+            // value term: rows of V^T (16 value rows x 16 nodes) x M, piece by piece
+            {
+                const __nv_bfloat16 *va = sV + ((lane & 7) + ((lane >> 4) << 3)) * vstride + tile * 16 + (lane & 8);
+#pragma unroll
+                for (int kk = 0; kk < LY::NK / 16; ++kk) {
+                    if (LY::NK > 16 && kk >= nk) break;
+                    uint32_t a[4];
+                    ldsm_x4_t(a, va + kk * 16 * vstride);
+#pragma unroll
+                    for (int i = 0; i < NTP; ++i) {
+                        if (NTP > 1 && i >= ntp) break;
+                        if (8 * (i0 + i) + 7 < 16 * kk) continue;       // a node's path holds no later node
+                        float lo[4], hi[4];
+#pragma unroll
+                        for (int pc = 2; pc >= 0; --pc) {
+                            const __nv_bfloat16 *mb = sM + (pc * N + 8 * (i0 + i) + g) * LY::MS + 16 * kk + 2 * t4;
+                            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(mb);
+                            const uint32_t b1 = *reinterpret_cast<const uint32_t *>(mb + 8);
+                            if (pc == 2) warp_mma_bf16_first(lo, a, b0, b1);
+                            else if (pc == 1) warp_mma_bf16(lo, a, b0, b1);
+                            else warp_mma_bf16_first(hi, a, b0, b1);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) { hh[i][e] += hi[e]; xx[i][e] += lo[e]; }
+                    }
+                }
+            }
+            float *ot = o0 + tile * 16;
+#pragma unroll
+            for (int i = 0; i < NTP; ++i) {
+                if (NTP > 1 && i >= ntp) break;
+                const int n0 = 8 * (i0 + i) + 2 * t4;
+                float *od = ot + n0 * node_stride;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    hh[i][e] += xx[i][e];
+                    zero = fmaf(hh[i][e], 0.f, zero);
+                }
+                if (n0 < n) { od[0] = hh[i][0]; od[8] = hh[i][2]; }
+                if (n0 + 1 < n) { od[node_stride] = hh[i][1]; od[node_stride + 8] = hh[i][3]; }
+            }
         }
-        // Where the effective queries are uneven, tiles that do not fit fp16 pairs, or all of them if the queries do not: once
-        // more, in TF32 as below 17 nodes.  (Looking for such tiles in the loop above cost 2 to 10 % of a call.)
-        if (LY::kHalf && *sUneven != 0) {
+        // Where the effective queries are uneven, the tiles that do not fit fp16 pairs, or all of them if the queries do not, are
+        // done once more.  (Looking for such tiles in the loop above cost 2 to 10 % of a call, doing them there up to 20 %.)
+        if constexpr (LY::kHalf) {
             const int uneven = *sUneven;                         // (bits 8 ..: steps with queries that do not fit)
 #pragma unroll 1
-            for (int tile = warp / PARTS; tile < tile_end; tile += STRIDE) {
+            for (int tile = warp / PARTS; uneven != 0 && tile < tile_end; tile += STRIDE) {
                 const float *cur = Su + long(tile) * 16 * DK;
-                bool loses = uneven >= 256;
-#pragma unroll 1
-                for (int q = 0; q < NS && uneven < 256; ++q) {
-                    if (!(uneven >> q & 1)) continue;
-                    float xa[8], xb[8];
-                    ld_state(xa, cur + 32 * q);
-                    ld_state(xb, cur + 32 * q + 8 * DK);
-                    const HalfScale scale_a(row_max(xa)), scale_b(row_max(xb));
-                    loses |= scale_a.loses(xa) || scale_b.loses(xb);
-                }
-                if (!__any_sync(0xffffffffu, loses)) continue;
-                float hh[NTP][4] = {}, xx[NTP][4] = {};
-#pragma unroll 1
-                for (int q = 0; q < NS; ++q) {
-                    float part[NTP][4] = {};
-#pragma unroll 1
-                    for (int e = 32 * q; e < 32 * q + 8; e += 2) {
-                        const float2 xa = *reinterpret_cast<const float2 *>(cur + e), xb = *reinterpret_cast<const float2 *>(cur + e + 8 * DK);
-                        const uint32_t ah[4] = {tf32_head(xa.x), tf32_head(xb.x), tf32_head(xa.y), tf32_head(xb.y)};
-                        const uint32_t al[4] = {tf32_tail(xa.x), tf32_tail(xb.x), tf32_tail(xa.y), tf32_tail(xb.y)};
+                if (uneven < 256 && !loses_bits<DK>(cur, uneven)) continue;
+                float x[NTP][4];
+                state_in_tf32<LY, NTP>(x, cur, hh_p, hl_p, sSc + 8 * i0 + g, ntp);
+                // the value term in plain fp32, node by node up the path
 #pragma unroll
-                        for (int i = 0; i < NTP; ++i) {
-                            if (NTP > 1 && i >= ntp) break;
-                            const uint32_t hi = *reinterpret_cast<const uint32_t *>(hh_p + 8 * i * LY::BSH + e);
-                            const uint32_t lo = *reinterpret_cast<const uint32_t *>(hl_p + 8 * i * LY::BSH + e);
-                            const float sc = sSc[q * N + 8 * (i0 + i) + g];
-                            const float2 h = __half22float2(as_half2(hi)), l = __half22float2(as_half2(lo));
-                            constexpr float kOne = 0x1p-14f / kUndoQuery;        // of a scaled value, under what undoes its scale
-                            float w0 = fmaf(l.x, kLowPiece, h.x) * kOne * sc, w1 = fmaf(l.y, kLowPiece, h.y) * kOne * sc;
-                            w0 = sc != 0.f ? w0 : __uint_as_float(__byte_perm(lo, hi, 0x5410));
-                            w1 = sc != 0.f ? w1 : __uint_as_float(__byte_perm(lo, hi, 0x7632));
-                            const uint32_t b0 = tf32_head(w0), b1 = tf32_head(w1);
-                            warp_mma_tf32(xx[i], al, b0, b1);
-                            warp_mma_tf32(xx[i], ah, tf32_tail(w0), tf32_tail(w1));
-                            warp_mma_tf32(part[i], ah, b0, b1);
+                for (int i = 0; i < NTP; ++i)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int node = 8 * (i0 + i) + 2 * t4 + (e & 1), r = 16 * tile + (e & 2) * 4;
+                        if (node >= n) continue;
+                        for (int a = node; a >= 0; a = sPar[a]) {
+                            const __nv_bfloat16 *m = sM + node * LY::MS + a;
+                            const float low = __bfloat162float(m[N * LY::MS]) + __bfloat162float(m[2 * N * LY::MS]);
+                            x[i][e] = fmaf(__bfloat162float(m[0]) + low, __bfloat162float(sV[a * vstride + r + g]), x[i][e]);
                         }
+                        zero = fmaf(x[i][e], 0.f, zero);
+                        o0[node * node_stride + r] = x[i][e];
                     }
-#pragma unroll
-                    for (int i = 0; i < NTP; ++i)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) hh[i][e] += part[i][e];
-                }
-                finish_tile(tile, hh, xx);
             }
         }
         const bool odd = __syncthreads_or(!(zero == 0.f));
