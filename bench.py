@@ -1011,7 +1011,7 @@ def run_sweep(args):
         torch.cuda.synchronize()
         return e0.elapsed_time(e1) / reps
 
-    S = synth.device_state(1, L, B, H, dk, dv, 0.02, dev)
+    S = synth.device_state(1, L, B, H, dk, dv, 0.02, dev) if args.sweep != "role-waits" else None
     status = torch.zeros(1, dtype=torch.int32, device=dev)
     rows = []
     if args.sweep == "commit-len":
@@ -1037,22 +1037,33 @@ def run_sweep(args):
                               "SPECA_NVCC_FLAGS=-DSPECA_PROF python -m paper_2607_16673_b200.build --force"}))
             return
         L = args.layers or 4
-        S = synth.device_state(1, L, B, H, dk, dv, 0.02, dev)
-        effective = {0: "state TMA", 1: "state product issuer", 2: "Gram and second product issuer", 3: "records TMA",
-                     4: "split group 0", 8: "split group 1", 12: "epilogue, even chunks", 16: "epilogue, odd chunks", 20: "solver"}
-        roles = {0: effective, 4: effective,
-                 3: {0: "TMA producer", 1: "MMA issuer", 2: "preparation", 6: "epilogue group 0", 10: "epilogue group 1"}}
+        first = {0: "state TMA", 1: "state product issuer", 2: "Gram and second product issuer", 3: "records TMA", 4: "split group 0"}
+        single_pass = {0: "TMA producer", 1: "MMA issuer", 2: "preparation", 6: "epilogue group 0", 10: "epilogue group 1"}
+        # the effective-query kernel has two split groups up to 8 levels, beyond that one
+        effective = {8: {**first, 8: "split group 1", 12: "epilogue, even chunks", 16: "epilogue, odd chunks", 20: "solver"},
+                     16: {**first, 8: "epilogue, even chunks", 12: "epilogue, odd chunks", 16: "solver"}}
         sm = torch.cuda.get_device_properties(dev).multi_processor_count
-        for wl in ("chains8", "trees64", "cfg5"):
-            hi = host_round_inputs(wl, B, 5000)
-            q, k, v, al, be = synth.device_records(7, L, hi["T"], H, dk, dv, dev)
+        rng = np.random.default_rng(5000)
+        units = [("chains8", dk, 8, None), ("trees64", dk, 8, None), ("cfg5", dk, 8, None)]
+        if args.route != speca.ROUTE_TF32:
+            units += [("trees of 64, 16 levels", dk, 16, 64), ("trees of 30, d_k = 256", 256, 8, 30)]
+        for wl, width, levels, nodes in units:
+            if nodes is None:
+                hi = host_round_inputs(wl, B, 5000)
+            else:
+                trees = [synth.random_tree_parent(nodes, levels, 4, rng) for _ in range(B)]
+                hi = dict(node_offsets=np.arange(0, nodes * B + 1, nodes, dtype=np.int32), T=nodes * B,
+                          parent=np.concatenate(trees).astype(np.int32))
+            if S is None or S.shape[-1] != width:
+                S = synth.device_state(1, L, B, H, width, dv, 0.02, dev)
+            q, k, v, al, be = synth.device_records(7, L, hi["T"], H, width, dv, dev)
             offs, par = t(hi["node_offsets"]), t(hi["parent"])
             o = torch.empty(L, hi["T"], H, dv, device=dev)
-            dims = speca.Dims(L, B, H, dk, dv, 1.0, 8, 64, args.route)
+            dims = speca.Dims(L, B, H, width, dv, 1.0, levels, 64 if width < 256 else 32, args.route)
             ws = speca.alloc_workspace(dims, hi["T"], dev)
             ms = timed(lambda: speca.verify_tree(dims, S, q, k, v, al, be, offs, hi["T"], par, None, o, None, ws, status), reps=1)
             ctrl = ws[:2048].cpu().numpy().view(np.int64)
-            for w, name in roles.get(args.route, roles[0]).items():
+            for w, name in (single_pass if args.route == speca.ROUTE_TF32 else effective[levels]).items():
                 vals = ctrl[8 + w * 9: 8 + w * 9 + 9]
                 if vals[8] > 0:
                     rows.append({"units": wl, "warp": w, "role": name, "life_kcycles": float(vals[8]) / 1e3,
