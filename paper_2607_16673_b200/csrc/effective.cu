@@ -327,18 +327,7 @@ __device__ __forceinline__ void plan_paths(const Params &p, int warp, int n_warp
         }
         if (!fault)
             for (int i = lane; i < n; i += 32) {
-                uint32_t up[4] = {0u, 0u, 0u, 0u}, lo = 0u, hi = 0u;
-                int d = 0;
-                for (int a = i; a >= 0; a = par[a], ++d) {
-                    const uint32_t byte = uint32_t(a) << (8 * (d & 3));
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) up[w] |= (d >> 2) == w ? byte : 0u;
-                    if (a < 32) lo |= 1u << a;
-                    else hi |= 1u << (a - 32);
-                }
-                p.ws.depth[base + i] = d;
-                reinterpret_cast<int4 *>(p.ws.up)[base + i] = make_int4(int(up[0]), int(up[1]), int(up[2]), int(up[3]));
-                reinterpret_cast<int2 *>(p.ws.set)[base + i] = make_int2(int(lo), int(hi));
+                const int d = write_path(p.ws, base, i, par);
                 if (d > p.max_depth) fault |= SPECA_STATUS_TOO_DEEP;
                 if (p.depth_in != nullptr && p.depth_in[base + i] != d) fault |= SPECA_STATUS_BAD_DEPTH;
             }

@@ -71,18 +71,7 @@ plan_kernel(const int32_t *node_offsets, const int32_t *parent,
         // one 3.5 us, in front of 0.5 ms of verification.
         int flag = 0;
         for (int i = tid; i < n; i += kPlanThreads) {
-            uint32_t up[4] = {0u, 0u, 0u, 0u}, lo = 0u, hi = 0u;
-            int d = 0;
-            for (int a = i; a >= 0; a = par[a], ++d) {
-                const uint32_t byte = uint32_t(a) << (8 * (d & 3));
-#pragma unroll
-                for (int w = 0; w < 4; ++w) up[w] |= (d >> 2) == w ? byte : 0u;
-                if (a < 32) lo |= 1u << a;
-                else hi |= 1u << (a - 32);
-            }
-            ws.depth[base + i] = d;
-            reinterpret_cast<int4 *>(ws.up)[base + i] = make_int4(int(up[0]), int(up[1]), int(up[2]), int(up[3]));
-            reinterpret_cast<int2 *>(ws.set)[base + i] = make_int2(int(lo), int(hi));
+            const int d = write_path(ws, base, i, par);
             if (d > max_depth) flag |= SPECA_STATUS_TOO_DEEP;
             if (depth_in != nullptr && depth_in[base + i] != d) flag |= SPECA_STATUS_BAD_DEPTH;
         }

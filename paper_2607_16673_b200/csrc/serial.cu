@@ -372,14 +372,13 @@ template <int DK, int RS, int WARPS> struct LaunchCommit {
         const long tiles = n_units(p) * (p.DV / ROWS);
         // Two tiles a CTA from four rounds of such CTAs on (d_k = 128, d_v = 256, 1536 units: 74.8 -> 72.0 us); below that
         // twice the CTAs serve the device better, and a 64-wide tile is done before its second is there (24576 units of
-        // d_k = d_v = 64: 162 us, two tiles 166).  Two neighbouring heads of 64 x 64, which share the path, do pay (us, one / two, paths
-        // of three nodes: 4608 units 26.0 / 25.7, 6144 41.7 / 40.6, 9216 61.1 / 57.6, 18432 117.5 / 103.3; of one node 21.4 / 21.7,
-        // 35.1 / 34.7, 51.8 / 52.0, 100.3 / 97.2).
+        // d_k = d_v = 64: 162 us, two tiles 166).  Two neighbouring heads of 64 x 64, which share the path, do pay (us, one /
+        // two, paths of three nodes: 4608 units 26.0 / 25.7, 6144 41.7 / 40.6, 9216 61.1 / 57.6, 18432 117.5 / 103.3; of one
+        // node 21.4 / 21.7, 35.1 / 34.7, 51.8 / 52.0, 100.3 / 97.2).
+        constexpr int HEADS = DK == 64 ? 2 : 1;
         const long round = long(sm_count_of_current_device()) * (2048 / (WARPS * 32) / 2);
-        if (DK > 64 && p.DV % (2 * ROWS) == 0 && tiles >= 8 * round)
-            launch(commit_kernel<DK, RS, WARPS, 2, 1>, unsigned(tiles / 2), WARPS * 32, 0, st, p);
-        else if (DK == 64 && p.DV == ROWS && p.H % 2 == 0 && tiles >= 5 * round)
-            launch(commit_kernel<DK, RS, WARPS, DK == 64 ? 2 : 1, DK == 64 ? 2 : 1>, unsigned(tiles / 2), WARPS * 32, 0, st, p);
+        if (HEADS == 2 ? p.DV == ROWS && p.H % 2 == 0 && tiles >= 5 * round : p.DV % (2 * ROWS) == 0 && tiles >= 8 * round)
+            launch(commit_kernel<DK, RS, WARPS, 2, HEADS>, unsigned(tiles / 2), WARPS * 32, 0, st, p);
         else
             launch(commit_kernel<DK, RS, WARPS, 1, 1>, unsigned(tiles), WARPS * 32, 0, st, p);
         return int(cudaGetLastError());

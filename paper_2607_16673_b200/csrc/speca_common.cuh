@@ -66,6 +66,24 @@ inline Workspace carve_workspace(void *base, int32_t batch, int32_t total_nodes)
     return w;
 }
 
+// Root path of node i of a sequence of at most 64 nodes, upward and as a set, and its depth, into the workspace; the depth.
+template <class Int> __device__ __forceinline__ int write_path(const Workspace &ws, int base, int i, const Int *par)
+{
+    uint32_t up[4] = {0u, 0u, 0u, 0u}, lo = 0u, hi = 0u;
+    int d = 0;
+    for (int a = i; a >= 0; a = par[a], ++d) {
+        const uint32_t byte = uint32_t(a) << (8 * (d & 3));
+#pragma unroll
+        for (int w = 0; w < 4; ++w) up[w] |= (d >> 2) == w ? byte : 0u;
+        if (a < 32) lo |= 1u << a;
+        else hi |= 1u << (a - 32);
+    }
+    ws.depth[base + i] = d;
+    reinterpret_cast<int4 *>(ws.up)[base + i] = make_int4(int(up[0]), int(up[1]), int(up[2]), int(up[3]));
+    reinterpret_cast<int2 *>(ws.set)[base + i] = make_int2(int(lo), int(hi));
+    return d;
+}
+
 // Packed schedule entry written by the plan kernel, one per node, in the order
 // the serial tree walk processes the nodes of a sequence.
 //   bits  0..15  node index (local to the sequence)

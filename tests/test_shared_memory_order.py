@@ -59,8 +59,8 @@ HANDED_OVER = [
     ("plan.cu", "prune_small_kernel", None, "q[lane + 32 * k] = mine[k];", "q[par[k]]"),
     ("plan.cu", "prune_small_kernel", "while (done", "q[lane + 32 * k] = mine[k];", "q[par[k]]"),
     ("plan.cu", "prune_small_kernel", "while (done", "q[par[k]]", "q[lane + 32 * k] = mine[k];"),
-    ("effective.cu", "plan_paths", None, "par[i] = int8_t(pa);", "a = par[a]"),
-    ("effective.cu", "plan_paths", "for (int b = warp;", "a = par[a]", "par[i] = int8_t(pa);"),
+    ("effective.cu", "plan_paths", None, "par[i] = int8_t(pa);", "write_path("),
+    ("effective.cu", "plan_paths", "for (int b = warp;", "write_path(", "par[i] = int8_t(pa);"),
 ]
 
 
