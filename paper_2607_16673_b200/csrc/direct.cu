@@ -44,11 +44,13 @@
 // over 16-row tiles needs two 32-column steps of registers in flight, not whole tiles: 24 warps fit an SM.  Holding
 // whole tiles in registers through the set-up (16 warps) took 5.1 us per 8-node unit and SM instead of 3.9, at 16
 // nodes 8.0 instead of 4.4.
-// Measured (d_k = 128, d_v = 256, 12288 units, the pipelined kernel with its plan in brackets): 8 nodes 298 us = 6.1 TB/s
-// (344 us), 16 nodes 369 us = 5.5 TB/s (377); d_k = d_v = 64, 24576 units of 8 / 30 nodes: 148 / 335 us (serial walk 316 /
-// 1244).  At d_k = 64 a unit of 17 nodes is 6400 warp instructions around 16 KB of state (half of the issue slots, 22 % of HBM);
-// several heads a CTA with their records loaded ahead, or five CTAs an SM instead of four, gained nothing there.  What bounds it: the state stream at 8 nodes (93 % of the copy rate; 83 % at 16), above that the set-up (some
-// thousand instructions a warp between ten barriers, issued every seventh cycle) and at 32 nodes the MMAs.  For a few users, 384 chains of 8: 8.8 us.
+// Measured (d_k = 128, d_v = 256, 12288 units, the pipelined kernel with its plan in brackets): 8 nodes 296 us = 6.1 TB/s
+// (293 us), 16 nodes 372 us = 5.5 TB/s (324 to 357); d_k = d_v = 64, 24576 units of 8 / 17 / 30 nodes: 143 / 270 / 305 us (serial
+// walk 312 / 689 / 1288).  At d_k = 64 a unit of 17 nodes is 6400 warp instructions around 16 KB of state (half of the issue
+// slots, 22 % of HBM); several heads a CTA with their records loaded ahead, or five CTAs an SM instead of four, gained nothing
+// there.  What bounds it: the state stream at 8 nodes (93 % of the copy rate; 83 % at 16), above that the set-up (some thousand
+// instructions a warp between ten barriers, issued every seventh cycle) and at 32 nodes the MMAs.  For a few users, 384 chains
+// of 8: 10.1 us out of HBM.
 #include <algorithm>
 #include <atomic>
 
@@ -87,14 +89,17 @@ __device__ __forceinline__ void warp_mma_bf16_first(float (&d)[4], const uint32_
                  : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
-template <bool FIRST> __device__ __forceinline__ void warp_mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+template <bool FIRST>
+__device__ __forceinline__ void warp_mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     if (FIRST)
-        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+            "{%10, %10, %10, %10};"
             : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
             : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
     else
-        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+            "{%0, %1, %2, %3};"
             : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
             : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -194,19 +199,22 @@ template <int DK, int NT, int MAXD> struct Lay {
     static constexpr bool kHalf = NT >= 4;
     static constexpr int NS = DK / 32;                          // 32-column steps
     static constexpr int BS = DK + 4;                           // floats per effective-query row (16 bytes of padding)
-    static constexpr int BSH = DK + 32;                         // fp16 per effective-query row (64 bytes: eight lanes, two rows, no
-                                                                // conflict)
+    static constexpr int BSH = DK + 32;                         // fp16 per effective-query row (64 bytes: eight lanes, two
+                                                                // rows, no conflict)
     static constexpr int MS = NK + 8;                           // bf16 per row of a piece of M
     static constexpr int GS = N + 1;
     static constexpr int NR = NK;                               // rows of the weight pieces: whole MMA row blocks
     // a node's path holds no later node, so row block m of the weights ends with column 16 m + 15
-    __host__ __device__ static constexpr int w_row(int r) { return 128 * (r >> 4) * ((r >> 4) + 2) + (r & 15) * (16 * (r >> 4) + 24); }
+    __host__ __device__ static constexpr int w_row(int r)
+    {
+        return 128 * (r >> 4) * ((r >> 4) + 2) + (r & 15) * (16 * (r >> 4) + 24);
+    }
     static constexpr int WP = w_row(NR);                        // bf16 per piece
     static constexpr int OffKQ = 0;                             // bf16 [2N][KQS]: key rows, query rows
     static constexpr int OffHi = OffKQ + 2 * N * KQS * 2;       // float [N][BS]
     static constexpr int OffLo = OffHi + (kHalf ? N * BSH * 2 : N * BS * 4);
-    static constexpr int OffS = OffLo + N * BSH * 2;            // kHalf: float [NS][N], what undoes the scale of a node's 32 columns
-    static constexpr int OffG = OffHi;                          // float [2N][GS]: Gram rows of keys, queries (dead before Hi is written)
+    static constexpr int OffS = OffLo + N * BSH * 2;            // kHalf: float [NS][N], undoes the scale of a node's 32 columns
+    static constexpr int OffG = OffHi;                          // float [2N][GS]: Gram rows of keys, queries (dead before Hi)
     static constexpr int kQEnd = kHalf ? OffS + NS * N * 4 : OffLo + N * BS * 4;
     static constexpr int kREnd = kQEnd > OffG + 2 * N * GS * 4 ? kQEnd : (OffG + 2 * N * GS * 4 + 15) & ~15;
     static constexpr int OffM = kREnd;                          // bf16 [3][N][MS]
@@ -587,8 +595,9 @@ verify_direct_kernel(const __grid_constant__ DirectArgs da)
 #pragma unroll
                 for (int c = 0; c < CB; ++c) {
                     // rows past the staged ones weigh nothing; clamp keeps the read inside the buffer
-                    const uint32_t q0 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r0, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
-                    const uint32_t q1 = *reinterpret_cast<const uint32_t *>(sKQ + (N + min(r1, N - 1)) * LY::KQS + c0 + 8 * c + 2 * t4);
+                    const __nv_bfloat16 *pq = sKQ + N * LY::KQS + c0 + 8 * c + 2 * t4;
+                    const uint32_t q0 = *reinterpret_cast<const uint32_t *>(pq + min(r0, N - 1) * LY::KQS);
+                    const uint32_t q1 = *reinterpret_cast<const uint32_t *>(pq + min(r1, N - 1) * LY::KQS);
                     acc[c][0] = g0 * __uint_as_float(q0 << 16); acc[c][1] = g0 * __uint_as_float(q0 & 0xffff0000u);
                     acc[c][2] = r1 < 8 * nt ? g1 * __uint_as_float(q1 << 16) : 0.f;
                     acc[c][3] = r1 < 8 * nt ? g1 * __uint_as_float(q1 & 0xffff0000u) : 0.f;
@@ -897,8 +906,8 @@ int launch_width(const Params &p, int hi, int lo, bool all, int sms, cudaStream_
         return launch_one<DK, 8, MAXD, 8, 2>(p, lo, all, sms, st);
     } else {
         // between two and three units per SM one wave of smaller CTAs beats two of the others (d_k = d_v = 128, 32 nodes: 384
-        // units 24.6 us, with eight warps 26.6; 432 units the same; 576 units take two waves either way; d_v = 256, 384 units of 24 /
-        // 32 nodes 22.1 / 25.6, with eight warps 25.1 / 29.0)
+        // units 24.6 us, with eight warps 26.6; 432 units the same; 576 units take two waves either way; d_v = 256, 384 units
+        // of 24 / 32 nodes 22.1 / 25.6, with eight warps 25.1 / 29.0)
         const long units = long(p.L) * p.B * p.H;
         if constexpr (DK == 128)
             if (p.DV <= 256 && units > 2 * sms && units <= 3 * sms) return launch_one<DK, 4, MAXD, 4, 3>(p, lo, all, sms, st);
@@ -915,11 +924,11 @@ int direct_limit(const Params &p, int d_k, int most, bool piped, bool chain)
     if (!piped) {
         // The alternative is the serial walk, whose time grows with the nodes where this kernel's hardly does.  A chain needs
         // no plan there, so short ones stay with it; how short, by the elements of a unit and of the call.  us, serial / this
-        // one: 64 x 64, 16 units of 4 / 5 / 8 nodes 3.6 / 4.1, 4.1 / 4.1, 5.5 / 4.1, 12288 units of 2 / 3 / 4 nodes 55 / 74,
-        // 72 / 74, 88 / 74; 64 x 32, 12288 units of 4 / 6 nodes 47 / 64, 65 / 65; 128 x 64, 12288 units of 1 / 2 nodes 70 / 92,
-        // 102 / 93, 192 units of 3 / 4 nodes 5.0 / 5.2, 5.9 / 5.3; 64 x 512, 1536 units of 1 / 2 nodes 37 / 49, 54 / 50.  Trees
-        // (with their plan): 64 x 32, 1536 units of 3 / 4 nodes 9.9 / 10.3, 11.7 / 10.3; 128 x 512, 1536 units of 1 / 2 nodes
-        // 71 / 76, 106 / 77, 16 units of 1 node 5.0 / 4.7.
+        // one: 64 x 64, 16 units of 4 / 5 / 8 nodes 3.8 / 4.0, 4.3 / 4.1, 5.8 / 4.0, 12288 units of 2 / 3 / 4 nodes 56 / 71,
+        // 72 / 71, 90 / 71; 64 x 32, 12288 units of 4 / 6 nodes 48 / 64, 65 / 65; 128 x 64, 12288 units of 1 / 2 nodes 72 / 92,
+        // 106 / 93, 192 units of 3 / 4 nodes 5.3 / 5.5, 6.3 / 5.5; 64 x 512, 1536 units of 1 / 2 nodes 37 / 42, 54 / 42.  Trees
+        // (with their plan): 64 x 32, 1536 units of 2 / 3 / 4 nodes 9.9 / 11.5, 11.9 / 11.5, 12.8 / 11.4; 128 x 512, 1536 units
+        // of 1 / 2 nodes 73 / 77, 108 / 78, 16 units of 1 node 5.6 / 5.1.
         const long unit = long(p.DV) * d_k, call = unit * p.L * p.B * p.H;
         const int small_unit = int((d_k == 128 || !chain ? 8191 : 8192) / unit);
         const int few = chain ? std::min(1 + small_unit + (call < 8L << 20) + (call <= 1L << 20), 5)
@@ -927,15 +936,17 @@ int direct_limit(const Params &p, int d_k, int most, bool piped, bool chain)
         // many chains take the time of the mean one, a few that of the longest
         if (chain && call >= 2L << 20 ? p.T <= long(few) * p.B : most <= few) return 0;
         // In a small call the walk of the largest tree is the whole time: where the mean says that there is one left for it, the
-        // others may as well go along (18 units at 64 x 512, trees of up to 68 nodes 47 us, after a launch of this kernel 57).
+        // others may as well go along (18 units at 64 x 512, trees of up to 70 nodes 58 us, after a launch of this kernel 70).
         const int limit = d_k == 64 ? 64 : 32;
         return p.T > long(limit) * p.B && small_batch(p, sm_count_of_current_device()) ? 0 : limit;
     }
-    // us per unit and SM in a large batch, this kernel / the pipelined one with its plan: d_k = 128, d_v = 256: 3.6 / 4.1 at 8
-    // nodes, 4.2 / 4.5 at 12, 4.4 / 4.5 at 16, d_v = 128: 2.1 / 3.6 at 8, 2.5 / 3.5 at 16.  Above that its set-up is the longer
-    // one (6.1 / 5.0 at 20..24 nodes; 8.2 / 6.6 at d_k = 256, 8 nodes; both kernels before their large sums were taken apart,
-    // which costs either 2 to 6 %).  A few users, us per call: d_k = 128, d_v = 128, 384 units of 8 / 16 / 32 nodes 8.8 / 15.8,
-    // 14.8 / 15.4, 16.5 / 16.6; d_k = 256, 8 nodes, 192 units 14.2 / 16.8, 384 units 26.4 / 26.4.
+    // us per unit and SM in a large batch, this kernel / the pipelined one with its plan: d_k = 128, d_v = 256: 3.6 / 3.6 at 8
+    // nodes, 4.1 / 4.0 at 12, 4.5 / 3.9 to 4.3 at 16, 5.6 / 4.3 at 20; d_v = 128: 2.0 / 3.3 at 8, 2.6 / 3.0 at 12 and 16, 3.9 /
+    // 3.1 at 20; d_k = 256, 8 nodes 7.5 / 6.4.  A few users, us per call: d_k = d_v = 128, 384 units of 8 / 16 / 24 / 32 nodes
+    // 10.1 / 14.0, 15.3 / 14.4, 13.3 / 15.3, 15.2 / 15.4; d_v = 256, 192 units 10.1 / 13.9, 15.4 / 14.3, 13.4 / 15.2, 16.1 /
+    // 15.3, 384 units 14.1 / 16.8, 24.0 / 17.4, 20.0 / 19.1, 23.0 / 19.5; d_k = 256, 8 nodes, 192 units 16.3 / 16.0, 384 units
+    // 27.6 / 24.2.  Up to the lines it is the faster kernel or the more accurate one: its error against 64 bits is half of the
+    // other's or less (x 10^-8, 8..32 nodes at d_k = 128 7.3 to 7.9 against 14.5 to 16.4, 8 nodes at d_k = 256 7.9 against 22).
     const bool few = small_batch(p, sm_count_of_current_device());
     const int cap = d_k == 128 ? (few ? 32 : 16) : (few ? 8 : 0);
     return most <= cap ? cap : 0;

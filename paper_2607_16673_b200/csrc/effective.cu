@@ -989,9 +989,11 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     if (sms <= 0) return int(cudaErrorInvalidDevice);
     // Few units leave SMs idle, or with one unit while others work on two.  A head of two value tiles then counts as two
     // heads of one tile that share keys, queries and gates: states, value rows and outputs already lie that way.  The
-    // coefficients are made twice, and a unit's solve takes as long whatever its value rows, so this pays while every half has an SM
-    // of its own (48 units, d_k = 128, 64 nodes: verification 17.4 us, whole units 19.5) and, for up to 8 levels, where
-    // the busiest SM walks fewer tiles of few (192 units: 27.7, whole 29.7; at 16 levels 35.8 / 33.8).
+    // coefficients are made twice, and a unit's solve takes as long whatever its value rows, so this pays while every half has
+    // an SM of its own (us, split / whole, d_k = 128, 64 nodes, 48 units: 10.5 / 12.3, at 16 levels 11.6 / 13.2; d_k = 256, 32
+    // nodes 9.8 / 11.4, 10.7 / 12.3) and, for up to 8 levels, where the busiest SM walks fewer tiles of few (192 units 18.6 /
+    // 19.2 and 17.8 / 18.6, at 16 levels 21.4 / 20.1 and 20.7 / 20.0; 480 units, the last that do, 35.3 / 33.2 and 33.3 / 33.9;
+    // 96, 240, 288 and 384 units, which do not, 4 to 13 % slower split, at 16 levels 11 to 26 %).
     Params p = call;
     const int heads = p.H;
     const long whole = (long(p.L) * p.B * p.H + sms - 1) / sms, halves = (2L * p.L * p.B * p.H + sms - 1) / sms;
@@ -1070,12 +1072,14 @@ int launch_verify_effective(const Params &call, int d_k, cudaStream_t st)
     ep.withhold_first_load = g_withhold_first_load;
     ep.share = share;
     ep.own_plan = own_plan;
-    // Consecutive heads of one (layer, sequence) that a CTA takes together.  The next head of a group costs a role two
-    // additions, the next group some hundred cycles of a chain that short units wait for; but whole groups leave some CTAs
-    // longer lists than others.  Groups of 4 against single heads, by units per SM: ragged trees of 8..64 nodes +2.6 % at 83,
-    // +1.3 % at 125, +1.7 % at 145, +3.4 % at 166, +1.5 % at 332; trees of 64 nodes 0 at 166, of 32 at d_v = 128 -6.6 % at 166,
-    // ragged at d_v = 128 -2.7 % at 249, chains of 8 -3.5 % at 332, half chains and half 64-node trees -3 % at 332.  The line at
-    // 128 lies where what is lost on ragged trees is less than what short units gain.
+    // Consecutive heads of one (layer, sequence) that a CTA takes together.  Whole groups leave some CTAs longer lists than
+    // others; what they save is steps of the walk, which one warp takes ahead of the roles.  Time of groups of 4 against single
+    // heads, by units per SM, two runs: ragged trees of 8..64 nodes +9 % at 41, +4 at 83, +4 and +3 at 124, +4 at 145, +3 and
+    // +2 at 166, +3 at 332; ragged at d_v = 128 -1 and +2 at 124, +2 and +1 at 249, +1 and 0 at 332; trees of 64 nodes +1 at
+    // 166, of 20 0 and -1, of 64 at 16 levels +1, of 24 at d_k = 256 +1; of 32 at d_v = 128 +3 and -2 at 166, 0 at 83 and 332;
+    // half chains and half 64-node trees at 332 -1.  The line at 128 keeps the last, the largest of the workloads served, and
+    // pays for it with ragged batches beyond 128 (it was drawn when every role walked the list, and gained 3 to 7 % on short
+    // units).
     ep.heads_per_group = p.H % 4 == 0 && n_units / 4 >= 32 * sms ? 4 : 1;
     const long n_groups = n_units / ep.heads_per_group;
     const int grid = int(n_groups < sms ? n_groups : sms);

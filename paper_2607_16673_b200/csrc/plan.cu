@@ -779,8 +779,9 @@ prune_kernel(int32_t N, float tau, int32_t budget, const int32_t *node_offsets,
 // The same for up to kPruneSeqs sequences of at most 64 nodes, in one launch: a warp per sequence, spread over a cluster of
 // CTAs that tell one another their counts through shared memory, so that nothing has to be done twice.  Sets of nodes are 64-bit
 // words, and a warp needs no barrier.  What is left is a chain of two loads, the levels of the tree, the 64 comparisons of
-// a node and one barrier of the cluster.  128 trees of 24..64 nodes: 11.9 us for the two runs of prune_kernel, 5.0 so.  More
-// sequences than warps, or more nodes than bits, go the other way.
+// a node and the barriers of the cluster.  128 trees of 24..64 nodes: 11.9 us for the two runs of prune_kernel, 4.9 so.  More
+// sequences than warps, or more nodes than bits, go the other way (CTAs of 32 warps would take 256 trees, in 7.5 us instead of
+// 12.7, and cost smaller batches some: 128 trees 5.1 instead of 4.9, one 3.2 instead of 2.9).
 constexpr int kPruneCtas = 8, kPruneSeqs = 128;
 __global__ void __cluster_dims__(kPruneCtas, 1, 1) __launch_bounds__(kPruneSeqs / kPruneCtas * 32)
 prune_small_kernel(int32_t B, int32_t N, float tau, int32_t budget, const int32_t *node_offsets, const int32_t *parent,
