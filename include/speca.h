@@ -93,10 +93,11 @@ extern "C" {
  * (d_k = 256).  Everything the tensor core multiplies is split into exact pieces, so outputs carry fp32 accuracy
  * whatever the magnitude of the state.  AUTO uses it whenever it applies and the serial route otherwise; asking for
  * it explicitly outside these shapes is SPECA_ERR_UNSUPPORTED.  Without u both run the effective-query kernel, and AUTO
- * sends small trees to a kernel of their own at the same accuracy: up to 64 nodes at d_k = 64 and up to 32 at the value
- * widths that FACTORIZED does not take (the shortest drafts among these stay with the serial route), elsewhere up to 16
- * at d_k = 128, and in calls of up to four units per multiprocessor 32 at d_k = 128 and 8 at d_k = 256.  The substitution
- * kernel serves the calls that ask for u.
+ * sends small trees to a kernel of their own at the same accuracy (two pieces that lose at most 2^-23 of a value, or what
+ * is less than 2^-23 of the products of its 32 columns): up to 64 nodes at d_k = 64 and up to 32 at the value widths that
+ * FACTORIZED does not take (the shortest drafts among these stay with the serial route), elsewhere up to 16 at d_k = 128,
+ * and in calls of up to four units per multiprocessor 32 at d_k = 128 and 8 at d_k = 256.  The substitution kernel serves
+ * the calls that ask for u.
  * SPECA_ROUTE_TF32 is never picked by AUTO: it reads the fp32 state through a single TF32 pass (10 mantissa
  * bits, truncated), which leaves errors of about 2^-11 of the output's scale, growing with the state; it takes
  * max_depth <= 8 with max_nodes <= 64 (d_k = 128) or <= 32 (d_k = 256), or max_depth <= 16 with max_nodes <=

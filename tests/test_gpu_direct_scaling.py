@@ -99,3 +99,27 @@ def test_results_inside_the_range_stay_inside(d_k, d_v, n, depth, state, query):
     prob.S0 *= np.float32(2.0 ** state)
     prob.q[:] = synth.f32_to_bf16_bits((synth.bf16_bits_to_f32(prob.q) * np.float32(2.0 ** query)).astype(np.float32))
     assert error_norm(prob, n) <= TOL_PRODUCTS
+
+
+@pytest.mark.parametrize("d_k,d_v,n,depth", SHAPES)
+def test_values_of_tiles_that_are_done_again(d_k, d_v, n, depth):
+    """The same large column with values beside the state, and one of these not finite: the nodes that have it on their path are
+    not finite in that row, everything else is right."""
+    rng = np.random.default_rng(n)
+    trees = [synth.random_tree_parent(max(1, m), depth, 4, rng) for m in (n, n - 7)]
+    prob = synth.make_problem(95 + n, 1, 3, d_k, d_v, trees, max_depth=depth, state_std=0.5)
+    for a in (prob.q, prob.k):
+        a[..., 5] = 0
+    prob.S0[..., 5] *= 2.0 ** 40
+    assert error_norm(prob, n) <= TOL_PRODUCTS
+    ref = oracle_verify(prob)
+    node, head, row = n // 2, 1, d_v - 1
+    prob.v[0, node, head, row] = 0x7f80                              # infinity
+    dp = DevProblem(prob, max_nodes=n)
+    dp.verify_tree()
+    assert dp.status_value() == 0
+    o = dp.o.cpu().numpy().astype(np.float64)
+    hit = np.zeros(o.shape, bool)
+    hit[0, [t for t in range(n) if node in synth.root_path(trees[0], t)], head, row] = True
+    assert not np.isfinite(o[hit]).any() and np.isfinite(o[~hit]).all()
+    assert np.linalg.norm(o[~hit] - ref[~hit]) <= TOL_PRODUCTS * np.linalg.norm(ref[~hit])
